@@ -1,4 +1,5 @@
-"""ctypes binding of include/lce.h.  Argument marshalling only."""
+"""Binding of include/lce.h.  Argument marshalling only: ctypes for the calls made while a model is loaded,
+the extension module _lce_host (csrc/host/binding.cpp) for those made per layer."""
 from __future__ import annotations
 
 import ctypes
@@ -29,6 +30,25 @@ class BConv2dDesc(ctypes.Structure):
 
 
 _lib = None
+
+
+class _NotLoaded:
+    """Stands in for the extension module until the first call: loads it and makes that call."""
+
+    def __getattr__(self, name):
+        global _native
+        library()
+        try:
+            from . import _lce_host
+        except ImportError as e:
+            raise ImportError(f"{_LIB_PATH.parent / '_lce_host.so'} cannot be loaded ({e}): run "
+                              "`python -m paper_2011_09398_b200.build` (there is no fallback path)") from e
+        _lce_host.setup(LceError)
+        _native = _lce_host
+        return getattr(_lce_host, name)
+
+
+_native = _NotLoaded()
 
 
 def library() -> ctypes.CDLL:
@@ -122,21 +142,12 @@ def lce_bconv2d_out_shape(desc: BConv2dDesc) -> Tuple[int, int]:
 
 def lce_bitpack(x: torch.Tensor, out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """LceQuantize: fp32 [..., C] -> int32-typed words [..., ceil(C/32)] (bit pattern of uint32)."""
-    C = x.shape[-1]
-    rows = x.numel() // C if C else 0
-    if out is None:
-        out = torch.empty(x.shape[:-1] + (_words(C),), dtype=torch.int32, device=x.device)
-    _check(library().lce_bitpack(_dev(x, torch.float32, "x"), _dev(out, torch.int32, "out"), rows, C, _stream()), "lce_bitpack")
-    return out
+    return _native.bitpack(x, out)
 
 
 def lce_unpack(words: torch.Tensor, channels: int, out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """LceDequantize: words [..., ceil(C/32)] -> fp32 [..., C] of +-1.0."""
-    rows = words.numel() // _words(channels)
-    if out is None:
-        out = torch.empty(words.shape[:-1] + (channels,), dtype=torch.float32, device=words.device)
-    _check(library().lce_unpack(_dev(words, torch.int32, "words"), _dev(out, torch.float32, "out"), rows, channels, _stream()), "lce_unpack")
-    return out
+    return _native.unpack(words, channels, out)
 
 
 def pack_weights(w_ohwi: torch.Tensor) -> torch.Tensor:
@@ -149,52 +160,14 @@ def lce_bconv2d(desc: BConv2dDesc, input: torch.Tensor, weights: torch.Tensor,
                 multiplier: Optional[torch.Tensor] = None, bias: Optional[torch.Tensor] = None,
                 thresholds: Optional[torch.Tensor] = None, out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """LceBConv2d on packed words; allocates `out` with torch when not given."""
-    oh, ow = lce_bconv2d_out_shape(desc)
-    if out is None:
-        if desc.out_type == OUT_FLOAT32:
-            out = torch.empty((desc.batch, oh, ow, desc.out_c), dtype=torch.float32, device=input.device)
-        elif desc.out_type == OUT_BITPACKED:
-            out = torch.empty((desc.batch, oh, ow, _words(desc.out_c)), dtype=torch.int32, device=input.device)
-        else:
-            out = torch.empty((desc.batch, oh, ow, desc.out_c), dtype=torch.int32, device=input.device)
-    expect_in = desc.batch * desc.in_h * desc.in_w * _words(desc.in_c)
-    expect_w = desc.out_c * desc.kernel_h * desc.kernel_w * _words(desc.in_c)
-    if desc.weights_packed:
-        expect_w = lce_bconv2d_packed_weights_bytes(desc) // 4
-    if input.numel() != expect_in or weights.numel() != expect_w:
-        raise ValueError("input / weights size does not match the descriptor")
-    out_dtype = torch.float32 if desc.out_type == OUT_FLOAT32 else torch.int32
-    _check(library().lce_bconv2d(
-        ctypes.byref(desc), _dev(input, torch.int32, "input"), _dev(weights, torch.int32, "weights"),
-        _dev(multiplier, torch.float32, "multiplier") if multiplier is not None else None,
-        _dev(bias, torch.float32, "bias") if bias is not None else None,
-        _dev(thresholds, torch.int32, "thresholds") if thresholds is not None else None,
-        _dev(out, out_dtype, "out"), _stream()), "lce_bconv2d")
-    return out
+    return _native.bconv2d(desc, input, weights, multiplier, bias, thresholds, out)
 
 
 def lce_bconv2d_f32(desc: BConv2dDesc, input: torch.Tensor, weights: torch.Tensor,
                     multiplier: Optional[torch.Tensor] = None, bias: Optional[torch.Tensor] = None,
                     thresholds: Optional[torch.Tensor] = None, out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """LceQuantize + LceBConv2d in one kernel: `input` is the fp32 tensor [batch][in_h][in_w][in_c]."""
-    oh, ow = lce_bconv2d_out_shape(desc)
-    if out is None:
-        last = _words(desc.out_c) if desc.out_type == OUT_BITPACKED else desc.out_c
-        out = torch.empty((desc.batch, oh, ow, last), dtype=torch.float32 if desc.out_type == OUT_FLOAT32 else torch.int32,
-                          device=input.device)
-    expect_w = desc.out_c * desc.kernel_h * desc.kernel_w * _words(desc.in_c)
-    if desc.weights_packed:
-        expect_w = lce_bconv2d_packed_weights_bytes(desc) // 4
-    if input.numel() != desc.batch * desc.in_h * desc.in_w * desc.in_c or weights.numel() != expect_w:
-        raise ValueError("input / weights size does not match the descriptor")
-    out_dtype = torch.float32 if desc.out_type == OUT_FLOAT32 else torch.int32
-    _check(library().lce_bconv2d_f32(
-        ctypes.byref(desc), _dev(input, torch.float32, "input"), _dev(weights, torch.int32, "weights"),
-        _dev(multiplier, torch.float32, "multiplier") if multiplier is not None else None,
-        _dev(bias, torch.float32, "bias") if bias is not None else None,
-        _dev(thresholds, torch.int32, "thresholds") if thresholds is not None else None,
-        _dev(out, out_dtype, "out"), _stream()), "lce_bconv2d_f32")
-    return out
+    return _native.bconv2d_f32(desc, input, weights, multiplier, bias, thresholds, out)
 
 
 class BConv2dPlanInfo(ctypes.Structure):
@@ -241,7 +214,7 @@ def lce_bconv2d_plan_create(desc: BConv2dDesc, input: torch.Tensor, weights: tor
 
 def lce_plan_run(plan: BConv2dPlan) -> torch.Tensor:
     """Launches the planned convolution on torch's current stream; returns the plan's output tensor."""
-    _check(library().lce_plan_run(plan.handle, _stream()), "lce_plan_run")
+    _native.plan_run(plan.handle)
     return plan.out
 
 
@@ -254,12 +227,7 @@ def lce_bconv2d_fused(desc: BConv2dDesc, input, weights, multiplier, bias, resid
                       out_packed=None) -> None:
     """LceBConv2d (float output) with the shortcut add and/or the next LceQuantize fused in; the
     caller supplies whichever of out_float / out_packed it wants."""
-    opt = lambda t, dt, n: _dev(t, dt, n) if t is not None else None
-    _check(library().lce_bconv2d_fused(
-        ctypes.byref(desc), _dev(input, torch.int32, "input"), _dev(weights, torch.int32, "weights"),
-        _dev(multiplier, torch.float32, "multiplier"), _dev(bias, torch.float32, "bias"),
-        opt(residual, torch.float32, "residual"), opt(out_float, torch.float32, "out_float"),
-        opt(out_packed, torch.int32, "out_packed"), _stream()), "lce_bconv2d_fused")
+    _native.bconv2d_fused(desc, input, weights, multiplier, bias, residual, out_float, out_packed)
 
 
 def lce_bconv2d_packed_weights_bytes(desc: BConv2dDesc) -> int:
@@ -292,23 +260,13 @@ def _host(t: Optional[torch.Tensor], dtype, name: str):
 def lce_bconv2d_host(desc: BConv2dDesc, input, weights, multiplier, bias, thresholds, out, workspace: torch.Tensor) -> None:
     """Host-buffer form: all tensors on the host (pinned for asynchronous copies) except `workspace`
     (a CUDA uint8 tensor of at least lce_bconv2d_host_workspace_bytes(desc))."""
-    out_dtype = torch.float32 if desc.out_type == OUT_FLOAT32 else torch.int32
-    _check(library().lce_bconv2d_host(
-        ctypes.byref(desc), _host(input, torch.int32, "input"), _host(weights, torch.int32, "weights"),
-        _host(multiplier, torch.float32, "multiplier"), _host(bias, torch.float32, "bias"),
-        _host(thresholds, torch.int32, "thresholds"), _host(out, out_dtype, "out"),
-        _dev(workspace, torch.uint8, "workspace"), workspace.numel(), _stream()), "lce_bconv2d_host")
+    _native.bconv2d_host(desc, input, weights, multiplier, bias, thresholds, out, workspace)
 
 
 def lce_bconv2d_host_async(desc: BConv2dDesc, input, weights, multiplier, bias, thresholds, out, workspace: torch.Tensor) -> None:
     """lce_bconv2d_host that only enqueues its copies and kernel on the current stream; the caller
     synchronises the stream before touching `out` (or reusing `workspace`)."""
-    out_dtype = torch.float32 if desc.out_type == OUT_FLOAT32 else torch.int32
-    _check(library().lce_bconv2d_host_async(
-        ctypes.byref(desc), _host(input, torch.int32, "input"), _host(weights, torch.int32, "weights"),
-        _host(multiplier, torch.float32, "multiplier"), _host(bias, torch.float32, "bias"),
-        _host(thresholds, torch.int32, "thresholds"), _host(out, out_dtype, "out"),
-        _dev(workspace, torch.uint8, "workspace"), workspace.numel(), _stream()), "lce_bconv2d_host_async")
+    _native.bconv2d_host_async(desc, input, weights, multiplier, bias, thresholds, out, workspace)
 
 
 def lce_bconv2d_host_noalloc_max_bytes() -> int:
@@ -329,30 +287,11 @@ def lce_bconv2d_host_noalloc(desc: BConv2dDesc, input, weights, multiplier, bias
 def lce_bmaxpool(words: torch.Tensor, channels: int, pool=(2, 2), stride=(2, 2), padding=PAD_VALID,
                  out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """LceBMaxPool2d on packed words [N,H,W,ceil(C/32)]."""
-    N, H, W, Cw = words.shape
-    if Cw != _words(channels):
-        raise ValueError("last dimension does not match channels")
-
-    def osz(size, k, s):
-        if padding == PAD_VALID:
-            return (size - k) // s + 1 if size >= k else 0
-        return -(-size // s)
-
-    if out is None:
-        out = torch.empty((N, osz(H, pool[0], stride[0]), osz(W, pool[1], stride[1]), Cw), dtype=torch.int32, device=words.device)
-    _check(library().lce_bmaxpool(_dev(words, torch.int32, "words"), _dev(out, torch.int32, "out"), N, H, W, channels,
-                                  pool[0], pool[1], stride[0], stride[1], padding, _stream()), "lce_bmaxpool")
-    return out
+    return _native.bmaxpool(words, channels, pool[0], pool[1], stride[0], stride[1], padding, out)
 
 
 def lce_add_f32(a: torch.Tensor, b: torch.Tensor, out: Optional[torch.Tensor] = None) -> torch.Tensor:
-    if out is None:
-        out = torch.empty_like(a)
-    if a.numel() != b.numel() or a.numel() != out.numel():
-        raise ValueError("size mismatch")
-    _check(library().lce_add_f32(_dev(a, torch.float32, "a"), _dev(b, torch.float32, "b"), _dev(out, torch.float32, "out"),
-                                 a.numel(), _stream()), "lce_add_f32")
-    return out
+    return _native.add_f32(a, b, out)
 
 
 def lce_device_status() -> int:
