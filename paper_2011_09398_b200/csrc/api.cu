@@ -27,11 +27,13 @@ size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 size_t plain_weight_bytes(const ConvGeom &g) { return round_up((size_t)g.Cout * g.KH * g.KW * g.Cw * 4, 256); }
 
 // A packed-weights buffer = [plain words][operand image of the tiled XOR/POPC kernel][operand image of
-// the tensor-core kernel], each part rounded up to 256 bytes; a part a kernel does not cover is empty.
+// the tensor-core kernel][tile image of the latency kernel], each part rounded up to 256 bytes; a part a kernel
+// does not cover is empty.
 struct WeightViews {
     const uint32_t *plain;
     const uint32_t *tiled;
     const void *tensor;
+    const uint32_t *small;
 };
 
 lce_status weight_views(const lce_bconv2d_desc *desc, const ConvGeom &g, const uint32_t *weights, WeightViews *v)
@@ -39,6 +41,7 @@ lce_status weight_views(const lce_bconv2d_desc *desc, const ConvGeom &g, const u
     v->plain = weights;
     v->tiled = nullptr;
     v->tensor = nullptr;
+    v->small = nullptr;
     if (!desc->weights_packed) return LCE_OK;
     if (!aligned(weights, 256)) return LCE_ERR_ALIGNMENT;
     const char *base = reinterpret_cast<const char *>(weights);
@@ -47,6 +50,8 @@ lce_status weight_views(const lce_bconv2d_desc *desc, const ConvGeom &g, const u
     if (tiled > 0) v->tiled = reinterpret_cast<const uint32_t *>(base + off);
     off += round_up(tiled, 256);
     if (tensor > 0) v->tensor = base + off;
+    off += round_up(tensor, 256);
+    if (small_weight_image_bytes(g) > 0) v->small = reinterpret_cast<const uint32_t *>(base + off);
     return LCE_OK;
 }
 
@@ -73,7 +78,18 @@ bool tensor_preferred(const ConvGeom &g)
     return macs >= (t.weights_resident ? 268435456.0 : 536870912.0);
 }
 
-enum KernelPick { PICK_NONE = 0, PICK_DIRECT, PICK_PATCH, PICK_TILED, PICK_TENSOR };
+// AUTO takes the latency kernel for layers with load-time packed weights below 2^29 binary MACs, as long as its
+// 64-pixel tiles make no more than 600 CTAs.  Measured (us, latency / tiled / tensor-core kernel): one image of
+// 14x14x64 1.7 / 3.1 / 3.9, of 28x28x128 2.4 / 4.2 / 4.1, of 7x7x512 2.9 / 9.3 / 8.9; four images of 14x14x256
+// (2^28.8) 4.3 / 5.2 / 5.2, of 7x7x512 4.2 / 11.6 / 8.6; 64 images of 16x16x64 (2^29.2, 512 CTAs) 5.6 / 4.9 / 4.9;
+// layers of little depth and many outputs are cheaper per output elsewhere: 16 images of 28x28x64, 1x1 to 256
+// (1568 CTAs) 9.0 / 5.4 / 4.6.
+bool small_preferred(const ConvGeom &g)
+{
+    return small_covers(g) && (double)g.M * g.Cout * g.KH * g.KW * g.Cin < 536870912.0 && small_ctas(g) <= 600;
+}
+
+enum KernelPick { PICK_NONE = 0, PICK_DIRECT, PICK_PATCH, PICK_TILED, PICK_TENSOR, PICK_SMALL };
 
 // One place decides which kernel a call gets; lce_bconv2d_plan shows the same decision.
 KernelPick pick_kernel(const lce_bconv2d_desc *desc, const ConvGeom &g, bool have_tensor_image, bool tiled_buffers_ok)
@@ -87,6 +103,7 @@ KernelPick pick_kernel(const lce_bconv2d_desc *desc, const ConvGeom &g, bool hav
             return tiled_buffers_ok && tiled_plan_info(g, &info) == LCE_OK ? PICK_TILED : PICK_NONE;
         default: break;
     }
+    if (desc->weights_packed && small_preferred(g)) return PICK_SMALL;
     if (have_tensor_image && tensor_preferred(g) && tensor_covers(g)) return PICK_TENSOR;
     if (patch_covers(g)) return PICK_PATCH;
     if (tiled_buffers_ok && tiled_plan_info(g, &info) == LCE_OK) return PICK_TILED;
@@ -106,6 +123,7 @@ lce_status dispatch(const lce_bconv2d_desc *desc, const ConvGeom &g, const uint3
         case PICK_PATCH: return launch_bconv_patch(g, input, v.plain, multiplier, bias, thresholds, output, s);
         case PICK_TILED: return launch_bconv_tiled(g, input, v.plain, v.tiled, multiplier, bias, thresholds, output, s);
         case PICK_TENSOR: return launch_bconv_tensor(g, input, v.tensor, multiplier, bias, thresholds, output, s);
+        case PICK_SMALL: return launch_bconv_small(g, input, v.plain, v.small, multiplier, bias, thresholds, output, s);
         default: return LCE_ERR_UNSUPPORTED;
     }
 }
@@ -191,6 +209,7 @@ extern "C" lce_status lce_bconv2d_plan(const lce_bconv2d_desc *desc, lce_bconv2d
     *plan = lce_bconv2d_plan_info{};
     // the decision dispatch() makes, for 16-byte aligned buffers
     const bool have_tensor_image = desc->weights_packed && tensor_weight_image_bytes(g) > 0;
+    TiledPlanInfo info{};
     switch (pick_kernel(desc, g, have_tensor_image, true)) {
         case PICK_DIRECT: plan->kernel = LCE_KERNEL_DIRECT; return LCE_OK;
         case PICK_PATCH: plan->kernel = LCE_KERNEL_TILED; plan->patch = 1; return LCE_OK;
@@ -206,12 +225,13 @@ extern "C" lce_status lce_bconv2d_plan(const lce_bconv2d_desc *desc, lce_bconv2d
             plan->shared_bytes = t.shared_bytes;
             return LCE_OK;
         }
-        case PICK_TILED: break;
+        case PICK_TILED:
+            st = tiled_plan_info(g, &info);
+            if (st != LCE_OK) return st;
+            break;
+        case PICK_SMALL: small_plan_info(g, &info); break;
         default: return LCE_ERR_UNSUPPORTED;
     }
-    TiledPlanInfo info{};
-    st = tiled_plan_info(g, &info);
-    if (st != LCE_OK) return st;
     plan->kernel = LCE_KERNEL_TILED;
     plan->pointwise = info.pointwise;
     plan->warps_per_cta = info.warps_per_cta;
@@ -312,8 +332,10 @@ extern "C" lce_status lce_bconv2d_fused(const lce_bconv2d_desc *desc, const uint
     // the tensor-core kernel fuses the same neighbours when whole 32-channel words and 16-byte rows allow it
     const bool tensor_ok = v.tensor && tensor_covers(g) && (g.Cout & 31) == 0 && aligned(out_float, 16) && aligned(residual, 16);
     if (desc->kernel == LCE_KERNEL_TENSOR && !tensor_ok) return LCE_ERR_UNSUPPORTED;
-    if (tensor_ok && (desc->kernel == LCE_KERNEL_TENSOR || (desc->kernel == LCE_KERNEL_AUTO && tensor_preferred(g))))
+    if (tensor_ok && (desc->kernel == LCE_KERNEL_TENSOR || (desc->kernel == LCE_KERNEL_AUTO && tensor_preferred(g) && !small_preferred(g))))
         return launch_bconv_tensor(g, input, v.tensor, multiplier, bias, nullptr, out_float, s, residual, out_packed);
+    if (v.small && desc->kernel == LCE_KERNEL_AUTO && tiled_weight_image_bytes(g) > 0 && small_preferred(g))
+        return launch_bconv_small(g, input, v.plain, v.small, multiplier, bias, nullptr, out_float, s, residual, out_packed);
     return launch_bconv_tiled(g, input, v.plain, v.tiled, multiplier, bias, nullptr, out_float, s, residual, out_packed);
 }
 
@@ -341,7 +363,8 @@ extern "C" size_t lce_bconv2d_packed_weights_bytes(const lce_bconv2d_desc *desc)
 {
     lce::ConvGeom g;
     if (lce::make_geom(desc, &g) != LCE_OK) return 0;
-    return lce::plain_weight_bytes(g) + lce::round_up(lce::tiled_weight_image_bytes(g), 256) + lce::tensor_weight_image_bytes(g);
+    return lce::plain_weight_bytes(g) + lce::round_up(lce::tiled_weight_image_bytes(g), 256) + lce::round_up(lce::tensor_weight_image_bytes(g), 256) +
+           lce::round_up(lce::small_weight_image_bytes(g), 256);
 }
 
 extern "C" lce_status lce_bconv2d_pack_weights(const lce_bconv2d_desc *desc, const uint32_t *weights, void *packed,
@@ -363,7 +386,12 @@ extern "C" lce_status lce_bconv2d_pack_weights(const lce_bconv2d_desc *desc, con
         if (st != LCE_OK) return st;
     }
     off += round_up(tiled, 256);
-    if (tensor > 0) return launch_pack_weights_tensor(g, weights, static_cast<char *>(packed) + off, s);
+    if (tensor > 0) {
+        st = launch_pack_weights_tensor(g, weights, static_cast<char *>(packed) + off, s);
+        if (st != LCE_OK) return st;
+    }
+    off += round_up(tensor, 256);
+    if (small_weight_image_bytes(g) > 0) return launch_pack_weights_small(g, weights, reinterpret_cast<uint32_t *>(static_cast<char *>(packed) + off), s);
     return LCE_OK;
 }
 

@@ -1351,16 +1351,6 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
     return found;
 }
 
-// floor(n / d) = (n * mul) >> sh for every 0 <= n < 2^31: sh = 31 + ceil(log2 d), mul = floor(2^sh / d) + 1
-// (the excess mul * d - 2^sh is at most d <= 2^(sh - 31), so n * excess < 2^sh)
-void fast_div_constants(uint32_t d, uint32_t *mul, uint32_t *sh)
-{
-    uint32_t l = 0;
-    while ((1ull << l) < d) ++l;
-    *sh = 31 + l;
-    *mul = (uint32_t)(((1ull << (31 + l)) / d) + 1);
-}
-
 template <int EPI>
 lce_status launch_mx(const MxParams &p, dim3 grid, size_t smem, cudaStream_t s)
 {

@@ -66,6 +66,16 @@ inline lce_status make_geom(const lce_bconv2d_desc *d, ConvGeom *g)
 
 inline bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
 
+// floor(n / d) = (n * mul) >> sh for every 0 <= n < 2^31: sh = 31 + ceil(log2 d), mul = floor(2^sh / d) + 1
+// (the excess mul * d - 2^sh is at most d <= 2^(sh - 31), so n * excess < 2^sh)
+inline void fast_div_constants(uint32_t d, uint32_t *mul, uint32_t *sh)
+{
+    uint32_t l = 0;
+    while ((1ull << l) < d) ++l;
+    *sh = 31 + l;
+    *mul = (uint32_t)(((1ull << (31 + l)) / d) + 1);
+}
+
 inline lce_status launch_status()
 {
     return cudaGetLastError() == cudaSuccess ? LCE_OK : LCE_ERR_CUDA;
@@ -109,6 +119,18 @@ lce_status launch_bconv_tiled(const ConvGeom &g, const uint32_t *in, const uint3
 bool patch_covers(const ConvGeom &g);
 lce_status launch_bconv_patch(const ConvGeom &g, const uint32_t *in, const uint32_t *w, const float *mult,
                               const float *bias, const int32_t *thr, void *out, cudaStream_t s);
+// Latency kernel for small layers (any filter, stride and channel count whose tile fits in shared memory).
+// w_image: the part of a packed-weights buffer launch_pack_weights_small wrote, or null to use the plain words.
+// residual / out_packed as for the tiled kernel.
+struct TiledPlanInfo;
+bool small_covers(const ConvGeom &g);
+int64_t small_ctas(const ConvGeom &g);
+void small_plan_info(const ConvGeom &g, TiledPlanInfo *info);
+size_t small_weight_image_bytes(const ConvGeom &g);
+lce_status launch_pack_weights_small(const ConvGeom &g, const uint32_t *w, uint32_t *image, cudaStream_t s);
+lce_status launch_bconv_small(const ConvGeom &g, const uint32_t *in, const uint32_t *w, const uint32_t *w_image, const float *mult,
+                              const float *bias, const int32_t *thr, void *out, cudaStream_t s,
+                              const float *residual = nullptr, uint32_t *out_packed = nullptr);
 // Tensor-core kernel (tcgen05 kind::mxf4 on e2m1 operands): any filter of up to 64 taps, equal strides
 // of 1 or 2, every padding mode; needs the weight image that launch_pack_weights_tensor writes at load
 // time (w_image; null -> LCE_ERR_UNSUPPORTED).  residual / out_packed as for the tiled kernel (float

@@ -41,7 +41,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)
 // The waiting itself is one copy of code shared by all call sites (inlined and unrolled, the loops below were
 // 4 KB per call site and two thirds of the kernel: four roles running side by side then miss the
 // instruction caches all the time).
-__device__ __noinline__ bool mbar_wait_slow(uint64_t *bar, uint32_t parity, uint64_t limit_ns)
+static __device__ __noinline__ bool mbar_wait_slow(uint64_t *bar, uint32_t parity, uint64_t limit_ns)
 {
 #pragma unroll 1
     for (int i = 0; i < 16; ++i)
