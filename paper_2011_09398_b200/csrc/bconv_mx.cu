@@ -83,7 +83,6 @@ constexpr int kOffSlot = 1000;       // TMEM base address; 1004 fills issued, 10
 constexpr int kOffPix = 1024;
 constexpr int kOffTbl = 8192;        // uint2[1024]: operand offsets (A, B; 16-byte units) of the MMAs of a tile
 constexpr int kOffDyn = 16384;      // raw words, weight ring, position buffers
-constexpr int kMaxTblMmas = kMaxTaps * 16;                   // 64 taps x 16 K steps (in_c <= 1024): every shape the kernel covers
 
 enum { BAR_FULL_X0 = 0, BAR_FULL_X3 = 3, BAR_TILE_DONE0, BAR_TILE_DONE3 = BAR_TILE_DONE0 + 3, BAR_FULL_D0, BAR_FULL_D1, BAR_EMPTY_D0, BAR_EMPTY_D1, BAR_DONE, BAR_DONE_B,
        BAR_SCALES, BAR_FULL_W0,
@@ -160,6 +159,11 @@ int *mx_flag_for_launch(cudaStream_t s)
     return arr ? arr + dev : nullptr;
 }
 
+// an advance by a fixed number of grid positions
+struct MxStep {
+    int n, r, c;
+};
+
 struct MxParams {
     const uint32_t *in;
     const uint8_t *wimg;
@@ -174,7 +178,8 @@ struct MxParams {
     int32_t OH, OW, KH, KW, stride, pt, pl, K;
     int32_t Wg, Hg, n_phase;
     uint32_t Wg_mul, Wg_sh, Hg_mul, Hg_sh;                // divisions by Wg, Hg as multiply + shift
-    uint32_t c0_mul, c0_sh, c1_mul, c1_sh;                // ... by the items per phase of a first / later chunk
+    MxStep step_across, step_tile, step_tile_super;       // kLoaders positions; to the next tile of a super-tile, of the next super-tile
+    MxStep step_chunk_first, step_chunk_super;            // from a super-tile's first chunk to its second; from its last one to the next super-tile's first
     int32_t Nt, P;           // tile width; rows of a position buffer per phase and channel word = T * Nt + halo
     int32_t T, halo;         // tiles that share a position buffer; positions a tile reads beyond its own
     int32_t n_tiles, n_super, total_q;
@@ -191,251 +196,230 @@ struct MxParams {
 // n / d for 0 <= n < 2^31 with (mul, sh) from the host: floor(n * mul / 2^sh), exact
 __device__ __forceinline__ int fast_div(int n, uint32_t mul, uint32_t sh) { return (int)(((uint64_t)(uint32_t)n * mul) >> sh); }
 
-// what the loaders need of the geometry, in registers (kernel parameters read inside their loops cost
-// more than the arithmetic)
-struct MxGeo {
-    int N, H, W, Cw, Cw2, Wg, Hg, P, n_phase, stride, pt, pl, pad_zero, cp_words;
-    uint32_t Wg_mul, Wg_sh, Hg_mul, Hg_sh;
-    const uint32_t *in;
+// ---- loaders --------------------------------------------------------------------------------------------
+// A grid position as image, grid row inside the image and grid column; a thread's positions advance by a few
+// fixed numbers of positions (to the next chunk, the next super-tile, its next position of a chunk), so the
+// coordinates are carried along with two compares instead of being divided out of the position every time (two
+// 64-bit multiply-shift divisions per position and one more pair per output column were most of a loader's
+// instructions: a tile of a 64-channel layer took 2550 clocks, its matrix instructions 1320).
+struct MxPos {
+    int n, r, c;
 };
 
-// A chunk of a position buffer: rows lo .. lo + count - 1 (of every phase), which hold the grid positions
-// q0 + lo ..; (mul, sh) divide by count.
-struct MxChunk {
-    int q0, lo, count;
-    uint32_t mul, sh;
-};
+__device__ __forceinline__ void mx_advance(MxPos &a, const MxStep &d, int Wg, int Hg)
+{
+    a.c += d.c;
+    a.r += d.r;
+    a.n += d.n;
+    if (a.c >= Wg) { a.c -= Wg; ++a.r; }
+    if (a.r >= Hg) { a.r -= Hg; ++a.n; }
+}
 
-// What the loader threads keep in registers for the whole kernel (read from the kernel parameters once).
+__device__ __forceinline__ MxPos mx_position(int f, const MxParams &p)
+{
+    MxPos a;
+    const int row = fast_div(f, p.Wg_mul, p.Wg_sh);
+    a.c = f - row * p.Wg;
+    a.n = fast_div(row, p.Hg_mul, p.Hg_sh);
+    a.r = row - a.n * p.Hg;
+    return a;
+}
+
+// What the loader threads keep in registers for the whole kernel (kernel parameters read inside their loops
+// cost more than the arithmetic).
 struct MxLoad {
-    MxGeo geo;
-    int Nt, T, halo, n_tiles, n_super, OH, OW, raw_words, fast_words, n_xbuf, ahead;
-    uint32_t c0_mul, c0_sh, c1_mul, c1_sh;
+    int N, H, W, Cw, Wg, Hg, P, pt, pl, origin;  // origin: the words from pixel (-pt, -pl) to pixel (0, 0)
+    int row_words, image_words;                  // words of an input row and of an image
+    const uint32_t *in;
+    MxStep across;                               // kLoaders positions
 };
 
-// the chunk of tile k of the super-tile that starts at position q0: the first tile brings the halo
-__device__ __forceinline__ MxChunk mx_chunk_of(const MxLoad &l, int q0, int k)
-{
-    MxChunk c;
-    c.q0 = q0;
-    c.lo = k ? k * l.Nt + l.halo : 0;
-    c.count = k ? l.Nt : l.Nt + l.halo;
-    c.mul = k ? l.c1_mul : l.c0_mul;
-    c.sh = k ? l.c1_sh : l.c0_sh;
-    return c;
-}
+// How a position's words are brought in and expanded.  CW: channel words, 0 = any number, read in pieces of
+// cp_words.  FORM: stride 1; stride 2 with its four phases one by one; stride 2 where image width and left pad
+// are even, so that the pixels of the two column phases are neighbours in memory (one copy of 2 CW words).
+enum { MX_S1 = 0, MX_S2 = 1, MX_S2_PAIR = 2 };
 
-// position j of the tile that starts at q0, phase ph -> inside the image? and the pixel's word offset
-__device__ __forceinline__ bool mx_locate(const MxGeo &p, int q0, int ph, int j, int64_t *word_offset)
+template <int CW>
+__device__ __forceinline__ void mx_copy_words(uint32_t *dst, const uint32_t *src, int words, int cp_words, bool ok)
 {
-    const int f = q0 + j;
-    const int r = fast_div(f, p.Wg_mul, p.Wg_sh), c = f - r * p.Wg;
-    const int n = fast_div(r, p.Hg_mul, p.Hg_sh), rr = r - n * p.Hg;
-    const int py = p.stride == 2 ? (ph >> 1) : 0, px = p.stride == 2 ? (ph & 1) : 0;
-    const int y = rr * p.stride + py - p.pt, x = c * p.stride + px - p.pl;
-    const bool ok = n < p.N && (unsigned)y < (unsigned)p.H && (unsigned)x < (unsigned)p.W;
-    *word_offset = ok ? (((int64_t)n * p.H + y) * p.W + x) * p.Cw : 0;
-    return ok;
-}
-
-// packed words of the chunk's positions -> raw[item][Cw] (pad positions: zero words), asynchronously
-__device__ __forceinline__ void mx_prefetch(const MxGeo &p, const MxChunk &c, uint32_t *raw, int ltid)
-{
-    const int items = p.n_phase * c.count;
-    for (int i = ltid; i < items; i += kLoaders) {
-        const int ph = p.n_phase == 1 ? 0 : fast_div(i, c.mul, c.sh), j = i - ph * c.count;
-        int64_t off;
-        const bool ok = mx_locate(p, c.q0 + c.lo, ph, j, &off);
-        const uint32_t *src = p.in + off;
-        uint32_t *dst = raw + (size_t)i * p.Cw;
-        if (p.cp_words == 4) {
-            for (int cw = 0; cw < p.Cw; cw += 4) cp_async_zfill<16>(dst + cw, src + cw, ok);
-        } else if (p.cp_words == 2) {
-            for (int cw = 0; cw < p.Cw; cw += 2) cp_async_zfill<8>(dst + cw, src + cw, ok);
-        } else {
-            for (int cw = 0; cw < p.Cw; ++cw) cp_async_zfill<4>(dst + cw, src + cw, ok);
-        }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-}
-
-// every thread expands the words it prefetched itself (same item mapping): waiting for its own copies is enough
-__device__ __forceinline__ void mx_expand(const MxGeo &p, const MxChunk &c, const uint32_t *raw, uint8_t *X, int ltid)
-{
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    const int items = p.n_phase * c.count;
-    for (int i = ltid; i < items; i += kLoaders) {
-        const int ph = p.n_phase == 1 ? 0 : fast_div(i, c.mul, c.sh), j = i - ph * c.count;
-        bool zero = false;
-        if (p.pad_zero) {
-            int64_t off;
-            zero = !mx_locate(p, c.q0 + c.lo, ph, j, &off);
-        }
-        const uint32_t *src = raw + (size_t)i * p.Cw;
-        uint4 *dst = reinterpret_cast<uint4 *>(X) + (size_t)ph * p.Cw2 * p.P + c.lo + j;
-        for (int cw = 0; cw < p.Cw; ++cw) {
-            uint4 v = mx_expand_word(src[cw]);
-            if (zero) v = make_uint4(0u, 0u, 0u, 0u);
-            dst[(size_t)cw * p.P] = v;
-        }
-    }
-}
-
-// The common cases (no zero-padding, aligned input; stride 1 with 2 / 4 / 8 / 16 channel words, stride 2 with
-// 1 / 2 / 4 / 8) with everything about the words and the phases known at compile time: one asynchronous copy of
-// 4 or 8 bytes or CW / 4 of 16 bytes per position, vector reads of the staged words, no loop or branch per
-// word, the phase of an item by comparison instead of division.
-template <int CW, int NPH>
-__device__ __forceinline__ void mx_fast_item(const MxChunk &c, int i, int *ph, int *j)
-{
-    if (NPH == 1) {
-        *ph = 0;
-        *j = i;
+    if (CW == 1) {
+        cp_async_zfill<4>(dst, src, ok);
+    } else if (CW == 2) {
+        cp_async_zfill<8>(dst, src, ok);
+    } else if (CW > 2) {
+#pragma unroll
+        for (int w = 0; w < CW; w += 4) cp_async_zfill<16>(dst + w, src + w, ok);
+    } else if (cp_words == 4) {
+        for (int w = 0; w < words; w += 4) cp_async_zfill<16>(dst + w, src + w, ok);
+    } else if (cp_words == 2) {
+        for (int w = 0; w < words; w += 2) cp_async_zfill<8>(dst + w, src + w, ok);
     } else {
-        const int h = i >= 2 * c.count ? 2 : 0;
-        const int r = i - h * c.count;
-        const int q = r >= c.count ? 1 : 0;
-        *ph = h + q;
-        *j = r - q * c.count;
+        for (int w = 0; w < words; ++w) cp_async_zfill<4>(dst + w, src + w, ok);
     }
 }
 
-template <int CW, int NPH>
-__device__ __forceinline__ void mx_prefetch_fast(const MxGeo &p, const MxChunk &c, uint32_t *raw, int ltid)
+// packed words of the chunk's `count` positions, of which this thread's first is `a` -> raw (pad positions:
+// zero words), asynchronously; raw holds the phases of a position one after the other
+template <int CW, int FORM>
+__device__ __forceinline__ void mx_prefetch(const MxLoad &l, MxPos a, int count, uint32_t *raw, int ltid, int cp_words)
 {
-    const int items = NPH * c.count;
-    for (int i = ltid; i < items; i += kLoaders) {
-        int ph, j;
-        mx_fast_item<CW, NPH>(c, i, &ph, &j);
-        int64_t off;
-        const bool ok = mx_locate(p, c.q0 + c.lo, ph, j, &off);
-        const uint32_t *src = p.in + off;
-        uint32_t *dst = raw + i * CW;
-        if (CW == 1) {
-            cp_async_zfill<4>(dst, src, ok);
-        } else if (CW == 2) {
-            cp_async_zfill<8>(dst, src, ok);
+    const int cw = CW ? CW : l.Cw;
+    for (int j = ltid; j < count; j += kLoaders) {
+        const bool image = a.n < l.N;
+        if (FORM == MX_S1) {
+            const bool ok = image && (unsigned)(a.r - l.pt) < (unsigned)l.H && (unsigned)(a.c - l.pl) < (unsigned)l.W;
+            const int off = a.n * l.image_words + a.r * l.row_words + a.c * cw - l.origin;
+            mx_copy_words<CW>(raw + j * cw, l.in + (ok ? off : 0), cw, cp_words, ok);
         } else {
+            const int y = 2 * a.r - l.pt, x = 2 * a.c - l.pl;
+            const int off = a.n * l.image_words + 2 * (a.r * l.row_words + a.c * cw) - l.origin;
 #pragma unroll
-            for (int w = 0; w < CW; w += 4) cp_async_zfill<16>(dst + w, src + w, ok);
+            for (int py = 0; py < 2; ++py) {
+                const bool row_ok = image && (unsigned)(y + py) < (unsigned)l.H;
+                uint32_t *dst = raw + (j * 4 + 2 * py) * cw;
+                if (FORM == MX_S2_PAIR) {
+                    const bool ok = row_ok && (unsigned)x < (unsigned)l.W;  // column phase 0; phase 1 is the next pixel, inside with it
+                    mx_copy_words<2 * CW>(dst, l.in + (ok ? off + py * l.row_words : 0), 2 * cw, cp_words, ok);
+                } else {
+#pragma unroll
+                    for (int px = 0; px < 2; ++px) {
+                        const bool ok = row_ok && (unsigned)(x + px) < (unsigned)l.W;
+                        mx_copy_words<CW>(dst + px * cw, l.in + (ok ? off + py * l.row_words + px * cw : 0), cw, cp_words, ok);
+                    }
+                }
+            }
         }
+        mx_advance(a, l.across, l.Wg, l.Hg);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-template <int CW, int NPH>
-__device__ __forceinline__ void mx_expand_fast(const MxGeo &p, const MxChunk &c, const uint32_t *raw, uint8_t *X, int ltid)
+// one phase of a position: cw words from src -> cw chunks of 16 bytes, P positions apart
+template <int CW>
+__device__ __forceinline__ void mx_expand_phase(uint4 *dst, int P, const uint32_t *src, int words, bool zero)
+{
+    if (CW == 0) {
+        for (int k = 0; k < words; ++k) {
+            uint4 v = mx_expand_word(src[k]);
+            if (zero) v = make_uint4(0u, 0u, 0u, 0u);
+            dst[k * P] = v;
+        }
+        return;
+    }
+    uint32_t w[CW ? CW : 1];
+    if (CW == 1) {
+        w[0] = *src;
+    } else if (CW == 2) {
+        const uint2 q = *reinterpret_cast<const uint2 *>(src);
+        w[0] = q.x; w[1] = q.y;
+    } else {
+#pragma unroll
+        for (int k = 0; k < CW; k += 4) {
+            const uint4 q = *reinterpret_cast<const uint4 *>(src + k);
+            w[k] = q.x; w[k + 1] = q.y; w[k + 2] = q.z; w[k + 3] = q.w;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < CW; ++k) {
+        uint4 v = mx_expand_word(w[k]);
+        if (zero) v = make_uint4(0u, 0u, 0u, 0u);
+        dst[k * P] = v;
+    }
+}
+
+// The chunk's words -> e2m1 in the position buffer, from row `lo` on.  Every thread expands the words it
+// prefetched itself (same item mapping): waiting for its own copies is enough.  With zero-padding the positions
+// outside the image become 0.0; `a` is the thread's first position again.
+template <int CW, int FORM>
+__device__ __forceinline__ void mx_expand(const MxLoad &l, MxPos a, int count, const uint32_t *raw, uint4 *X, int plane, int ltid, bool pad_zero)
 {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-    const int items = NPH * c.count;
-    for (int i = ltid; i < items; i += kLoaders) {
-        int ph, j;
-        mx_fast_item<CW, NPH>(c, i, &ph, &j);
-        uint32_t w[CW];
-        if (CW == 1) {
-            w[0] = raw[i];
-        } else if (CW == 2) {
-            const uint2 q = *reinterpret_cast<const uint2 *>(raw + i * 2);
-            w[0] = q.x; w[1] = q.y;
-        } else {
+    const int cw = CW ? CW : l.Cw;
+    for (int j = ltid; j < count; j += kLoaders) {
+        bool zero_y[2] = {false, false}, zero_x[2] = {false, false};
+        if (pad_zero) {
+            const int y = FORM == MX_S1 ? a.r - l.pt : 2 * a.r - l.pt, x = FORM == MX_S1 ? a.c - l.pl : 2 * a.c - l.pl;
 #pragma unroll
-            for (int k = 0; k < CW; k += 4) {
-                const uint4 q = *reinterpret_cast<const uint4 *>(raw + i * CW + k);
-                w[k] = q.x; w[k + 1] = q.y; w[k + 2] = q.z; w[k + 3] = q.w;
+            for (int k = 0; k < (FORM == MX_S1 ? 1 : 2); ++k) {
+                zero_y[k] = a.n >= l.N || (unsigned)(y + k) >= (unsigned)l.H;
+                zero_x[k] = (unsigned)(x + k) >= (unsigned)l.W;
             }
+            mx_advance(a, l.across, l.Wg, l.Hg);
         }
-        uint4 *dst = reinterpret_cast<uint4 *>(X) + (size_t)ph * p.Cw2 * p.P + c.lo + j;
-#pragma unroll
-        for (int k = 0; k < CW; ++k) dst[(size_t)k * p.P] = mx_expand_word(w[k]);
-    }
-}
-
-// Stride 2 with an even image width and an even left pad: the pixels of the column phases 0 and 1 of a grid
-// position are neighbours in memory, so one item is a row phase and a position, one copy of 2 CW words brings
-// both column phases, and the address arithmetic is done once for the two.
-template <int CW>
-__device__ __forceinline__ void mx_prefetch_pair(const MxGeo &p, const MxChunk &c, uint32_t *raw, int ltid)
-{
-    const int items = 2 * c.count;
-    for (int i = ltid; i < items; i += kLoaders) {
-        const int py = i >= c.count ? 1 : 0, j = i - py * c.count;
-        int64_t off;
-        const bool ok = mx_locate(p, c.q0 + c.lo, 2 * py, j, &off);  // column phase 0; phase 1 is the next pixel, inside with it
-        const uint32_t *src = p.in + off;
-        uint32_t *dst = raw + i * 2 * CW;
-        if (CW == 1) {
-            cp_async_zfill<8>(dst, src, ok);
+        if (FORM == MX_S1) {
+            mx_expand_phase<CW>(X + j, l.P, raw + j * cw, cw, zero_y[0] || zero_x[0]);
         } else {
 #pragma unroll
-            for (int w = 0; w < 2 * CW; w += 4) cp_async_zfill<16>(dst + w, src + w, ok);
-        }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-}
-
-template <int CW>
-__device__ __forceinline__ void mx_expand_pair(const MxGeo &p, const MxChunk &c, const uint32_t *raw, uint8_t *X, int ltid)
-{
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    const int items = 2 * c.count;
-    for (int i = ltid; i < items; i += kLoaders) {
-        const int py = i >= c.count ? 1 : 0, j = i - py * c.count;
-        uint32_t w[2 * CW];
-        if (CW == 1) {
-            const uint2 q = *reinterpret_cast<const uint2 *>(raw + i * 2);
-            w[0] = q.x; w[1] = q.y;
-        } else {
-#pragma unroll
-            for (int k = 0; k < 2 * CW; k += 4) {
-                const uint4 q = *reinterpret_cast<const uint4 *>(raw + i * 2 * CW + k);
-                w[k] = q.x; w[k + 1] = q.y; w[k + 2] = q.z; w[k + 3] = q.w;
-            }
-        }
-        uint4 *dst0 = reinterpret_cast<uint4 *>(X) + (size_t)(2 * py) * p.Cw2 * p.P + c.lo + j;  // column phase 0
-        uint4 *dst1 = dst0 + (size_t)p.Cw2 * p.P;                                                 // column phase 1
-#pragma unroll
-        for (int k = 0; k < CW; ++k) {
-            dst0[(size_t)k * p.P] = mx_expand_word(w[k]);
-            dst1[(size_t)k * p.P] = mx_expand_word(w[CW + k]);
+            for (int ph = 0; ph < 4; ++ph)
+                mx_expand_phase<CW>(X + ph * plane + j, l.P, raw + (j * 4 + ph) * cw, cw, zero_y[ph >> 1] || zero_x[ph & 1]);
         }
     }
 }
 
-// which form the loaders use: 0 the general one, else channel words (+ 32 for the stride-2 form, + 64 for the
-// stride-2 form that copies the two column phases together)
-__device__ __forceinline__ int mx_fast_words(const MxGeo &p)
+// which form the loaders use: channel words (0 = any) + 32 * FORM
+__device__ __forceinline__ int mx_form(const MxParams &p)
 {
     const bool words_ok = (p.Cw == 1) || (p.Cw == 2 && p.cp_words >= 2) || ((p.Cw == 4 || p.Cw == 8 || p.Cw == 16) && p.cp_words == 4);
-    if (p.pad_zero || !words_ok) return 0;
-    if (p.n_phase == 1) return p.Cw >= 2 ? p.Cw : 0;
-    const bool pairs = (p.W & 1) == 0 && (p.pl & 1) == 0 && (reinterpret_cast<uintptr_t>(p.in) & 15) == 0 && p.Cw <= 4;
-    return pairs ? 64 + p.Cw : p.Cw == 8 ? 40 : 0;
+    if (p.n_phase == 1) return words_ok && p.Cw >= 2 ? p.Cw : 0;
+    const bool pairs = (p.W & 1) == 0 && (p.pl & 1) == 0 && (reinterpret_cast<uintptr_t>(p.in) & 15) == 0 && words_ok && p.Cw <= 4;
+    return pairs ? 32 * MX_S2_PAIR + p.Cw : words_ok && p.Cw == 8 ? 32 * MX_S2 + 8 : 32 * MX_S2;
 }
 
-__device__ __forceinline__ void mx_prefetch_any(int fw, const MxGeo &p, const MxChunk &c, uint32_t *raw, int ltid)
-{
-    if (fw == 2) mx_prefetch_fast<2, 1>(p, c, raw, ltid);
-    else if (fw == 4) mx_prefetch_fast<4, 1>(p, c, raw, ltid);
-    else if (fw == 8) mx_prefetch_fast<8, 1>(p, c, raw, ltid);
-    else if (fw == 16) mx_prefetch_fast<16, 1>(p, c, raw, ltid);
-    else if (fw == 40) mx_prefetch_fast<8, 4>(p, c, raw, ltid);
-    else if (fw == 65) mx_prefetch_pair<1>(p, c, raw, ltid);
-    else if (fw == 66) mx_prefetch_pair<2>(p, c, raw, ltid);
-    else if (fw == 68) mx_prefetch_pair<4>(p, c, raw, ltid);
-    else mx_prefetch(p, c, raw, ltid);
-}
+#define LCE_MX_FORMS(CALL)                                                                                                       \
+    switch (form) {                                                                                                             \
+        case 2: CALL(2, MX_S1); break;                                                                                          \
+        case 4: CALL(4, MX_S1); break;                                                                                          \
+        case 8: CALL(8, MX_S1); break;                                                                                          \
+        case 16: CALL(16, MX_S1); break;                                                                                        \
+        case 32 * MX_S2 + 8: CALL(8, MX_S2); break;                                                                             \
+        case 32 * MX_S2: CALL(0, MX_S2); break;                                                                                 \
+        case 32 * MX_S2_PAIR + 1: CALL(1, MX_S2_PAIR); break;                                                                   \
+        case 32 * MX_S2_PAIR + 2: CALL(2, MX_S2_PAIR); break;                                                                   \
+        case 32 * MX_S2_PAIR + 4: CALL(4, MX_S2_PAIR); break;                                                                   \
+        default: CALL(0, MX_S1); break;                                                                                         \
+    }
 
-__device__ __forceinline__ void mx_expand_any(int fw, const MxGeo &p, const MxChunk &c, const uint32_t *raw, uint8_t *X, int ltid)
+// The loaders' loop over the CTA's tiles: expand the chunk whose words have arrived, work out which output pixel
+// each of the tile's columns is, hand the tile to the issuer, and only then ask for the words of the next chunk
+// (the tile's MMAs must not wait for loads they do not need).  False when a wait gave up.
+template <int CW, int FORM>
+__device__ __forceinline__ bool mx_load_tiles(const MxParams &p, const MxLoad &l, MxPos stage, uint64_t *bars, uint32_t *raw0, uint8_t *sX0, int32_t *sPix,
+                                              int tid, int first_tile, int tile_step)
 {
-    if (fw == 2) mx_expand_fast<2, 1>(p, c, raw, X, ltid);
-    else if (fw == 4) mx_expand_fast<4, 1>(p, c, raw, X, ltid);
-    else if (fw == 8) mx_expand_fast<8, 1>(p, c, raw, X, ltid);
-    else if (fw == 16) mx_expand_fast<16, 1>(p, c, raw, X, ltid);
-    else if (fw == 40) mx_expand_fast<8, 4>(p, c, raw, X, ltid);
-    else if (fw == 65) mx_expand_pair<1>(p, c, raw, X, ltid);
-    else if (fw == 66) mx_expand_pair<2>(p, c, raw, X, ltid);
-    else if (fw == 68) mx_expand_pair<4>(p, c, raw, X, ltid);
-    else mx_expand(p, c, raw, X, ltid);
+    const int Nt = p.Nt, T = p.T, halo = p.halo, n_tiles = p.n_tiles, n_super = p.n_super, raw_words = p.raw_words, n_xbuf = p.n_xbuf, ahead = p.ahead;
+    const int OH = p.OH, OW = p.OW, plane = p.Cw2 * p.P, cp_words = p.cp_words;
+    const uint32_t x_bytes = (uint32_t)p.x_bytes;
+    const bool pad_zero = p.pad_zero != 0;
+    const MxStep tile_d = p.step_tile, tile_super = p.step_tile_super, chunk_first = p.step_chunk_first, chunk_super = p.step_chunk_super;
+    MxPos pix = mx_position(first_tile * T * Nt + tid, p);  // this thread's column of the tile
+    int it = 0, xbuf = 0;
+    for (int st = first_tile; st < n_super; st += tile_step, xbuf = xbuf + 1 == n_xbuf ? 0 : xbuf + 1) {
+        uint4 *X = reinterpret_cast<uint4 *>(sX0 + xbuf * x_bytes);
+        for (int k = 0; k < T && st * T + k < n_tiles; ++k, ++it) {
+            if (it >= ahead) {
+                // At most `ahead` tiles in front of the finished MMAs: those of tile it - ahead are done (a
+                // ring of four barriers, one commit per tile).  That keeps the arrivals on the four full_x
+                // barriers within one phase of what the issuer has seen, and (the MMAs finish in order; ahead
+                // <= (n_xbuf - 1) * T + 1) it means that the super-tile whose position buffer this chunk
+                // overwrites has been read completely.
+                const int done = it - ahead;
+                if (!mbar_wait_bounded(&bars[BAR_TILE_DONE0 + (done & 3)], (uint32_t)(done >> 2) & 1u)) return false;
+            }
+            mx_expand<CW, FORM>(l, stage, k ? Nt : Nt + halo, raw0 + (it & 1) * raw_words, X + (k ? k * Nt + halo : 0), plane, tid, pad_zero);
+            if (tid < Nt)
+                sPix[(it & (kPixSlots - 1)) * kMaxNt + tid] = pix.n < l.N && pix.r < OH && pix.c < OW ? (pix.n * OH + pix.r) * OW + pix.c : -1;
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            mbar_arrive(&bars[BAR_FULL_X0 + (it & 3)]);
+            const bool more_here = k + 1 < T && st * T + k + 1 < n_tiles;
+            mx_advance(pix, more_here ? tile_d : tile_super, l.Wg, l.Hg);
+            if (more_here || st + tile_step < n_super) {
+                mx_advance(stage, !more_here ? chunk_super : k ? tile_d : chunk_first, l.Wg, l.Hg);
+                mx_prefetch<CW, FORM>(l, stage, more_here ? Nt : Nt + halo, raw0 + ((it + 1) & 1) * raw_words, tid, cp_words);
+            }
+        }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    return true;
 }
 
 // B operand of tap (ky, kx): its phase buffer (stride 2) shifted by the tap's position offset, in 16-byte units
@@ -959,23 +943,23 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
     // The loaders' first prefetch goes out before the CTA-wide barrier of the set-up: it needs the previous
     // kernel's output (hence the dependency wait) and plain shared memory, nothing that is set up above.
     MxLoad ld;
+    MxPos stage{0, 0, 0};
+    int form = 0;
     if (tid < kLoaders) {
-        MxGeo &geo = ld.geo;
-        geo.N = p.N; geo.H = p.H; geo.W = p.W; geo.Cw = p.Cw; geo.Cw2 = p.Cw2; geo.Wg = p.Wg; geo.Hg = p.Hg; geo.P = p.P;
-        geo.n_phase = p.n_phase; geo.stride = p.stride; geo.pt = p.pt; geo.pl = p.pl; geo.pad_zero = p.pad_zero; geo.cp_words = p.cp_words;
-        geo.Wg_mul = p.Wg_mul; geo.Wg_sh = p.Wg_sh; geo.Hg_mul = p.Hg_mul; geo.Hg_sh = p.Hg_sh;
-        geo.in = p.in;
-        ld.Nt = p.Nt; ld.T = p.T; ld.halo = p.halo; ld.n_tiles = p.n_tiles; ld.n_super = p.n_super; ld.OH = p.OH; ld.OW = p.OW;
-        ld.raw_words = p.raw_words; ld.n_xbuf = p.n_xbuf; ld.ahead = p.ahead;
-        ld.c0_mul = p.c0_mul; ld.c0_sh = p.c0_sh; ld.c1_mul = p.c1_mul; ld.c1_sh = p.c1_sh;
-        ld.fast_words = mx_fast_words(geo);
+        ld.N = p.N; ld.H = p.H; ld.W = p.W; ld.Cw = p.Cw; ld.Wg = p.Wg; ld.Hg = p.Hg; ld.P = p.P; ld.pt = p.pt; ld.pl = p.pl;
+        ld.in = p.in;
+        ld.row_words = p.W * p.Cw;
+        ld.image_words = p.H * ld.row_words;
+        ld.origin = p.pt * ld.row_words + p.pl * p.Cw;
+        ld.across = p.step_across;
+        form = mx_form(p);
+        stage = mx_position(first_tile * p.T * p.Nt + tid, p);
         asm volatile("griddepcontrol.wait;" ::: "memory");  // the activations may come from the previous kernel
-        if (first_tile < ld.n_super) {
-            // through the general form where its staging layout is the fast form's too (all but the paired stride-2
-            // form): one more inlined copy of every fast form costs more in code size than it saves here
-            const MxChunk c0 = mx_chunk_of(ld, first_tile * ld.T * ld.Nt, 0);
-            if (ld.fast_words >= 64) mx_prefetch_any(ld.fast_words, geo, c0, raw0, tid);
-            else mx_prefetch(geo, c0, raw0, tid);
+        if (first_tile < p.n_super) {
+            // through the general forms, whose staging layout is everybody's: one more copy of every special form
+            // costs more in code size than it saves here
+            if (p.n_phase == 1) mx_prefetch<0, MX_S1>(ld, stage, p.Nt + p.halo, raw0, tid, p.cp_words);
+            else mx_prefetch<0, MX_S2>(ld, stage, p.Nt + p.halo, raw0, tid, p.cp_words);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1000,44 +984,8 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
     bool ok = true;
     if (tid < kLoaders) {
         // ======================= loaders ==============================================================
-        const MxGeo &geo = ld.geo;
-        const int Nt = ld.Nt, T = ld.T, n_tiles = ld.n_tiles, n_super = ld.n_super, OH = ld.OH, OW = ld.OW, raw_words = ld.raw_words;
-        const size_t x_bytes = (size_t)p.x_bytes;
-        auto chunk_of = [&](int q0, int k) { return mx_chunk_of(ld, q0, k); };
-        const int n_xbuf = ld.n_xbuf, ahead = ld.ahead;
-        int it = 0, xbuf = 0;
-        for (int st = first_tile; st < n_super && ok; st += tile_step, xbuf = xbuf + 1 == n_xbuf ? 0 : xbuf + 1) {
-            const int q0 = st * T * Nt;
-            uint8_t *X = sX0 + xbuf * x_bytes;
-            for (int k = 0; k < T && st * T + k < n_tiles; ++k, ++it) {
-                if (it >= ahead) {
-                    // At most `ahead` tiles in front of the finished MMAs: those of tile it - ahead are done (a
-                    // ring of four barriers, one commit per tile).  That keeps the arrivals on the four full_x
-                    // barriers within one phase of what the issuer has seen, and (the MMAs finish in order; ahead
-                    // <= (n_xbuf - 1) * T + 1) it means that the super-tile whose position buffer this chunk
-                    // overwrites has been read completely.
-                    const int done = it - ahead;
-                    ok = mbar_wait_bounded(&bars[BAR_TILE_DONE0 + (done & 3)], (uint32_t)(done >> 2) & 1u);
-                    if (!ok) break;
-                }
-                mx_expand_any(ld.fast_words, geo, chunk_of(q0, k), raw0 + (it & 1) * raw_words, X, tid);
-                if (tid < Nt) {
-                    const int f = q0 + k * Nt + tid;
-                    const int r = fast_div(f, geo.Wg_mul, geo.Wg_sh), c = f - r * geo.Wg;
-                    const int n = fast_div(r, geo.Hg_mul, geo.Hg_sh), rr = r - n * geo.Hg;
-                    const bool col_ok = n < geo.N && rr < OH && c < OW;
-                    sPix[(it & (kPixSlots - 1)) * kMaxNt + tid] = col_ok ? (n * OH + rr) * OW + c : -1;
-                }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                mbar_arrive(&bars[BAR_FULL_X0 + (it & 3)]);
-                // only now the words of the next chunk: the MMAs of this tile must not wait for loads they do not need
-                const bool more_here = k + 1 < T && st * T + k + 1 < n_tiles;
-                if (more_here || st + tile_step < n_super)
-                    mx_prefetch_any(ld.fast_words, geo, more_here ? chunk_of(q0, k + 1) : chunk_of((st + tile_step) * T * Nt, 0),
-                                    raw0 + ((it + 1) & 1) * raw_words, tid);
-            }
-        }
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
+#define LCE_MX_LOAD(CW, FORM) ok = mx_load_tiles<CW, FORM>(p, ld, stage, bars, raw0, sX0, sPix, tid, first_tile, tile_step)
+        LCE_MX_FORMS(LCE_MX_LOAD)
     } else if (tid < kLoaders + kFinishers) {
         // ======================= finishers ============================================================
         const int fw = warp - kLoaders / 32;  // 0..15: lane quarter fw & 3 (= warp & 3), column group fw >> 2
@@ -1325,7 +1273,7 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
             // per tap (wait for the stage, issue, hand the stage back: about 600 clocks on top of the MMAs;
             // measured on a nine-tap, one-MMA-per-tap layer: 6000 clocks per tile whether 2 or 4 stages)
             const double stream = resident ? 0.0 : (double)groups * fmax(fmax(group_taps * pl->tap_bytes / 19.0, 1300.0 / stages), 600.0 + group_taps * ksteps * mma1);
-            // stride 2: four phases per position, staged two at a time where the geometry allows (mx_prefetch_pair)
+            // stride 2: four phases per position, staged two at a time where the geometry allows (MX_S2_PAIR)
             const double per_position = s == 1 ? 1.0 : ((g.W & 1) == 0 && (g.pl & 1) == 0 && g.Cw <= 4) ? 2.0 : 3.0;
             const double load = 400.0 + 8.0 * per_position * (nt + (double)halo / T);
             const double cost = per_cta * (fmax(fmax(mma, stream), load) + 150.0);
@@ -1440,8 +1388,16 @@ lce_status launch_bconv_tensor(const ConvGeom &g, const uint32_t *in, const void
     p.Wg = pl.Wg; p.Hg = pl.Hg; p.n_phase = pl.n_phase;
     fast_div_constants((uint32_t)pl.Wg, &p.Wg_mul, &p.Wg_sh);
     fast_div_constants((uint32_t)pl.Hg, &p.Hg_mul, &p.Hg_sh);
-    fast_div_constants((uint32_t)(pl.Nt + pl.halo), &p.c0_mul, &p.c0_sh);
-    fast_div_constants((uint32_t)pl.Nt, &p.c1_mul, &p.c1_sh);
+    const auto step = [&](int64_t positions) {
+        const int64_t rows = positions / pl.Wg;
+        return MxStep{(int)(rows / pl.Hg), (int)(rows % pl.Hg), (int)(positions % pl.Wg)};
+    };
+    const int64_t last_chunk = pl.T > 1 ? (int64_t)(pl.T - 1) * pl.Nt + pl.halo : 0, super_step = (int64_t)pl.ctas_x * pl.T * pl.Nt;
+    p.step_across = step(kLoaders);
+    p.step_tile = step(pl.Nt);
+    p.step_tile_super = step(super_step - (int64_t)(pl.T - 1) * pl.Nt);
+    p.step_chunk_first = step(pl.Nt + pl.halo);
+    p.step_chunk_super = step(super_step - last_chunk);
     p.Nt = pl.Nt; p.P = pl.P; p.T = pl.T; p.halo = pl.halo; p.n_tiles = pl.n_tiles; p.n_super = pl.n_super; p.total_q = pl.total_q;
     p.taps = pl.taps; p.ksteps = pl.Cw2 / 2; p.stages = pl.stages; p.resident = pl.resident; p.group_taps = pl.group_taps; p.groups = pl.groups;
     p.tap_bytes = (int32_t)pl.tap_bytes; p.raw_words = (int32_t)pl.raw_words; p.x_bytes = (int32_t)pl.x_bytes;
