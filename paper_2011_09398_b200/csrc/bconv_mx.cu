@@ -81,8 +81,7 @@ constexpr int kOffSlot = 1000;       // TMEM base address; 1004 fills issued, 10
 // accumulator back before they have stored its values, so the loaders can be up to four tiles ahead
 // of a finisher that still reads its tile's slot (tile t + 5 cannot be staged before finisher t is done).
 constexpr int kOffPix = 1024;
-constexpr int kOffTbl = 8192;        // uint2[1024]: operand offsets (A, B; 16-byte units) of the MMAs of a tile
-constexpr int kOffDyn = 16384;      // raw words, weight ring, position buffers
+constexpr int kOffDyn = 8192;       // raw words, uint2[MMAs of a tile]: operand offsets (A, B; 16-byte units), weight ring, position buffers
 
 enum { BAR_FULL_X0 = 0, BAR_FULL_X3 = 3, BAR_TILE_DONE0, BAR_TILE_DONE3 = BAR_TILE_DONE0 + 3, BAR_FULL_D0, BAR_FULL_D1, BAR_EMPTY_D0, BAR_EMPTY_D1, BAR_DONE, BAR_DONE_B,
        BAR_SCALES, BAR_FULL_W0,
@@ -187,7 +186,7 @@ struct MxParams {
     int32_t group_taps, groups;  // streamed weights: taps per ring stage, stages' worth of taps per tile = ceil(taps / group_taps)
     int32_t tap_bytes, raw_words, x_bytes;
     int32_t n_xbuf, ahead;   // position buffers (2..4); tiles the loaders may be ahead of the finished MMAs (2..4)
-    int32_t off_w, off_x;    // byte offsets in shared memory
+    int32_t off_tbl, off_w, off_x;    // byte offsets in shared memory
     int32_t cp_words;        // words per cp.async: 4, 2 or 1
     int32_t pad_zero, out_type, activation, write_float;
     int32_t dup_log2;        // log2 of the copies of the channel block in the 128 rows: 1 for out_c <= 64, 2 for out_c <= 32, else 0
@@ -872,7 +871,6 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + kOffSlot);
     int32_t *fills = reinterpret_cast<int32_t *>(smem + kOffSlot + 4);  // [0] issued by the producer, [1] consumed by the issuer
     int32_t *sPix = reinterpret_cast<int32_t *>(smem + kOffPix);
-    uint2 *tbl = reinterpret_cast<uint2 *>(smem + kOffTbl);
     uint32_t *raw0 = reinterpret_cast<uint32_t *>(smem + kOffDyn);
     uint8_t *sW = smem + p.off_w;
     uint8_t *sX0 = smem + p.off_x;
@@ -932,6 +930,7 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
             fills[1] = 0;
         }
     } else if (tid >= kLoaders) {
+        uint2 *tbl = reinterpret_cast<uint2 *>(smem + p.off_tbl);
         for (int e = tid - kLoaders; e < n_mma; e += kFinishers) {
             const int tap = e / p.ksteps, kk = e - tap * p.ksteps;
             const int ky = tap / p.KW, kx = tap - ky * p.KW;
@@ -1016,6 +1015,7 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
         // two take alternate tiles (one accumulator buffer each), so that one warp's per-tile bookkeeping and
         // waits run while the other's MMAs are in the pipe.
         const int my_parity = warp - kIssuerWarp;
+        const uint2 *tbl = reinterpret_cast<const uint2 *>(smem + p.off_tbl);
         // instruction descriptor (block-scaled kinds): A, B = e2m1 (1), both K-major, N >> 3 at bit 17,
         // scales ue8m0 (bit 23), M >> 4 at bit 24, scale-factor ids 0
         const uint32_t idesc = (1u << 7) | (1u << 10) | ((uint32_t)(p.Nt >> 3) << 17) | (1u << 23) | ((uint32_t)(128 >> 4) << 24);
@@ -1166,7 +1166,7 @@ __global__ void mx_pack_weights_kernel(const uint32_t *w, uint4 *image, int Cout
 
 struct MxPlan {
     int Nt, P, T, stages, resident, group_taps, groups, n_blocks, ctas_x, n_tiles, n_super, total_q, Wg, Hg, n_phase, Cw2, taps, halo, n_xbuf, ahead;
-    size_t raw_words, x_bytes, tap_bytes, off_w, off_x, smem;
+    size_t raw_words, x_bytes, tap_bytes, off_tbl, off_w, off_x, smem;
 };
 
 constexpr size_t kSmemLimit = 227 * 1024;
@@ -1243,7 +1243,8 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
             if (T > 1 && (T - 1) * ctas_max >= n_tiles) break;   // no CTA would have that many tiles
             const size_t raw_words = (((size_t)pl->n_phase * (nt + halo) * g.Cw + 3) / 4) * 4;
             const size_t x_bytes = (size_t)pl->n_phase * pl->Cw2 * P * 16;
-            const size_t fixed = kOffDyn + 2 * raw_words * 4;
+            const size_t off_tbl = kOffDyn + 2 * raw_words * 4;
+            const size_t fixed = off_tbl + (size_t)taps * ksteps * 8;  // the table no longer than it is: at 512 channels 3x3 the 8 KB saved are a wider tile
             const size_t off_w = (fixed + 127) / 128 * 128;
             const size_t rest = 2 * x_bytes + 256;
             if (off_w + rest + (taps > 1 ? 2 : 1) * pl->tap_bytes > kSmemLimit) break;
@@ -1268,11 +1269,10 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
             // position and tile
             const double mma1 = fmax(100.0, 43.0 + nt / 2.0);
             const double mma = (double)taps * ksteps * mma1;
-            // a streamed tap: its bytes from L2 (every SM streams at once: the L2 gives each about 19 bytes per clock,
-            // 5.5 TB/s in all), or its share of a copy's latency, or what the single issuer needs
+            // a streamed group: its bytes from L2 (with all SMs streaming at least 38 bytes per clock each), or its share of a copy's latency, or what the single issuer needs
             // per tap (wait for the stage, issue, hand the stage back: about 600 clocks on top of the MMAs;
             // measured on a nine-tap, one-MMA-per-tap layer: 6000 clocks per tile whether 2 or 4 stages)
-            const double stream = resident ? 0.0 : (double)groups * fmax(fmax(group_taps * pl->tap_bytes / 19.0, 1300.0 / stages), 600.0 + group_taps * ksteps * mma1);
+            const double stream = resident ? 0.0 : (double)groups * fmax(fmax(group_taps * pl->tap_bytes / 38.0, 1300.0 / stages), 600.0 + group_taps * ksteps * mma1);
             // stride 2: four phases per position, staged two at a time where the geometry allows (MX_S2_PAIR)
             const double per_position = s == 1 ? 1.0 : ((g.W & 1) == 0 && (g.pl & 1) == 0 && g.Cw <= 4) ? 2.0 : 3.0;
             const double load = 400.0 + 8.0 * per_position * (nt + (double)halo / T);
@@ -1283,6 +1283,7 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
                 pl->Nt = nt; pl->P = P; pl->T = T; pl->stages = stages; pl->resident = resident ? 1 : 0; pl->group_taps = group_taps; pl->groups = groups;
                 pl->n_tiles = n_tiles; pl->n_super = n_super; pl->ctas_x = ctas_x;
                 pl->raw_words = raw_words; pl->x_bytes = x_bytes;
+                pl->off_tbl = off_tbl;
                 pl->off_w = off_w;
                 pl->off_x = (off_w + (size_t)stages * group_taps * pl->tap_bytes + 127) / 128 * 128;
                 // More position buffers where shared memory is left over (thin layers): the loaders may then be
@@ -1402,7 +1403,7 @@ lce_status launch_bconv_tensor(const ConvGeom &g, const uint32_t *in, const void
     p.taps = pl.taps; p.ksteps = pl.Cw2 / 2; p.stages = pl.stages; p.resident = pl.resident; p.group_taps = pl.group_taps; p.groups = pl.groups;
     p.tap_bytes = (int32_t)pl.tap_bytes; p.raw_words = (int32_t)pl.raw_words; p.x_bytes = (int32_t)pl.x_bytes;
     p.n_xbuf = pl.n_xbuf; p.ahead = pl.ahead;
-    p.off_w = (int32_t)pl.off_w; p.off_x = (int32_t)pl.off_x;
+    p.off_tbl = (int32_t)pl.off_tbl; p.off_w = (int32_t)pl.off_w; p.off_x = (int32_t)pl.off_x;
     p.cp_words = (g.Cw % 4 == 0 && aligned(in, 16)) ? 4 : (g.Cw % 2 == 0 && aligned(in, 8)) ? 2 : 1;
     p.pad_zero = g.padding == LCE_PAD_SAME_ZERO;
     p.out_type = g.out_type; p.activation = g.activation;
