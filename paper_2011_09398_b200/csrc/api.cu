@@ -2,24 +2,30 @@
 // host-buffer forms).  All argument checks happen here, before anything is launched.
 #include "common.cuh"
 
+#include <string.h>
+
 #include <atomic>
+#include <memory>
 #include <new>
 
 namespace lce {
 namespace {
 
-lce_status check_conv_args(const lce_bconv2d_desc *desc, ConvGeom *g, const void *input, const void *weights,
-                           const void *multiplier, const void *bias, const void *thresholds, const void *output)
+lce_status check_conv_buffers(const ConvGeom &g, const void *input, const void *weights, const void *multiplier, const void *bias,
+                              const void *thresholds, const void *output)
 {
-    lce_status st = make_geom(desc, g);
-    if (st != LCE_OK) return st;
     if (!input || !weights || !output) return LCE_ERR_INVALID_ARG;
-    if (g->out_type == LCE_OUT_FLOAT32 && (!multiplier || !bias)) return LCE_ERR_INVALID_ARG;
-    if (g->out_type == LCE_OUT_BITPACKED) {
+    if (g.out_type == LCE_OUT_FLOAT32 && (!multiplier || !bias)) return LCE_ERR_INVALID_ARG;
+    if (g.out_type == LCE_OUT_BITPACKED) {
         if (!thresholds) return LCE_ERR_INVALID_ARG;
-        if (g->activation != LCE_ACT_NONE) return LCE_ERR_INVALID_ARG;
+        if (g.activation != LCE_ACT_NONE) return LCE_ERR_INVALID_ARG;
     }
     return LCE_OK;
+}
+
+bool conv_buffers_aligned(const void *input, const void *weights, const void *multiplier, const void *bias, const void *thresholds, const void *output)
+{
+    return aligned(input, 4) && aligned(weights, 4) && aligned(output, 4) && aligned(multiplier, 4) && aligned(bias, 4) && aligned(thresholds, 4);
 }
 
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -29,37 +35,22 @@ size_t plain_weight_bytes(const ConvGeom &g) { return round_up((size_t)g.Cout * 
 // A packed-weights buffer = [plain words][operand image of the tiled XOR/POPC kernel][operand image of
 // the tensor-core kernel][tile image of the latency kernel], each part rounded up to 256 bytes; a part a kernel
 // does not cover is empty.
-struct WeightViews {
-    const uint32_t *plain;
-    const uint32_t *tiled;
-    const void *tensor;
-    const uint32_t *small;
+struct WeightParts {
+    size_t tiled, tensor, small, total;  // byte offsets; 0: no such part
 };
 
-lce_status weight_views(const lce_bconv2d_desc *desc, const ConvGeom &g, const uint32_t *weights, WeightViews *v)
+WeightParts weight_parts(const ConvGeom &g)
 {
-    v->plain = weights;
-    v->tiled = nullptr;
-    v->tensor = nullptr;
-    v->small = nullptr;
-    if (!desc->weights_packed) return LCE_OK;
-    if (!aligned(weights, 256)) return LCE_ERR_ALIGNMENT;
-    const char *base = reinterpret_cast<const char *>(weights);
+    WeightParts w{};
     size_t off = plain_weight_bytes(g);
-    const size_t tiled = tiled_weight_image_bytes(g), tensor = tensor_weight_image_bytes(g);
-    if (tiled > 0) v->tiled = reinterpret_cast<const uint32_t *>(base + off);
+    const size_t tiled = tiled_weight_image_bytes(g), tensor = tensor_weight_image_bytes(g), small = small_weight_image_bytes(g);
+    if (tiled > 0) w.tiled = off;
     off += round_up(tiled, 256);
-    if (tensor > 0) v->tensor = base + off;
+    if (tensor > 0) w.tensor = off;
     off += round_up(tensor, 256);
-    if (small_weight_image_bytes(g) > 0) v->small = reinterpret_cast<const uint32_t *>(base + off);
-    return LCE_OK;
-}
-
-// The tiled kernels write float / int32 rows with 128-bit accesses when the channel count allows it,
-// and then need 16-byte aligned buffers.
-bool tiled_accepts(const ConvGeom &g, const void *out, const void *residual)
-{
-    return !((g.Cout & 3) == 0 && g.out_type != LCE_OUT_BITPACKED && (!aligned(out, 16) || !aligned(residual, 16)));
+    if (small > 0) w.small = off;
+    w.total = off + round_up(small, 256);
+    return w;
 }
 
 // AUTO takes the tensor-core kernel when the weights were packed at load time (its operand image exists)
@@ -92,6 +83,8 @@ bool small_preferred(const ConvGeom &g)
 enum KernelPick { PICK_NONE = 0, PICK_DIRECT, PICK_PATCH, PICK_TILED, PICK_TENSOR, PICK_SMALL };
 
 // One place decides which kernel a call gets; lce_bconv2d_plan shows the same decision.
+// tiled_buffers_ok: the tiled kernels write float / int32 rows with 128-bit accesses when the channel count allows it,
+// and then need 16-byte aligned buffers.
 KernelPick pick_kernel(const lce_bconv2d_desc *desc, const ConvGeom &g, bool have_tensor_image, bool tiled_buffers_ok)
 {
     TiledPlanInfo info{};
@@ -110,20 +103,94 @@ KernelPick pick_kernel(const lce_bconv2d_desc *desc, const ConvGeom &g, bool hav
     return PICK_DIRECT;
 }
 
-lce_status dispatch(const lce_bconv2d_desc *desc, const ConvGeom &g, const uint32_t *input, const uint32_t *weights,
-                    const float *multiplier, const float *bias, const int32_t *thresholds, void *output,
-                    cudaStream_t s)
+// The fused form (shortcut, re-quantised copy): the shapes the tiled kernels cover; the tensor-core kernel wants whole
+// 32-channel words and 16-byte rows.
+KernelPick pick_fused(const lce_bconv2d_desc *desc, const ConvGeom &g, const WeightParts &parts, bool rows_aligned)
+{
+    if (desc->kernel == LCE_KERNEL_DIRECT || patch_covers(g)) return PICK_NONE;
+    const bool tensor_ok = desc->weights_packed && parts.tensor && tensor_covers(g) && (g.Cout & 31) == 0 && rows_aligned;
+    if (desc->kernel == LCE_KERNEL_TENSOR) return tensor_ok ? PICK_TENSOR : PICK_NONE;
+    if (desc->kernel == LCE_KERNEL_AUTO && desc->weights_packed && tiled_weight_image_bytes(g) > 0 && small_preferred(g)) return PICK_SMALL;
+    if (desc->kernel == LCE_KERNEL_AUTO && tensor_ok && tensor_preferred(g)) return PICK_TENSOR;
+    return PICK_TILED;
+}
+
+// Everything about a call that follows from its descriptor: geometry, parts of the packed weights, which kernel and
+// the launch worked out for it.
+struct Prepared {
+    lce_bconv2d_desc desc;
+    int device;
+    uint32_t form;      // FORM_*: what else the choice depends on
+    lce_status status;
+    ConvGeom g;
+    WeightParts parts;
+    KernelPick pick;
+    PreparedLaunch launch;
+};
+enum { FORM_FUSED = 1, FORM_ROWS_UNALIGNED = 2 };  // float / int32 rows that are not on 16 bytes (relevant for out_c % 4 == 0)
+
+void prepare(const lce_bconv2d_desc *desc, int device, uint32_t form, Prepared *p)
+{
+    p->desc = *desc;
+    p->device = device;
+    p->form = form;
+    p->status = make_geom(desc, &p->g);
+    if (p->status != LCE_OK) return;
+    p->parts = weight_parts(p->g);
+    const bool rows_aligned = !(form & FORM_ROWS_UNALIGNED);
+    p->pick = form & FORM_FUSED ? pick_fused(desc, p->g, p->parts, rows_aligned) : pick_kernel(desc, p->g, desc->weights_packed && p->parts.tensor, rows_aligned);
+    if (p->pick == PICK_SMALL) p->status = prepare_bconv_small(p->g, &p->launch);
+    if (p->pick == PICK_TENSOR) p->status = prepare_bconv_tensor(p->g, &p->launch);
+}
+
+// A network repeats few descriptors: the last ones of each host thread are kept.  Working a call out costs 1 - 2 us of
+// host time, against 2.4 us for the launch itself.
+const Prepared &prepared_for(const lce_bconv2d_desc *desc, uint32_t form)
+{
+    constexpr int kSlots = 64, kWays = 4;
+    struct Cache {
+        Prepared slots[kSlots] = {};
+        bool used[kSlots] = {};
+        uint32_t turn = 0;
+    };
+    static thread_local std::unique_ptr<Cache> cache;
+    if (!cache) cache.reset(new Cache);
+    int device = -1;
+    if (cudaGetDevice(&device) != cudaSuccess) device = -1;
+    uint32_t hash = form * 2654435761u;
+    int32_t fields[sizeof(lce_bconv2d_desc) / 4];
+    memcpy(fields, desc, sizeof(fields));
+    for (int32_t f : fields) hash = (hash ^ (uint32_t)f) * 16777619u;
+    const uint32_t base = (hash >> 16) % (kSlots / kWays) * kWays;
+    for (uint32_t i = base; i < base + kWays; ++i) {
+        const Prepared &p = cache->slots[i];
+        if (cache->used[i] && p.device == device && p.form == form && memcmp(&p.desc, desc, sizeof(*desc)) == 0) return p;
+    }
+    const uint32_t i = base + cache->turn++ % kWays;
+    prepare(desc, device, form, &cache->slots[i]);
+    cache->used[i] = true;
+    return cache->slots[i];
+}
+
+uint32_t rows_form(const lce_bconv2d_desc *desc, const void *out, const void *residual)
+{
+    const bool wide_rows = (desc->out_c & 3) == 0 && desc->out_type != LCE_OUT_BITPACKED;
+    return wide_rows && (!aligned(out, 16) || !aligned(residual, 16)) ? FORM_ROWS_UNALIGNED : 0;
+}
+
+lce_status dispatch(const Prepared &p, const uint32_t *input, const uint32_t *weights, const float *multiplier, const float *bias,
+                    const int32_t *thresholds, void *output, cudaStream_t s, const float *residual = nullptr, uint32_t *out_packed = nullptr)
 {
     if (tensor_timeout_flagged()) return LCE_ERR_DEVICE_TIMEOUT;  // an earlier kernel on this device gave up a wait
-    WeightViews v;
-    lce_status st = weight_views(desc, g, weights, &v);
-    if (st != LCE_OK) return st;
-    switch (pick_kernel(desc, g, v.tensor != nullptr, tiled_accepts(g, output, nullptr))) {
-        case PICK_DIRECT: return launch_bconv_direct(g, input, v.plain, multiplier, bias, thresholds, output, s);
-        case PICK_PATCH: return launch_bconv_patch(g, input, v.plain, multiplier, bias, thresholds, output, s);
-        case PICK_TILED: return launch_bconv_tiled(g, input, v.plain, v.tiled, multiplier, bias, thresholds, output, s);
-        case PICK_TENSOR: return launch_bconv_tensor(g, input, v.tensor, multiplier, bias, thresholds, output, s);
-        case PICK_SMALL: return launch_bconv_small(g, input, v.plain, v.small, multiplier, bias, thresholds, output, s);
+    const bool packed = p.desc.weights_packed != 0;
+    if (packed && !aligned(weights, 256)) return LCE_ERR_ALIGNMENT;
+    const auto part = [&](size_t off) { return packed && off ? reinterpret_cast<const uint32_t *>(reinterpret_cast<const char *>(weights) + off) : nullptr; };
+    switch (p.pick) {
+        case PICK_DIRECT: return launch_bconv_direct(p.g, input, weights, multiplier, bias, thresholds, output, s);
+        case PICK_PATCH: return launch_bconv_patch(p.g, input, weights, multiplier, bias, thresholds, output, s);
+        case PICK_TILED: return launch_bconv_tiled(p.g, input, weights, part(p.parts.tiled), multiplier, bias, thresholds, output, s, residual, out_packed);
+        case PICK_TENSOR: return launch_bconv_tensor(p.launch, input, part(p.parts.tensor), multiplier, bias, thresholds, output, s, residual, out_packed);
+        case PICK_SMALL: return launch_bconv_small(p.launch, input, weights, part(p.parts.small), multiplier, bias, thresholds, output, s, residual, out_packed);
         default: return LCE_ERR_UNSUPPORTED;
     }
 }
@@ -250,20 +317,18 @@ extern "C" lce_status lce_bconv2d(const lce_bconv2d_desc *desc, const uint32_t *
                                   void *output, void *stream)
 {
     using namespace lce;
-    ConvGeom g;
-    lce_status st = check_conv_args(desc, &g, input, weights, multiplier, bias, thresholds, output);
+    if (!desc) return LCE_ERR_INVALID_ARG;
+    const Prepared &p = prepared_for(desc, rows_form(desc, output, nullptr));
+    if (p.status != LCE_OK) return p.status;
+    const lce_status st = check_conv_buffers(p.g, input, weights, multiplier, bias, thresholds, output);
     if (st != LCE_OK) return st;
-    if (!aligned(input, 4) || !aligned(weights, 4) || !aligned(output, 4) ||
-        (multiplier && !aligned(multiplier, 4)) || (bias && !aligned(bias, 4)) ||
-        (thresholds && !aligned(thresholds, 4)))
-        return LCE_ERR_ALIGNMENT;
-    return dispatch(desc, g, input, weights, multiplier, bias, thresholds, output, static_cast<cudaStream_t>(stream));
+    if (!conv_buffers_aligned(input, weights, multiplier, bias, thresholds, output)) return LCE_ERR_ALIGNMENT;
+    return dispatch(p, input, weights, multiplier, bias, thresholds, output, static_cast<cudaStream_t>(stream));
 }
 
 // ---- plan objects: the checks of lce_bconv2d once, the launch many times ---------------------------
 struct lce_plan {
-    lce_bconv2d_desc desc;
-    lce::ConvGeom geom;
+    lce::Prepared prepared;
     const uint32_t *input, *weights;
     const float *multiplier, *bias;
     const int32_t *thresholds;
@@ -277,24 +342,20 @@ extern "C" lce_status lce_bconv2d_plan_create(const lce_bconv2d_desc *desc, cons
     using namespace lce;
     if (!plan) return LCE_ERR_INVALID_ARG;
     *plan = nullptr;
-    ConvGeom g;
-    lce_status st = check_conv_args(desc, &g, input, weights, multiplier, bias, thresholds, output);
+    if (!desc) return LCE_ERR_INVALID_ARG;
+    const Prepared &p = prepared_for(desc, rows_form(desc, output, nullptr));
+    if (p.status != LCE_OK) return p.status;
+    const lce_status st = check_conv_buffers(p.g, input, weights, multiplier, bias, thresholds, output);
     if (st != LCE_OK) return st;
-    if (!aligned(input, 4) || !aligned(weights, 4) || !aligned(output, 4) ||
-        (multiplier && !aligned(multiplier, 4)) || (bias && !aligned(bias, 4)) ||
-        (thresholds && !aligned(thresholds, 4)))
-        return LCE_ERR_ALIGNMENT;
+    if (!conv_buffers_aligned(input, weights, multiplier, bias, thresholds, output)) return LCE_ERR_ALIGNMENT;
     // is there a kernel for this shape, these buffers and a forced kernel choice?  (A float / int32 output
-    // that is only 4-byte aligned rules the tiled kernel out: AUTO then records the direct kernel, a
+    // that is only 4-byte aligned rules the tiled kernel out: AUTO then records another kernel, a
     // forced LCE_KERNEL_TILED fails here rather than at every run.)
-    WeightViews v;
-    st = weight_views(desc, g, weights, &v);
-    if (st != LCE_OK) return st;
-    if (pick_kernel(desc, g, v.tensor != nullptr, tiled_accepts(g, output, nullptr)) == PICK_NONE) return LCE_ERR_UNSUPPORTED;
+    if (desc->weights_packed && !aligned(weights, 256)) return LCE_ERR_ALIGNMENT;
+    if (p.pick == PICK_NONE) return LCE_ERR_UNSUPPORTED;
     lce_plan *h = new (std::nothrow) lce_plan;
     if (!h) return LCE_ERR_CUDA;
-    h->desc = *desc;
-    h->geom = g;
+    h->prepared = p;
     h->input = input; h->weights = weights; h->multiplier = multiplier; h->bias = bias; h->thresholds = thresholds;
     h->output = output;
     *plan = h;
@@ -303,9 +364,13 @@ extern "C" lce_status lce_bconv2d_plan_create(const lce_bconv2d_desc *desc, cons
 
 extern "C" lce_status lce_plan_run(const lce_plan *plan, void *stream)
 {
+    using namespace lce;
     if (!plan) return LCE_ERR_INVALID_ARG;
-    return lce::dispatch(&plan->desc, plan->geom, plan->input, plan->weights, plan->multiplier, plan->bias, plan->thresholds,
-                         plan->output, static_cast<cudaStream_t>(stream));
+    int device = -1;
+    // on another device than the plan was made on: its launch is worked out for that one
+    const bool same = cudaGetDevice(&device) == cudaSuccess && device == plan->prepared.device;
+    const Prepared &p = same ? plan->prepared : prepared_for(&plan->prepared.desc, plan->prepared.form);
+    return dispatch(p, plan->input, plan->weights, plan->multiplier, plan->bias, plan->thresholds, plan->output, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" void lce_plan_destroy(lce_plan *plan) { delete plan; }
@@ -315,28 +380,13 @@ extern "C" lce_status lce_bconv2d_fused(const lce_bconv2d_desc *desc, const uint
                                         float *out_float, uint32_t *out_packed, void *stream)
 {
     using namespace lce;
-    ConvGeom g;
-    lce_status st = make_geom(desc, &g);
-    if (st != LCE_OK) return st;
-    if (g.out_type != LCE_OUT_FLOAT32) return LCE_ERR_INVALID_ARG;
+    if (!desc) return LCE_ERR_INVALID_ARG;
+    const Prepared &p = prepared_for(desc, FORM_FUSED | (aligned(out_float, 16) && aligned(residual, 16) ? 0 : FORM_ROWS_UNALIGNED));
+    if (p.status != LCE_OK) return p.status;
+    if (p.g.out_type != LCE_OUT_FLOAT32) return LCE_ERR_INVALID_ARG;
     if (!input || !weights || !multiplier || !bias || (!out_float && !out_packed)) return LCE_ERR_INVALID_ARG;
-    if (!aligned(input, 4) || !aligned(weights, 4) || !aligned(multiplier, 4) || !aligned(bias, 4) ||
-        !aligned(residual, 4) || !aligned(out_float, 4) || !aligned(out_packed, 4))
-        return LCE_ERR_ALIGNMENT;
-    if (tensor_timeout_flagged()) return LCE_ERR_DEVICE_TIMEOUT;
-    WeightViews v;
-    st = weight_views(desc, g, weights, &v);
-    if (st != LCE_OK) return st;
-    if (desc->kernel == LCE_KERNEL_DIRECT || patch_covers(g)) return LCE_ERR_UNSUPPORTED;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // the tensor-core kernel fuses the same neighbours when whole 32-channel words and 16-byte rows allow it
-    const bool tensor_ok = v.tensor && tensor_covers(g) && (g.Cout & 31) == 0 && aligned(out_float, 16) && aligned(residual, 16);
-    if (desc->kernel == LCE_KERNEL_TENSOR && !tensor_ok) return LCE_ERR_UNSUPPORTED;
-    if (tensor_ok && (desc->kernel == LCE_KERNEL_TENSOR || (desc->kernel == LCE_KERNEL_AUTO && tensor_preferred(g) && !small_preferred(g))))
-        return launch_bconv_tensor(g, input, v.tensor, multiplier, bias, nullptr, out_float, s, residual, out_packed);
-    if (v.small && desc->kernel == LCE_KERNEL_AUTO && tiled_weight_image_bytes(g) > 0 && small_preferred(g))
-        return launch_bconv_small(g, input, v.plain, v.small, multiplier, bias, nullptr, out_float, s, residual, out_packed);
-    return launch_bconv_tiled(g, input, v.plain, v.tiled, multiplier, bias, nullptr, out_float, s, residual, out_packed);
+    if (!conv_buffers_aligned(input, weights, multiplier, bias, out_packed, out_float) || !aligned(residual, 4)) return LCE_ERR_ALIGNMENT;
+    return dispatch(p, input, weights, multiplier, bias, nullptr, out_float, static_cast<cudaStream_t>(stream), residual, out_packed);
 }
 
 extern "C" lce_status lce_bconv2d_f32(const lce_bconv2d_desc *desc, const float *input, const uint32_t *weights,
@@ -345,26 +395,28 @@ extern "C" lce_status lce_bconv2d_f32(const lce_bconv2d_desc *desc, const float 
 {
     using namespace lce;
     ConvGeom g;
-    lce_status st = check_conv_args(desc, &g, input, weights, multiplier, bias, thresholds, output);
+    lce_status st = make_geom(desc, &g);
     if (st != LCE_OK) return st;
-    if (!aligned(input, 4) || !aligned(weights, 4) || !aligned(output, 4) ||
-        (multiplier && !aligned(multiplier, 4)) || (bias && !aligned(bias, 4)) ||
-        (thresholds && !aligned(thresholds, 4)))
-        return LCE_ERR_ALIGNMENT;
-    WeightViews v;
-    st = weight_views(desc, g, weights, &v);
+    st = check_conv_buffers(g, input, weights, multiplier, bias, thresholds, output);
     if (st != LCE_OK) return st;
+    if (!conv_buffers_aligned(input, weights, multiplier, bias, thresholds, output)) return LCE_ERR_ALIGNMENT;
+    const uint32_t *image = nullptr;
+    if (desc->weights_packed) {
+        if (!aligned(weights, 256)) return LCE_ERR_ALIGNMENT;
+        const size_t off = weight_parts(g).tiled;
+        if (off) image = reinterpret_cast<const uint32_t *>(reinterpret_cast<const char *>(weights) + off);
+    }
     if (desc->kernel == LCE_KERNEL_DIRECT || desc->kernel == LCE_KERNEL_TENSOR) return LCE_ERR_UNSUPPORTED;
-    return launch_bconv_tiled(g, nullptr, v.plain, v.tiled, multiplier, bias, thresholds, output,
+    return launch_bconv_tiled(g, nullptr, weights, image, multiplier, bias, thresholds, output,
                               static_cast<cudaStream_t>(stream), nullptr, nullptr, input);
 }
 
 extern "C" size_t lce_bconv2d_packed_weights_bytes(const lce_bconv2d_desc *desc)
 {
-    lce::ConvGeom g;
-    if (lce::make_geom(desc, &g) != LCE_OK) return 0;
-    return lce::plain_weight_bytes(g) + lce::round_up(lce::tiled_weight_image_bytes(g), 256) + lce::round_up(lce::tensor_weight_image_bytes(g), 256) +
-           lce::round_up(lce::small_weight_image_bytes(g), 256);
+    using namespace lce;
+    if (!desc) return 0;
+    const Prepared &p = prepared_for(desc, 0);
+    return p.status == LCE_OK ? p.parts.total : 0;
 }
 
 extern "C" lce_status lce_bconv2d_pack_weights(const lce_bconv2d_desc *desc, const uint32_t *weights, void *packed,
@@ -379,19 +431,11 @@ extern "C" lce_status lce_bconv2d_pack_weights(const lce_bconv2d_desc *desc, con
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const size_t plain = (size_t)g.Cout * g.KH * g.KW * g.Cw * 4;
     if (cudaMemcpyAsync(packed, weights, plain, cudaMemcpyDeviceToDevice, s) != cudaSuccess) return LCE_ERR_CUDA;
-    size_t off = plain_weight_bytes(g);
-    const size_t tiled = tiled_weight_image_bytes(g), tensor = tensor_weight_image_bytes(g);
-    if (tiled > 0) {
-        st = launch_pack_weights_tiled(g, weights, reinterpret_cast<uint32_t *>(static_cast<char *>(packed) + off), s);
-        if (st != LCE_OK) return st;
-    }
-    off += round_up(tiled, 256);
-    if (tensor > 0) {
-        st = launch_pack_weights_tensor(g, weights, static_cast<char *>(packed) + off, s);
-        if (st != LCE_OK) return st;
-    }
-    off += round_up(tensor, 256);
-    if (small_weight_image_bytes(g) > 0) return launch_pack_weights_small(g, weights, reinterpret_cast<uint32_t *>(static_cast<char *>(packed) + off), s);
+    const WeightParts parts = weight_parts(g);
+    char *base = static_cast<char *>(packed);
+    if (parts.tiled && (st = launch_pack_weights_tiled(g, weights, reinterpret_cast<uint32_t *>(base + parts.tiled), s)) != LCE_OK) return st;
+    if (parts.tensor && (st = launch_pack_weights_tensor(g, weights, base + parts.tensor, s)) != LCE_OK) return st;
+    if (parts.small) return launch_pack_weights_small(g, weights, reinterpret_cast<uint32_t *>(base + parts.small), s);
     return LCE_OK;
 }
 
@@ -409,7 +453,8 @@ lce_status host_conv(const lce_bconv2d_desc *desc, const uint32_t *input, const 
                      void *stream, bool synchronise)
 {
     ConvGeom g;
-    lce_status st = check_conv_args(desc, &g, input, weights, multiplier, bias, thresholds, output);
+    lce_status st = make_geom(desc, &g);
+    if (st == LCE_OK) st = check_conv_buffers(g, input, weights, multiplier, bias, thresholds, output);
     if (st != LCE_OK) return st;
     if (!workspace || desc->weights_packed) return LCE_ERR_INVALID_ARG;
     if (!aligned(workspace, 256)) return LCE_ERR_ALIGNMENT;
@@ -423,7 +468,9 @@ lce_status host_conv(const lce_bconv2d_desc *desc, const uint32_t *input, const 
     if (bias) ok = ok && cudaMemcpyAsync(ws + L.bias, bias, L.ch_bytes, cudaMemcpyHostToDevice, s) == cudaSuccess;
     if (thresholds) ok = ok && cudaMemcpyAsync(ws + L.thr, thresholds, L.ch_bytes, cudaMemcpyHostToDevice, s) == cudaSuccess;
     if (!ok) return LCE_ERR_CUDA;
-    st = dispatch(desc, g, reinterpret_cast<const uint32_t *>(ws + L.in), reinterpret_cast<const uint32_t *>(ws + L.w),
+    const Prepared &p = prepared_for(desc, 0);
+    if (p.status != LCE_OK) return p.status;
+    st = dispatch(p, reinterpret_cast<const uint32_t *>(ws + L.in), reinterpret_cast<const uint32_t *>(ws + L.w),
                   multiplier ? reinterpret_cast<const float *>(ws + L.mult) : nullptr,
                   bias ? reinterpret_cast<const float *>(ws + L.bias) : nullptr,
                   thresholds ? reinterpret_cast<const int32_t *>(ws + L.thr) : nullptr, ws + L.out, s);
@@ -477,7 +524,8 @@ extern "C" lce_status lce_bconv2d_host_noalloc(const lce_bconv2d_desc *desc, con
 {
     using namespace lce;
     ConvGeom g;
-    lce_status st = check_conv_args(desc, &g, input, weights, multiplier, bias, thresholds, output);
+    lce_status st = make_geom(desc, &g);
+    if (st == LCE_OK) st = check_conv_buffers(g, input, weights, multiplier, bias, thresholds, output);
     if (st != LCE_OK) return st;
     if (desc->weights_packed) return LCE_ERR_INVALID_ARG;
     if (host_layout(g).total > LCE_STATIC_WORKSPACE_BYTES) return LCE_ERR_WORKSPACE;  // this call does not fit the built-in array

@@ -113,6 +113,8 @@ bconv1x1_kernel(const TiledParams p)
         for (int e = tid * 4; e < w_words; e += kThreads * 4) cp_async16(smem + e, src + e);
         asm volatile("cp.async.commit_group;" ::: "memory");
     } else {
+        // plain words may come from the kernel before (LceQuantize of the weights), which may still be running
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         for (int e = tid; e < kChanPerCta * groups; e += kThreads) {
             const int ch = e / groups;
             const int g = e - ch * groups;

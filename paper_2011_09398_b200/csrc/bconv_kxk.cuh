@@ -166,6 +166,8 @@ bconv3x3_kernel(const TiledParams p)
         for (int e = tid * 4; e < words; e += kThreads * 4) cp_async16(smem + e, src + e);
         asm volatile("cp.async.commit_group;" ::: "memory");
     } else {
+        // plain words may come from the kernel before (LceQuantize of the weights), which may still be running
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         for (int e = tid; e < kChanPerCta * p.Cw * kNG; e += kThreads) {
             const int g = e % kNG;
             const int cw = (e / kNG) % p.Cw;

@@ -1305,25 +1305,7 @@ lce_status launch_mx(const MxParams &p, dim3 grid, size_t smem, cudaStream_t s)
 {
     static SmemOptIn opted;
     if (!opted.ensure(bconv_mx_kernel<EPI>, smem)) return LCE_ERR_CUDA;
-    // Programmatic dependent launch: the CTAs of this grid may be scheduled while the previous kernel of the
-    // stream is still draining; they set themselves up and fetch their weights (constants of the model),
-    // and wait for the previous kernel's completion (griddepcontrol.wait) before they touch anything it may
-    // have written or may still read: the activations, the shortcut tensor, the outputs.
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(kMxThreads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, bconv_mx_kernel<EPI>, p) != cudaSuccess) {
-        cudaGetLastError();
-        return LCE_ERR_CUDA;
-    }
-    return LCE_OK;
+    return launch_dependent(bconv_mx_kernel<EPI>, grid, kMxThreads, smem, s, p);
 }
 
 int mx_dup(const ConvGeom &g) { return g.Cout <= 32 ? 4 : g.Cout <= 64 ? 2 : 1; }
@@ -1374,15 +1356,24 @@ lce_status tensor_plan_info(const ConvGeom &g, TensorPlanInfo *info)
     return LCE_OK;
 }
 
-lce_status launch_bconv_tensor(const ConvGeom &g, const uint32_t *in, const void *w_image, const float *mult, const float *bias,
-                               const int32_t *thr, void *out, cudaStream_t s, const float *residual, uint32_t *out_packed)
+namespace {
+struct MxLaunch {
+    MxParams params;
+    dim3 grid;
+    size_t smem;
+};
+static_assert(sizeof(MxLaunch) <= sizeof(PreparedLaunch), "PreparedLaunch too small");
+}  // namespace
+
+lce_status prepare_bconv_tensor(const ConvGeom &g, PreparedLaunch *prepared)
 {
     MxPlan pl;
-    if (!w_image || !mx_plan(g, device_sms(), &pl)) return LCE_ERR_UNSUPPORTED;
-    MxParams p{};
-    p.in = in; p.wimg = static_cast<const uint8_t *>(w_image); p.mult = mult; p.bias = bias; p.thr = thr; p.out = out;
-    p.residual = residual; p.out_packed = out_packed;
-    p.host_flag = mx_flag_for_launch(s);
+    if (!mx_plan(g, device_sms(), &pl)) return LCE_ERR_UNSUPPORTED;
+    MxLaunch &l = *reinterpret_cast<MxLaunch *>(prepared->bytes);
+    l.params = MxParams{};
+    l.grid = dim3((unsigned)pl.ctas_x, (unsigned)pl.n_blocks);
+    l.smem = pl.smem;
+    MxParams &p = l.params;
     p.N = g.N; p.H = g.H; p.W = g.W; p.Cw = g.Cw; p.Cw2 = pl.Cw2; p.Cout = g.Cout; p.Cow = g.Cow;
     p.OH = g.OH; p.OW = g.OW; p.KH = g.KH; p.KW = g.KW; p.stride = g.sh; p.pt = g.pt; p.pl = g.pl;
     p.K = g.KH * g.KW * g.Cin;
@@ -1404,18 +1395,28 @@ lce_status launch_bconv_tensor(const ConvGeom &g, const uint32_t *in, const void
     p.tap_bytes = (int32_t)pl.tap_bytes; p.raw_words = (int32_t)pl.raw_words; p.x_bytes = (int32_t)pl.x_bytes;
     p.n_xbuf = pl.n_xbuf; p.ahead = pl.ahead;
     p.off_tbl = (int32_t)pl.off_tbl; p.off_w = (int32_t)pl.off_w; p.off_x = (int32_t)pl.off_x;
-    p.cp_words = (g.Cw % 4 == 0 && aligned(in, 16)) ? 4 : (g.Cw % 2 == 0 && aligned(in, 8)) ? 2 : 1;
     p.pad_zero = g.padding == LCE_PAD_SAME_ZERO;
     p.out_type = g.out_type; p.activation = g.activation;
-    p.write_float = out != nullptr;
     p.dup_log2 = mx_dup(g) == 4 ? 2 : mx_dup(g) == 2 ? 1 : 0;
-    if (!aligned(w_image, 16)) return LCE_ERR_ALIGNMENT;
-    const dim3 grid((unsigned)pl.ctas_x, (unsigned)pl.n_blocks);
-    if (g.out_type == LCE_OUT_FLOAT32 && (residual || out_packed || !out || g.activation != LCE_ACT_NONE))
-        return launch_mx<EPI_FLOAT_FUSED>(p, grid, pl.smem, s);
-    return launch_mx<EPI_PLAIN>(p, grid, pl.smem, s);
+    return LCE_OK;
 }
 
+lce_status launch_bconv_tensor(const PreparedLaunch &prepared, const uint32_t *in, const void *w_image, const float *mult, const float *bias,
+                               const int32_t *thr, void *out, cudaStream_t s, const float *residual, uint32_t *out_packed)
+{
+    if (!w_image) return LCE_ERR_UNSUPPORTED;
+    if (!aligned(w_image, 16)) return LCE_ERR_ALIGNMENT;
+    const MxLaunch &l = *reinterpret_cast<const MxLaunch *>(prepared.bytes);
+    MxParams p = l.params;
+    p.in = in; p.wimg = static_cast<const uint8_t *>(w_image); p.mult = mult; p.bias = bias; p.thr = thr; p.out = out;
+    p.residual = residual; p.out_packed = out_packed;
+    p.host_flag = mx_flag_for_launch(s);
+    p.cp_words = (p.Cw % 4 == 0 && aligned(in, 16)) ? 4 : (p.Cw % 2 == 0 && aligned(in, 8)) ? 2 : 1;
+    p.write_float = out != nullptr;
+    if (p.out_type == LCE_OUT_FLOAT32 && (residual || out_packed || !out || p.activation != LCE_ACT_NONE))
+        return launch_mx<EPI_FLOAT_FUSED>(p, l.grid, l.smem, s);
+    return launch_mx<EPI_PLAIN>(p, l.grid, l.smem, s);
+}
 
 // ---- status of the bounded waits ----------------------------------------------------------------------
 namespace {

@@ -138,6 +138,8 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) bconv_small_kernel(const __
         const uint32_t *src = p.w + (int64_t)blockIdx.y * image_words;
         for (int e = tid; e < n; e += n_threads) cp_async_zfill<16>(sW + 4 * e, src + 4 * e, true);
     } else {
+        // plain words may come from the kernel before (LceQuantize of the weights), which may still be running
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         for (int r = warp; r < kChannels; r += n_warps) {
             const bool valid = ch0 + r < p.Cout;
             const uint32_t *src = p.w + (valid ? (int64_t)(ch0 + r) * p.K : 0);
@@ -383,29 +385,29 @@ lce_status launch_small_mode(const SmallParams &p, const SmallShape &shape, cuda
 {
     static SmemOptIn opted;
     if (!opted.ensure(bconv_small_kernel<MODE, NT>, shape.smem)) return LCE_ERR_CUDA;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)((p.M + shape.tile - 1) / shape.tile), (unsigned)p.Cow);
-    cfg.blockDim = dim3(32 * shape.warps);
-    cfg.dynamicSmemBytes = shape.smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, bconv_small_kernel<MODE, NT>, p) != cudaSuccess) {
-        cudaGetLastError();
-        return LCE_ERR_CUDA;
-    }
-    return LCE_OK;
+    return launch_dependent(bconv_small_kernel<MODE, NT>, dim3((unsigned)((p.M + shape.tile - 1) / shape.tile), (unsigned)p.Cow), 32 * shape.warps, shape.smem, s, p);
 }
 
-lce_status launch_small_as(const ConvGeom &g, const SmallShape &shape, const uint32_t *in, const uint32_t *w, const uint32_t *w_image, const float *mult,
-                           const float *bias, const int32_t *thr, void *out, cudaStream_t s, const float *residual, uint32_t *out_packed)
+struct SmallLaunch {
+    SmallParams params;
+    SmallShape shape;
+};
+static_assert(sizeof(SmallLaunch) <= sizeof(PreparedLaunch), "PreparedLaunch too small");
+
+// the activations are copied in pieces of `vec` words
+void small_set_vec(SmallParams *p, int vec)
 {
-    SmallParams p{};
-    p.in = in; p.w = w_image ? w_image : w; p.image = w_image != nullptr;
-    p.mult = mult; p.bias = bias; p.thr = thr; p.residual = residual; p.out = out; p.out_packed = out_packed;
+    p->vec = vec;
+    p->pieces = p->W * p->Cw / vec;
+    p->by_pieces = fast_div((uint32_t)p->pieces);
+    p->by_px_pieces = fast_div((uint32_t)(p->Cw / vec));
+}
+
+void prepare_small_as(const ConvGeom &g, const SmallShape &shape, SmallLaunch *l)
+{
+    l->shape = shape;
+    l->params = SmallParams{};
+    SmallParams &p = l->params;
     p.N = g.N; p.H = g.H; p.W = g.W; p.Cw = g.Cw; p.Cin = g.Cin; p.Cout = g.Cout; p.Cow = g.Cow; p.KH = g.KH; p.KW = g.KW; p.taps = g.KH * g.KW;
     p.sh = g.sh; p.sw = g.sw; p.OH = g.OH; p.OW = g.OW; p.pt = g.pt; p.pl = g.pl;
     p.M = (int32_t)g.M; p.K = p.taps * g.Cw; p.KD = p.taps * g.Cin;
@@ -415,16 +417,24 @@ lce_status launch_small_as(const ConvGeom &g, const SmallShape &shape, const uin
     while ((1 << p.slices_sh) < shape.slices) ++p.slices_sh;
     p.raw_words = (int32_t)small_raw_words(g, shape.tile);
     p.padded = g.padding != LCE_PAD_VALID && (g.KH > 1 || g.KW > 1);
-    p.vec = (g.Cw % 4 == 0 && aligned(in, 16)) ? 4 : (g.Cw % 2 == 0 && aligned(in, 8)) ? 2 : 1;
-    p.pieces = g.W * g.Cw / p.vec;
-    p.by_pieces = fast_div((uint32_t)p.pieces); p.by_px_pieces = fast_div((uint32_t)(g.Cw / p.vec)); p.by_cw = fast_div((uint32_t)g.Cw);
+    small_set_vec(&p, g.Cw % 4 == 0 ? 4 : g.Cw % 2 == 0 ? 2 : 1);
+    p.by_cw = fast_div((uint32_t)g.Cw);
     p.by_kw = fast_div((uint32_t)g.KW); p.by_ow = fast_div((uint32_t)g.OW); p.by_oh = fast_div((uint32_t)g.OH); p.by_hp = fast_div((uint32_t)p.Hp);
     p.zero_pad = g.padding == LCE_PAD_SAME_ZERO; p.out_type = g.out_type; p.relu = g.activation == LCE_ACT_RELU;
-    const bool wide = shape.groups == 2;
-    if (g.out_type == LCE_OUT_BITPACKED) return wide ? launch_small_mode<SMALL_BITS, 2>(p, shape, s) : launch_small_mode<SMALL_BITS, 1>(p, shape, s);
-    if (g.out_type == LCE_OUT_FLOAT32 && !residual && !out_packed)
-        return wide ? launch_small_mode<SMALL_FLOAT, 2>(p, shape, s) : launch_small_mode<SMALL_FLOAT, 1>(p, shape, s);
-    return wide ? launch_small_mode<SMALL_GENERAL, 2>(p, shape, s) : launch_small_mode<SMALL_GENERAL, 1>(p, shape, s);
+}
+
+lce_status launch_small_as(const SmallLaunch &l, const uint32_t *in, const uint32_t *w, const uint32_t *w_image, const float *mult,
+                           const float *bias, const int32_t *thr, void *out, cudaStream_t s, const float *residual, uint32_t *out_packed)
+{
+    SmallParams p = l.params;
+    p.in = in; p.w = w_image ? w_image : w; p.image = w_image != nullptr;
+    p.mult = mult; p.bias = bias; p.thr = thr; p.residual = residual; p.out = out; p.out_packed = out_packed;
+    while (!aligned(in, 4 * (size_t)p.vec)) small_set_vec(&p, p.vec / 2);
+    const bool wide = l.shape.groups == 2;
+    if (p.out_type == LCE_OUT_BITPACKED) return wide ? launch_small_mode<SMALL_BITS, 2>(p, l.shape, s) : launch_small_mode<SMALL_BITS, 1>(p, l.shape, s);
+    if (p.out_type == LCE_OUT_FLOAT32 && !residual && !out_packed)
+        return wide ? launch_small_mode<SMALL_FLOAT, 2>(p, l.shape, s) : launch_small_mode<SMALL_FLOAT, 1>(p, l.shape, s);
+    return wide ? launch_small_mode<SMALL_GENERAL, 2>(p, l.shape, s) : launch_small_mode<SMALL_GENERAL, 1>(p, l.shape, s);
 }
 
 constexpr size_t kSmallSmem = 100 * 1024;  // two CTAs per SM, so that a CTA of the next kernel finds room to prepare itself
@@ -490,11 +500,17 @@ lce_status launch_pack_weights_small(const ConvGeom &g, const uint32_t *w, uint3
     return launch_status();
 }
 
-lce_status launch_bconv_small(const ConvGeom &g, const uint32_t *in, const uint32_t *w, const uint32_t *w_image, const float *mult,
-                              const float *bias, const int32_t *thr, void *out, cudaStream_t s, const float *residual, uint32_t *out_packed)
+lce_status prepare_bconv_small(const ConvGeom &g, PreparedLaunch *prepared)
 {
     if (!small_covers(g)) return LCE_ERR_UNSUPPORTED;
-    return launch_small_as(g, small_shape(g), in, w, w_image, mult, bias, thr, out, s, residual, out_packed);
+    prepare_small_as(g, small_shape(g), reinterpret_cast<SmallLaunch *>(prepared->bytes));
+    return LCE_OK;
+}
+
+lce_status launch_bconv_small(const PreparedLaunch &prepared, const uint32_t *in, const uint32_t *w, const uint32_t *w_image, const float *mult,
+                              const float *bias, const int32_t *thr, void *out, cudaStream_t s, const float *residual, uint32_t *out_packed)
+{
+    return launch_small_as(*reinterpret_cast<const SmallLaunch *>(prepared.bytes), in, w, w_image, mult, bias, thr, out, s, residual, out_packed);
 }
 
 }  // namespace lce

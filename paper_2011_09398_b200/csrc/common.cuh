@@ -104,6 +104,36 @@ struct SmemOptIn {
     }
 };
 
+// Launches a kernel with programmatic stream serialization: its CTAs may be scheduled while the previous kernel
+// of the stream drains (if that kernel lets its dependents start early), and wait for its completion themselves
+// (griddepcontrol.wait) before they touch anything it may have written or may still read.  Also the cheaper launch
+// for the host (2.4 us against 2.9 us measured).
+template <typename... Params, typename... Args>
+lce_status launch_dependent(void (*kernel)(Params...), dim3 grid, int threads, size_t smem_bytes, cudaStream_t s, const Args &...args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.dynamicSmemBytes = smem_bytes;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...) != cudaSuccess) {
+        cudaGetLastError();
+        return LCE_ERR_CUDA;
+    }
+    return LCE_OK;
+}
+
+// A launch worked out ahead of time for a geometry: everything but the buffers (filled in by the prepare functions,
+// read by the launch functions of the same kernel).
+struct PreparedLaunch {
+    alignas(16) unsigned char bytes[640];
+};
+
 // Kernel entry points implemented in the other translation units.
 lce_status launch_bconv_direct(const ConvGeom &g, const uint32_t *in, const uint32_t *w, const float *mult,
                                const float *bias, const int32_t *thr, void *out, cudaStream_t s);
@@ -128,7 +158,8 @@ int64_t small_ctas(const ConvGeom &g);
 void small_plan_info(const ConvGeom &g, TiledPlanInfo *info);
 size_t small_weight_image_bytes(const ConvGeom &g);
 lce_status launch_pack_weights_small(const ConvGeom &g, const uint32_t *w, uint32_t *image, cudaStream_t s);
-lce_status launch_bconv_small(const ConvGeom &g, const uint32_t *in, const uint32_t *w, const uint32_t *w_image, const float *mult,
+lce_status prepare_bconv_small(const ConvGeom &g, PreparedLaunch *prepared);
+lce_status launch_bconv_small(const PreparedLaunch &prepared, const uint32_t *in, const uint32_t *w, const uint32_t *w_image, const float *mult,
                               const float *bias, const int32_t *thr, void *out, cudaStream_t s,
                               const float *residual = nullptr, uint32_t *out_packed = nullptr);
 // Tensor-core kernel (tcgen05 kind::mxf4 on e2m1 operands): any filter of up to 64 taps, equal strides
@@ -138,7 +169,8 @@ lce_status launch_bconv_small(const ConvGeom &g, const uint32_t *in, const uint3
 bool tensor_covers(const ConvGeom &g);
 size_t tensor_weight_image_bytes(const ConvGeom &g);
 lce_status launch_pack_weights_tensor(const ConvGeom &g, const uint32_t *w, void *image, cudaStream_t s);
-lce_status launch_bconv_tensor(const ConvGeom &g, const uint32_t *in, const void *w_image, const float *mult,
+lce_status prepare_bconv_tensor(const ConvGeom &g, PreparedLaunch *prepared);
+lce_status launch_bconv_tensor(const PreparedLaunch &prepared, const uint32_t *in, const void *w_image, const float *mult,
                                const float *bias, const int32_t *thr, void *out, cudaStream_t s,
                                const float *residual = nullptr, uint32_t *out_packed = nullptr);
 struct TensorPlanInfo {

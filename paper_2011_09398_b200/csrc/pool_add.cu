@@ -1,6 +1,7 @@
 // LceBMaxPool2d (paper Section 3.2: max-pool on packed bits is the bitwise AND of the window,
 // because a 0 bit is +1 and max(sign X) = sign(max X)) and the fp32 residual add that the
-// shortcut pattern of Section 5.3 places between a float-output conv and the next LceQuantize.
+// shortcut pattern of Section 5.3 places between a float-output conv and the next LceQuantize.  Launched as
+// programmatic dependents: they wait for the previous kernel before their first access.
 #include "common.cuh"
 
 namespace lce {
@@ -18,6 +19,7 @@ bmaxpool_kernel(const uint32_t *__restrict__ in, uint32_t *__restrict__ out, int
                 int32_t Cw, int32_t OH, int32_t OW, int32_t PH, int32_t PW, int32_t sh, int32_t sw, int32_t pt,
                 int32_t pl)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int32_t cv = Cw / VEC;            // vectors per pixel
     const int32_t row_vecs = OW * cv;       // vectors per output row
     const int32_t rows = N * OH;  // < 2^31: checked on the host
@@ -69,6 +71,7 @@ bmaxpool_kernel(const uint32_t *__restrict__ in, uint32_t *__restrict__ out, int
 __global__ void __launch_bounds__(kThreads)
 add_f32_vec4_kernel(const float4 *a, const float4 *b, float4 *out, int64_t n4)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n4; i += (int64_t)gridDim.x * kThreads) {
         const float4 u = __ldcs(a + i), v = __ldcs(b + i);
         out[i] = make_float4(__fadd_rn(u.x, v.x), __fadd_rn(u.y, v.y), __fadd_rn(u.z, v.z), __fadd_rn(u.w, v.w));
@@ -78,6 +81,7 @@ add_f32_vec4_kernel(const float4 *a, const float4 *b, float4 *out, int64_t n4)
 __global__ void __launch_bounds__(kThreads)
 add_f32_scalar_kernel(const float *a, const float *b, float *out, int64_t begin, int64_t n)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int64_t i = begin + (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kThreads)
         out[i] = __fadd_rn(a[i], b[i]);
 }
@@ -114,13 +118,9 @@ extern "C" lce_status lce_bmaxpool(const uint32_t *in, uint32_t *out, int32_t ba
     int64_t blocks = (int64_t)batch * ah.out;  // one block per output row, grid-stride beyond 8 waves of 8 blocks per SM
     if (blocks > 148 * 8 * 8) blocks = 148 * 8 * 8;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (Cw % 4 == 0 && aligned(in, 16) && aligned(out, 16))
-        bmaxpool_kernel<4><<<(unsigned)blocks, kThreads, 0, s>>>(in, out, batch, in_h, in_w, Cw, ah.out, aw.out, pool_h, pool_w,
-                                                                stride_h, stride_w, ah.pad_before, aw.pad_before);
-    else
-        bmaxpool_kernel<1><<<(unsigned)blocks, kThreads, 0, s>>>(in, out, batch, in_h, in_w, Cw, ah.out, aw.out, pool_h, pool_w,
-                                                                stride_h, stride_w, ah.pad_before, aw.pad_before);
-    return launch_status();
+    const bool vec = Cw % 4 == 0 && aligned(in, 16) && aligned(out, 16);
+    return launch_dependent(vec ? bmaxpool_kernel<4> : bmaxpool_kernel<1>, dim3((unsigned)blocks), kThreads, 0, s, in, out, batch, in_h, in_w, Cw, ah.out,
+                            aw.out, pool_h, pool_w, stride_h, stride_w, ah.pad_before, aw.pad_before);
 }
 
 extern "C" lce_status lce_add_f32(const float *a, const float *b, float *out, int64_t n, void *stream)
@@ -134,10 +134,10 @@ extern "C" lce_status lce_add_f32(const float *a, const float *b, float *out, in
     int64_t done = 0;
     if (aligned(a, 16) && aligned(b, 16) && aligned(out, 16) && n >= 4) {
         const int64_t n4 = n / 4;
-        add_f32_vec4_kernel<<<grid_for(n4, 148 * 8), kThreads, 0, s>>>(
-            reinterpret_cast<const float4 *>(a), reinterpret_cast<const float4 *>(b), reinterpret_cast<float4 *>(out), n4);
+        const lce_status st = launch_dependent(add_f32_vec4_kernel, dim3(grid_for(n4, 148 * 8)), kThreads, 0, s, reinterpret_cast<const float4 *>(a),
+                                               reinterpret_cast<const float4 *>(b), reinterpret_cast<float4 *>(out), n4);
         done = n4 * 4;
+        if (st != LCE_OK || done == n) return st;
     }
-    if (done < n) add_f32_scalar_kernel<<<grid_for(n - done, 148 * 8), kThreads, 0, s>>>(a, b, out, done, n);
-    return launch_status();
+    return launch_dependent(add_f32_scalar_kernel, dim3(grid_for(n - done, 148 * 8)), kThreads, 0, s, a, b, out, done, n);
 }

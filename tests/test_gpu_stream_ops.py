@@ -1,0 +1,54 @@
+"""LceQuantize and LceDequantize at channel counts that are not whole words, against the oracle: rows shorter and longer
+than a word, runs of rows that end inside a 16-byte piece or a group of sixteen loads, rows longer than a block's run,
+outputs that are only 4-byte aligned, and LceQuantize straight before a convolution that reads its output as weights."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2011_09398_b200 as lce
+from gpu_util import DEV, guarded, guards_intact, run_bconv, to_dev, words_to_host
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("rows,channels", [(1, 1), (5, 3), (7, 4), (3, 5), (1, 31), (9, 33), (4001, 7), (2500, 100), (700, 513), (30000, 38), (2, 8191),
+                                           (3, 8193), (2, 20001), (5000, 16)])
+def test_quantize_and_back(rows, channels, offset):
+    rng = np.random.default_rng(rows * 7 + channels)
+    x = rng.standard_normal((rows, channels)).astype(np.float32)
+    x[0, 0] = -0.0
+    words = (channels + 31) // 32
+    src = torch.empty(rows * channels + 1, dtype=torch.float32, device=DEV)[offset:offset + rows * channels].view(rows, channels)
+    src.copy_(torch.from_numpy(x))
+    whole, out = guarded((rows, words), torch.int32, 0x5A5A5A5A)
+    if offset:
+        whole = torch.full((rows * words + 129,), 0x5A5A5A5A, dtype=torch.int32, device=DEV)
+        out = whole[65:65 + rows * words].view(rows, words)
+    lce.lce_bitpack(src, out)
+    assert guards_intact(whole, 0x5A5A5A5A)
+    want = oracle.bitpack(x)
+    np.testing.assert_array_equal(words_to_host(out), want)
+    whole_f = torch.full((rows * channels + 129,), 7.0, dtype=torch.float32, device=DEV)
+    back = whole_f[64 + offset:64 + offset + rows * channels].view(rows, channels)
+    lce.lce_unpack(out, channels, back)
+    assert guards_intact(whole_f, 7.0)
+    np.testing.assert_array_equal(back.cpu().numpy(), np.where(x < 0, -1.0, 1.0).astype(np.float32))
+
+
+@pytest.mark.parametrize("cin,k", [(64, 3), (96, 1)])
+def test_weights_quantized_right_before_the_convolution(cin, k):
+    """Plain weights may be the output of the kernel just launched: many rounds, other weights each time."""
+    rng = np.random.default_rng(cin)
+    a = (2 * rng.integers(0, 2, size=(2, 12, 12, cin)) - 1).astype(np.int8)
+    ws = [(2 * rng.integers(0, 2, size=(160, k, k, cin)) - 1).astype(np.int8) for _ in range(6)]
+    desc = lce.make_desc(2, 12, 12, cin, 160, (k, k), out_type=lce.OUT_INT32)
+    x, floats = lce.lce_bitpack(to_dev(a.astype(np.float32))), [to_dev(w.astype(np.float32)) for w in ws]
+    words = torch.zeros(ws[0].shape[:3] + ((cin + 31) // 32,), dtype=torch.int32, device=DEV)
+    outs = []
+    for f in floats:
+        lce.lce_bitpack(f, words)
+        outs.append(lce.lce_bconv2d(desc, x, words))
+    for w, out in zip(ws, outs):
+        np.testing.assert_array_equal(out.cpu().numpy(), oracle.bconv2d_acc(a, w))
