@@ -184,7 +184,7 @@ struct MxParams {
     int32_t n_tiles, n_super, total_q;
     int32_t taps, ksteps, stages, resident;
     int32_t group_taps, groups;  // streamed weights: taps per ring stage, stages' worth of taps per tile = ceil(taps / group_taps)
-    int32_t tap_bytes, raw_words, x_bytes;
+    int32_t tap_bytes, x_bytes;
     int32_t n_xbuf, ahead;   // position buffers (2..4); tiles the loaders may be ahead of the finished MMAs (2..4)
     int32_t off_tbl, off_w, off_x;    // byte offsets in shared memory
     int32_t cp_words;        // words per cp.async: 4, 2 or 1
@@ -258,7 +258,8 @@ __device__ __forceinline__ void mx_copy_words(uint32_t *dst, const uint32_t *src
 }
 
 // packed words of the chunk's `count` positions, of which this thread's first is `a` -> raw (pad positions:
-// zero words), asynchronously; raw holds the phases of a position one after the other
+// zero words), asynchronously; raw holds the phases of a position one after the other.  One buffer is enough: every
+// thread fetches only into places whose words it has itself just expanded.
 template <int CW, int FORM>
 __device__ __forceinline__ void mx_prefetch(const MxLoad &l, MxPos a, int count, uint32_t *raw, int ltid, int cp_words)
 {
@@ -385,7 +386,7 @@ template <int CW, int FORM>
 __device__ __forceinline__ bool mx_load_tiles(const MxParams &p, const MxLoad &l, MxPos stage, uint64_t *bars, uint32_t *raw0, uint8_t *sX0, int32_t *sPix,
                                               int tid, int first_tile, int tile_step)
 {
-    const int Nt = p.Nt, T = p.T, halo = p.halo, n_tiles = p.n_tiles, n_super = p.n_super, raw_words = p.raw_words, n_xbuf = p.n_xbuf, ahead = p.ahead;
+    const int Nt = p.Nt, T = p.T, halo = p.halo, n_tiles = p.n_tiles, n_super = p.n_super, n_xbuf = p.n_xbuf, ahead = p.ahead;
     const int OH = p.OH, OW = p.OW, plane = p.Cw2 * p.P, cp_words = p.cp_words;
     const uint32_t x_bytes = (uint32_t)p.x_bytes;
     const bool pad_zero = p.pad_zero != 0;
@@ -404,7 +405,7 @@ __device__ __forceinline__ bool mx_load_tiles(const MxParams &p, const MxLoad &l
                 const int done = it - ahead;
                 if (!mbar_wait_bounded(&bars[BAR_TILE_DONE0 + (done & 3)], (uint32_t)(done >> 2) & 1u)) return false;
             }
-            mx_expand<CW, FORM>(l, stage, k ? Nt : Nt + halo, raw0 + (it & 1) * raw_words, X + (k ? k * Nt + halo : 0), plane, tid, pad_zero);
+            mx_expand<CW, FORM>(l, stage, k ? Nt : Nt + halo, raw0, X + (k ? k * Nt + halo : 0), plane, tid, pad_zero);
             if (tid < Nt)
                 sPix[(it & (kPixSlots - 1)) * kMaxNt + tid] = pix.n < l.N && pix.r < OH && pix.c < OW ? (pix.n * OH + pix.r) * OW + pix.c : -1;
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -413,7 +414,7 @@ __device__ __forceinline__ bool mx_load_tiles(const MxParams &p, const MxLoad &l
             mx_advance(pix, more_here ? tile_d : tile_super, l.Wg, l.Hg);
             if (more_here || st + tile_step < n_super) {
                 mx_advance(stage, !more_here ? chunk_super : k ? tile_d : chunk_first, l.Wg, l.Hg);
-                mx_prefetch<CW, FORM>(l, stage, more_here ? Nt : Nt + halo, raw0 + ((it + 1) & 1) * raw_words, tid, cp_words);
+                mx_prefetch<CW, FORM>(l, stage, more_here ? Nt : Nt + halo, raw0, tid, cp_words);
             }
         }
     }
@@ -934,9 +935,9 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
         for (int e = tid - kLoaders; e < n_mma; e += kFinishers) {
             const int tap = e / p.ksteps, kk = e - tap * p.ksteps;
             const int ky = tap / p.KW, kx = tap - ky * p.KW;
-            // A: K step (+ the tap's ring stage when all taps are resident: stage = tap); B: the tap's offset + K step
+            // A: the tap's place among the resident taps or in its group of streamed ones + K step; B: the tap's offset + K step
             const uint32_t b_off = tap_b_offset(p, ky, kx);
-            tbl[e] = make_uint2((p.resident ? (uint32_t)tap * ((uint32_t)p.tap_bytes >> 4) : 0u) + 256u * kk, b_off + 2u * (uint32_t)p.P * kk);
+            tbl[e] = make_uint2((uint32_t)(p.resident ? tap : tap % p.group_taps) * ((uint32_t)p.tap_bytes >> 4) + 256u * kk, b_off + 2u * (uint32_t)p.P * kk);
         }
     }
     // The loaders' first prefetch goes out before the CTA-wide barrier of the set-up: it needs the previous
@@ -1027,8 +1028,7 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
         const bool resident = p.resident != 0;
         const uint32_t w_lo0 = ((uint32_t)p.off_w >> 4) + (smem_u32(smem) >> 4) + (128u << 16);
         const uint32_t x_lo_buf0 = ((uint32_t)p.off_x >> 4) + (smem_u32(smem) >> 4) + ((uint32_t)p.P << 16);
-        const uint32_t x_units = (uint32_t)p.x_bytes >> 4, tap_units = (uint32_t)p.tap_bytes >> 4;
-        const uint32_t group_units = tap_units * (uint32_t)p.group_taps;
+        const uint32_t x_units = (uint32_t)p.x_bytes >> 4, group_units = ((uint32_t)p.tap_bytes >> 4) * (uint32_t)p.group_taps;
         const uint32_t sfa = tmem_base + kSfaCol, sfb = tmem_base + kSfbCol;
         uint32_t par_empty_d[2] = {0, 0};
         const int n_xbuf = p.n_xbuf;
@@ -1064,9 +1064,9 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
                 }
                 mx_issue_table(tmem_d, tbl, n_mma, w_lo0, x_lo0, desc_hi, idesc, sfa, sfb, accumulate);
             } else {
-                // the taps stream through the ring a group at a time: wait for the group, issue its taps' MMAs,
-                // hand its stage back (the wait, the commit and the bookkeeping cost this warp about 600 clocks,
-                // as much as six MMAs: hence groups, not single taps)
+                // the taps stream through the ring a group at a time: wait for the group, issue its MMAs in one run, hand
+                // its stage back (the wait, the commit and the bookkeeping cost this warp as much as some MMAs: hence
+                // groups, not single taps; issued tap by tap, a group of five taps cost 600 clocks more than its MMAs)
                 int tap = 0;
                 while (tap < taps) {
                     ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bars[BAR_FULL_W0 + stage_i], w_parity));
@@ -1074,10 +1074,9 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
                     ++g;
                     if (lane == 0) fills[1] = g;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    uint32_t a_tap = w_lo0 + (uint32_t)stage_i * group_units;
-                    const int group_end = min(taps, tap + group_taps);
-                    for (; tap < group_end; ++tap, a_tap += tap_units)
-                        mx_issue_table(tmem_d, tbl + tap * ksteps, ksteps, a_tap, x_lo0, desc_hi, idesc, sfa, sfb, accumulate);
+                    const int n_taps = min(group_taps, taps - tap);
+                    mx_issue_table(tmem_d, tbl + tap * ksteps, n_taps * ksteps, w_lo0 + (uint32_t)stage_i * group_units, x_lo0, desc_hi, idesc, sfa, sfb, accumulate);
+                    tap += n_taps;
                     if (elect_one()) mma_commit(&bars[BAR_EMPTY_W0 + stage_i]);
                     if (++stage_i == stages) { stage_i = 0; w_parity ^= 1u; }
                 }
@@ -1243,7 +1242,7 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
             if (T > 1 && (T - 1) * ctas_max >= n_tiles) break;   // no CTA would have that many tiles
             const size_t raw_words = (((size_t)pl->n_phase * (nt + halo) * g.Cw + 3) / 4) * 4;
             const size_t x_bytes = (size_t)pl->n_phase * pl->Cw2 * P * 16;
-            const size_t off_tbl = kOffDyn + 2 * raw_words * 4;
+            const size_t off_tbl = kOffDyn + raw_words * 4;
             const size_t fixed = off_tbl + (size_t)taps * ksteps * 8;  // the table no longer than it is: at 512 channels 3x3 the 8 KB saved are a wider tile
             const size_t off_w = (fixed + 127) / 128 * 128;
             const size_t rest = 2 * x_bytes + 256;
@@ -1270,13 +1269,14 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
             const double mma1 = fmax(100.0, 43.0 + nt / 2.0);
             const double mma = (double)taps * ksteps * mma1;
             // a streamed group: its bytes from L2 (with all SMs streaming at least 38 bytes per clock each), or its share of a copy's latency, or what the single issuer needs
-            // per tap (wait for the stage, issue, hand the stage back: about 600 clocks on top of the MMAs;
-            // measured on a nine-tap, one-MMA-per-tap layer: 6000 clocks per tile whether 2 or 4 stages)
-            const double stream = resident ? 0.0 : (double)groups * fmax(fmax(group_taps * pl->tap_bytes / 38.0, 1300.0 / stages), 600.0 + group_taps * ksteps * mma1);
+            // per group (wait for the stage, issue, hand the stage back: about 250 clocks on top of the MMAs)
+            const double stream = resident ? 0.0 : (double)groups * fmax(fmax(group_taps * pl->tap_bytes / 38.0, 1300.0 / stages), 250.0 + group_taps * ksteps * mma1);
             // stride 2: four phases per position, staged two at a time where the geometry allows (MX_S2_PAIR)
             const double per_position = s == 1 ? 1.0 : ((g.W & 1) == 0 && (g.pl & 1) == 0 && g.Cw <= 4) ? 2.0 : 3.0;
             const double load = 400.0 + 8.0 * per_position * (nt + (double)halo / T);
-            const double cost = per_cta * (fmax(fmax(mma, stream), load) + 150.0);
+            // with streamed weights the hand-overs of the ring and of the loaders do not hide each other (112x112x32 stride 2
+            // at batch 256: 71 us streamed, 36 us resident, where the three terms alone call it a tie)
+            const double cost = per_cta * (fmax(fmax(mma, stream), load) + 0.5 * fmin(stream, load) + 150.0);
             if (cost < best) {
                 best = cost;
                 found = true;
@@ -1392,7 +1392,7 @@ lce_status prepare_bconv_tensor(const ConvGeom &g, PreparedLaunch *prepared)
     p.step_chunk_super = step(super_step - last_chunk);
     p.Nt = pl.Nt; p.P = pl.P; p.T = pl.T; p.halo = pl.halo; p.n_tiles = pl.n_tiles; p.n_super = pl.n_super; p.total_q = pl.total_q;
     p.taps = pl.taps; p.ksteps = pl.Cw2 / 2; p.stages = pl.stages; p.resident = pl.resident; p.group_taps = pl.group_taps; p.groups = pl.groups;
-    p.tap_bytes = (int32_t)pl.tap_bytes; p.raw_words = (int32_t)pl.raw_words; p.x_bytes = (int32_t)pl.x_bytes;
+    p.tap_bytes = (int32_t)pl.tap_bytes; p.x_bytes = (int32_t)pl.x_bytes;
     p.n_xbuf = pl.n_xbuf; p.ahead = pl.ahead;
     p.off_tbl = (int32_t)pl.off_tbl; p.off_w = (int32_t)pl.off_w; p.off_x = (int32_t)pl.off_x;
     p.pad_zero = g.padding == LCE_PAD_SAME_ZERO;
