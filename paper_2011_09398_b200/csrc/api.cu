@@ -96,7 +96,9 @@ KernelPick pick_kernel(const lce_bconv2d_desc *desc, const ConvGeom &g, bool hav
             return tiled_buffers_ok && tiled_plan_info(g, &info) == LCE_OK ? PICK_TILED : PICK_NONE;
         default: break;
     }
-    if (desc->weights_packed && small_preferred(g)) return PICK_SMALL;
+    // a stem's patch kernel beats the latency kernel at every batch (one 224x224x3 image 2.0 against 4.1 us)
+    const bool stem = patch_covers(g) && g.out_type == LCE_OUT_BITPACKED && g.padding != LCE_PAD_SAME_ZERO;
+    if (desc->weights_packed && !stem && small_preferred(g)) return PICK_SMALL;
     if (have_tensor_image && tensor_preferred(g) && tensor_covers(g)) return PICK_TENSOR;
     if (patch_covers(g)) return PICK_PATCH;
     if (tiled_buffers_ok && tiled_plan_info(g, &info) == LCE_OK) return PICK_TILED;
@@ -187,7 +189,7 @@ lce_status dispatch(const Prepared &p, const uint32_t *input, const uint32_t *we
     const auto part = [&](size_t off) { return packed && off ? reinterpret_cast<const uint32_t *>(reinterpret_cast<const char *>(weights) + off) : nullptr; };
     switch (p.pick) {
         case PICK_DIRECT: return launch_bconv_direct(p.g, input, weights, multiplier, bias, thresholds, output, s);
-        case PICK_PATCH: return launch_bconv_patch(p.g, input, weights, multiplier, bias, thresholds, output, s);
+        case PICK_PATCH: return launch_bconv_patch(p.g, input, weights, packed, multiplier, bias, thresholds, output, s);
         case PICK_TILED: return launch_bconv_tiled(p.g, input, weights, part(p.parts.tiled), multiplier, bias, thresholds, output, s, residual, out_packed);
         case PICK_TENSOR: return launch_bconv_tensor(p.launch, input, part(p.parts.tensor), multiplier, bias, thresholds, output, s, residual, out_packed);
         case PICK_SMALL: return launch_bconv_small(p.launch, input, weights, part(p.parts.small), multiplier, bias, thresholds, output, s, residual, out_packed);

@@ -4,9 +4,19 @@
 // output on 27 useful bits; here the taps' Cin bits are first gathered into a single "patch"
 // word per pixel (im2col at bit granularity), the weights of a channel into a matching word, and
 // the accumulator is K - 2*popcount(patch XOR weight word): one XOR + POPC per output.
-// A thread owns one output pixel and walks all output channels, 32 at a time, so that it can
-// write whole bit-packed output words without any cross-lane traffic.
+//
+// Bit-packed output (the stem of a binarized network) runs on the warp-level integer matrix instruction: a patch word
+// is exactly its depth of 32, so one m16n8k32 gives 128 popcount(a AND w) for 16 channels x 8 pixels (the bit encoding
+// of bconv_small.cu, with lane q of a quad taking the bits q and q + 4 of every byte).  Up to 27 bits (3x3x3) leave
+// five bits of the word free: they carry popcount(a) in binary, with weights that take 64 of it off, and the
+// threshold is the instruction's third operand, so an output bit is the sign of a matrix result with no arithmetic
+// behind it.  What bounds it is the logic pipe: the gather (nine words per pixel) and collecting those signs.
+// 224x224x3 -> 32, stride 2: batch 256 43 -> 36 us (the popcount loop before it was bound by the popcount unit), batch
+// 64 17 -> 11 us, one image 4.6 -> 2.0 us.
+// Other outputs and zero-padding: a thread owns one output pixel and walks all output channels, 32 at a time.
 #include "common.cuh"
+#include "mx_common.cuh"
+#include "u8_mma.cuh"
 
 namespace lce {
 namespace {
@@ -33,7 +43,6 @@ bconv_patch_kernel(const PatchParams p)
     uint32_t *sWord = smem;                                             // [cout_pad] weight patch words
     int32_t *sThr = reinterpret_cast<int32_t *>(smem + cout_pad);       // [cout_pad]
     int32_t *sWsum = reinterpret_cast<int32_t *>(smem + 2 * cout_pad);  // [cout_pad][taps], zero-padding only
-    // then [cout_pad] (word, popcount threshold) pairs for the bit-packed fast path
     const uint32_t mask = p.Cin >= 32 ? 0xffffffffu : ((1u << p.Cin) - 1u);
 
     for (int o = threadIdx.x; o < cout_pad; o += kThreads) {
@@ -53,91 +62,6 @@ bconv_patch_kernel(const PatchParams p)
     __syncthreads();
 
     const int K = taps * p.Cin;
-
-    if (p.out_type == LCE_OUT_BITPACKED && p.padding != LCE_PAD_SAME_ZERO) {
-        // Bit-packed output without a zero-padding correction (the stem of a binarized network):
-        // acc < thr  <=>  K - 2*popc < thr  <=>  popc > floor((K - thr) / 2), so a channel is one
-        // 64-bit shared-memory read (weight word, popcount threshold), XOR, POPC, compare, OR.  Two
-        // pixels per thread share that read.
-        __syncthreads();  // sWord / sThr are complete; rewrite them as (word, popcount threshold) pairs
-        uint2 *sPair = reinterpret_cast<uint2 *>(smem + (2 + taps) * cout_pad);
-        for (int o = threadIdx.x; o < cout_pad; o += kThreads) {
-            int32_t t = INT32_MAX;  // pad channels: never set
-            if (o < p.Cout) t = (int32_t)(((int64_t)K - (int64_t)sThr[o]) >> 1);
-            sPair[o] = make_uint2(sWord[o], (uint32_t)t);
-        }
-        __syncthreads();
-        const int64_t stride = (int64_t)gridDim.x * kThreads;
-        // (image, row, column) of the thread's two pixels, advanced by 2*stride pixels per iteration
-        // with carries instead of two divisions per pixel
-        const int64_t step = 2 * stride;
-        const int step_ow = (int)(step % p.OW);
-        const int64_t step_rows = step / p.OW;
-        const int step_oh = (int)(step_rows % p.OH), step_n = (int)(step_rows / p.OH);
-        int pn[2], poh[2], pow_[2];
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int64_t m = (int64_t)blockIdx.x * kThreads + threadIdx.x + q * stride;
-            const int64_t r = m / p.OW;
-            pow_[q] = (int)(m - r * p.OW);
-            pn[q] = (int)(r / p.OH);
-            poh[q] = (int)(r - (int64_t)pn[q] * p.OH);
-        }
-        for (int64_t m0 = (int64_t)blockIdx.x * kThreads + threadIdx.x; m0 < p.M; m0 += step) {
-            const int64_t mm[2] = {m0, m0 + stride};
-            uint32_t patch[2] = {0u, 0u};
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const int n = pn[q], oh = poh[q], ow = pow_[q];
-                pow_[q] += step_ow;
-                poh[q] += step_oh;
-                pn[q] += step_n;
-                if (pow_[q] >= p.OW) { pow_[q] -= p.OW; ++poh[q]; }
-                if (poh[q] >= p.OH) { poh[q] -= p.OH; ++pn[q]; }
-                if (mm[q] >= p.M) continue;
-                const int iy0 = oh * p.sh - p.pt, ix0 = ow * p.sw - p.pl;
-                const uint32_t *img = p.in + (int64_t)n * p.H * p.W;
-                if (taps == 9 && p.KW == 3 && iy0 >= 0 && iy0 + 2 < p.H && ix0 >= 0 && ix0 + 2 < p.W) {
-                    // 3x3 window inside the image (all but the border pixels): nine loads from three row
-                    // pointers, nothing to test per tap
-                    const uint32_t *r0 = img + iy0 * p.W + ix0, *r1 = r0 + p.W, *r2 = r1 + p.W;
-                    uint32_t v[9];
-#pragma unroll
-                    for (int kx = 0; kx < 3; ++kx) {
-                        v[kx] = __ldg(r0 + kx);
-                        v[3 + kx] = __ldg(r1 + kx);
-                        v[6 + kx] = __ldg(r2 + kx);
-                    }
-                    uint32_t acc_patch = 0u;
-#pragma unroll
-                    for (int t = 8; t >= 0; --t) acc_patch = (acc_patch << p.Cin) | (v[t] & mask);  // Horner: tap t ends at bit t*Cin
-                    patch[q] = acc_patch;
-                    continue;
-                }
-                for (int ky = 0; ky < p.KH; ++ky) {
-                    const int iy = iy0 + ky;
-                    for (int kx = 0; kx < p.KW; ++kx) {
-                        const int ix = ix0 + kx;
-                        if (iy >= 0 && iy < p.H && ix >= 0 && ix < p.W)
-                            patch[q] |= (__ldg(img + iy * p.W + ix) & mask) << ((ky * p.KW + kx) * p.Cin);
-                    }
-                }
-            }
-            for (int wd = 0; wd < p.Cow; ++wd) {
-                uint32_t bits0 = 0u, bits1 = 0u;
-#pragma unroll
-                for (int j = 31; j >= 0; --j) {
-                    // popc > t  <=>  t - popc < 0: the output bit is a sign bit, shifted in from the top
-                    const uint2 wt = sPair[wd * 32 + j];
-                    bits0 = __funnelshift_l(wt.y - (uint32_t)__popc(patch[0] ^ wt.x), bits0, 1);
-                    bits1 = __funnelshift_l(wt.y - (uint32_t)__popc(patch[1] ^ wt.x), bits1, 1);
-                }
-                static_cast<uint32_t *>(p.out)[mm[0] * p.Cow + wd] = bits0;
-                if (mm[1] < p.M) static_cast<uint32_t *>(p.out)[mm[1] * p.Cow + wd] = bits1;
-            }
-        }
-        return;
-    }
 
     for (int m = blockIdx.x * kThreads + threadIdx.x; m < p.M; m += gridDim.x * kThreads) {
         const int r = m / p.OW, ow = m - r * p.OW;
@@ -187,6 +111,197 @@ bconv_patch_kernel(const PatchParams p)
     }
 }
 
+// The taps' Cin bits of one output pixel as one word: tap t at bit t * Cin, taps outside the image zero (= +1.0).
+// 3x3 filters: the nine words are asked for (PatchWords) well before they are put together, so that the loads of a
+// warp's next pixels are in flight while it works on these.
+struct PatchWords {
+    uint32_t v[9];
+};
+
+__device__ __forceinline__ PatchWords load_patch3(const PatchParams &p, int n, int oh, int ow, bool exists)
+{
+    const int y = oh * p.sh - p.pt, x = ow * p.sw - p.pl;
+    const uint32_t *at = p.in + ((int64_t)n * p.H + y) * p.W + x;
+    PatchWords w;
+    if (__all_sync(0xffffffffu, exists && y >= 0 && x >= 0 && y + 2 < p.H && x + 2 < p.W)) {  // nothing to test
+#pragma unroll
+        for (int kx = 0; kx < 3; ++kx) {
+            w.v[kx] = __ldg(at + kx);
+            w.v[3 + kx] = __ldg(at + p.W + kx);
+            w.v[6 + kx] = __ldg(at + 2 * p.W + kx);
+        }
+        return w;
+    }
+#pragma unroll
+    for (int ky = 0; ky < 3; ++ky) {
+        const bool row = exists && (unsigned)(y + ky) < (unsigned)p.H;
+#pragma unroll
+        for (int kx = 0; kx < 3; ++kx) w.v[3 * ky + kx] = row && (unsigned)(x + kx) < (unsigned)p.W ? __ldg(at + kx) : 0u;
+        at += p.W;
+    }
+    return w;
+}
+
+// Horner with `scale` = 2^Cin: tap t ends at bit t * Cin (pad bits of a word are 0).  Multiply-adds: the logic pipe is the
+// busy one.
+__device__ __forceinline__ uint32_t put_together(const PatchWords &w, uint32_t scale)
+{
+    uint32_t patch = w.v[8];
+#pragma unroll
+    for (int t = 7; t >= 0; --t) asm("mad.lo.u32 %0, %0, %1, %2;" : "+r"(patch) : "r"(scale), "r"(w.v[t]));
+    return patch;
+}
+
+__device__ __forceinline__ uint32_t gather_patch(const PatchParams &p, int n, int oh, int ow, uint32_t mask)
+{
+    const int iy0 = oh * p.sh - p.pt, ix0 = ow * p.sw - p.pl;
+    const uint32_t *img = p.in + (int64_t)n * p.H * p.W;
+    uint32_t patch = 0u;
+    for (int ky = 0; ky < p.KH; ++ky) {
+        const int iy = iy0 + ky;
+        for (int kx = 0; kx < p.KW; ++kx) {
+            const int ix = ix0 + kx;
+            if (iy >= 0 && iy < p.H && ix >= 0 && ix < p.W) patch |= (__ldg(img + iy * p.W + ix) & mask) << ((ky * p.KW + kx) * p.Cin);
+        }
+    }
+    return patch;
+}
+
+// Bit-packed output, one-padding or none.  A warp takes 32 consecutive output pixels at a time: lane = pixel for the
+// gather, then four groups of 8 pixels x 32 channels.  Row r of matrix tile t is channel 4 (r % 8) + 2 t + r / 8 of the
+// word, so that a lane's four sums of a pixel are four neighbouring bits; three exchanges put the word together, and
+// every lane ends up with the word of one of the 32 pixels.  COUNTED: K <= 27, popcount(a) travels in the word.
+constexpr int kLaneWords = 12;  // per lane and 32 channels: eight operand registers, four compare constants
+
+template <bool ONE_WORD, bool COUNTED>
+__global__ void __launch_bounds__(kThreads)
+bconv_patch_bits_kernel(const PatchParams p, int packed)
+{
+    extern __shared__ __align__(16) uint32_t smem[];  // [Cow][3][32 lanes][4]
+    const int taps = p.KH * p.KW, K = taps * p.Cin;
+    const uint32_t mask = p.Cin >= 32 ? 0xffffffffu : ((1u << p.Cin) - 1u);
+    const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // load-time packed weights are constants of the model; plain words may come from the kernel before
+    if (!packed) asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (int wd = threadIdx.x >> 5; wd < p.Cow; wd += kThreads / 32) {
+        uint32_t a[8];
+        int32_t c[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int o = wd * 32 + 4 * g + i;
+            uint32_t word = 0u;
+            int32_t thr = -K - 1;  // pad channels: bit 0
+            if (o < p.Cout) {
+                for (int t = 0; t < taps; ++t) word |= (__ldg(p.w + (int64_t)o * taps + t) & mask) << (t * p.Cin);
+                thr = max(-K - 1, min(K + 1, __ldg(p.thr + o)));
+            }
+            // K - 2 popc(a) - 2 popc(w) + 4 popc(a AND w) < thr  <=>  0 < L + 64 popc(a) - 128 popc(a AND w), all
+            // multiples of 32, so the output bit is the complement of the sign of that minus one
+            c[i] = 32 * (thr - K) + 64 * __popc(word) - 1;
+            // minus 2^(7 - b) for bit b of a byte, as signed bytes; the five count bits 27 .. 31 (bits 3 .. 7 of the last
+            // byte, 2^(3 + i) for the digit 2^i): 8
+            const auto operand = [&](int b) {
+                uint32_t v = 0u;
+                for (int byte = 0; byte < 4; ++byte) {
+                    const int bit = 8 * byte + b;
+                    const uint32_t x = bit >= 27 ? 8u : (word >> bit & 1u) ? (uint32_t)(-(1 << (7 - b))) & 0xFFu : 0u;
+                    v |= x << (8 * byte);
+                }
+                return v;
+            };
+            a[(i >> 1) * 4 + (i & 1)] = COUNTED ? operand(q) : reverse_in_bytes(word) & (0x80808080u >> q);
+            a[(i >> 1) * 4 + 2 + (i & 1)] = COUNTED ? operand(q + 4) : reverse_in_bytes(word) & (0x08080808u >> q);
+        }
+        uint4 *slot = reinterpret_cast<uint4 *>(smem) + wd * 96 + lane;
+        slot[0] = make_uint4(a[0], a[1], a[2], a[3]);
+        slot[32] = make_uint4(a[4], a[5], a[6], a[7]);
+        slot[64] = make_uint4((uint32_t)c[0], (uint32_t)c[1], (uint32_t)c[2], (uint32_t)c[3]);
+    }
+    const uint32_t a_lo = 0x01010101u << q, a_hi = 0x10101010u << q;
+    // image, row and column of the lane's pixel, advanced by the grid's stride with carries
+    const int step = gridDim.x * kThreads;
+    const int step_ow = step % p.OW, step_rows = step / p.OW, step_oh = step_rows % p.OH, step_n = step_rows / p.OH;
+    int64_t m0 = blockIdx.x * kThreads + (int)(threadIdx.x & ~31u);
+    int n, oh, ow;
+    {
+        const int m = (int)m0 + lane, r = m / p.OW;
+        ow = m - r * p.OW;
+        n = r / p.OH;
+        oh = r - n * p.OH;
+    }
+    __syncthreads();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const uint4 *slots = reinterpret_cast<const uint4 *>(smem) + lane;
+    uint4 w0 = slots[0], w1 = slots[32], c = slots[64];
+    const uint32_t scale = 1u << p.Cin, nibble_at = 1u << (4 * g);
+    const bool square3 = p.KH == 3 && p.KW == 3;
+    PatchWords next{};
+    if (square3) next = load_patch3(p, n, oh, ow, m0 + lane < p.M);
+    for (; m0 < p.M; m0 += step) {
+        const uint32_t patch = square3 ? put_together(next, scale) : m0 + lane < p.M ? gather_patch(p, n, oh, ow, mask) : 0u;
+        ow += step_ow;
+        oh += step_oh;
+        n += step_n;
+        if (ow >= p.OW) { ow -= p.OW; ++oh; }
+        if (oh >= p.OH) { oh -= p.OH; ++n; }
+        if (square3) next = load_patch3(p, n, oh, ow, m0 + step + lane < p.M);
+        const int ones = __popc(patch);
+        const uint32_t operand = COUNTED ? patch | (uint32_t)ones << 27 : patch;
+        uint32_t b0[4], b1[4];
+        int p0[4], p1[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t word = __shfl_sync(0xffffffffu, operand, 8 * i + g);
+            b0[i] = word & a_lo;
+            b1[i] = word & a_hi;
+            if (!COUNTED) {
+                p0[i] = __shfl_sync(0xffffffffu, 64 * ones, 8 * i + 2 * q);
+                p1[i] = __shfl_sync(0xffffffffu, 64 * ones, 8 * i + 2 * q + 1);
+            }
+        }
+        const int64_t pixel = m0 + (g >> 1) * 8 + 2 * q + (g & 1);
+        for (int wd = 0; wd < (ONE_WORD ? 1 : p.Cow); ++wd) {
+            if (!ONE_WORD) { w0 = slots[wd * 96]; w1 = slots[wd * 96 + 32]; c = slots[wd * 96 + 64]; }
+            uint32_t mine = 0u;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                int d0[4], d1[4];
+                if (COUNTED) {
+                    mma_s8u8(d0, w0.x, w0.y, w0.z, w0.w, b0[i], b1[i], (int)c.x, (int)c.x, (int)c.y, (int)c.y);
+                    mma_s8u8(d1, w1.x, w1.y, w1.z, w1.w, b0[i], b1[i], (int)c.z, (int)c.z, (int)c.w, (int)c.w);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) d0[k] = d1[k] = 0;
+                    mma_u8(d0, w0.x, w0.y, w0.z, w0.w, b0[i], b1[i]);
+                    mma_u8(d1, w1.x, w1.y, w1.z, w1.w, b0[i], b1[i]);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int more = k & 1 ? p1[i] : p0[i];
+                        d0[k] = (int)(k & 2 ? c.y : c.x) + more - d0[k];
+                        d1[k] = (int)(k & 2 ? c.w : c.z) + more - d1[k];
+                    }
+                }
+                // the sign bits of four channels of a pixel, the lowest channel last
+                const auto nibble = [&](int x0, int x1, int x2, int x3) {
+                    uint32_t v = (uint32_t)x3 >> 31;
+                    v = __funnelshift_l((uint32_t)x2, v, 1);
+                    v = __funnelshift_l((uint32_t)x1, v, 1);
+                    v = __funnelshift_l((uint32_t)x0, v, 1);
+                    asm("mul.lo.u32 %0, %0, %1;" : "+r"(v) : "r"(nibble_at));
+                    return v;
+                };
+                const uint32_t n0 = nibble(d0[0], d0[2], d1[0], d1[2]), n1 = nibble(d0[1], d0[3], d1[1], d1[3]);
+                uint32_t v = (g & 1 ? n1 : n0) | __shfl_xor_sync(0xffffffffu, g & 1 ? n0 : n1, 4);
+                v |= __shfl_xor_sync(0xffffffffu, v, 8);
+                v |= __shfl_xor_sync(0xffffffffu, v, 16);
+                if ((g >> 1) == i) mine = ~v;
+            }
+            if (pixel < p.M) static_cast<uint32_t *>(p.out)[pixel * p.Cow + wd] = mine;
+        }
+    }
+}
+
 }  // namespace
 
 bool patch_covers(const ConvGeom &g)
@@ -194,7 +309,7 @@ bool patch_covers(const ConvGeom &g)
     return g.Cw == 1 && g.KH * g.KW > 1 && g.KH * g.KW * g.Cin <= 32 && g.M < (1ll << 31) - 4096 && g.Cow <= 256;
 }
 
-lce_status launch_bconv_patch(const ConvGeom &g, const uint32_t *in, const uint32_t *w, const float *mult,
+lce_status launch_bconv_patch(const ConvGeom &g, const uint32_t *in, const uint32_t *w, bool packed, const float *mult,
                               const float *bias, const int32_t *thr, void *out, cudaStream_t s)
 {
     if (!patch_covers(g)) return LCE_ERR_UNSUPPORTED;
@@ -203,7 +318,24 @@ lce_status launch_bconv_patch(const ConvGeom &g, const uint32_t *in, const uint3
     p.N = g.N; p.H = g.H; p.W = g.W; p.Cin = g.Cin; p.Cout = g.Cout; p.Cow = g.Cow;
     p.KH = g.KH; p.KW = g.KW; p.sh = g.sh; p.sw = g.sw; p.OH = g.OH; p.OW = g.OW; p.pt = g.pt; p.pl = g.pl;
     p.M = (int32_t)g.M; p.padding = g.padding; p.out_type = g.out_type; p.activation = g.activation;
-    const size_t smem = (size_t)g.Cow * 32 * (4 + g.KH * g.KW) * 4;
+    if (g.out_type == LCE_OUT_BITPACKED && g.padding != LCE_PAD_SAME_ZERO) {
+        // the blocks that fit at once (64 registers: four per SM), grid-stride beyond that: a block begins with its operands
+        const int64_t bits_blocks = (g.M + kThreads - 1) / kThreads;
+        const dim3 grid((unsigned)(bits_blocks < 148 * 4 ? bits_blocks : 148 * 4));
+        const size_t bits_smem = (size_t)g.Cow * 32 * kLaneWords * 4;
+        const bool counted = g.KH * g.KW * g.Cin <= 27;
+        if (g.Cow == 1)
+            return counted ? launch_dependent(bconv_patch_bits_kernel<true, true>, grid, kThreads, bits_smem, s, p, (int)packed)
+                           : launch_dependent(bconv_patch_bits_kernel<true, false>, grid, kThreads, bits_smem, s, p, (int)packed);
+        static SmemOptIn opted, opted_counted;
+        if (counted) {
+            if (!opted_counted.ensure(bconv_patch_bits_kernel<false, true>, bits_smem)) return LCE_ERR_CUDA;
+            return launch_dependent(bconv_patch_bits_kernel<false, true>, grid, kThreads, bits_smem, s, p, (int)packed);
+        }
+        if (!opted.ensure(bconv_patch_bits_kernel<false, false>, bits_smem)) return LCE_ERR_CUDA;
+        return launch_dependent(bconv_patch_bits_kernel<false, false>, grid, kThreads, bits_smem, s, p, (int)packed);
+    }
+    const size_t smem = (size_t)g.Cow * 32 * (2 + g.KH * g.KW) * 4;
     if (smem > 48 * 1024) return LCE_ERR_UNSUPPORTED;
     // one wave of resident blocks (8 x 256 threads per SM), grid-stride beyond that: every block pays
     // for building the weight words in shared memory, so fewer, longer-lived blocks are cheaper

@@ -29,6 +29,7 @@
 //     kernel of the stream drains.
 #include "common.cuh"
 #include "mx_common.cuh"
+#include "u8_mma.cuh"
 
 namespace lce {
 namespace {
@@ -91,22 +92,6 @@ __device__ __forceinline__ int load_early(const void *p)
     int v;
     asm volatile("ld.global.nc.b32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
-}
-
-// D += A B on 16 x 8 outputs, 32 deep: unsigned bytes, 32-bit sums
-__device__ __forceinline__ void mma_u8(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
-{
-    asm("mma.sync.aligned.m16n8k32.row.col.s32.u8.u8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
-                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-// the bits of every byte in reverse order
-__host__ __device__ __forceinline__ uint32_t reverse_in_bytes(uint32_t w)
-{
-    w = ((w >> 4) & 0x0F0F0F0Fu) | ((w & 0x0F0F0F0Fu) << 4);
-    w = ((w >> 2) & 0x33333333u) | ((w & 0x33333333u) << 2);
-    return ((w >> 1) & 0x55555555u) | ((w & 0x55555555u) << 1);
 }
 
 enum { SMALL_BITS = 0, SMALL_FLOAT = 1, SMALL_GENERAL = 2 };  // GENERAL: int32 output, shortcut add, re-quantised copy

@@ -145,9 +145,10 @@ lce_status launch_bconv_tiled(const ConvGeom &g, const uint32_t *in, const uint3
                               const float *mult, const float *bias, const int32_t *thr, void *out, cudaStream_t s,
                               const float *residual = nullptr, uint32_t *out_packed = nullptr,
                               const float *in_f32 = nullptr);
-// One-word-patch kernel for tiny channel counts (KH*KW*Cin <= 32); plain weights only.
+// One-word-patch kernel for tiny channel counts (KH*KW*Cin <= 32); plain words, `packed` when they are the first part
+// of a packed-weights buffer.
 bool patch_covers(const ConvGeom &g);
-lce_status launch_bconv_patch(const ConvGeom &g, const uint32_t *in, const uint32_t *w, const float *mult,
+lce_status launch_bconv_patch(const ConvGeom &g, const uint32_t *in, const uint32_t *w, bool packed, const float *mult,
                               const float *bias, const int32_t *thr, void *out, cudaStream_t s);
 // Latency kernel for small layers (any filter, stride and channel count whose tile fits in shared memory).
 // w_image: the part of a packed-weights buffer launch_pack_weights_small wrote, or null to use the plain words.
