@@ -221,9 +221,11 @@ lce_status lce_bconv2d_pack_weights(const lce_bconv2d_desc *desc, const uint32_t
 /* Host-buffer form of lce_bconv2d, for callers whose tensors live in host memory: every data
  * pointer is a HOST pointer (pinned memory makes the copies asynchronous); `workspace` is a
  * DEVICE buffer of at least lce_bconv2d_host_workspace_bytes(desc) bytes that the call uses
- * for the device copies of input, weights, per-channel arrays and output.  Copies in, runs
- * the same kernel as lce_bconv2d (weights_packed must be 0), copies the output back, all on `stream`, and returns after
- * synchronising that stream.  LCE_ERR_WORKSPACE if workspace_bytes is too small. */
+ * for the device copies of input, weights, per-channel arrays and output, and where it pays for a packed
+ * copy of the weights (without that room, which earlier versions did not ask for, the call still runs, on
+ * the kernel for plain weights).  Copies in, runs the convolution (weights_packed must be 0; kernel
+ * AUTO also takes the kernels that want packed weights), copies the output back, all on `stream`, and
+ * returns after synchronising that stream.  LCE_ERR_WORKSPACE if workspace_bytes is too small. */
 size_t lce_bconv2d_host_workspace_bytes(const lce_bconv2d_desc *desc);
 lce_status lce_bconv2d_host(const lce_bconv2d_desc *desc, const uint32_t *input, const uint32_t *weights,
                             const float *multiplier, const float *bias, const int32_t *thresholds,

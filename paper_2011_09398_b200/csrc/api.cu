@@ -117,6 +117,18 @@ KernelPick pick_fused(const lce_bconv2d_desc *desc, const ConvGeom &g, const Wei
     return PICK_TILED;
 }
 
+// The host-buffer form brings plain weights along: the kernels that want packed ones are open to it, too, if there is
+// room in the workspace to pack them (`image_fits`; the latency kernel reads plain words).  28x28x128 at batch 64: the
+// XOR/POPC kernel 38 us, packing and the tensor-core kernel 10 us.
+KernelPick pick_host(const lce_bconv2d_desc *desc, const ConvGeom &g, bool image_fits)
+{
+    if (desc->kernel != LCE_KERNEL_AUTO) return pick_kernel(desc, g, false, true);
+    const bool stem = patch_covers(g);
+    if (!stem && small_preferred(g)) return PICK_SMALL;
+    if (!stem && image_fits && tensor_weight_image_bytes(g) > 0 && tensor_preferred(g)) return PICK_TENSOR;
+    return pick_kernel(desc, g, false, true);
+}
+
 // Everything about a call that follows from its descriptor: geometry, parts of the packed weights, which kernel and
 // the launch worked out for it.
 struct Prepared {
@@ -129,7 +141,7 @@ struct Prepared {
     KernelPick pick;
     PreparedLaunch launch;
 };
-enum { FORM_FUSED = 1, FORM_ROWS_UNALIGNED = 2 };  // float / int32 rows that are not on 16 bytes (relevant for out_c % 4 == 0)
+enum { FORM_FUSED = 1, FORM_ROWS_UNALIGNED = 2, FORM_HOST = 4, FORM_NO_IMAGE = 8 };  // float / int32 rows that are not on 16 bytes (relevant for out_c % 4 == 0)
 
 void prepare(const lce_bconv2d_desc *desc, int device, uint32_t form, Prepared *p)
 {
@@ -140,7 +152,7 @@ void prepare(const lce_bconv2d_desc *desc, int device, uint32_t form, Prepared *
     if (p->status != LCE_OK) return;
     p->parts = weight_parts(p->g);
     const bool rows_aligned = !(form & FORM_ROWS_UNALIGNED);
-    p->pick = form & FORM_FUSED ? pick_fused(desc, p->g, p->parts, rows_aligned) : pick_kernel(desc, p->g, desc->weights_packed && p->parts.tensor, rows_aligned);
+    p->pick = form & FORM_HOST ? pick_host(desc, p->g, !(form & FORM_NO_IMAGE)) : form & FORM_FUSED ? pick_fused(desc, p->g, p->parts, rows_aligned) : pick_kernel(desc, p->g, desc->weights_packed && p->parts.tensor, rows_aligned);
     if (p->pick == PICK_SMALL) p->status = prepare_bconv_small(p->g, &p->launch);
     if (p->pick == PICK_TENSOR) p->status = prepare_bconv_tensor(p->g, &p->launch);
 }
@@ -198,7 +210,8 @@ lce_status dispatch(const Prepared &p, const uint32_t *input, const uint32_t *we
 }
 
 struct HostLayout {
-    size_t in, w, mult, bias, thr, out, total;
+    size_t in, w, mult, bias, thr, out, total;  // total: what a call needs at least
+    size_t image;                               // beyond that, room for packed weights (0: of no use to this layer)
     size_t in_bytes, w_bytes, ch_bytes, out_bytes;
 };
 
@@ -217,6 +230,7 @@ HostLayout host_layout(const ConvGeom &g)
     L.thr = off;  off += round_up(L.ch_bytes, 256);
     L.out = off;  off += round_up(L.out_bytes, 256);
     L.total = off;
+    if (!patch_covers(g) && !small_preferred(g) && tensor_preferred(g)) L.image = round_up(tensor_weight_image_bytes(g), 256);
     return L;
 }
 
@@ -445,7 +459,8 @@ extern "C" size_t lce_bconv2d_host_workspace_bytes(const lce_bconv2d_desc *desc)
 {
     lce::ConvGeom g;
     if (lce::make_geom(desc, &g) != LCE_OK) return 0;
-    return lce::host_layout(g).total;
+    const lce::HostLayout L = lce::host_layout(g);
+    return L.total + L.image;
 }
 
 namespace lce {
@@ -464,18 +479,24 @@ lce_status host_conv(const lce_bconv2d_desc *desc, const uint32_t *input, const 
     if (workspace_bytes < L.total) return LCE_ERR_WORKSPACE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     char *ws = static_cast<char *>(workspace);
-    bool ok = cudaMemcpyAsync(ws + L.in, input, L.in_bytes, cudaMemcpyHostToDevice, s) == cudaSuccess;
-    ok = ok && cudaMemcpyAsync(ws + L.w, weights, L.w_bytes, cudaMemcpyHostToDevice, s) == cudaSuccess;
-    if (multiplier) ok = ok && cudaMemcpyAsync(ws + L.mult, multiplier, L.ch_bytes, cudaMemcpyHostToDevice, s) == cudaSuccess;
-    if (bias) ok = ok && cudaMemcpyAsync(ws + L.bias, bias, L.ch_bytes, cudaMemcpyHostToDevice, s) == cudaSuccess;
-    if (thresholds) ok = ok && cudaMemcpyAsync(ws + L.thr, thresholds, L.ch_bytes, cudaMemcpyHostToDevice, s) == cudaSuccess;
-    if (!ok) return LCE_ERR_CUDA;
-    const Prepared &p = prepared_for(desc, 0);
+    // the largest copy first: the rest is prepared while it runs
+    const auto copy_in = [&](size_t off, const void *src, size_t bytes) { return !src || cudaMemcpyAsync(ws + off, src, bytes, cudaMemcpyHostToDevice, s) == cudaSuccess; };
+    if (!copy_in(L.in, input, L.in_bytes) || !copy_in(L.w, weights, L.w_bytes) || !copy_in(L.mult, multiplier, L.ch_bytes) ||
+        !copy_in(L.bias, bias, L.ch_bytes) || !copy_in(L.thr, thresholds, L.ch_bytes))
+        return LCE_ERR_CUDA;
+    const Prepared &p = prepared_for(desc, FORM_HOST | (workspace_bytes < L.total + L.image ? FORM_NO_IMAGE : 0));
     if (p.status != LCE_OK) return p.status;
-    st = dispatch(p, reinterpret_cast<const uint32_t *>(ws + L.in), reinterpret_cast<const uint32_t *>(ws + L.w),
-                  multiplier ? reinterpret_cast<const float *>(ws + L.mult) : nullptr,
-                  bias ? reinterpret_cast<const float *>(ws + L.bias) : nullptr,
-                  thresholds ? reinterpret_cast<const int32_t *>(ws + L.thr) : nullptr, ws + L.out, s);
+    const auto at = [&](size_t off) { return reinterpret_cast<uint32_t *>(ws + off); };
+    const uint32_t *d_in = at(L.in), *d_w = at(L.w);
+    const float *d_mult = multiplier ? reinterpret_cast<const float *>(ws + L.mult) : nullptr, *d_bias = bias ? reinterpret_cast<const float *>(ws + L.bias) : nullptr;
+    const int32_t *d_thr = thresholds ? reinterpret_cast<const int32_t *>(ws + L.thr) : nullptr;
+    if (p.pick == PICK_TENSOR) {
+        if (tensor_timeout_flagged()) return LCE_ERR_DEVICE_TIMEOUT;
+        st = launch_pack_weights_tensor(g, d_w, ws + L.total, s);
+        if (st == LCE_OK) st = launch_bconv_tensor(p.launch, d_in, ws + L.total, d_mult, d_bias, d_thr, ws + L.out, s);
+    } else {
+        st = dispatch(p, d_in, d_w, d_mult, d_bias, d_thr, ws + L.out, s);
+    }
     if (st != LCE_OK) return st;
     if (cudaMemcpyAsync(output, ws + L.out, L.out_bytes, cudaMemcpyDeviceToHost, s) != cudaSuccess) return LCE_ERR_CUDA;
     if (synchronise && cudaStreamSynchronize(s) != cudaSuccess) return LCE_ERR_CUDA;

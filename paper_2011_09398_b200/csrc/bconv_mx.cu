@@ -1134,6 +1134,7 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
 // finisher warp
 __global__ void mx_pack_weights_kernel(const uint32_t *w, uint4 *image, int Cout, int Cin, int Cw, int Cw2, int taps, int n_blocks, int dup)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int64_t total = (int64_t)n_blocks * taps * Cw2 * 128;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int row = (int)(e & 127);
@@ -1339,9 +1340,9 @@ lce_status launch_pack_weights_tensor(const ConvGeom &g, const uint32_t *w, void
     const int64_t total = (int64_t)pl.n_blocks * pl.taps * pl.Cw2 * 128;
     const int64_t want = (total + 255) / 256;
     const int blocks = (int)(want < 4096 ? want : 4096);
-    mx_pack_weights_kernel<<<blocks, 256, 0, s>>>(w, static_cast<uint4 *>(image), g.Cout, g.Cin, g.Cw, pl.Cw2, pl.taps, pl.n_blocks, mx_dup(g));
+    const lce_status st = launch_dependent(mx_pack_weights_kernel, dim3((unsigned)blocks), 256, 0, s, w, static_cast<uint4 *>(image), g.Cout, g.Cin, g.Cw, pl.Cw2, pl.taps, pl.n_blocks, mx_dup(g));
     mx_flag_array(false);  // load time is the moment to set up the host-visible status word (it cannot be done under stream capture)
-    return launch_status();
+    return st;
 }
 
 lce_status tensor_plan_info(const ConvGeom &g, TensorPlanInfo *info)
