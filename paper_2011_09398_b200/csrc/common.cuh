@@ -185,6 +185,16 @@ lce_status tensor_device_status(int *status);
 lce_status tensor_device_status_reset();
 bool tensor_timeout_flagged();
 lce_status tensor_wait_probe(uint64_t limit_ns, cudaStream_t s);
+// Small copies from pinned host memory in one kernel; destinations on 16 bytes, sizes multiples of 4 below 2^31 in
+// all, empty ones allowed.  pinned_host_view: the device's view of a pinned host pointer, null for any other memory.
+constexpr int kHostCopies = 5;
+struct HostCopy {
+    const void *src;
+    void *dst;
+    size_t bytes;
+};
+void *pinned_host_view(const void *host);
+lce_status launch_host_copies(const HostCopy (&copies)[kHostCopies], cudaStream_t s);
 // Bytes of the tiled kernel's weight image for this geometry (0 if the kernel does not cover it).
 // Launch plan of the tiled kernels for a geometry (no buffers involved), for lce_bconv2d_plan.
 struct TiledPlanInfo {
