@@ -228,7 +228,7 @@ __device__ __forceinline__ MxPos mx_position(int f, const MxParams &p)
 // cost more than the arithmetic).
 struct MxLoad {
     int N, H, W, Cw, Wg, Hg, P, pt, pl, origin;  // origin: the words from pixel (-pt, -pl) to pixel (0, 0)
-    int row_words, image_words;                  // words of an input row and of an image
+    int col_words, row_words, image_words;       // words between positions of a grid column, row and image
     const uint32_t *in;
     MxStep across;                               // kLoaders positions
 };
@@ -268,7 +268,7 @@ __device__ __forceinline__ void mx_prefetch(const MxLoad &l, MxPos a, int count,
         const bool image = a.n < l.N;
         if (FORM == MX_S1) {
             const bool ok = image && (unsigned)(a.r - l.pt) < (unsigned)l.H && (unsigned)(a.c - l.pl) < (unsigned)l.W;
-            const int off = a.n * l.image_words + a.r * l.row_words + a.c * cw - l.origin;
+            const int off = a.n * l.image_words + a.r * l.row_words + a.c * l.col_words - l.origin;
             mx_copy_words<CW>(raw + j * cw, l.in + (ok ? off : 0), cw, cp_words, ok);
         } else {
             const int y = 2 * a.r - l.pt, x = 2 * a.c - l.pl;
@@ -948,9 +948,15 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
     if (tid < kLoaders) {
         ld.N = p.N; ld.H = p.H; ld.W = p.W; ld.Cw = p.Cw; ld.Wg = p.Wg; ld.Hg = p.Hg; ld.P = p.P; ld.pt = p.pt; ld.pl = p.pl;
         ld.in = p.in;
+        ld.col_words = p.Cw;
         ld.row_words = p.W * p.Cw;
         ld.image_words = p.H * ld.row_words;
         ld.origin = p.pt * ld.row_words + p.pl * p.Cw;
+        if (p.stride == 2 && p.n_phase == 1) {  // 1x1: every second pixel of every second row, none of them padding
+            ld.H = p.OH; ld.W = p.OW;
+            ld.col_words *= 2;
+            ld.row_words *= 2;
+        }
         ld.across = p.step_across;
         form = mx_form(p);
         stage = mx_position(first_tile * p.T * p.Nt + tid, p);
@@ -1167,6 +1173,7 @@ __global__ void mx_pack_weights_kernel(const uint32_t *w, uint4 *image, int Cout
 struct MxPlan {
     int Nt, P, T, stages, resident, group_taps, groups, n_blocks, ctas_x, n_tiles, n_super, total_q, Wg, Hg, n_phase, Cw2, taps, halo, n_xbuf, ahead;
     size_t raw_words, x_bytes, tap_bytes, off_tbl, off_w, off_x, smem;
+    double clocks;  // of a CTA's tiles by the cost model
 };
 
 constexpr size_t kSmemLimit = 227 * 1024;
@@ -1225,7 +1232,9 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
     const int64_t total_q = (int64_t)g.N * Hg * Wg;
     if (total_q >= (1ll << 31) - 4096 || g.M >= (1ll << 31)) return false;
     pl->Wg = Wg; pl->Hg = Hg; pl->halo = halo; pl->total_q = (int)total_q;
-    pl->n_phase = s * s;
+    // a 1x1 filter at stride 2 reads one phase of the four: staging that one alone took 64 images of 28x28x512 -> 512 from
+    // 19.5 to 7.3 us, of 56x56x256 -> 256 from 13.7 to 9.0
+    pl->n_phase = taps == 1 ? 1 : s * s;
     pl->Cw2 = g.Cw + (g.Cw & 1);
     pl->taps = taps;
     pl->tap_bytes = (size_t)pl->Cw2 * 2048;
@@ -1273,13 +1282,13 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
             // per group (wait for the stage, issue, hand the stage back: about 250 clocks on top of the MMAs)
             const double stream = resident ? 0.0 : (double)groups * fmax(fmax(group_taps * pl->tap_bytes / 38.0, 1300.0 / stages), 250.0 + group_taps * ksteps * mma1);
             // stride 2: four phases per position, staged two at a time where the geometry allows (MX_S2_PAIR)
-            const double per_position = s == 1 ? 1.0 : ((g.W & 1) == 0 && (g.pl & 1) == 0 && g.Cw <= 4) ? 2.0 : 3.0;
+            const double per_position = pl->n_phase == 1 ? 1.0 : ((g.W & 1) == 0 && (g.pl & 1) == 0 && g.Cw <= 4) ? 2.0 : 3.0;
             const double load = 400.0 + 8.0 * per_position * (nt + (double)halo / T);
             // with streamed weights the hand-overs of the ring and of the loaders do not hide each other (112x112x32 stride 2
             // at batch 256: 71 us streamed, 36 us resident, where the three terms alone call it a tie)
             const double cost = per_cta * (fmax(fmax(mma, stream), load) + 0.5 * fmin(stream, load) + 150.0);
             if (cost < best) {
-                best = cost;
+                best = pl->clocks = cost;
                 found = true;
                 pl->Nt = nt; pl->P = P; pl->T = T; pl->stages = stages; pl->resident = resident ? 1 : 0; pl->group_taps = group_taps; pl->groups = groups;
                 pl->n_tiles = n_tiles; pl->n_super = n_super; pl->ctas_x = ctas_x;
@@ -1354,6 +1363,8 @@ lce_status tensor_plan_info(const ConvGeom &g, TensorPlanInfo *info)
     info->weight_stages = pl.stages;
     info->weights_resident = pl.resident;
     info->shared_bytes = (int64_t)pl.smem;
+    info->clocks = pl.clocks;
+    info->phases = pl.n_phase;
     return LCE_OK;
 }
 

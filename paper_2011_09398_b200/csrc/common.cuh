@@ -175,8 +175,9 @@ lce_status launch_bconv_tensor(const PreparedLaunch &prepared, const uint32_t *i
                                const float *bias, const int32_t *thr, void *out, cudaStream_t s,
                                const float *residual = nullptr, uint32_t *out_packed = nullptr);
 struct TensorPlanInfo {
-    int32_t tile_positions, ctas, weight_stages, weights_resident;
+    int32_t tile_positions, ctas, weight_stages, weights_resident, phases;
     int64_t shared_bytes;
+    double clocks;  // of a CTA's share, by the cost model of the plan
 };
 lce_status tensor_plan_info(const ConvGeom &g, TensorPlanInfo *info);
 // Bounded device-side waits: status word, its reset, the host-visible flag (no synchronisation), and a
