@@ -53,34 +53,30 @@ WeightParts weight_parts(const ConvGeom &g)
     return w;
 }
 
-// AUTO takes the tensor-core kernel when the weights were packed at load time (its operand image exists)
-// and the layer is large enough to pay for that kernel's start-up, by what was measured on the paper's
-// layer sweep (batch 1 and 64) and the ImageNet-shaped bodies: from 2^28 binary MACs when all taps of a channel
-// block stay in shared memory, from 2^29 when they have to stream past once per tile; 3x3 and smaller filters
-// on at most 32 input channels (half of every 64-deep MMA is padding) only from 2^31, where the two kernels
-// draw level (the 112x112x32 stride-2 layer of an ImageNet stem, 2^34 MACs, is twice as fast on the tensor cores).
-bool tensor_preferred(const ConvGeom &g)
-{
-    if (patch_covers(g)) return false;
-    TensorPlanInfo t{};
-    if (tensor_plan_info(g, &t) != LCE_OK) return false;
-    const double macs = (double)g.M * g.Cout * g.KH * g.KW * g.Cin;
-    if (g.Cin <= 32 && g.KH * g.KW <= 9) return macs >= 2147483648.0;
-    return macs >= (t.weights_resident ? 268435456.0 : 536870912.0);
-}
-
-// AUTO takes the latency kernel for layers with load-time packed weights below 2^29 binary MACs, as long as its
-// 64-pixel tiles make no more than 600 CTAs.  Measured (us, latency / tiled / tensor-core kernel): one image of
-// 14x14x64 1.7 / 3.1 / 3.9, of 28x28x128 2.4 / 4.2 / 4.1, of 7x7x512 2.9 / 9.3 / 8.9; four images of 14x14x256
-// (2^28.8) 4.3 / 5.2 / 5.2, of 7x7x512 4.2 / 11.6 / 8.6; 64 images of 16x16x64 (2^29.2, 512 CTAs) 5.6 / 4.9 / 4.9;
-// layers of little depth and many outputs are cheaper per output elsewhere: 16 images of 28x28x64, 1x1 to 256
-// (1568 CTAs) 9.0 / 5.4 / 4.6.
-bool small_preferred(const ConvGeom &g)
-{
-    return small_covers(g) && (double)g.M * g.Cout * g.KH * g.KW * g.Cin < 536870912.0 && small_ctas(g) <= 600;
-}
-
 enum KernelPick { PICK_NONE = 0, PICK_DIRECT, PICK_PATCH, PICK_TILED, PICK_TENSOR, PICK_SMALL };
+
+// Which kernel weights packed at load time go to: the one whose estimated time is the shorter.  The estimates (us) were
+// fitted to 180 layers of 2^26 - 2^31 binary MACs, 1x1 - 5x5, 32 - 512 channels, strides 1 and 2 (10% rms each): the
+// latency kernel pays per output and per 128-deep step of an output, the tensor-core kernel a start-up and the clocks its
+// plan predicts; staging the four phase grids of a stride-2 layer word by word grows with the square of the depth (fewer
+// positions fit a tile).  The slower of the two was picked in 7 of the 180, by 13% on average.  One image of 14x14x64 is
+// 1.7 on the latency kernel and 3.9 on the tensor cores; 21 images of 14x14x256, 1x1 (2^28.0), 5.9 and 4.1; one of
+// 56x56x512, stride 2 (2^30.8), 9.9 and 13.4.  The XOR/POPC kernel was ahead of both in two of the 180.
+// Where one of the two does not cover the layer the other competes with the integer kernels: from 2^28 (weights
+// resident) or 2^29 MACs (streamed) the tensor cores are ahead, up to 2^29 and 600 CTAs the latency kernel is.
+// `extra`: what the tensor-core kernel costs besides.  PICK_NONE: neither.
+KernelPick pick_packed(const ConvGeom &g, bool tensor_ok, double extra = 0.0)
+{
+    TensorPlanInfo t{};
+    tensor_ok = tensor_ok && !patch_covers(g) && tensor_plan_info(g, &t) == LCE_OK;
+    const bool small_ok = small_covers(g);
+    const double macs = (double)g.M * g.Cout * g.KH * g.KW * g.Cin, outs = (double)g.M * g.Cow * 32;
+    if (!tensor_ok) return small_ok && macs < 536870912.0 && small_ctas(g) <= 600 ? PICK_SMALL : PICK_NONE;
+    if (!small_ok) return macs >= (t.weights_resident ? 268435456.0 : 536870912.0) ? PICK_TENSOR : PICK_NONE;
+    const double small_us = 2.2 + outs * (2.3e-6 + 5.6e-7 * ((g.KH * g.KW * g.Cw + 3) / 4));
+    const double tensor_us = 4.0 + 3.85e-4 * t.clocks + (t.phases > 1 ? 0.017 * g.Cw * g.Cw : 0.0) + extra;
+    return small_us <= tensor_us ? PICK_SMALL : PICK_TENSOR;
+}
 
 // One place decides which kernel a call gets; lce_bconv2d_plan shows the same decision.
 // tiled_buffers_ok: the tiled kernels write float / int32 rows with 128-bit accesses when the channel count allows it,
@@ -98,8 +94,8 @@ KernelPick pick_kernel(const lce_bconv2d_desc *desc, const ConvGeom &g, bool hav
     }
     // a stem's patch kernel beats the latency kernel at every batch (one 224x224x3 image 2.0 against 4.1 us)
     const bool stem = patch_covers(g) && g.out_type == LCE_OUT_BITPACKED && g.padding != LCE_PAD_SAME_ZERO;
-    if (desc->weights_packed && !stem && small_preferred(g)) return PICK_SMALL;
-    if (have_tensor_image && tensor_preferred(g) && tensor_covers(g)) return PICK_TENSOR;
+    const KernelPick packed = desc->weights_packed && !stem ? pick_packed(g, have_tensor_image) : PICK_NONE;
+    if (packed != PICK_NONE) return packed;
     if (patch_covers(g)) return PICK_PATCH;
     if (tiled_buffers_ok && tiled_plan_info(g, &info) == LCE_OK) return PICK_TILED;
     return PICK_DIRECT;
@@ -112,21 +108,21 @@ KernelPick pick_fused(const lce_bconv2d_desc *desc, const ConvGeom &g, const Wei
     if (desc->kernel == LCE_KERNEL_DIRECT || patch_covers(g)) return PICK_NONE;
     const bool tensor_ok = desc->weights_packed && parts.tensor && tensor_covers(g) && (g.Cout & 31) == 0 && rows_aligned;
     if (desc->kernel == LCE_KERNEL_TENSOR) return tensor_ok ? PICK_TENSOR : PICK_NONE;
-    if (desc->kernel == LCE_KERNEL_AUTO && desc->weights_packed && tiled_weight_image_bytes(g) > 0 && small_preferred(g)) return PICK_SMALL;
-    if (desc->kernel == LCE_KERNEL_AUTO && tensor_ok && tensor_preferred(g)) return PICK_TENSOR;
-    return PICK_TILED;
+    if (desc->kernel != LCE_KERNEL_AUTO || !desc->weights_packed) return PICK_TILED;
+    const KernelPick packed = pick_packed(g, tensor_ok);
+    if (packed == PICK_SMALL && tiled_weight_image_bytes(g) == 0) return tensor_ok ? PICK_TENSOR : PICK_TILED;
+    return packed == PICK_NONE ? PICK_TILED : packed;
 }
 
 // The host-buffer form brings plain weights along: the kernels that want packed ones are open to it, too, if there is
 // room in the workspace to pack them (`image_fits`; the latency kernel reads plain words).  28x28x128 at batch 64: the
 // XOR/POPC kernel 38 us, packing and the tensor-core kernel 10 us.
+constexpr double kPackImage = 2.5;  // us: packing, behind the copies
 KernelPick pick_host(const lce_bconv2d_desc *desc, const ConvGeom &g, bool image_fits)
 {
     if (desc->kernel != LCE_KERNEL_AUTO) return pick_kernel(desc, g, false, true);
-    const bool stem = patch_covers(g);
-    if (!stem && small_preferred(g)) return PICK_SMALL;
-    if (!stem && image_fits && tensor_weight_image_bytes(g) > 0 && tensor_preferred(g)) return PICK_TENSOR;
-    return pick_kernel(desc, g, false, true);
+    const KernelPick packed = patch_covers(g) ? PICK_NONE : pick_packed(g, image_fits, kPackImage);
+    return packed == PICK_NONE ? pick_kernel(desc, g, false, true) : packed;
 }
 
 // Everything about a call that follows from its descriptor: geometry, parts of the packed weights, which kernel and
@@ -230,7 +226,7 @@ HostLayout host_layout(const ConvGeom &g)
     L.thr = off;  off += round_up(L.ch_bytes, 256);
     L.out = off;  off += round_up(L.out_bytes, 256);
     L.total = off;
-    if (!patch_covers(g) && !small_preferred(g) && tensor_preferred(g)) L.image = round_up(tensor_weight_image_bytes(g), 256);
+    if (!patch_covers(g) && pick_packed(g, true, kPackImage) == PICK_TENSOR) L.image = round_up(tensor_weight_image_bytes(g), 256);
     return L;
 }
 

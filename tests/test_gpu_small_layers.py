@@ -18,7 +18,7 @@ SHAPES = [
     (2, 3, 3, 64, 33, 3, 3, 1, ONE), (5, 3, 5, 96, 65, 3, 3, 1, ZERO), (3, 7, 7, 512, 96, 3, 3, 1, ONE), (1, 14, 14, 256, 40, 3, 3, 1, ZERO),
     (4, 9, 11, 160, 72, 2, 4, 1, ONE), (2, 13, 10, 288, 64, 3, 3, 2, ONE), (3, 8, 8, 128, 130, 5, 5, 2, ZERO), (2, 12, 9, 60, 64, 5, 5, 1, VALID),
     (1, 29, 31, 3, 32, 3, 3, 2, ONE), (7, 5, 5, 224, 100, 1, 1, 1, VALID), (2, 16, 16, 64, 64, 3, 3, 3, VALID), (6, 17, 19, 100, 64, 3, 3, 1, ZERO),
-    (1, 8, 8, 1024, 32, 3, 3, 1, ONE), (2, 15, 15, 64, 128, 7, 7, 2, ONE), (20, 24, 24, 32, 64, 3, 3, 1, ZERO),
+    (1, 8, 8, 1024, 32, 3, 3, 1, ONE), (2, 15, 15, 64, 128, 7, 7, 2, ONE), (10, 60, 60, 32, 64, 3, 3, 3, ZERO), (20, 60, 60, 32, 64, 3, 3, 3, ONE),
 ]
 
 
