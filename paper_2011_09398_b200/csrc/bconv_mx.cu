@@ -1008,13 +1008,11 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
         const MxFin fin = mx_fin_context(p, fw, lane, ch0);
         asm volatile("griddepcontrol.wait;" ::: "memory");  // outputs and the shortcut tensor: only after the previous kernel
         const int T = p.T, n_tiles = p.n_tiles, n_super = p.n_super, out_type = p.out_type;
-        uint32_t par_full_d[2] = {0, 0};
         int it = 0;
         for (int st = first_tile; st < n_super && ok; st += tile_step) {
             for (int k = 0; k < T && st * T + k < n_tiles; ++k, ++it) {
                 const int buf = it & 1;
-                ok = mbar_wait_bounded(&bars[BAR_FULL_D0 + buf], par_full_d[buf]);
-                par_full_d[buf] ^= 1u;
+                ok = mbar_wait_bounded(&bars[BAR_FULL_D0 + buf], (uint32_t)(it >> 1) & 1u);
                 ok = __all_sync(0xffffffffu, ok);  // the warp goes on together (its epilogue uses warp-wide shuffles and ballots)
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -1046,7 +1044,6 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
         const uint32_t x_lo_buf0 = ((uint32_t)p.off_x >> 4) + (smem_u32(smem) >> 4) + ((uint32_t)p.P << 16);
         const uint32_t x_units = (uint32_t)p.x_bytes >> 4, group_units = ((uint32_t)p.tap_bytes >> 4) * (uint32_t)p.group_taps;
         const uint32_t sfa = tmem_base + kSfaCol, sfb = tmem_base + kSfbCol;
-        uint32_t par_empty_d[2] = {0, 0};
         const int n_xbuf = p.n_xbuf;
         ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bars[BAR_SCALES], 0));  // the block scales are in TMEM
         int g = 0, stage_i = 0;
@@ -1059,8 +1056,7 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
             if (resident && buf != my_parity) continue;
             ok = mbar_wait_bounded(&bars[BAR_FULL_X0 + (it & 3)], (uint32_t)(it >> 2) & 1u);
             if (ok && it >= 2) {  // the accumulator buffer must have been read out
-                ok = mbar_wait_bounded(&bars[BAR_EMPTY_D0 + buf], par_empty_d[buf]);
-                par_empty_d[buf] ^= 1u;
+                ok = mbar_wait_bounded(&bars[BAR_EMPTY_D0 + buf], (uint32_t)((it >> 1) - 1) & 1u);
             }
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
