@@ -64,10 +64,10 @@ typedef enum { LCE_ACT_NONE = 0, LCE_ACT_RELU = 1 } lce_activation;
  *          integer below 2^24).  Filters of up to 64 taps, equal strides of 1 or 2, in_c <= 1024, every
  *          padding mode and output type.  Needs weights packed by lce_bconv2d_pack_weights;
  *   DIRECT one thread per output, any shape (fallback, not tuned);
- *   AUTO   TENSOR when the weights are packed and the layer is large enough to pay for that kernel's
- *          start-up (at least 2^28 binary MACs, 2^29 when the filter does not fit in shared memory, 2^31
- *          for 3x3 or smaller filters on at most 32 input channels), otherwise TILED where it covers the
- *          shape, otherwise DIRECT.  lce_bconv2d_plan tells which.
+ *   AUTO   with packed weights TENSOR or, for small layers, a latency kernel of any filter size and stride
+ *          (bits on the warp-level integer matrix instruction), whichever is estimated to be the faster;
+ *          otherwise, and for plain weights, TILED where it covers the shape, else DIRECT.  lce_bconv2d_plan
+ *          tells which.
  * Forcing a kernel on a shape (or on plain weights) it does not cover returns LCE_ERR_UNSUPPORTED. */
 typedef enum { LCE_KERNEL_AUTO = 0, LCE_KERNEL_DIRECT = 1, LCE_KERNEL_TILED = 2, LCE_KERNEL_TENSOR = 3 } lce_kernel;
 
@@ -164,7 +164,9 @@ lce_status lce_bconv2d_f32(const lce_bconv2d_desc *desc, const float *input, con
  * paper's engine picks its kernel and tiling per layer when the model is loaded (Section 3.1); this
  * is that choice made visible.  Fields that do not apply to the chosen kernel are 0.
  *   kernel              LCE_KERNEL_DIRECT, LCE_KERNEL_TILED or LCE_KERNEL_TENSOR (the one-word patch
- *                       kernel for very few input channels reports LCE_KERNEL_TILED with patch = 1).
+ *                       kernel for very few input channels reports LCE_KERNEL_TILED with patch = 1, the
+ *                       latency kernel of AUTO LCE_KERNEL_TILED with pixels_per_thread = 0 and tile_pixels,
+ *                       warps_per_cta, ctas, shared_bytes).
  *                       For LCE_KERNEL_TENSOR: tile_pixels = grid positions per tile, ctas, shared_bytes,
  *                       weights_resident = 1 when every tap of a channel block stays in shared memory
  *                       (fetched once per CTA; weight_stages = taps), 0 when they stream past once per
@@ -206,8 +208,8 @@ void lce_plan_destroy(lce_plan *plan);
  * time for its access pattern; Section 3.1: weights are converted once, when the model is built).  Rewrites
  * the plain packed weights into the operand layout the tiled kernel copies straight into shared
  * memory, so that none of that work is repeated per call.  The packed buffer also keeps a copy of
- * the plain words, and, where the tensor-core kernel covers the geometry, that kernel's operand image
- * (every weight bit expanded to a 4-bit +-1, pad channels 0).  It is valid for every padding mode, output
+ * the plain words, and, where the tensor-core and the latency kernel cover the geometry, their operand images
+ * (every weight bit expanded to a 4-bit +-1, pad channels 0; words in the order the latency kernel stages them).  It is valid for every padding mode, output
  * type and activation of the same geometry (batch, sizes, channels, kernel, stride).  The first call in a
  * process also sets up a few bytes of pinned host memory for the device-timeout flag: make it outside
  * any stream capture.
