@@ -461,12 +461,14 @@ extern "C" size_t lce_bconv2d_host_workspace_bytes(const lce_bconv2d_desc *desc)
 
 namespace lce {
 namespace {
-// An engine copy costs about 4 us however short; one kernel over pinned memory moves all the small arrays in about 3 us and
-// keeps up with the engine to some 256 KB.  Outputs written by the convolution itself save that copy's start-up as well:
-// one 20x20x32 image 33 -> 21 us a call, 51 KB of floats 28.4 -> 21.6, 86 KB 31.0 -> 27.6.
-constexpr size_t kSmallCopy = 256 * 1024;
+// An engine copy costs about 4 us however short, and where a kernel follows or goes before it some 8 us more; one kernel
+// over pinned memory moves all the arrays of a call in about 3 us and the PCIe time (0.8 MB: 20.6 us, the engine 18.0),
+// so the two draw level at some 2.5 MB.  28x28x128, 64 images, 0.8 MB in and out: 64 -> 61 us a call; 56x56x128, 8 images:
+// 55 -> 43.  An output written by the convolution itself saves the copy's launch as well: one 20x20x32 image 33 -> 21 us,
+// 51 KB of floats 28.4 -> 21.6, 86 KB 31.0 -> 27.6.
+constexpr size_t kKernelCopy = 2048 * 1024;
 // float / int32 rows leave as 128-byte lines, bit-packed words four bytes at a time (0.8 MB of them straight to the host:
-// 203 us a call instead of 63)
+// 203 us a call)
 constexpr size_t kSmallRows = 256 * 1024, kSmallWords = 32 * 1024;
 
 lce_status host_conv(const lce_bconv2d_desc *desc, const uint32_t *input, const uint32_t *weights, const float *multiplier,
@@ -483,13 +485,13 @@ lce_status host_conv(const lce_bconv2d_desc *desc, const uint32_t *input, const 
     if (workspace_bytes < L.total) return LCE_ERR_WORKSPACE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     char *ws = static_cast<char *>(workspace);
-    // arrays of up to kSmallCopy bytes in pinned memory travel together in one kernel, the others (first: the rest is
+    // arrays of up to kKernelCopy bytes in pinned memory travel together in one kernel, the others (first: the rest is
     // prepared while they run) by the copy engine
     HostCopy copies[kHostCopies] = {{input, ws + L.in, L.in_bytes}, {weights, ws + L.w, L.w_bytes}, {multiplier, ws + L.mult, L.ch_bytes},
                                     {bias, ws + L.bias, L.ch_bytes}, {thresholds, ws + L.thr, L.ch_bytes}};
     for (HostCopy &c : copies) {
         if (!c.src) c.bytes = 0;
-        const void *view = c.bytes > 0 && c.bytes <= kSmallCopy ? pinned_host_view(c.src) : nullptr;
+        const void *view = c.bytes > 0 && c.bytes <= kKernelCopy ? pinned_host_view(c.src) : nullptr;
         if (view) {
             c.src = view;
             continue;
@@ -516,7 +518,14 @@ lce_status host_conv(const lce_bconv2d_desc *desc, const uint32_t *input, const 
         st = dispatch(p, d_in, d_w, d_mult, d_bias, d_thr, d_out, s);
     }
     if (st != LCE_OK) return st;
-    if (!out_view && cudaMemcpyAsync(output, ws + L.out, L.out_bytes, cudaMemcpyDeviceToHost, s) != cudaSuccess) return LCE_ERR_CUDA;
+    void *back_view = !out_view && L.out_bytes <= kKernelCopy ? pinned_host_view(output) : nullptr;
+    if (back_view) {
+        const HostCopy back[kHostCopies] = {{ws + L.out, back_view, L.out_bytes}};
+        st = launch_host_copies(back, s);
+        if (st != LCE_OK) return st;
+    } else if (!out_view && cudaMemcpyAsync(output, ws + L.out, L.out_bytes, cudaMemcpyDeviceToHost, s) != cudaSuccess) {
+        return LCE_ERR_CUDA;
+    }
     if (synchronise && cudaStreamSynchronize(s) != cudaSuccess) return LCE_ERR_CUDA;
     return LCE_OK;
 }

@@ -1,8 +1,9 @@
-// The small host-to-device copies of lce_bconv2d_host in one kernel.  What bounds the call for a small layer is the
-// number of stream operations: each cudaMemcpyAsync costs about 4 us of the stream whatever its size, and a layer
-// brings weights and one or two per-channel arrays beside its input.  Pinned host memory is visible to the device, so
-// one kernel fetches them all over PCIe (its latency once, about 4 us together).  The copy engine is a little faster
-// for large arrays (0.8 MB: 18.0 against 20.6 us), which stay with it.
+// The copies of lce_bconv2d_host in one kernel each way.  What bounds the call for a small layer is the number of stream
+// operations: each cudaMemcpyAsync costs about 4 us of the stream whatever its size, more where the stream changes between
+// copy engine and SMs, and a layer brings weights and one or two per-channel arrays beside its input.  Pinned host memory
+// is visible to the device, so one kernel fetches them all over PCIe (its latency once, about 4 us together), and one
+// brings the output back.  The copy engine is a little faster per byte (0.8 MB: 18.0 against 20.6 us): large arrays stay
+// with it.
 #include "common.cuh"
 
 namespace lce {
@@ -33,7 +34,7 @@ __global__ void __launch_bounds__(kCopyThreads) host_copy_kernel(const CopyParam
                 words = p.words[k];
             }
         }
-        if (at + 4 <= words && (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+        if (at + 4 <= words && ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0) {
             *reinterpret_cast<uint4 *>(dst + at) = *reinterpret_cast<const uint4 *>(src + at);
         } else {
             for (int k = at; k < min(at + 4, words); ++k) dst[k] = src[k];
