@@ -208,7 +208,7 @@ void lce_plan_destroy(lce_plan *plan);
  * time for its access pattern; Section 3.1: weights are converted once, when the model is built).  Rewrites
  * the plain packed weights into the operand layout the tiled kernel copies straight into shared
  * memory, so that none of that work is repeated per call.  The packed buffer also keeps a copy of
- * the plain words, and, where the tensor-core and the latency kernel cover the geometry, their operand images
+ * the plain words, and, where the tensor-core and the latency kernel cover the geometry (under any padding mode), their operand images
  * (every weight bit expanded to a 4-bit +-1, pad channels 0; words in the order the latency kernel stages them).  It is valid for every padding mode, output
  * type and activation of the same geometry (batch, sizes, channels, kernel, stride).  The first call in a
  * process also sets up a few bytes of pinned host memory for the device-timeout flag: make it outside

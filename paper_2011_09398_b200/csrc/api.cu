@@ -33,8 +33,8 @@ size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 size_t plain_weight_bytes(const ConvGeom &g) { return round_up((size_t)g.Cout * g.KH * g.KW * g.Cw * 4, 256); }
 
 // A packed-weights buffer = [plain words][operand image of the tiled XOR/POPC kernel][operand image of
-// the tensor-core kernel][tile image of the latency kernel], each part rounded up to 256 bytes; a part a kernel
-// does not cover is empty.
+// the tensor-core kernel][tile image of the latency kernel], each part rounded up to 256 bytes; a part is
+// empty if its kernel covers the geometry under no padding mode (the buffer is the same under all of them).
 struct WeightParts {
     size_t tiled, tensor, small, total;  // byte offsets; 0: no such part
 };

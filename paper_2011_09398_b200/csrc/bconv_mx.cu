@@ -1183,6 +1183,7 @@ struct MxPlan {
 };
 
 constexpr size_t kSmemLimit = 227 * 1024;
+constexpr int kMaxPositions = 16383;  // of a position buffer: descriptor strides are 14-bit counts of 16 bytes
 
 bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl);
 
@@ -1217,34 +1218,77 @@ bool mx_plan(const ConvGeom &g, int sms, MxPlan *pl)
     return e.found;
 }
 
-bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
+int mx_channel_words(const ConvGeom &g) { return g.Cw + (g.Cw & 1); }
+int mx_channel_blocks(const ConvGeom &g) { return (g.Cout + 127) / 128; }
+
+// The grid of positions and everything else of a plan that does not depend on the tile; false where the kernel does not
+// cover the layer.
+bool mx_frame(const ConvGeom &g, MxPlan *pl)
 {
     if (g.sh != g.sw || (g.sh != 1 && g.sh != 2)) return false;
     if (g.Cw > 32) return false;
     const int taps = g.KH * g.KW;
     if (taps > kMaxTaps) return false;
     const int s = g.sh;
-    int Wg, Hg, halo;
+    int Wg, Hg;
+    int64_t halo;
     if (s == 1) {
         const int pr = max(0, (g.OW - 1) + g.KW - g.W - g.pl), pb = max(0, (g.OH - 1) + g.KH - g.H - g.pt);
         Wg = g.W + max(g.pl, pr);
         Hg = g.H + max(g.pt, pb);
-        halo = (g.KH - 1) * Wg + (g.KW - 1);
+        halo = (int64_t)(g.KH - 1) * Wg + (g.KW - 1);
     } else {
         Wg = g.OW + (g.KW - 1) / 2;
         Hg = g.OH + (g.KH - 1) / 2;
-        halo = ((g.KH - 1) / 2) * Wg + (g.KW - 1) / 2;
+        halo = (int64_t)((g.KH - 1) / 2) * Wg + (g.KW - 1) / 2;
     }
     const int64_t total_q = (int64_t)g.N * Hg * Wg;
-    if (total_q >= (1ll << 31) - 4096 || g.M >= (1ll << 31)) return false;
-    pl->Wg = Wg; pl->Hg = Hg; pl->halo = halo; pl->total_q = (int)total_q;
+    if (total_q >= (1ll << 31) - 4096 || g.M >= (1ll << 31) || halo > kMaxPositions) return false;
+    pl->Wg = Wg; pl->Hg = Hg; pl->halo = (int)halo; pl->total_q = (int)total_q;
     // a 1x1 filter at stride 2 reads one phase of the four: staging that one alone took 64 images of 28x28x512 -> 512 from
     // 19.5 to 7.3 us, of 56x56x256 -> 256 from 13.7 to 9.0
     pl->n_phase = taps == 1 ? 1 : s * s;
-    pl->Cw2 = g.Cw + (g.Cw & 1);
+    pl->Cw2 = mx_channel_words(g);
     pl->taps = taps;
     pl->tap_bytes = (size_t)pl->Cw2 * 2048;
-    pl->n_blocks = (g.Cout + 127) / 128;
+    pl->n_blocks = mx_channel_blocks(g);
+    return true;
+}
+
+// Shared memory of a tile of nt positions, T of them to a position buffer; false if it does not fit beside two taps
+// (one of a 1x1 filter).
+struct MxRoom {
+    int P;
+    size_t raw_words, x_bytes, off_tbl, off_w, rest;
+};
+
+bool mx_room(const MxPlan &pl, int Cw, int nt, int T, MxRoom *r)
+{
+    // T tiles share one position buffer of T * nt + halo rows: the halo is staged once per T tiles
+    r->P = T * nt + pl.halo;
+    if (r->P > kMaxPositions) return false;
+    r->raw_words = (((size_t)pl.n_phase * (nt + pl.halo) * Cw + 3) / 4) * 4;
+    r->x_bytes = (size_t)pl.n_phase * pl.Cw2 * r->P * 16;
+    r->off_tbl = kOffDyn + r->raw_words * 4;
+    const size_t fixed = r->off_tbl + (size_t)pl.taps * (pl.Cw2 / 2) * 8;  // the table no longer than it is: at 512 channels 3x3 the 8 KB saved are a wider tile
+    r->off_w = (fixed + 127) / 128 * 128;
+    r->rest = 2 * r->x_bytes + 256;
+    return r->off_w + r->rest + (pl.taps > 1 ? 2 : 1) * pl.tap_bytes <= kSmemLimit;
+}
+
+// a larger tile never takes less room, so a layer has a plan if the smallest one fits
+bool mx_covers(const ConvGeom &g)
+{
+    MxPlan pl;
+    MxRoom r;
+    return mx_frame(g, &pl) && mx_room(pl, g.Cw, 16, 1, &r);
+}
+
+bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
+{
+    if (!mx_frame(g, pl)) return false;
+    const int taps = pl->taps, halo = pl->halo;
+    const int64_t total_q = pl->total_q;
     const int ctas_max = max(1, sms / pl->n_blocks);
     const int ksteps = pl->Cw2 / 2;
     double best = 1e30;
@@ -1252,21 +1296,13 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
     for (int nt = 16; nt <= kMaxNt; nt += 16) {
         const int n_tiles = (int)((total_q + nt - 1) / nt);
         for (int T = 1; T <= 8; ++T) {
-            // T tiles share one position buffer of T * nt + halo rows: the halo is staged once per T tiles
-            const int P = T * nt + halo;
-            if (P > 16383) break;  // descriptor strides are 14-bit counts of 16 bytes
             if (T > 1 && (T - 1) * ctas_max >= n_tiles) break;   // no CTA would have that many tiles
-            const size_t raw_words = (((size_t)pl->n_phase * (nt + halo) * g.Cw + 3) / 4) * 4;
-            const size_t x_bytes = (size_t)pl->n_phase * pl->Cw2 * P * 16;
-            const size_t off_tbl = kOffDyn + raw_words * 4;
-            const size_t fixed = off_tbl + (size_t)taps * ksteps * 8;  // the table no longer than it is: at 512 channels 3x3 the 8 KB saved are a wider tile
-            const size_t off_w = (fixed + 127) / 128 * 128;
-            const size_t rest = 2 * x_bytes + 256;
-            if (off_w + rest + (taps > 1 ? 2 : 1) * pl->tap_bytes > kSmemLimit) break;
+            MxRoom room;
+            if (!mx_room(*pl, g.Cw, nt, T, &room)) break;
             // taps that fit beside the position buffers: all of them -> resident (one stage per tap, one barrier);
             // otherwise a ring of two stages of half the fitting taps each (a group costs the issuer one wait and
             // one commit, whatever its size: two large groups measured better than three or four smaller ones)
-            const int slots = (int)((kSmemLimit - off_w - rest) / pl->tap_bytes);
+            const int slots = (int)((kSmemLimit - room.off_w - room.rest) / pl->tap_bytes);
             const bool resident = slots >= taps;
             int stages, group_taps, groups;
             if (resident) {
@@ -1296,20 +1332,20 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
             if (cost < best) {
                 best = pl->clocks = cost;
                 found = true;
-                pl->Nt = nt; pl->P = P; pl->T = T; pl->stages = stages; pl->resident = resident ? 1 : 0; pl->group_taps = group_taps; pl->groups = groups;
+                pl->Nt = nt; pl->P = room.P; pl->T = T; pl->stages = stages; pl->resident = resident ? 1 : 0; pl->group_taps = group_taps; pl->groups = groups;
                 pl->n_tiles = n_tiles; pl->n_super = n_super; pl->ctas_x = ctas_x;
-                pl->raw_words = raw_words; pl->x_bytes = x_bytes;
-                pl->off_tbl = off_tbl;
-                pl->off_w = off_w;
-                pl->off_x = (off_w + (size_t)stages * group_taps * pl->tap_bytes + 127) / 128 * 128;
+                pl->raw_words = room.raw_words; pl->x_bytes = room.x_bytes;
+                pl->off_tbl = room.off_tbl;
+                pl->off_w = room.off_w;
+                pl->off_x = (room.off_w + (size_t)stages * group_taps * pl->tap_bytes + 127) / 128 * 128;
                 // More position buffers where shared memory is left over (thin layers): the loaders may then be
                 // up to four tiles ahead, ahead <= (n_xbuf - 1) * T + 1, and the hand-overs between the roles
                 // (a few hundred clocks each) drop out of the per-tile cycle.
                 int n_xbuf = 2;
-                while (n_xbuf < 4 && (n_xbuf - 1) * T + 1 < 4 && pl->off_x + (size_t)(n_xbuf + 1) * x_bytes <= kSmemLimit) ++n_xbuf;
+                while (n_xbuf < 4 && (n_xbuf - 1) * T + 1 < 4 && pl->off_x + (size_t)(n_xbuf + 1) * room.x_bytes <= kSmemLimit) ++n_xbuf;
                 pl->n_xbuf = n_xbuf;
                 pl->ahead = min(4, (n_xbuf - 1) * T + 1);
-                pl->smem = pl->off_x + (size_t)n_xbuf * x_bytes;
+                pl->smem = pl->off_x + (size_t)n_xbuf * room.x_bytes;
             }
         }
     }
@@ -1335,27 +1371,20 @@ int device_sms()
 
 }  // namespace
 
-bool tensor_covers(const ConvGeom &g)
-{
-    MxPlan pl;
-    return mx_plan(g, 148, &pl);
-}
+bool tensor_covers(const ConvGeom &g) { return mx_covers(g); }
 
 size_t tensor_weight_image_bytes(const ConvGeom &g)
 {
-    MxPlan pl;
-    if (!mx_plan(g, 148, &pl)) return 0;
-    return (size_t)pl.n_blocks * pl.taps * pl.tap_bytes;
+    return covers_some_padding(g, mx_covers) ? (size_t)mx_channel_blocks(g) * g.KH * g.KW * mx_channel_words(g) * 2048 : 0;
 }
 
 lce_status launch_pack_weights_tensor(const ConvGeom &g, const uint32_t *w, void *image, cudaStream_t s)
 {
-    MxPlan pl;
-    if (!mx_plan(g, 148, &pl)) return LCE_ERR_UNSUPPORTED;
-    const int64_t total = (int64_t)pl.n_blocks * pl.taps * pl.Cw2 * 128;
+    const int n_blocks = mx_channel_blocks(g), taps = g.KH * g.KW, Cw2 = mx_channel_words(g);
+    const int64_t total = (int64_t)n_blocks * taps * Cw2 * 128;
     const int64_t want = (total + 255) / 256;
     const int blocks = (int)(want < 4096 ? want : 4096);
-    const lce_status st = launch_dependent(mx_pack_weights_kernel, dim3((unsigned)blocks), 256, 0, s, w, static_cast<uint4 *>(image), g.Cout, g.Cin, g.Cw, pl.Cw2, pl.taps, pl.n_blocks, mx_dup(g));
+    const lce_status st = launch_dependent(mx_pack_weights_kernel, dim3((unsigned)blocks), 256, 0, s, w, static_cast<uint4 *>(image), g.Cout, g.Cin, g.Cw, Cw2, taps, n_blocks, mx_dup(g));
     mx_flag_array(false);  // load time is the moment to set up the host-visible status word (it cannot be done under stream capture)
     return st;
 }

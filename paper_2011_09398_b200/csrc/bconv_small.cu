@@ -475,7 +475,7 @@ void small_plan_info(const ConvGeom &g, TiledPlanInfo *info)
 
 size_t small_weight_image_bytes(const ConvGeom &g)
 {
-    return small_covers(g) ? (size_t)g.Cow * kChannels * (small_pitch(g) + 1 + g.KH * g.KW) * 4 : 0;
+    return covers_some_padding(g, small_covers) ? (size_t)g.Cow * kChannels * (small_pitch(g) + 1 + g.KH * g.KW) * 4 : 0;
 }
 
 lce_status launch_pack_weights_small(const ConvGeom &g, const uint32_t *w, uint32_t *image, cudaStream_t s)

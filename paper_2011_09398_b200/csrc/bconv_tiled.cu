@@ -202,14 +202,13 @@ bool choose_tile(const ConvGeom &g, int chan_blocks, SmemFn smem_for_tile, TileC
 
 size_t tiled_weight_image_bytes(const ConvGeom &g)
 {
-    if (!tiled_covers(g)) return 0;
+    if (!covers_some_padding(g, tiled_covers)) return 0;
     const int chan_blocks = (g.Cout + kChanPerCta - 1) / kChanPerCta;
     return (size_t)chan_blocks * image_block_words(image_groups(g)) * 4;
 }
 
 lce_status launch_pack_weights_tiled(const ConvGeom &g, const uint32_t *w, uint32_t *image, cudaStream_t s)
 {
-    if (!tiled_covers(g)) return LCE_ERR_UNSUPPORTED;
     const int chan_blocks = (g.Cout + kChanPerCta - 1) / kChanPerCta;
     const int groups = image_groups(g);
     const int64_t entries = (int64_t)chan_blocks * kChanPerCta * groups;

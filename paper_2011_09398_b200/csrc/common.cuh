@@ -35,6 +35,34 @@ struct ConvGeom {
     int64_t M;  // N*OH*OW output pixels
 };
 
+// Output extents under a padding mode.  The index arithmetic of the kernels is 32-bit on words: every tensor stays below
+// 2^31 words.
+inline lce_status set_padding(ConvGeom *g, int32_t padding)
+{
+    const Axis ah = axis_geometry(g->H, g->KH, g->sh, padding), aw = axis_geometry(g->W, g->KW, g->sw, padding);
+    if (ah.out <= 0 || aw.out <= 0) return LCE_ERR_INVALID_ARG;
+    g->padding = padding;
+    g->OH = ah.out; g->OW = aw.out; g->pt = ah.pad_before; g->pl = aw.pad_before;
+    g->M = (int64_t)g->N * g->OH * g->OW;
+    const int64_t in_words = (int64_t)g->N * g->H * g->W * g->Cw;
+    const int64_t out_elems = g->M * g->Cout;
+    const int64_t w_words = (int64_t)g->Cout * g->KH * g->KW * g->Cw;
+    return in_words >= (1ll << 31) || out_elems >= (1ll << 31) || w_words >= (1ll << 31) ? LCE_ERR_UNSUPPORTED : LCE_OK;
+}
+
+// Whether `covers` holds for the geometry under one padding mode at least.  Packed weights serve every padding mode, so
+// which parts their buffer has must not depend on the mode they are packed under: a part is there for all modes if its
+// kernel covers any of them (the kernels' limits on shared memory and taps differ between the modes).
+template <typename Covers>
+bool covers_some_padding(const ConvGeom &g, Covers covers)
+{
+    for (const int32_t padding : {LCE_PAD_VALID, LCE_PAD_SAME_ONE, LCE_PAD_SAME_ZERO}) {
+        ConvGeom t = g;
+        if (set_padding(&t, padding) == LCE_OK && covers(t)) return true;
+    }
+    return false;
+}
+
 inline lce_status make_geom(const lce_bconv2d_desc *d, ConvGeom *g)
 {
     if (!d) return LCE_ERR_INVALID_ARG;
@@ -46,22 +74,11 @@ inline lce_status make_geom(const lce_bconv2d_desc *d, ConvGeom *g)
     if (d->activation < LCE_ACT_NONE || d->activation > LCE_ACT_RELU) return LCE_ERR_INVALID_ARG;
     if (d->kernel < LCE_KERNEL_AUTO || d->kernel > LCE_KERNEL_TENSOR) return LCE_ERR_INVALID_ARG;
     if (d->weights_packed != 0 && d->weights_packed != 1) return LCE_ERR_INVALID_ARG;
-    Axis ah = axis_geometry(d->in_h, d->kernel_h, d->stride_h, d->padding);
-    Axis aw = axis_geometry(d->in_w, d->kernel_w, d->stride_w, d->padding);
-    if (ah.out <= 0 || aw.out <= 0) return LCE_ERR_INVALID_ARG;
     g->N = d->batch; g->H = d->in_h; g->W = d->in_w; g->Cin = d->in_c; g->Cw = (d->in_c + 31) / 32;
     g->Cout = d->out_c; g->Cow = (d->out_c + 31) / 32;
     g->KH = d->kernel_h; g->KW = d->kernel_w; g->sh = d->stride_h; g->sw = d->stride_w;
-    g->OH = ah.out; g->OW = aw.out; g->pt = ah.pad_before; g->pl = aw.pad_before;
-    g->padding = d->padding; g->out_type = d->out_type; g->activation = d->activation;
-    g->M = (int64_t)g->N * g->OH * g->OW;
-    // the index arithmetic of the kernels is 32-bit on words: keep every tensor below 2^31 words
-    int64_t in_words = (int64_t)g->N * g->H * g->W * g->Cw;
-    int64_t out_elems = g->M * g->Cout;
-    int64_t w_words = (int64_t)g->Cout * g->KH * g->KW * g->Cw;
-    if (in_words >= (1ll << 31) || out_elems >= (1ll << 31) || w_words >= (1ll << 31))
-        return LCE_ERR_UNSUPPORTED;
-    return LCE_OK;
+    g->out_type = d->out_type; g->activation = d->activation;
+    return set_padding(g, d->padding);
 }
 
 inline bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }

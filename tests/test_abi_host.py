@@ -188,6 +188,32 @@ def test_packed_weights_buffer_holds_the_three_parts(lib):
     assert lce.lce_bconv2d_packed_weights_bytes(odd) >= 130 * 9 * 3 * 4 + 2 * 9 * 4 * 2048
 
 
+def test_packed_weights_are_the_same_buffer_under_every_padding_mode(lib):
+    """lce.h: packed weights are valid for every padding mode, output type and activation of their geometry.  So the size
+    and the parts of the buffer may depend on none of them, also where a kernel covers one mode and not another
+    (14x14x64 7x7: the latency kernel takes VALID and one-padding, not zero-padding)."""
+    rng = np.random.default_rng(11)
+    shapes = [(1, 14, 14, 64, 64, 7, 7, 1)]
+    while len(shapes) < 1500:
+        k = int(rng.choice([1, 2, 3, 5, 6, 7, 8]))
+        n, c, o = int(rng.integers(1, 9)), int(rng.integers(1, 512)), int(rng.integers(1, 300))
+        kw = int(rng.choice([k, rng.integers(1, 9)]))
+        shapes.append((n, int(rng.integers(1, 80)), int(rng.integers(1, 80)), c, o, k, kw, int(rng.integers(1, 3))))
+    # a row so long that only VALID, which needs no halo of its own, leaves the tensor-core kernel room
+    shapes += [(1, 1, 16000, 32, 32, 1, 3, 1), (1, 2, 8100, 32, 32, 3, 3, 1), (1, 40, 16, 1024, 32, 5, 5, 1), (1, 9, 9, 1024, 32, 8, 8, 1)]
+    differing = []
+    for n, h, w, c, o, kh, kw, s in shapes:
+        sizes = {}
+        for pad in (lce.PAD_VALID, lce.PAD_SAME_ONE, lce.PAD_SAME_ZERO):
+            for out_type, act in ((lce.OUT_BITPACKED, lce.ACT_NONE), (lce.OUT_FLOAT32, lce.ACT_RELU), (lce.OUT_INT32, lce.ACT_NONE)):
+                d = lce.make_desc(n, h, w, c, o, (kh, kw), (s, s), pad, out_type, act, weights_packed=1)
+                sizes[pad, out_type] = lce.lce_bconv2d_packed_weights_bytes(d)
+        if pad_sizes := {v for v in sizes.values() if v}:   # 0: the descriptor is malformed (VALID, image smaller than the filter)
+            if len(pad_sizes) > 1:
+                differing.append(((n, h, w, c, o, kh, kw, s), sizes))
+    assert not differing, f"{len(differing)} geometries, the first: {differing[0]}"
+
+
 def test_plans_are_remembered_per_geometry_not_mixed_up(lib):
     """The library keeps the last few plans of a host thread: a repeated geometry must give the same
     plan as the first time, with more distinct geometries in between than it keeps."""

@@ -72,3 +72,33 @@ def test_small_fused_layers_match_the_oracle(cout, parts):
         np.testing.assert_array_equal(out.cpu().numpy(), want)
     if packed is not None:
         np.testing.assert_array_equal(words_to_host(packed), oracle.bitpack(want))
+
+
+# n, h, w, cin, cout, k, stride: a kernel covers them under some padding modes only (the latency kernel 7x7 not under
+# zero-padding, the tensor-core kernel the other two under VALID alone: longer rows leave it no room)
+@pytest.mark.parametrize("shape", [(1, 14, 14, 64, 64, 7, 1), (1, 4, 30, 1000, 40, 3, 1), (2, 6, 13, 1000, 40, 5, 1)], ids=lambda s: "x".join(map(str, s)))
+def test_weights_packed_under_one_padding_mode_run_under_every_other(shape):
+    n, h, w, cin, cout, k, s = shape
+    rng = np.random.default_rng(sum(shape))
+    a = (2 * rng.integers(0, 2, size=(n, h, w, cin)) - 1).astype(np.int8)
+    wt = (2 * rng.integers(0, 2, size=(cout, k, k, cin)) - 1).astype(np.int8)
+    x, plain = to_dev_words(oracle.bitpack_pm1(a)), to_dev_words(oracle.bitpack_pm1(wt))
+    desc = lambda pad, choice: lce.make_desc(n, h, w, cin, cout, (k, k), (s, s), pad, lce.OUT_INT32, lce.ACT_NONE, choice, 1)
+    choices, covered = (lce.KERNEL_AUTO, lce.KERNEL_TENSOR, lce.KERNEL_TILED), set()
+    packed = {pad: lce.lce_bconv2d_pack_weights(desc(pad, lce.KERNEL_AUTO), plain) for pad in (VALID, ONE, ZERO)}
+    for pad in (VALID, ONE, ZERO):
+        want = oracle.bconv2d_acc(a, wt, (s, s), pad)
+        for choice in choices:
+            try:
+                lce.lce_bconv2d_plan(desc(pad, choice))
+            except lce.LceError as e:
+                assert e.status == 2
+                continue
+            covered.add((pad, choice))
+            for under in (VALID, ONE, ZERO):
+                got = lce.lce_bconv2d(desc(pad, choice), x, packed[under])
+                np.testing.assert_array_equal(got.cpu().numpy(), want, err_msg=f"packed under {under}, run under {pad}, kernel {choice}")
+    assert (VALID, lce.KERNEL_AUTO) in covered
+    if k != 7:
+        assert (VALID, lce.KERNEL_TENSOR) in covered and (ONE, lce.KERNEL_TENSOR) not in covered
+    assert lce.lce_device_status() == 0
