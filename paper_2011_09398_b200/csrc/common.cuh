@@ -204,7 +204,8 @@ lce_status tensor_device_status_reset();
 bool tensor_timeout_flagged();
 lce_status tensor_wait_probe(uint64_t limit_ns, cudaStream_t s);
 // Copies between pinned host memory and the device in one kernel; arrays on 4 bytes, sizes multiples of 4 below 2^31 in
-// all, empty ones allowed.  pinned_host_view: the device's view of a pinned host pointer, null for any other memory.
+// all, empty ones allowed.  pinned_host_view: where a kernel may access a host array, null where the array is the copy
+// engine's (host_view.cuh).
 constexpr int kHostCopies = 5;
 struct HostCopy {
     const void *src;
