@@ -491,7 +491,7 @@ lce_status host_conv(const lce_bconv2d_desc *desc, const uint32_t *input, const 
                                     {bias, ws + L.bias, L.ch_bytes}, {thresholds, ws + L.thr, L.ch_bytes}};
     for (HostCopy &c : copies) {
         if (!c.src) c.bytes = 0;
-        const void *view = c.bytes > 0 && c.bytes <= kKernelCopy ? pinned_host_view(c.src) : nullptr;
+        const void *view = c.bytes > 0 && c.bytes <= kKernelCopy ? pinned_host_view(c.src, c.bytes, false) : nullptr;
         if (view) {
             c.src = view;
             continue;
@@ -502,7 +502,7 @@ lce_status host_conv(const lce_bconv2d_desc *desc, const uint32_t *input, const 
     st = launch_host_copies(copies, s);
     if (st != LCE_OK) return st;
     // a small output in pinned memory is written there directly
-    void *out_view = L.out_bytes <= (g.out_type == LCE_OUT_BITPACKED ? kSmallWords : kSmallRows) && aligned(output, 16) ? pinned_host_view(output) : nullptr;
+    void *out_view = L.out_bytes <= (g.out_type == LCE_OUT_BITPACKED ? kSmallWords : kSmallRows) && aligned(output, 16) ? pinned_host_view(output, L.out_bytes, true) : nullptr;
     void *d_out = out_view ? out_view : ws + L.out;
     const Prepared &p = prepared_for(desc, FORM_HOST | (workspace_bytes < L.total + L.image ? FORM_NO_IMAGE : 0));
     if (p.status != LCE_OK) return p.status;
@@ -518,7 +518,7 @@ lce_status host_conv(const lce_bconv2d_desc *desc, const uint32_t *input, const 
         st = dispatch(p, d_in, d_w, d_mult, d_bias, d_thr, d_out, s);
     }
     if (st != LCE_OK) return st;
-    void *back_view = !out_view && L.out_bytes <= kKernelCopy ? pinned_host_view(output) : nullptr;
+    void *back_view = !out_view && L.out_bytes <= kKernelCopy ? pinned_host_view(output, L.out_bytes, true) : nullptr;
     if (back_view) {
         const HostCopy back[kHostCopies] = {{ws + L.out, back_view, L.out_bytes}};
         st = launch_host_copies(back, s);

@@ -204,15 +204,15 @@ lce_status tensor_device_status_reset();
 bool tensor_timeout_flagged();
 lce_status tensor_wait_probe(uint64_t limit_ns, cudaStream_t s);
 // Copies between pinned host memory and the device in one kernel; arrays on 4 bytes, sizes multiples of 4 below 2^31 in
-// all, empty ones allowed.  pinned_host_view: where a kernel may access a host array, null where the array is the copy
-// engine's (host_view.cuh).
+// all, empty ones allowed.  pinned_host_view: where a kernel may access a host array (`write`: store to it), null
+// where the array is the copy engine's (host_view.cuh).
 constexpr int kHostCopies = 5;
 struct HostCopy {
     const void *src;
     void *dst;
     size_t bytes;
 };
-void *pinned_host_view(const void *host);
+void *pinned_host_view(const void *host, size_t bytes, bool write);
 lce_status launch_host_copies(const HostCopy (&copies)[kHostCopies], cudaStream_t s);
 // Bytes of the tiled kernel's weight image for this geometry (0 if the kernel does not cover it).
 // Launch plan of the tiled kernels for a geometry (no buffers involved), for lce_bconv2d_plan.

@@ -14,21 +14,30 @@ pytestmark = pytest.mark.gpu
 
 ONE, ZERO = lce.PAD_SAME_ONE, lce.PAD_SAME_ZERO
 FILL = 0xA5
+READ_ONLY = 8   # cudaHostRegisterReadOnly
 
 
 class Buffer:
-    """Host memory, pinned or pageable, that starts `offset` bytes past a 64-byte boundary, guard bytes on both sides."""
+    """Host memory that starts `offset` bytes past a page boundary, guard bytes on both sides.  How: "pinned", "pageable",
+    or "registered" / "read-only": pageable memory of which the array's bytes and no others are registered."""
 
-    def __init__(self, nbytes, pinned, offset=0):
-        self.whole = torch.full((nbytes + 320,), FILL, dtype=torch.uint8)
-        if pinned:
+    def __init__(self, nbytes, how, offset=0):
+        self.whole = torch.full((nbytes + 3 * 4096,), FILL, dtype=torch.uint8)
+        if how == "pinned":
             self.whole = self.whole.pin_memory()
-        self.first = -self.whole.data_ptr() % 64 + 64 + offset
+        self.first = -self.whole.data_ptr() % 4096 + 4096 + offset
         self.nbytes, self.ptr = nbytes, self.whole.data_ptr() + self.first
+        self.registered = how in ("registered", "read-only")
+        if self.registered:
+            assert int(torch.cuda.cudart().cudaHostRegister(self.ptr, nbytes, READ_ONLY if how == "read-only" else 0)) == 0
+
+    def release(self):
+        if self.registered:
+            assert int(torch.cuda.cudart().cudaHostUnregister(self.ptr)) == 0
 
     @classmethod
-    def of(cls, array, pinned, offset=0):
-        b = cls(array.nbytes, pinned, offset)
+    def of(cls, array, how, offset=0):
+        b = cls(array.nbytes, how, offset)
         b.whole[b.first:b.first + b.nbytes] = torch.from_numpy(np.ascontiguousarray(array).view(np.uint8).reshape(-1).copy())
         return b
 
@@ -45,8 +54,8 @@ def least_workspace(n, h, w, cin, cout, k, out_words):
     return up(n * h * w * words * 4) + up(cout * k * k * words * 4) + 3 * up(cout * 4) + up(out_words * 4)
 
 
-def check(shape, out_type, place=lambda name: (True, 0), workspace="full", entry="lce_bconv2d_host"):
-    """One call; `place` gives (pinned, offset) of an array by its name; `workspace`: what the call asks for, or the least
+def check(shape, out_type, place=lambda name: ("pinned", 0), workspace="full", entry="lce_bconv2d_host"):
+    """One call; `place` gives (how, offset) of an array by its name; `workspace`: what the call asks for, or the least
     it accepts (no room to pack weights)."""
     n, h, w, cin, cout, k, s, pad = shape
     rng = np.random.default_rng(sum(shape) + out_type)
@@ -81,6 +90,9 @@ def check(shape, out_type, place=lambda name: (True, 0), workspace="full", entry
     assert out.guards_intact() and all(b is None or b.guards_intact() for b in held.values())
     assert bool((ws[room:] == FILL).all().item()), "wrote past the workspace"
     assert lce.lce_device_status() == 0
+    for b in (out, *held.values()):
+        if b is not None:
+            b.release()
     return asked > least
 
 
@@ -88,6 +100,13 @@ def check(shape, out_type, place=lambda name: (True, 0), workspace="full", entry
 @pytest.mark.parametrize("which", ["input", "weights", "multiplier", "bias", "thresholds", "output", "all"])
 def test_pinned_arrays_that_start_on_any_byte(which, offset):
     out_type = lce.OUT_BITPACKED if which == "thresholds" else lce.OUT_FLOAT32
-    check((2, 9, 11, 40, 36, 3, 1, ONE), out_type, lambda name: (True, offset if which in (name, "all") else 0))
+    check((2, 9, 11, 40, 36, 3, 1, ONE), out_type, lambda name: ("pinned", offset if which in (name, "all") else 0))
     if which in ("output", "all"):
-        check((2, 9, 11, 40, 36, 3, 1, ONE), lce.OUT_BITPACKED, lambda name: (True, offset if which in (name, "all") else 0))
+        check((2, 9, 11, 40, 36, 3, 1, ONE), lce.OUT_BITPACKED, lambda name: ("pinned", offset if which in (name, "all") else 0))
+
+
+@pytest.mark.parametrize("offset", [0, 4, 100])
+def test_arrays_the_caller_has_registered(offset):
+    for out_type in (lce.OUT_FLOAT32, lce.OUT_BITPACKED):
+        check((2, 9, 11, 40, 36, 3, 1, ONE), out_type, lambda name: ("registered", offset))
+        check((2, 9, 11, 40, 36, 3, 1, ONE), out_type, lambda name: ("registered" if name == "output" else "read-only", offset))
