@@ -45,10 +45,6 @@ __global__ void __launch_bounds__(kCopyThreads) host_copy_kernel(const CopyParam
     }
 }
 
-}  // namespace
-
-namespace {
-
 // cuPointerGetAttributes, which tells all of HostMemory in one call (0.6 us); null if the driver has none.
 using PointerAttributes = CUresult (*)(unsigned int, CUpointer_attribute *, void **, CUdeviceptr);
 PointerAttributes pointer_attributes()
@@ -67,10 +63,7 @@ PointerAttributes pointer_attributes()
 void *pinned_host_view(const void *host, size_t bytes, bool write)
 {
     const PointerAttributes query = pointer_attributes();
-    unsigned int type = 0, access = 0;
-    int managed = 0;
-    CUdeviceptr view = 0, first = 0;
-    size_t size = 0;
+    uint64_t type = 0, managed = 0, view = 0, first = 0, size = 0, access = 0;  // as wide as the widest value the driver writes
     CUpointer_attribute names[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
                                    CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE, CU_POINTER_ATTRIBUTE_ACCESS_FLAGS};
     void *values[] = {&type, &managed, &view, &first, &size, &access};
@@ -83,7 +76,7 @@ void *pinned_host_view(const void *host, size_t bytes, bool write)
         if (cudaPointerGetAttributes(&a, host) != cudaSuccess) cudaGetLastError();
         if (query(kNames, names, values, address) != CUDA_SUCCESS) return nullptr;
     }
-    const HostMemory m{type == CU_MEMORYTYPE_HOST && !managed, view, first, size, access == CU_POINTER_ATTRIBUTE_ACCESS_FLAG_READWRITE};
+    const HostMemory m{type == CU_MEMORYTYPE_HOST && !managed, (uintptr_t)view, (uintptr_t)first, (size_t)size, access == CU_POINTER_ATTRIBUTE_ACCESS_FLAG_READWRITE};
     return reinterpret_cast<void *>(kernel_view(reinterpret_cast<uintptr_t>(host), bytes, write, m));
 }
 
