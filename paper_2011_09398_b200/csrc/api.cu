@@ -164,9 +164,14 @@ const Prepared &prepared_for(const lce_bconv2d_desc *desc, uint32_t form)
         uint32_t turn = 0;
     };
     static thread_local std::unique_ptr<Cache> cache;
-    if (!cache) cache.reset(new Cache);
+    static thread_local Prepared uncached;  // where there is no memory for the cache
+    if (!cache) cache.reset(new (std::nothrow) Cache);
     int device = -1;
     if (cudaGetDevice(&device) != cudaSuccess) device = -1;
+    if (!cache) {
+        prepare(desc, device, form, &uncached);
+        return uncached;
+    }
     uint32_t hash = form * 2654435761u;
     int32_t fields[sizeof(lce_bconv2d_desc) / 4];
     memcpy(fields, desc, sizeof(fields));

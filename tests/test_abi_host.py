@@ -1,7 +1,10 @@
 """Host-side checks of the C-ABI library that need no GPU: it loads, exports every symbol the
 header declares, and rejects malformed calls before touching the device."""
 import ctypes
+import os
 import re
+import subprocess
+import sys
 from pathlib import Path
 
 import numpy as np
@@ -231,6 +234,40 @@ def test_plans_are_remembered_per_geometry_not_mixed_up(lib):
     b = _plan(4, 20, 20, 64, 96, 3, 1, padding=lce.PAD_VALID)[0]
     c = _plan(4, 20, 20, 64, 96, 3, 1, out_type=lce.OUT_FLOAT32)[0]
     assert a == c and b["kernel"] == lce.KERNEL_TILED
+
+
+NO_MEMORY = r'''
+#include <cstdlib>
+#include <new>
+static bool failing = false;
+extern "C" void fail_allocations(int on) { failing = on != 0; }
+void *operator new(std::size_t n) { void *p = failing ? nullptr : std::malloc(n); if (!p) throw std::bad_alloc(); return p; }
+void *operator new(std::size_t n, const std::nothrow_t &) noexcept { return failing ? nullptr : std::malloc(n); }
+void operator delete(void *p) noexcept { std::free(p); }
+void operator delete(void *p, std::size_t) noexcept { std::free(p); }
+'''
+NO_MEMORY_CALLS = r'''
+import ctypes, sys
+shim, lib = ctypes.CDLL(sys.argv[1]), ctypes.CDLL(sys.argv[2])
+lib.lce_bconv2d_packed_weights_bytes.restype = ctypes.c_size_t
+desc = (ctypes.c_int32 * 14)(1, 14, 14, 64, 64, 3, 3, 1, 1, 1, 1, 0, 0, 1)
+out, other = ctypes.c_void_p(), (ctypes.c_int32 * 14)(2, 14, 14, 64, 64, 3, 3, 1, 1, 1, 1, 0, 0, 1)
+shim.fail_allocations(1)
+without = [lib.lce_bconv2d_packed_weights_bytes(d) for d in (desc, other, desc)]
+fake = ctypes.c_void_p(256)
+assert lib.lce_bconv2d_plan_create(desc, fake, fake, None, None, fake, fake, ctypes.byref(out)) == 4 and not out.value
+shim.fail_allocations(0)
+assert without == [lib.lce_bconv2d_packed_weights_bytes(d) for d in (desc, other, desc)] and min(without) > 0
+'''
+
+
+def test_a_failed_allocation_does_not_throw_through_the_c_interface(lib, tmp_path):
+    (tmp_path / "no_memory.cpp").write_text(NO_MEMORY)
+    shim = tmp_path / "no_memory.so"
+    subprocess.run(["g++", "-shared", "-fPIC", "-o", str(shim), str(tmp_path / "no_memory.cpp")], check=True)
+    done = subprocess.run([sys.executable, "-c", NO_MEMORY_CALLS, str(shim), str(lce_build.LIB)], env={**os.environ, "LD_PRELOAD": str(shim)},
+                          capture_output=True, text=True, timeout=120)
+    assert done.returncode == 0, done.stderr
 
 
 def test_plan_objects_check_their_arguments_on_the_host(lib):
