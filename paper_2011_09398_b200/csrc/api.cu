@@ -488,6 +488,10 @@ lce_status host_conv(const lce_bconv2d_desc *desc, const uint32_t *input, const 
     if (!aligned(workspace, 256)) return LCE_ERR_ALIGNMENT;
     const HostLayout L = host_layout(g);
     if (workspace_bytes < L.total) return LCE_ERR_WORKSPACE;
+    const Prepared &p = prepared_for(desc, FORM_HOST | (workspace_bytes < L.total + L.image ? FORM_NO_IMAGE : 0));
+    if (p.status != LCE_OK) return p.status;
+    if (p.pick == PICK_NONE) return LCE_ERR_UNSUPPORTED;
+    if (tensor_timeout_flagged()) return LCE_ERR_DEVICE_TIMEOUT;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     char *ws = static_cast<char *>(workspace);
     // arrays of up to kKernelCopy bytes in pinned memory travel together in one kernel, the others (first: the rest is
@@ -509,14 +513,11 @@ lce_status host_conv(const lce_bconv2d_desc *desc, const uint32_t *input, const 
     // a small output in pinned memory is written there directly
     void *out_view = L.out_bytes <= (g.out_type == LCE_OUT_BITPACKED ? kSmallWords : kSmallRows) && aligned(output, 16) ? pinned_host_view(output, L.out_bytes, true) : nullptr;
     void *d_out = out_view ? out_view : ws + L.out;
-    const Prepared &p = prepared_for(desc, FORM_HOST | (workspace_bytes < L.total + L.image ? FORM_NO_IMAGE : 0));
-    if (p.status != LCE_OK) return p.status;
     const auto at = [&](size_t off) { return reinterpret_cast<uint32_t *>(ws + off); };
     const uint32_t *d_in = at(L.in), *d_w = at(L.w);
     const float *d_mult = multiplier ? reinterpret_cast<const float *>(ws + L.mult) : nullptr, *d_bias = bias ? reinterpret_cast<const float *>(ws + L.bias) : nullptr;
     const int32_t *d_thr = thresholds ? reinterpret_cast<const int32_t *>(ws + L.thr) : nullptr;
     if (p.pick == PICK_TENSOR) {
-        if (tensor_timeout_flagged()) return LCE_ERR_DEVICE_TIMEOUT;
         st = launch_pack_weights_tensor(g, d_w, ws + L.total, s);
         if (st == LCE_OK) st = launch_bconv_tensor(p.launch, d_in, ws + L.total, d_mult, d_bias, d_thr, d_out, s);
     } else {

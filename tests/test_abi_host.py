@@ -84,6 +84,12 @@ def test_argument_errors_come_back_as_status_codes(lib):
     assert lib.lce_add_f32(fake, fake, fake, 0, null) == 0
     assert lib.lce_add_f32(null, fake, fake, 4, null) == 1
     assert lib.lce_bconv2d_host_workspace_bytes(ctypes.byref(bad)) == 0
+    # host-buffer form: a kernel that does not cover the call is refused before a copy is enqueued (which needs a GPU: status 4)
+    lib.lce_bconv2d_host_async.argtypes = lib.lce_bconv2d_host.argtypes
+    for choice, kernel in ((lce.KERNEL_TENSOR, (3, 3)), (lce.KERNEL_TILED, (7, 7))):
+        forced = lce.make_desc(1, 9, 9, 64, 64, kernel, kernel_choice=choice)
+        for fn in (lib.lce_bconv2d_host, lib.lce_bconv2d_host_async):
+            assert fn(ctypes.byref(forced), fake, fake, fake, fake, null, fake, fake, 1 << 20, null) == 2
     assert lib.lce_bconv2d_host_workspace_bytes(ctypes.byref(d)) >= 4 * 4 * 4 + 32 * 9 * 4 + 4 * 4 * 32 * 4
 
 
