@@ -110,3 +110,54 @@ def test_arrays_the_caller_has_registered(offset):
     for out_type in (lce.OUT_FLOAT32, lce.OUT_BITPACKED):
         check((2, 9, 11, 40, 36, 3, 1, ONE), out_type, lambda name: ("registered", offset))
         check((2, 9, 11, 40, 36, 3, 1, ONE), out_type, lambda name: ("registered" if name == "output" else "read-only", offset))
+
+
+# n, h, w, cin, cout, k, stride, padding: arrays of 1, 2 and 3 words past a 16-byte piece, one word in all, and more
+RAGGED = [(1, 1, 1, 1, 1, 1, 1, ONE), (1, 1, 5, 32, 3, 1, 1, ONE), (1, 3, 5, 40, 5, 3, 1, ZERO), (1, 7, 1, 96, 2, 1, 1, ONE), (3, 5, 7, 70, 33, 3, 2, ONE)]
+
+
+@pytest.mark.parametrize("out_type", [lce.OUT_FLOAT32, lce.OUT_BITPACKED, lce.OUT_INT32])
+@pytest.mark.parametrize("shape", RAGGED, ids=lambda s: "x".join(map(str, s)))
+def test_arrays_that_are_not_whole_pieces(shape, out_type):
+    check(shape, out_type)
+
+
+NAMES = ("input", "weights", "multiplier", "bias", "thresholds", "output")
+
+
+@pytest.mark.parametrize("entry", ["lce_bconv2d_host", "lce_bconv2d_host_noalloc"])
+@pytest.mark.parametrize("pageable", [{n} for n in NAMES] + [set(NAMES), {"input", "bias", "output"}, {"weights", "multiplier", "thresholds"}],
+                         ids=lambda s: "+".join(n for n in NAMES if n in s) if len(s) < 6 else "all")
+def test_pageable_arrays_beside_pinned_ones(pageable, entry):
+    for out_type in (lce.OUT_FLOAT32, lce.OUT_BITPACKED):
+        check((2, 9, 11, 40, 36, 3, 1, ONE), out_type, lambda name: ("pageable" if name in pageable else "pinned", 0), entry=entry)
+
+
+# around the limits of the two ways for small arrays: copied by a kernel up to 2 MB, outputs written in place up to 256 KB
+# of floats and 32 KB of bit-packed words; exactly at a limit and one word past it
+LIMITS = [(1, 512, 1024, 32, 1, lce.OUT_BITPACKED), (1, 1, 524289, 32, 1, lce.OUT_BITPACKED), (1, 512, 1024, 32, 1, lce.OUT_FLOAT32),
+          (1, 1, 524289, 32, 1, lce.OUT_INT32), (1, 2, 2, 8192, 2048, lce.OUT_FLOAT32), (1, 2, 2, 8192, 2049, lce.OUT_BITPACKED),
+          (1, 64, 128, 32, 32, lce.OUT_BITPACKED), (1, 3, 2731, 32, 32, lce.OUT_BITPACKED), (1, 256, 256, 32, 1, lce.OUT_FLOAT32),
+          (1, 1, 65537, 32, 1, lce.OUT_FLOAT32), (1, 1, 65537, 32, 1, lce.OUT_INT32)]
+
+
+@pytest.mark.parametrize("how", ["pinned", "pageable"])
+@pytest.mark.parametrize("case", LIMITS, ids=lambda c: "x".join(map(str, c)))
+def test_arrays_around_the_limits_of_the_copy_kernel_and_of_outputs_written_in_place(case, how):
+    n, h, w, cin, cout, out_type = case
+    check((n, h, w, cin, cout, 1, 1, ONE), out_type, lambda name: (how, 0))
+
+
+@pytest.mark.parametrize("out_type", [lce.OUT_FLOAT32, lce.OUT_BITPACKED, lce.OUT_INT32])
+@pytest.mark.parametrize("shape", [(16, 28, 28, 128, 128, 3, 1, ONE), (64, 27, 25, 100, 72, 3, 2, ZERO)], ids=lambda s: "x".join(map(str, s)))
+def test_workspace_with_and_without_room_for_packed_weights(shape, out_type):
+    assert check(shape, out_type, workspace="full") and check(shape, out_type, workspace="least")
+
+
+def test_built_in_workspace_without_room_for_packed_weights():
+    """The built-in array is enough for the call and not for the packed weights beside it: the call runs all the same."""
+    shape = (124, 16, 16, 64, 64, 3, 1, ONE)
+    limit = lce.lce_bconv2d_host_noalloc_max_bytes()
+    assert least_workspace(*shape[:6], 124 * 16 * 16 * 64) <= limit
+    assert lce.lce_bconv2d_host_workspace_bytes(lce.make_desc(*shape[:5])) > limit
+    check(shape, lce.OUT_FLOAT32, entry="lce_bconv2d_host_noalloc")
