@@ -225,7 +225,9 @@ lce_status lce_bconv2d_pack_weights(const lce_bconv2d_desc *desc, const uint32_t
  * DEVICE buffer of at least lce_bconv2d_host_workspace_bytes(desc) bytes that the call uses
  * for the device copies of input, weights, per-channel arrays and output, and where it pays for a packed
  * copy of the weights (without that room, which earlier versions did not ask for, the call still runs, on
- * the kernel for plain weights).  Copies in, runs the convolution (weights_packed must be 0; kernel
+ * the kernel for plain weights).  The arrays may start on any byte and lie in pageable memory; those of up to
+ * 2 MB that are pinned as a whole (one allocation or registration) and start on 4 bytes are copied by a kernel
+ * instead of the copy engine, and a small output that starts on 16 is written in place.  Copies in, runs the convolution (weights_packed must be 0; kernel
  * AUTO also takes the kernels that want packed weights), copies the output back, all on `stream`, and
  * returns after synchronising that stream.  LCE_ERR_WORKSPACE if workspace_bytes is too small. */
 size_t lce_bconv2d_host_workspace_bytes(const lce_bconv2d_desc *desc);
@@ -248,8 +250,9 @@ lce_status lce_bconv2d_host_async(const lce_bconv2d_desc *desc, const uint32_t *
  * staging area inside the library, in one fixed device array of
  * lce_bconv2d_host_noalloc_max_bytes() = 8 MiB per GPU, and calls no cudaMalloc, cudaFree or any
  * other allocating routine.  Arguments and result are those of lce_bconv2d_host without the
- * workspace; a call whose lce_bconv2d_host_workspace_bytes(desc) exceeds the array returns
- * LCE_ERR_WORKSPACE and does nothing.
+ * workspace; a call whose input, weights, per-channel arrays and output do not fit the array returns
+ * LCE_ERR_WORKSPACE and does nothing.  lce_bconv2d_host_workspace_bytes(desc) may be larger than the array all
+ * the same: where only the room for packed weights is missing, the call runs on the kernel for plain weights.
  *   - The first call on each device looks up the array's device address (with that device
  *     current).  The call synchronises `stream` before it returns, so it cannot be part of a stream
  *     capture anyway.
@@ -278,8 +281,8 @@ lce_status lce_add_f32(const float *a, const float *b, float *out, int64_t n, vo
  * (operands ready, MMAs complete, accumulator read out); every such wait is limited to 0.2 s, after
  * which the kernel stops working, waits (bounded) for its copies and MMAs in flight, frees its tensor
  * memory and returns, leaving its output incomplete.  It records that in a device word and in a word
- * of mapped host memory; from then on lce_bconv2d, lce_bconv2d_fused and lce_plan_run on that device
- * return LCE_ERR_DEVICE_TIMEOUT without launching, until lce_device_status_reset.
+ * of mapped host memory; from then on lce_bconv2d, its host-buffer forms, lce_bconv2d_fused and lce_plan_run on that
+ * device return LCE_ERR_DEVICE_TIMEOUT without launching, until lce_device_status_reset.
  *   lce_device_status        *status (HOST pointer) = 0 if no wait has given up on the current device
  *                            since load or the last reset, 1 otherwise.  Synchronous (reads the device word).
  *   lce_device_status_reset  clears both words for the current device.  Synchronous.

@@ -276,7 +276,7 @@ def lce_bconv2d_host_noalloc_max_bytes() -> int:
 def lce_bconv2d_host_noalloc(desc: BConv2dDesc, input, weights, multiplier, bias, thresholds, out) -> None:
     """lce_bconv2d_host without the workspace argument: for callers that cannot allocate device
     memory.  Every tensor is a host tensor; the staging area is a fixed array inside the library
-    (shared by all calls on the device, so do not overlap calls)."""
+    (shared by all calls on the device, so do not overlap calls), which has to hold the tensors themselves."""
     out_dtype = torch.float32 if desc.out_type == OUT_FLOAT32 else torch.int32
     _check(library().lce_bconv2d_host_noalloc(
         ctypes.byref(desc), _host(input, torch.int32, "input"), _host(weights, torch.int32, "weights"),
