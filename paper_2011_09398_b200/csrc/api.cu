@@ -447,12 +447,12 @@ extern "C" lce_status lce_bconv2d_pack_weights(const lce_bconv2d_desc *desc, con
     if (!aligned(weights, 4) || !aligned(packed, 256)) return LCE_ERR_ALIGNMENT;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const size_t plain = (size_t)g.Cout * g.KH * g.KW * g.Cw * 4;
-    if (cudaMemcpyAsync(packed, weights, plain, cudaMemcpyDeviceToDevice, s) != cudaSuccess) return LCE_ERR_CUDA;
     const WeightParts parts = weight_parts(g);
     char *base = static_cast<char *>(packed);
+    if (!parts.small && cudaMemcpyAsync(packed, weights, plain, cudaMemcpyDeviceToDevice, s) != cudaSuccess) return LCE_ERR_CUDA;
     if (parts.tiled && (st = launch_pack_weights_tiled(g, weights, reinterpret_cast<uint32_t *>(base + parts.tiled), s)) != LCE_OK) return st;
     if (parts.tensor && (st = launch_pack_weights_tensor(g, weights, base + parts.tensor, s)) != LCE_OK) return st;
-    if (parts.small) return launch_pack_weights_small(g, weights, reinterpret_cast<uint32_t *>(base + parts.small), s);
+    if (parts.small) return launch_pack_weights_small(g, weights, static_cast<uint32_t *>(packed), reinterpret_cast<uint32_t *>(base + parts.small), s);
     return LCE_OK;
 }
 

@@ -175,7 +175,7 @@ bool small_covers(const ConvGeom &g);
 int64_t small_ctas(const ConvGeom &g);
 void small_plan_info(const ConvGeom &g, TiledPlanInfo *info);
 size_t small_weight_image_bytes(const ConvGeom &g);
-lce_status launch_pack_weights_small(const ConvGeom &g, const uint32_t *w, uint32_t *image, cudaStream_t s);
+lce_status launch_pack_weights_small(const ConvGeom &g, const uint32_t *w, uint32_t *plain, uint32_t *image, cudaStream_t s);  // plain: a copy of w
 lce_status prepare_bconv_small(const ConvGeom &g, PreparedLaunch *prepared);
 lce_status launch_bconv_small(const PreparedLaunch &prepared, const uint32_t *in, const uint32_t *w, const uint32_t *w_image, const float *mult,
                               const float *bias, const int32_t *thr, void *out, cudaStream_t s,

@@ -102,3 +102,16 @@ def test_weights_packed_under_one_padding_mode_run_under_every_other(shape):
     if k != 7:
         assert (VALID, lce.KERNEL_TENSOR) in covered and (ONE, lce.KERNEL_TENSOR) not in covered
     assert lce.lce_device_status() == 0
+
+
+@pytest.mark.parametrize("cin,cout,k", [(1, 1, 1), (33, 31, 1), (64, 64, 3), (3, 32, 3), (512, 40, 3), (96, 130, 5), (7300, 5, 3), (4000, 33, 1)])
+def test_packed_weights_begin_with_the_plain_words(cin, cout, k):
+    """With the latency kernel's image its packing kernel copies them, without (the last but one) the copy engine does."""
+    rng = np.random.default_rng(cin + cout)
+    plain = to_dev_words(oracle.bitpack_pm1((2 * rng.integers(0, 2, size=(cout, k, k, cin)) - 1).astype(np.int8)))
+    desc = lce.make_desc(1, 9, 9, cin, cout, (k, k), weights_packed=1)
+    words = lce.lce_bconv2d_packed_weights_bytes(desc) // 4
+    whole = to_dev(np.full(words + 128, 0x5A5A5A5A, dtype=np.int32))
+    packed = lce.lce_bconv2d_pack_weights(desc, plain, whole[64:64 + words])
+    assert bool((packed[:plain.numel()] == plain.reshape(-1)).all().item())
+    assert bool((whole[:64] == 0x5A5A5A5A).all().item()) and bool((whole[64 + words:] == 0x5A5A5A5A).all().item())
