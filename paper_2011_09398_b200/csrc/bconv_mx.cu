@@ -682,7 +682,8 @@ __device__ __forceinline__ MxFin mx_fin_context(const MxParams &p, int fw, int l
 
 // Two additions in one instruction: the warps of a CTA share the issue slots (60% of them taken on a 64-channel layer),
 // and what one role saves is time for the others.  56x56x64, 256 images, bits: 29.7 -> 29.0 us.  (The float transforms
-// do not gain from the same for their multiply-adds: 14.1 -> 14.2 us on 56x56x64, 64 images; their stores set the pace.)
+// do not gain from the same for their multiply-adds: 14.1 -> 14.2 us on 56x56x64, 64 images, as graph replays (15.6 called
+// one after another); their stores set the pace.)
 __device__ __forceinline__ void add_pair(float &x, float &y, float c)
 {
     asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %2};\n\tadd.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}" : "+f"(x), "+f"(y) : "f"(c));
