@@ -1,5 +1,6 @@
 """lce_bconv2d_host against the oracle, every element, over the ways an array can reach the device and an output can come
 back: by the copy engine or by a kernel, or written by the convolution itself."""
+import concurrent.futures
 import ctypes
 
 import numpy as np
@@ -161,3 +162,12 @@ def test_built_in_workspace_without_room_for_packed_weights():
     assert least_workspace(*shape[:6], 124 * 16 * 16 * 64) <= limit
     assert lce.lce_bconv2d_host_workspace_bytes(lce.make_desc(*shape[:5])) > limit
     check(shape, lce.OUT_FLOAT32, entry="lce_bconv2d_host_noalloc")
+
+
+def test_calls_from_fresh_host_threads():
+    """A thread's first CUDA call may be this one; several at a time, each with arrays and a workspace of its own."""
+    shapes = [(2, 9, 11, 40, 36, 3, 1, ONE), (16, 28, 28, 128, 128, 3, 1, ONE), (1, 512, 1024, 32, 1, 1, 1, ONE), (3, 5, 7, 70, 33, 3, 2, ONE)]
+    with concurrent.futures.ThreadPoolExecutor(len(shapes)) as pool:
+        for done in [pool.submit(check, shape, out_type, workspace=room) for shape in shapes
+                     for out_type, room in ((lce.OUT_FLOAT32, "full"), (lce.OUT_BITPACKED, "least"))]:
+            done.result()
