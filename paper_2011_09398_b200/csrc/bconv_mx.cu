@@ -26,12 +26,16 @@
 //     buffer of T * Nt + halo rows, so the halo a tile reads beyond its own positions is staged once
 //     per T tiles; there are two to four such buffers (as many as shared memory has room for, up to what
 //     lets the loaders run four tiles ahead).
+//   * K is the taps' channel words, 32 values each, two to an instruction (mx_word): the two chunks of its B operand are
+//     rows of one buffer any distance apart, so the last words of an odd count pair up across taps.  A word of zeros
+//     per tap instead cost 9 MMAs for 9 words (32 channels, 3x3; now 5) and 75 for 125 (160 channels, 5x5; now 63:
+//     32x32x160, 64 images, float 36.4 -> 33.3 us).
 //   * the weights were expanded when the model was loaded (lce_bconv2d_pack_weights) into the exact
-//     operand image [channel block][tap][channel word][128 channels][16 bytes] (for out_c <= 64 the
+//     operand image [channel block][pair of words][2][128 channels][16 bytes] (for out_c <= 64 the
 //     channel block is repeated down the 128 rows, so that every TMEM lane quarter holds values a
-//     finisher warp can work on); the bulk-copy engine brings taps into a ring of shared-memory stages
-//     (cp.async.bulk + mbarrier transaction count).  If every tap fits they are fetched once per CTA,
-//     all counted on one barrier; otherwise they stream past once per tile, in groups of taps that
+//     finisher warp can work on); the bulk-copy engine brings pairs into a ring of shared-memory stages
+//     (cp.async.bulk + mbarrier transaction count).  If every pair fits they are fetched once per CTA,
+//     all counted on one barrier; otherwise they stream past once per tile, in groups of pairs that
 //     alternate between two stages (one copy, one wait and one commit per group).
 //   * roles: 8 loader warps (prefetch the packed words of the next chunk with cp.async, expand the
 //     current one), one warp that issues the MMAs (all lanes run the same code, the elected lane
@@ -71,6 +75,7 @@ constexpr int kMaxNt = 224;                                  // tile width (posi
 constexpr uint32_t kD1Col = 240;                             // TMEM column of the second accumulator buffer
 constexpr uint32_t kSfaCol = 480, kSfbCol = 496;             // block scales (all 1.0) of the A / B operand
 constexpr int kMaxTaps = 64;
+constexpr int kPairBytes = 4096;                             // weights of an MMA: two words of K, 128 rows, 16 bytes each
 constexpr int kMaxStages = 32;
 constexpr int kPixSlots = 8;                                 // see the note at kOffPix
 
@@ -173,7 +178,7 @@ struct MxParams {
     const float *residual;   // fused shortcut (float output), or null
     uint32_t *out_packed;    // fused LceQuantize of the float result, or null
     int *host_flag;          // host-mapped word set when a wait gives up, or null
-    int32_t N, H, W, Cw, Cw2, Cout, Cow;
+    int32_t N, H, W, Cw, Cout, Cow;
     int32_t OH, OW, KH, KW, stride, pt, pl, K;
     int32_t Wg, Hg, n_phase;
     uint32_t Wg_mul, Wg_sh, Hg_mul, Hg_sh;                // divisions by Wg, Hg as multiply + shift
@@ -182,13 +187,15 @@ struct MxParams {
     int32_t Nt, P;           // tile width; rows of a position buffer per phase and channel word = T * Nt + halo
     int32_t T, halo;         // tiles that share a position buffer; positions a tile reads beyond its own
     int32_t n_tiles, n_super, total_q;
-    int32_t taps, ksteps, stages, resident;
-    int32_t group_taps, groups;  // streamed weights: taps per ring stage, stages' worth of taps per tile = ceil(taps / group_taps)
-    int32_t tap_bytes, x_bytes;
+    int32_t pairs, stages, resident;
+    int32_t group_pairs, groups;  // streamed weights: pairs per ring stage, stages' worth of pairs per tile = ceil(pairs / group_pairs)
+    int32_t x_bytes;
     int32_t n_xbuf, ahead;   // position buffers (2..4); tiles the loaders may be ahead of the finished MMAs (2..4)
     int32_t off_tbl, off_w, off_x;    // byte offsets in shared memory
     int32_t cp_words;        // words per cp.async: 4, 2 or 1
     int32_t pad_zero, out_type, activation, write_float;
+    uint32_t even_mul, even_sh;            // divisions by the even number of channel words, as multiply + shift
+    uint16_t tap_rows[kMaxTaps];           // first row of a tap's words in a position buffer, taps in the order of mx_word
     int32_t dup_log2;        // log2 of the copies of the channel block in the 128 rows: 1 for out_c <= 64, 2 for out_c <= 32, else 0
 };
 
@@ -387,7 +394,7 @@ __device__ __forceinline__ bool mx_load_tiles(const MxParams &p, const MxLoad &l
                                               int tid, int first_tile, int tile_step)
 {
     const int Nt = p.Nt, T = p.T, halo = p.halo, n_tiles = p.n_tiles, n_super = p.n_super, n_xbuf = p.n_xbuf, ahead = p.ahead;
-    const int OH = p.OH, OW = p.OW, plane = p.Cw2 * p.P, cp_words = p.cp_words;
+    const int OH = p.OH, OW = p.OW, plane = p.Cw * p.P, cp_words = p.cp_words;
     const uint32_t x_bytes = (uint32_t)p.x_bytes;
     const bool pad_zero = p.pad_zero != 0;
     const MxStep tile_d = p.step_tile, tile_super = p.step_tile_super, chunk_first = p.step_chunk_first, chunk_super = p.step_chunk_super;
@@ -422,11 +429,44 @@ __device__ __forceinline__ bool mx_load_tiles(const MxParams &p, const MxLoad &l
     return true;
 }
 
-// B operand of tap (ky, kx): its phase buffer (stride 2) shifted by the tap's position offset, in 16-byte units
-__device__ __forceinline__ uint32_t tap_b_offset(const MxParams &p, int ky, int kx)
+// The order of K: word i of an output's taps x Cw words, as a tap (row, column) and a channel word.  Taps by their place
+// in a position buffer, which for stride 2 is phase by phase; every tap's channel words two by two; where their number
+// is odd, the taps' last ones at the end.  Two words of a pair are then one behind the other in the buffer (the distance
+// in the operand descriptor has no sign), and pairs are as few as the words allow.
+struct MxWord {
+    int ky, kx, cw;
+};
+
+__host__ __device__ __forceinline__ MxWord mx_word(int i, int KH, int KW, int Cw, int stride)
 {
-    if (p.stride == 2) return (uint32_t)((((ky & 1) * 2 + (kx & 1)) * p.Cw2) * p.P + (ky >> 1) * p.Wg + (kx >> 1));
-    return (uint32_t)(ky * p.Wg + kx);
+    const int even = Cw & ~1, paired = KH * KW * even;
+    MxWord w;
+    int tap = i < paired ? i / even : i - paired;
+    w.cw = i < paired ? i - tap * even : Cw - 1;
+    if (stride == 1) {
+        w.ky = tap / KW;
+        w.kx = tap - w.ky * KW;
+        return w;
+    }
+    w.ky = w.kx = 0;
+    for (int phase = 0; phase < 4; ++phase) {
+        const int py = phase >> 1, px = phase & 1, rows = (KH - py + 1) / 2, cols = (KW - px + 1) / 2;
+        if (tap < rows * cols) {
+            w.ky = py + 2 * (tap / cols);
+            w.kx = px + 2 * (tap % cols);
+            break;
+        }
+        tap -= rows * cols;
+    }
+    return w;
+}
+
+// its first row in a position buffer, in 16-byte units: the tap's (worked out on the host: dividing it out here, from cold
+// code, took 0.2 us of every launch) in the plane of its channel word
+__device__ __forceinline__ uint32_t word_b_offset(const MxParams &p, int i, int even, int paired)
+{
+    const int tap = i < paired ? fast_div(i, p.even_mul, p.even_sh) : i - paired;
+    return p.tap_rows[tap] + (uint32_t)((i < paired ? i - tap * even : even) * p.P);
 }
 
 // One lane of the converged warp, the same one every time
@@ -897,9 +937,9 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
     // ---- set-up, its parts side by side: the issuer warp allocates TMEM, the producer warp initialises the
     // barriers and starts the weight copies, the finisher warps fill the table of operand offsets, the
     // loaders fetch the first chunk of activations ---------------------------------------------------------
-    const int n_mma = p.taps * p.ksteps;
-    // the weight producer's progress (one thread): fills issued, ring stage and (tile-local) tap group of the next one
-    int prod_g = 0, prod_total = 0, prod_stage = 0, prod_tap = 0;
+    const int n_mma = p.pairs;
+    // the weight producer's progress (one thread): fills issued, ring stage and (tile-local) group of pairs of the next one
+    int prod_g = 0, prod_total = 0, prod_stage = 0, prod_group = 0;
     uint32_t prod_parity = 1;  // the first pass over the ring waits for nothing
     if (warp == kIssuerWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)) : "memory");
@@ -912,28 +952,28 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         __syncwarp();
         // The weights are constants of the model: their copies start at once, whatever the previous kernel of
-        // the stream is still doing, one lane per copy.  Resident: all taps, every copy counted on the same
+        // the stream is still doing, one lane per copy.  Resident: all pairs, every copy counted on the same
         // barrier; streamed: the first pass over the ring (stage = fill number; at most 32 stages).
-        const uint8_t *src = p.wimg + (size_t)blockIdx.y * p.taps * p.tap_bytes;
+        const uint8_t *src = p.wimg + (size_t)blockIdx.y * p.pairs * kPairBytes;
         if (p.resident) {
-            if (lane == 0) mbar_expect_tx(&bars[BAR_FULL_W0], (uint32_t)(p.taps * p.tap_bytes));
+            if (lane == 0) mbar_expect_tx(&bars[BAR_FULL_W0], (uint32_t)(p.pairs * kPairBytes));
             __syncwarp();
-            for (int tap = lane; tap < p.taps; tap += 32)
-                bulk_copy_g2s(sW + (size_t)tap * p.tap_bytes, src + (size_t)tap * p.tap_bytes, (uint32_t)p.tap_bytes, &bars[BAR_FULL_W0]);
+            const int share = (p.pairs + 31) >> 5, first = lane * share, n = min(share, p.pairs - first);
+            if (n > 0) bulk_copy_g2s(sW + (size_t)first * kPairBytes, src + (size_t)first * kPairBytes, (uint32_t)(n * kPairBytes), &bars[BAR_FULL_W0]);
             prod_g = 1;
         } else {
             int my_tiles = 0;
             for (int st = first_tile; st < p.n_super; st += tile_step) my_tiles += min(p.T, p.n_tiles - st * p.T);
-            // a fill = one group of up to group_taps consecutive taps (one copy: they are contiguous in the image)
+            // a fill = one group of up to group_pairs consecutive pairs (one copy: they are contiguous in the image)
             prod_total = my_tiles * p.groups;
             prod_g = min(p.stages, prod_total);
             if (lane < prod_g) {
-                const int first = (lane % p.groups) * p.group_taps;
-                const uint32_t bytes = (uint32_t)(min(p.group_taps, p.taps - first) * p.tap_bytes);
+                const int first = (lane % p.groups) * p.group_pairs;
+                const uint32_t bytes = (uint32_t)(min(p.group_pairs, p.pairs - first) * kPairBytes);
                 mbar_expect_tx(&bars[BAR_FULL_W0 + lane], bytes);
-                bulk_copy_g2s(sW + (size_t)lane * p.group_taps * p.tap_bytes, src + (size_t)first * p.tap_bytes, bytes, &bars[BAR_FULL_W0 + lane]);
+                bulk_copy_g2s(sW + (size_t)lane * p.group_pairs * kPairBytes, src + (size_t)first * kPairBytes, bytes, &bars[BAR_FULL_W0 + lane]);
             }
-            prod_tap = prod_g % p.groups;   // the next fill's group within its tile
+            prod_group = prod_g % p.groups;   // the next fill's group within its tile
             if (prod_g == p.stages) prod_parity ^= 1u; else prod_stage = prod_g;
         }
         __syncwarp();
@@ -943,12 +983,14 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
         }
     } else if (tid >= kLoaders) {
         uint2 *tbl = reinterpret_cast<uint2 *>(smem + p.off_tbl);
+        const int even = p.Cw & ~1, paired = p.KH * p.KW * even, words = p.KH * p.KW * p.Cw;
         for (int e = tid - kLoaders; e < n_mma; e += kFinishers) {
-            const int tap = e / p.ksteps, kk = e - tap * p.ksteps;
-            const int ky = tap / p.KW, kx = tap - ky * p.KW;
-            // A: the tap's place among the resident taps or in its group of streamed ones + K step; B: the tap's offset + K step
-            const uint32_t b_off = tap_b_offset(p, ky, kx);
-            tbl[e] = make_uint2((uint32_t)(p.resident ? tap : tap % p.group_taps) * ((uint32_t)p.tap_bytes >> 4) + 256u * kk, b_off + 2u * (uint32_t)p.P * kk);
+            // A: the pair's place among the resident ones or in its group of streamed ones.  B: the first word's rows, and in
+            // the upper half the distance from there to the second word's; an odd last word has a second one of zero
+            // weights, whose rows may be any (the next ones: a position buffer has one row to spare)
+            const uint32_t first = word_b_offset(p, 2 * e, even, paired);
+            const uint32_t apart = 2 * e < paired ? (uint32_t)p.P : 2 * e + 1 < words ? word_b_offset(p, 2 * e + 1, even, paired) - first : 1u;
+            tbl[e] = make_uint2((uint32_t)(p.resident ? e : e % p.group_pairs) * (kPairBytes >> 4), first | apart << 16);
         }
     }
     // The loaders' first prefetch goes out before the CTA-wide barrier of the set-up: it needs the previous
@@ -1035,15 +1077,15 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
         // instruction descriptor (block-scaled kinds): A, B = e2m1 (1), both K-major, N >> 3 at bit 17,
         // scales ue8m0 (bit 23), M >> 4 at bit 24, scale-factor ids 0
         const uint32_t idesc = (1u << 7) | (1u << 10) | ((uint32_t)(p.Nt >> 3) << 17) | (1u << 23) | ((uint32_t)(128 >> 4) << 24);
-        // shared-memory descriptors (units of 16 bytes): low = start | K-chunk stride << 16; high = 8-row
+        // shared-memory descriptors (units of 16 bytes): low = start | K-chunk stride << 16 (B: from the table); high = 8-row
         // group stride (128 bytes) | version 1 at bit 46; no swizzle
         const uint32_t desc_hi = 8u | (1u << 14);
         // everything the loops use, read from the kernel parameters once
-        const int T = p.T, n_tiles = p.n_tiles, n_super = p.n_super, Nt = p.Nt, ksteps = p.ksteps, stages = p.stages, taps = p.taps, group_taps = p.group_taps;
+        const int T = p.T, n_tiles = p.n_tiles, n_super = p.n_super, Nt = p.Nt, stages = p.stages, group_pairs = p.group_pairs;
         const bool resident = p.resident != 0;
         const uint32_t w_lo0 = ((uint32_t)p.off_w >> 4) + (smem_u32(smem) >> 4) + (128u << 16);
-        const uint32_t x_lo_buf0 = ((uint32_t)p.off_x >> 4) + (smem_u32(smem) >> 4) + ((uint32_t)p.P << 16);
-        const uint32_t x_units = (uint32_t)p.x_bytes >> 4, group_units = ((uint32_t)p.tap_bytes >> 4) * (uint32_t)p.group_taps;
+        const uint32_t x_lo_buf0 = ((uint32_t)p.off_x >> 4) + (smem_u32(smem) >> 4);
+        const uint32_t x_units = (uint32_t)p.x_bytes >> 4, group_units = (uint32_t)(kPairBytes >> 4) * (uint32_t)p.group_pairs;
         const uint32_t sfa = tmem_base + kSfaCol, sfb = tmem_base + kSfbCol;
         const int n_xbuf = p.n_xbuf;
         ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bars[BAR_SCALES], 0));  // the block scales are in TMEM
@@ -1067,7 +1109,7 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
             const uint32_t x_lo0 = x_lo_buf0 + (uint32_t)xbuf * x_units + (uint32_t)(k * Nt);
             uint32_t accumulate = 0;
             if (resident) {
-                // every tap stays in shared memory: one wait for all of them (a single barrier counts the bytes
+                // every pair stays in shared memory: one wait for all of them (a single barrier counts the bytes
                 // of all the copies) before the CTA's first tile, then nothing between the MMAs of a tile
                 if (it < 2) {  // this warp's first tile
                     ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bars[BAR_FULL_W0], 0));
@@ -1077,19 +1119,19 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
                 }
                 mx_issue_table(tmem_d, tbl, n_mma, w_lo0, x_lo0, desc_hi, idesc, sfa, sfb, accumulate);
             } else {
-                // the taps stream through the ring a group at a time: wait for the group, issue its MMAs in one run, hand
-                // its stage back (the wait, the commit and the bookkeeping cost this warp as much as some MMAs: hence
-                // groups, not single taps; issued tap by tap, a group of five taps cost 600 clocks more than its MMAs)
-                int tap = 0;
-                while (tap < taps) {
+                // the pairs stream through the ring a group at a time: wait for the group, issue its MMAs in one run, hand
+                // its stage back (the wait, the commit and the bookkeeping cost this warp as much as some MMAs: issued tap
+                // by tap, a group of five taps cost 600 clocks more than its MMAs)
+                int pair = 0;
+                while (pair < n_mma) {
                     ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bars[BAR_FULL_W0 + stage_i], w_parity));
                     if (!ok) break;
                     ++g;
                     if (lane == 0) fills[1] = g;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const int n_taps = min(group_taps, taps - tap);
-                    mx_issue_table(tmem_d, tbl + tap * ksteps, n_taps * ksteps, w_lo0 + (uint32_t)stage_i * group_units, x_lo0, desc_hi, idesc, sfa, sfb, accumulate);
-                    tap += n_taps;
+                    const int n = min(group_pairs, n_mma - pair);
+                    mx_issue_table(tmem_d, tbl + pair, n, w_lo0 + (uint32_t)stage_i * group_units, x_lo0, desc_hi, idesc, sfa, sfb, accumulate);
+                    pair += n;
                     if (elect_one()) mma_commit(&bars[BAR_EMPTY_W0 + stage_i]);
                     if (++stage_i == stages) { stage_i = 0; w_parity ^= 1u; }
                 }
@@ -1101,17 +1143,17 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
             }
         }
     } else if (tid == kProducerTid) {
-        // ======================= weight producer: one thread, the rest of the streamed taps ===========
-        const uint8_t *src = p.wimg + (size_t)blockIdx.y * p.taps * p.tap_bytes;
+        // ======================= weight producer: one thread, the rest of the streamed pairs ==========
+        const uint8_t *src = p.wimg + (size_t)blockIdx.y * p.pairs * kPairBytes;
         for (; !p.resident && prod_g < prod_total; ++prod_g) {
             ok = mbar_wait_bounded(&bars[BAR_EMPTY_W0 + prod_stage], prod_parity);
             if (!ok) break;
-            const int first = prod_tap * p.group_taps;
-            const uint32_t bytes = (uint32_t)(min(p.group_taps, p.taps - first) * p.tap_bytes);
+            const int first = prod_group * p.group_pairs;
+            const uint32_t bytes = (uint32_t)(min(p.group_pairs, p.pairs - first) * kPairBytes);
             mbar_expect_tx(&bars[BAR_FULL_W0 + prod_stage], bytes);
-            bulk_copy_g2s(sW + (size_t)prod_stage * p.group_taps * p.tap_bytes, src + (size_t)first * p.tap_bytes, bytes, &bars[BAR_FULL_W0 + prod_stage]);
+            bulk_copy_g2s(sW + (size_t)prod_stage * p.group_pairs * kPairBytes, src + (size_t)first * kPairBytes, bytes, &bars[BAR_FULL_W0 + prod_stage]);
             fills[0] = prod_g + 1;
-            if (++prod_tap == p.groups) prod_tap = 0;
+            if (++prod_group == p.groups) prod_group = 0;
             if (++prod_stage == p.stages) { prod_stage = 0; prod_parity ^= 1u; }
         }
     }
@@ -1141,34 +1183,33 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
 }
 
 // ---- load-time weight image -----------------------------------------------------------------------------
-// plain packed words [Cout][taps][Cw] -> e2m1 operand image [channel block][tap][Cw2][128 channels][16 bytes];
-// channels past Cout, the pad channel word of an odd Cw and channels past Cin inside a word are 0.0; with out_c
-// <= 64 (<= 32) the rows hold two (four) copies of the channels, so that every TMEM lane quarter has work for a
-// finisher warp
-__global__ void mx_pack_weights_kernel(const uint32_t *w, uint4 *image, int Cout, int Cin, int Cw, int Cw2, int taps, int n_blocks, int dup)
+// plain packed words [Cout][KH][KW][Cw] -> e2m1 operand image [channel block][pair of words of K][2][128 channels][16 bytes]
+// in the order of mx_word; channels past Cout, the second word of an odd last one and channels past Cin inside a word are
+// 0.0; with out_c <= 64 (<= 32) the rows hold two (four) copies of the channels, so that every TMEM lane quarter has work
+// for a finisher warp
+__global__ void mx_pack_weights_kernel(const uint32_t *w, uint4 *image, int Cout, int Cin, int Cw, int KH, int KW, int stride, int n_blocks, int dup)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int64_t total = (int64_t)n_blocks * taps * Cw2 * 128;
+    const int words = KH * KW * Cw, padded = words + (words & 1);
+    const int64_t total = (int64_t)n_blocks * padded * 128;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int row = (int)(e & 127);
-        int64_t t = e >> 7;
-        const int cw = (int)(t % Cw2);
-        t /= Cw2;
-        const int tap = (int)(t % taps);
-        const int blk = (int)(t / taps);
+        const int64_t t = e >> 7;
+        const int blk = (int)(t / padded), i = (int)(t - (int64_t)blk * padded);
         const int o = blk * 128 + (row & (128 / dup - 1));  // few output channels: the block is repeated down the 128 rows
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (o < Cout && cw < Cw) {
-            v = mx_expand_word(w[((int64_t)o * taps + tap) * Cw + cw]);
-            const int valid = Cin - cw * 32;  // channels of this word that exist
+        if (o < Cout && i < words) {
+            const MxWord at = mx_word(i, KH, KW, Cw, stride);
+            v = mx_expand_word(w[((int64_t)o * KH * KW + at.ky * KW + at.kx) * Cw + at.cw]);
+            const int valid = Cin - at.cw * 32;  // channels of this word that exist
             if (valid < 32) {
                 // value (register j, nibble i) is channel 4 i + j of the word
                 uint32_t m[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     m[j] = 0u;
-                    for (int i = 0; i < 8; ++i)
-                        if (4 * i + j < valid) m[j] |= 0xFu << (4 * i);
+                    for (int n = 0; n < 8; ++n)
+                        if (4 * n + j < valid) m[j] |= 0xFu << (4 * n);
                 }
                 v.x &= m[0]; v.y &= m[1]; v.z &= m[2]; v.w &= m[3];
             }
@@ -1178,8 +1219,8 @@ __global__ void mx_pack_weights_kernel(const uint32_t *w, uint4 *image, int Cout
 }
 
 struct MxPlan {
-    int Nt, P, T, stages, resident, group_taps, groups, n_blocks, ctas_x, n_tiles, n_super, total_q, Wg, Hg, n_phase, Cw2, taps, halo, n_xbuf, ahead;
-    size_t raw_words, x_bytes, tap_bytes, off_tbl, off_w, off_x, smem;
+    int Nt, P, T, stages, resident, group_pairs, groups, n_blocks, ctas_x, n_tiles, n_super, total_q, Wg, Hg, n_phase, Cw, pairs, taps, halo, cover_halo, n_xbuf, ahead;
+    size_t raw_words, x_bytes, off_tbl, off_w, off_x, smem;
     double clocks;  // of a CTA's tiles by the cost model
 };
 
@@ -1219,7 +1260,7 @@ bool mx_plan(const ConvGeom &g, int sms, MxPlan *pl)
     return e.found;
 }
 
-int mx_channel_words(const ConvGeom &g) { return g.Cw + (g.Cw & 1); }
+int mx_pairs(const ConvGeom &g) { return (g.KH * g.KW * g.Cw + 1) / 2; }
 int mx_channel_blocks(const ConvGeom &g) { return (g.Cout + 127) / 128; }
 
 // The grid of positions and everything else of a plan that does not depend on the tile; false where the kernel does not
@@ -1232,10 +1273,12 @@ bool mx_frame(const ConvGeom &g, MxPlan *pl)
     if (taps > kMaxTaps) return false;
     const int s = g.sh;
     int Wg, Hg;
-    int64_t halo;
+    int64_t halo, cover_halo = -1;
     if (s == 1) {
         const int pr = max(0, (g.OW - 1) + g.KW - g.W - g.pl), pb = max(0, (g.OH - 1) + g.KH - g.H - g.pt);
         Wg = g.W + max(g.pl, pr);
+        cover_halo = (int64_t)(g.KH - 1) * Wg + (g.KW - 1);
+        if (g.Cw & 1) Wg = max(Wg, g.KW);  // a tap's place in the buffer grows with its number (mx_word) as long as a row holds the window
         Hg = g.H + max(g.pt, pb);
         halo = (int64_t)(g.KH - 1) * Wg + (g.KW - 1);
     } else {
@@ -1245,53 +1288,57 @@ bool mx_frame(const ConvGeom &g, MxPlan *pl)
     }
     const int64_t total_q = (int64_t)g.N * Hg * Wg;
     if (total_q >= (1ll << 31) - 4096 || g.M >= (1ll << 31) || halo > kMaxPositions) return false;
-    pl->Wg = Wg; pl->Hg = Hg; pl->halo = (int)halo; pl->total_q = (int)total_q;
+    pl->Wg = Wg; pl->Hg = Hg; pl->halo = (int)halo; pl->cover_halo = (int)(cover_halo < 0 ? halo : cover_halo); pl->total_q = (int)total_q;
     // a 1x1 filter at stride 2 reads one phase of the four: staging that one alone took 64 images of 28x28x512 -> 512 from
     // 19.5 to 7.3 us, of 56x56x256 -> 256 from 13.7 to 9.0
     pl->n_phase = taps == 1 ? 1 : s * s;
-    pl->Cw2 = mx_channel_words(g);
+    pl->Cw = g.Cw;
     pl->taps = taps;
-    pl->tap_bytes = (size_t)pl->Cw2 * 2048;
+    pl->pairs = mx_pairs(g);
     pl->n_blocks = mx_channel_blocks(g);
     return true;
 }
 
-// Shared memory of a tile of nt positions, T of them to a position buffer; false if it does not fit beside two taps
-// (one of a 1x1 filter).
+// Shared memory of a tile of nt positions, T of them to a position buffer; false if it does not fit beside two pairs of
+// weight words (or the only one).
 struct MxRoom {
     int P;
     size_t raw_words, x_bytes, off_tbl, off_w, rest;
 };
 
-bool mx_room(const MxPlan &pl, int Cw, int nt, int T, MxRoom *r)
+bool mx_room(const MxPlan &pl, int nt, int T, MxRoom *r)
 {
     // T tiles share one position buffer of T * nt + halo rows: the halo is staged once per T tiles
     r->P = T * nt + pl.halo;
     if (r->P > kMaxPositions) return false;
-    r->raw_words = (((size_t)pl.n_phase * (nt + pl.halo) * Cw + 3) / 4) * 4;
-    r->x_bytes = (size_t)pl.n_phase * pl.Cw2 * r->P * 16;
+    r->raw_words = (((size_t)pl.n_phase * (nt + pl.halo) * pl.Cw + 3) / 4) * 4;
+    r->x_bytes = ((size_t)pl.n_phase * pl.Cw * r->P * 16 + 16 + 127) / 128 * 128;  // one row to spare: see the table of operand offsets
     r->off_tbl = kOffDyn + r->raw_words * 4;
-    const size_t fixed = r->off_tbl + (size_t)pl.taps * (pl.Cw2 / 2) * 8;  // the table no longer than it is: at 512 channels 3x3 the 8 KB saved are a wider tile
+    const size_t fixed = r->off_tbl + (size_t)pl.pairs * 8;  // the table no longer than it is: at 512 channels 3x3 the 8 KB saved are a wider tile
     r->off_w = (fixed + 127) / 128 * 128;
     r->rest = 2 * r->x_bytes + 256;
-    return r->off_w + r->rest + (pl.taps > 1 ? 2 : 1) * pl.tap_bytes <= kSmemLimit;
+    return r->off_w + r->rest + (size_t)min(2, pl.pairs) * kPairBytes <= kSmemLimit;
 }
 
-// a larger tile never takes less room, so a layer has a plan if the smallest one fits
+// Which layers the kernel takes: those whose smallest tile (16 positions) fits beside two whole taps (one of a 1x1 filter)
+// of an even number of words each.  Pairs take less room than that, and a larger tile never less than a smaller one, so
+// such a layer has a plan.
 bool mx_covers(const ConvGeom &g)
 {
     MxPlan pl;
-    MxRoom r;
-    return mx_frame(g, &pl) && mx_room(pl, g.Cw, 16, 1, &r);
+    if (!mx_frame(g, &pl)) return false;
+    const size_t Cw2 = g.Cw + (g.Cw & 1), P = 16 + pl.cover_halo;
+    const size_t raw = (pl.n_phase * P * g.Cw + 3) / 4 * 16, table = pl.taps * (Cw2 / 2) * 8;
+    return (kOffDyn + raw + table + 127) / 128 * 128 + 2 * pl.n_phase * Cw2 * P * 16 + 256 + (pl.taps > 1 ? 2 : 1) * Cw2 * 2048 <= kSmemLimit;
 }
 
 bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
 {
     if (!mx_frame(g, pl)) return false;
-    const int taps = pl->taps, halo = pl->halo;
+    if (!mx_covers(g)) return false;
+    const int pairs = pl->pairs, halo = pl->halo;
     const int64_t total_q = pl->total_q;
     const int ctas_max = max(1, sms / pl->n_blocks);
-    const int ksteps = pl->Cw2 / 2;
     double best = 1e30;
     bool found = false;
     for (int nt = 16; nt <= kMaxNt; nt += 16) {
@@ -1299,20 +1346,20 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
         for (int T = 1; T <= 8; ++T) {
             if (T > 1 && (T - 1) * ctas_max >= n_tiles) break;   // no CTA would have that many tiles
             MxRoom room;
-            if (!mx_room(*pl, g.Cw, nt, T, &room)) break;
-            // taps that fit beside the position buffers: all of them -> resident (one stage per tap, one barrier);
-            // otherwise a ring of two stages of half the fitting taps each (a group costs the issuer one wait and
-            // one commit, whatever its size: two large groups measured better than three or four smaller ones)
-            const int slots = (int)((kSmemLimit - room.off_w - room.rest) / pl->tap_bytes);
-            const bool resident = slots >= taps;
-            int stages, group_taps, groups;
+            if (!mx_room(*pl, nt, T, &room)) break;
+            // pairs that fit beside the position buffers: all of them -> resident (one barrier); otherwise a ring of two
+            // stages of half the fitting pairs each (a group costs the issuer one wait and one commit, whatever its
+            // size: two large groups measured better than three or four smaller ones)
+            const int slots = (int)((kSmemLimit - room.off_w - room.rest) / kPairBytes);
+            const bool resident = slots >= pairs;
+            int stages, group_pairs, groups;
             if (resident) {
-                stages = taps; group_taps = 1; groups = taps;
+                stages = groups = 1; group_pairs = pairs;
             } else {
-                group_taps = slots >= 4 ? slots / 2 : 1;
-                groups = (taps + group_taps - 1) / group_taps;
-                group_taps = (taps + groups - 1) / groups;  // even groups
-                stages = min(kMaxStages, slots / group_taps);
+                group_pairs = max(1, slots / 2);
+                groups = (pairs + group_pairs - 1) / group_pairs;
+                group_pairs = (pairs + groups - 1) / groups;  // even groups
+                stages = min(kMaxStages, slots / group_pairs);
             }
             const int n_super = (n_tiles + T - 1) / T;
             const int ctas_x = min(ctas_max, n_super);
@@ -1320,10 +1367,10 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
             // clocks per MMA: 43 + N/2, at least 100 (measured); the loaders need about 400 + 8 clocks per staged
             // position and tile
             const double mma1 = fmax(100.0, 43.0 + nt / 2.0);
-            const double mma = (double)taps * ksteps * mma1;
+            const double mma = (double)pairs * mma1;
             // a streamed group: its bytes from L2 (with all SMs streaming at least 38 bytes per clock each), or its share of a copy's latency, or what the single issuer needs
             // per group (wait for the stage, issue, hand the stage back: about 250 clocks on top of the MMAs)
-            const double stream = resident ? 0.0 : (double)groups * fmax(fmax(group_taps * pl->tap_bytes / 38.0, 1300.0 / stages), 250.0 + group_taps * ksteps * mma1);
+            const double stream = resident ? 0.0 : (double)groups * fmax(fmax(group_pairs * kPairBytes / 38.0, 1300.0 / stages), 250.0 + group_pairs * mma1);
             // stride 2: four phases per position, staged two at a time where the geometry allows (MX_S2_PAIR)
             const double per_position = pl->n_phase == 1 ? 1.0 : ((g.W & 1) == 0 && (g.pl & 1) == 0 && g.Cw <= 4) ? 2.0 : 3.0;
             const double load = 400.0 + 8.0 * per_position * (nt + (double)halo / T);
@@ -1333,12 +1380,12 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
             if (cost < best) {
                 best = pl->clocks = cost;
                 found = true;
-                pl->Nt = nt; pl->P = room.P; pl->T = T; pl->stages = stages; pl->resident = resident ? 1 : 0; pl->group_taps = group_taps; pl->groups = groups;
+                pl->Nt = nt; pl->P = room.P; pl->T = T; pl->stages = stages; pl->resident = resident ? 1 : 0; pl->group_pairs = group_pairs; pl->groups = groups;
                 pl->n_tiles = n_tiles; pl->n_super = n_super; pl->ctas_x = ctas_x;
                 pl->raw_words = room.raw_words; pl->x_bytes = room.x_bytes;
                 pl->off_tbl = room.off_tbl;
                 pl->off_w = room.off_w;
-                pl->off_x = (room.off_w + (size_t)stages * group_taps * pl->tap_bytes + 127) / 128 * 128;
+                pl->off_x = (room.off_w + (size_t)stages * group_pairs * kPairBytes + 127) / 128 * 128;
                 // More position buffers where shared memory is left over (thin layers): the loaders may then be
                 // up to four tiles ahead, ahead <= (n_xbuf - 1) * T + 1, and the hand-overs between the roles
                 // (a few hundred clocks each) drop out of the per-tile cycle.
@@ -1376,16 +1423,16 @@ bool tensor_covers(const ConvGeom &g) { return mx_covers(g); }
 
 size_t tensor_weight_image_bytes(const ConvGeom &g)
 {
-    return covers_some_padding(g, mx_covers) ? (size_t)mx_channel_blocks(g) * g.KH * g.KW * mx_channel_words(g) * 2048 : 0;
+    return covers_some_padding(g, mx_covers) ? (size_t)mx_channel_blocks(g) * mx_pairs(g) * kPairBytes : 0;
 }
 
 lce_status launch_pack_weights_tensor(const ConvGeom &g, const uint32_t *w, void *image, cudaStream_t s)
 {
-    const int n_blocks = mx_channel_blocks(g), taps = g.KH * g.KW, Cw2 = mx_channel_words(g);
-    const int64_t total = (int64_t)n_blocks * taps * Cw2 * 128;
+    const int n_blocks = mx_channel_blocks(g);
+    const int64_t total = (int64_t)n_blocks * mx_pairs(g) * 256;
     const int64_t want = (total + 255) / 256;
     const int blocks = (int)(want < 4096 ? want : 4096);
-    const lce_status st = launch_dependent(mx_pack_weights_kernel, dim3((unsigned)blocks), 256, 0, s, w, static_cast<uint4 *>(image), g.Cout, g.Cin, g.Cw, Cw2, taps, n_blocks, mx_dup(g));
+    const lce_status st = launch_dependent(mx_pack_weights_kernel, dim3((unsigned)blocks), 256, 0, s, w, static_cast<uint4 *>(image), g.Cout, g.Cin, g.Cw, g.KH, g.KW, g.sh, n_blocks, mx_dup(g));
     mx_flag_array(false);  // load time is the moment to set up the host-visible status word (it cannot be done under stream capture)
     return st;
 }
@@ -1396,7 +1443,7 @@ lce_status tensor_plan_info(const ConvGeom &g, TensorPlanInfo *info)
     if (!mx_plan(g, device_sms(), &pl)) return LCE_ERR_UNSUPPORTED;
     info->tile_positions = pl.Nt;
     info->ctas = pl.ctas_x * pl.n_blocks;
-    info->weight_stages = pl.stages;
+    info->weight_stages = pl.resident ? pl.taps : pl.stages;
     info->weights_resident = pl.resident;
     info->shared_bytes = (int64_t)pl.smem;
     info->clocks = pl.clocks;
@@ -1422,7 +1469,7 @@ lce_status prepare_bconv_tensor(const ConvGeom &g, PreparedLaunch *prepared)
     l.grid = dim3((unsigned)pl.ctas_x, (unsigned)pl.n_blocks);
     l.smem = pl.smem;
     MxParams &p = l.params;
-    p.N = g.N; p.H = g.H; p.W = g.W; p.Cw = g.Cw; p.Cw2 = pl.Cw2; p.Cout = g.Cout; p.Cow = g.Cow;
+    p.N = g.N; p.H = g.H; p.W = g.W; p.Cw = g.Cw; p.Cout = g.Cout; p.Cow = g.Cow;
     p.OH = g.OH; p.OW = g.OW; p.KH = g.KH; p.KW = g.KW; p.stride = g.sh; p.pt = g.pt; p.pl = g.pl;
     p.K = g.KH * g.KW * g.Cin;
     p.Wg = pl.Wg; p.Hg = pl.Hg; p.n_phase = pl.n_phase;
@@ -1439,8 +1486,14 @@ lce_status prepare_bconv_tensor(const ConvGeom &g, PreparedLaunch *prepared)
     p.step_chunk_first = step(pl.Nt + pl.halo);
     p.step_chunk_super = step(super_step - last_chunk);
     p.Nt = pl.Nt; p.P = pl.P; p.T = pl.T; p.halo = pl.halo; p.n_tiles = pl.n_tiles; p.n_super = pl.n_super; p.total_q = pl.total_q;
-    p.taps = pl.taps; p.ksteps = pl.Cw2 / 2; p.stages = pl.stages; p.resident = pl.resident; p.group_taps = pl.group_taps; p.groups = pl.groups;
-    p.tap_bytes = (int32_t)pl.tap_bytes; p.x_bytes = (int32_t)pl.x_bytes;
+    const uint32_t even = (uint32_t)max(2, g.Cw & ~1);
+    fast_div_constants(even, &p.even_mul, &p.even_sh);
+    for (int tap = 0; tap < pl.taps; ++tap) {  // word 0 of a tap of one word a tap: the tap itself
+        const MxWord w = mx_word(tap, g.KH, g.KW, 1, g.sh);
+        p.tap_rows[tap] = (uint16_t)(g.sh == 2 ? ((w.ky & 1) * 2 + (w.kx & 1)) * g.Cw * pl.P + (w.ky >> 1) * pl.Wg + (w.kx >> 1) : w.ky * pl.Wg + w.kx);
+    }
+    p.pairs = pl.pairs; p.stages = pl.stages; p.resident = pl.resident; p.group_pairs = pl.group_pairs; p.groups = pl.groups;
+    p.x_bytes = (int32_t)pl.x_bytes;
     p.n_xbuf = pl.n_xbuf; p.ahead = pl.ahead;
     p.off_tbl = (int32_t)pl.off_tbl; p.off_w = (int32_t)pl.off_w; p.off_x = (int32_t)pl.off_x;
     p.pad_zero = g.padding == LCE_PAD_SAME_ZERO;
