@@ -65,10 +65,10 @@
 namespace lce {
 namespace {
 
-constexpr int kLoaders = 256;                                // warps 0-7
-constexpr int kFinishers = 512;                              // warps 8-23 (warp % 4 = TMEM lane quarter, four column groups)
-constexpr int kMxThreads = kLoaders + kFinishers + 64;       // + MMA issuer warp + weight producer warp
-constexpr int kIssuerWarp = (kLoaders + kFinishers) / 32;
+constexpr int kFinishers = 512;                              // warps 0-15 (warp % 4 = TMEM lane quarter, four column groups)
+constexpr int kLoaders = 256;                                // warps 16-23
+constexpr int kMxThreads = kFinishers + kLoaders + 64;       // + MMA issuer warp + weight producer warp
+constexpr int kIssuerWarp = (kFinishers + kLoaders) / 32;
 constexpr int kProducerTid = (kIssuerWarp + 1) * 32;
 constexpr int kColGroups = kFinishers / 128;                 // finisher warps per TMEM lane quarter
 constexpr int kMaxNt = 224;                                  // tile width (positions); two accumulators + scales fit 512 columns
@@ -77,20 +77,16 @@ constexpr uint32_t kSfaCol = 480, kSfbCol = 496;             // block scales (al
 constexpr int kMaxTaps = 64;
 constexpr int kPairBytes = 4096;                             // weights of an MMA: two words of K, 128 rows, 16 bytes each
 constexpr int kMaxStages = 32;
-constexpr int kPixSlots = 8;                                 // see the note at kOffPix
-
 // shared-memory map (bytes)
 constexpr int kOffBars = 0;          // full_x[4] tile_done[4] full_d[2] empty_d[2] done[2] scales full_w[32] empty_w[32]
 constexpr int kOffSlot = 1000;       // TMEM base address; 1004 fills issued, 1008 fills consumed
-// int32[8][224]: output pixel of a column, or -1.  A ring of eight tiles: the finishers hand an
-// accumulator back before they have stored its values, so the loaders can be up to four tiles ahead
-// of a finisher that still reads its tile's slot (tile t + 5 cannot be staged before finisher t is done).
-constexpr int kOffPix = 1024;
-constexpr int kOffDyn = 8192;       // raw words, uint2[MMAs of a tile]: operand offsets (A, B; 16-byte units), weight ring, position buffers
+constexpr int kOffPix = 1024;        // int32[16][2][32]: for every finisher warp the output pixels of the positions it works on, two chunks of a tile at most; int32[32]: -1
+constexpr int kOffDyn = 5248;       // raw words, uint2[MMAs of a tile]: operand offsets (A, B; 16-byte units), weight ring, position buffers
 
 enum { BAR_FULL_X0 = 0, BAR_FULL_X3 = 3, BAR_TILE_DONE0, BAR_TILE_DONE3 = BAR_TILE_DONE0 + 3, BAR_FULL_D0, BAR_FULL_D1, BAR_EMPTY_D0, BAR_EMPTY_D1, BAR_DONE, BAR_DONE_B,
        BAR_SCALES, BAR_FULL_W0,
        BAR_EMPTY_W0 = BAR_FULL_W0 + kMaxStages, BAR_COUNT = BAR_EMPTY_W0 + kMaxStages };
+static_assert((kMaxNt + 31) / 32 <= 2 * kColGroups, "a finisher warp has two chunks of a tile at most");
 static_assert(BAR_COUNT * 8 <= kOffSlot, "barriers overlap the TMEM slot");
 
 
@@ -182,7 +178,7 @@ struct MxParams {
     int32_t OH, OW, KH, KW, stride, pt, pl, K;
     int32_t Wg, Hg, n_phase;
     uint32_t Wg_mul, Wg_sh, Hg_mul, Hg_sh;                // divisions by Wg, Hg as multiply + shift
-    MxStep step_across, step_tile, step_tile_super;       // kLoaders positions; to the next tile of a super-tile, of the next super-tile
+    MxStep step_across, step_tile;                        // kLoaders positions; to the next tile of a super-tile
     MxStep step_chunk_first, step_chunk_super;            // from a super-tile's first chunk to its second; from its last one to the next super-tile's first
     int32_t Nt, P;           // tile width; rows of a position buffer per phase and channel word = T * Nt + halo
     int32_t T, halo;         // tiles that share a position buffer; positions a tile reads beyond its own
@@ -386,19 +382,17 @@ __device__ __forceinline__ int mx_form(const MxParams &p)
         default: CALL(0, MX_S1); break;                                                                                         \
     }
 
-// The loaders' loop over the CTA's tiles: expand the chunk whose words have arrived, work out which output pixel
-// each of the tile's columns is, hand the tile to the issuer, and only then ask for the words of the next chunk
+// The loaders' loop over the CTA's tiles: expand the chunk whose words have arrived, hand the tile to the issuer, and only then ask for the words of the next chunk
 // (the tile's MMAs must not wait for loads they do not need).  False when a wait gave up.
 template <int CW, int FORM>
-__device__ __forceinline__ bool mx_load_tiles(const MxParams &p, const MxLoad &l, MxPos stage, uint64_t *bars, uint32_t *raw0, uint8_t *sX0, int32_t *sPix,
+__device__ __forceinline__ bool mx_load_tiles(const MxParams &p, const MxLoad &l, MxPos stage, uint64_t *bars, uint32_t *raw0, uint8_t *sX0,
                                               int tid, int first_tile, int tile_step)
 {
     const int Nt = p.Nt, T = p.T, halo = p.halo, n_tiles = p.n_tiles, n_super = p.n_super, n_xbuf = p.n_xbuf, ahead = p.ahead;
-    const int OH = p.OH, OW = p.OW, plane = p.Cw * p.P, cp_words = p.cp_words;
+    const int plane = p.Cw * p.P, cp_words = p.cp_words;
     const uint32_t x_bytes = (uint32_t)p.x_bytes;
     const bool pad_zero = p.pad_zero != 0;
-    const MxStep tile_d = p.step_tile, tile_super = p.step_tile_super, chunk_first = p.step_chunk_first, chunk_super = p.step_chunk_super;
-    MxPos pix = mx_position(first_tile * T * Nt + tid, p);  // this thread's column of the tile
+    const MxStep tile_d = p.step_tile, chunk_first = p.step_chunk_first, chunk_super = p.step_chunk_super;
     int it = 0, xbuf = 0;
     for (int st = first_tile; st < n_super; st += tile_step, xbuf = xbuf + 1 == n_xbuf ? 0 : xbuf + 1) {
         uint4 *X = reinterpret_cast<uint4 *>(sX0 + xbuf * x_bytes);
@@ -413,12 +407,9 @@ __device__ __forceinline__ bool mx_load_tiles(const MxParams &p, const MxLoad &l
                 if (!mbar_wait_bounded(&bars[BAR_TILE_DONE0 + (done & 3)], (uint32_t)(done >> 2) & 1u)) return false;
             }
             mx_expand<CW, FORM>(l, stage, k ? Nt : Nt + halo, raw0, X + (k ? k * Nt + halo : 0), plane, tid, pad_zero);
-            if (tid < Nt)
-                sPix[(it & (kPixSlots - 1)) * kMaxNt + tid] = pix.n < l.N && pix.r < OH && pix.c < OW ? (pix.n * OH + pix.r) * OW + pix.c : -1;
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             mbar_arrive(&bars[BAR_FULL_X0 + (it & 3)]);
             const bool more_here = k + 1 < T && st * T + k + 1 < n_tiles;
-            mx_advance(pix, more_here ? tile_d : tile_super, l.Wg, l.Hg);
             if (more_here || st + tile_step < n_super) {
                 mx_advance(stage, !more_here ? chunk_super : k ? tile_d : chunk_first, l.Wg, l.Hg);
                 mx_prefetch<CW, FORM>(l, stage, more_here ? Nt : Nt + halo, raw0, tid, cp_words);
@@ -628,25 +619,34 @@ __device__ __forceinline__ void mx_issue_table(uint32_t tmem_d, const uint2 *tbl
     }
 }
 
+// Two additions in one instruction
+__device__ __forceinline__ void add_pair(float &x, float &y, float c)
+{
+    asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %2};\n\tadd.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}" : "+f"(x), "+f"(y) : "f"(c));
+}
+
 // 32 x 32 bit transpose across the warp: in: lane = row, bit j = column j; out: lane j holds column j.
 // Five butterfly steps; in step k a lane keeps the bits under its mask and takes the others from its
 // partner's word rotated by k towards them (the bits that wrap around fall under the kept mask).  The
 // per-lane masks and rotation counts are worked out once per warp: a step is one shuffle, one funnel shift
-// and one three-input logic operation.
+// and one three-input logic operation, the first two (whole bytes) one shuffle and one byte permutation.
 struct Transpose32 {
-    uint32_t keep[5];   // bits this lane keeps in the steps k = 16, 8, 4, 2, 1
-    uint32_t rot[5];    // left-rotation of the partner's word
+    uint32_t bytes[2];  // byte selectors of the steps k = 16, 8
+    uint32_t keep[3];   // bits this lane keeps in the steps k = 4, 2, 1
+    uint32_t rot[3];    // left-rotation of the partner's word
 };
 
 __device__ __forceinline__ Transpose32 transpose32_setup(int lane)
 {
+    // a lane without bit k keeps its low halves and takes the partner's low halves moved up by k;
+    // a lane with bit k keeps its high halves and takes the partner's high halves moved down by k
     Transpose32 t;
+    t.bytes[0] = (lane & 16) ? 0x3276u : 0x5410u;
+    t.bytes[1] = (lane & 8) ? 0x3715u : 0x6240u;
 #pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        const int k = 16 >> i;
-        const uint32_t low = k == 16 ? 0x0000FFFFu : k == 8 ? 0x00FF00FFu : k == 4 ? 0x0F0F0F0Fu : k == 2 ? 0x33333333u : 0x55555555u;
-        // a lane without bit k keeps its low halves and takes the partner's low halves moved up by k;
-        // a lane with bit k keeps its high halves and takes the partner's high halves moved down by k
+    for (int i = 0; i < 3; ++i) {
+        const int k = 4 >> i;
+        const uint32_t low = k == 4 ? 0x0F0F0F0Fu : k == 2 ? 0x33333333u : 0x55555555u;
         t.keep[i] = (lane & k) ? ~low : low;
         t.rot[i] = (lane & k) ? 32u - (uint32_t)k : (uint32_t)k;
     }
@@ -655,15 +655,23 @@ __device__ __forceinline__ Transpose32 transpose32_setup(int lane)
 
 __device__ __forceinline__ uint32_t warp_transpose32(uint32_t m, const Transpose32 &t)
 {
+    m = __byte_perm(m, __shfl_xor_sync(0xffffffffu, m, 16), t.bytes[0]);
+    m = __byte_perm(m, __shfl_xor_sync(0xffffffffu, m, 8), t.bytes[1]);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        const uint32_t y = __shfl_xor_sync(0xffffffffu, m, 16 >> i);
+    for (int i = 0; i < 3; ++i) {
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, m, 4 >> i);
         const uint32_t moved = __funnelshift_l(y, y, t.rot[i]);
         m = (m & t.keep[i]) | (moved & ~t.keep[i]);
     }
     return m;
 }
 
+// The finishers.  All transforms take the accumulator 16 columns at a time (32 left no register free: the bit-packed one
+// spilled), know their positions' output pixels before the accumulator is there, and do one compare a position.  Instructions
+// bound the thin layers (5900 a tile of 208 positions on 56x56x64): 64 channels, 56x56, 256 images, bits 28.4 -> 26.5 us;
+// 64 images, float 14.0 -> 13.8.  Setting the accumulators to minus the threshold beforehand (tcgen05.st) instead of
+// adding it to every value was slower (28.4 -> 36 us): the store waits for the other tile's matrix instructions.
+//
 // What a finisher warp needs for every tile, worked out once before its tile loop (divisions and
 // kernel-parameter reads per tile cost a third of the warp's instructions when they sat in the epilogue).
 // TMEM lane quarter of the warp = warp % 4; with few output channels the 128 rows hold `dup` copies of
@@ -674,18 +682,21 @@ struct MxFin {
     int group, n_groups;     // this warp takes chunks group, group + n_groups, ...
     int last_chunk;          // its last one (-1: none: nothing to read for this warp)
     uint32_t lane_off;       // TMEM lane offset of its quarter
-    bool ch_ok;              // this lane's channel exists
     float minus_thr, mult, bias;  // this lane's channel: minus its threshold (inf if it does not exist), multiplier, bias
-    int64_t cout, cow;
+    int cout, cow;
     uint32_t *out_words;     // bit-packed output, at this warp's channel word
     float *outp;             // float / int32 output, at this lane's channel
     const float *resp;       // shortcut tensor at this lane's channel, or null
     uint32_t *packp;         // re-quantised copy at this warp's channel word, or null
     bool relu, write_float;
-    Transpose32 tr;          // bit-packed output: the transpose's per-lane constants
+    int N, OH, OW, Wg, Hg;   // position -> output pixel
+    uint32_t Wg_mul, Wg_sh, Hg_mul, Hg_sh;
+    int lane_step;           // from lane_pixels of the first chunk to that of the second
+    int32_t *pixels;         // shared memory: output pixels of the two chunks' positions (one array per warp)
+    const int32_t *lane_pixels;  // the same for this lane; a row of -1 if its channel does not exist
 };
 
-__device__ __forceinline__ MxFin mx_fin_context(const MxParams &p, int fw, int lane, int ch0)
+__device__ __forceinline__ MxFin mx_fin_context(const MxParams &p, int32_t *sPix, int fw, int lane, int ch0)
 {
     MxFin f;
     const int quarter = fw & 3, dl = p.dup_log2;                    // dup = 1 << dl copies of the channel block
@@ -698,16 +709,16 @@ __device__ __forceinline__ MxFin mx_fin_context(const MxParams &p, int fw, int l
     const bool real = ch0 + cq * 32 < p.Cout && f.group < f.n_chunks;
     f.last_chunk = real ? f.group + ((f.n_chunks - 1 - f.group) & ~(f.n_groups - 1)) : -1;
     f.lane_off = (uint32_t)(quarter * 32) << 16;
-    f.ch_ok = channel < p.Cout;
+    const bool ch_ok = channel < p.Cout;
     // this lane's constants straight from global memory (constants of the model, never the previous kernel's
     // output): their latency passes while the first tile is being staged
     f.minus_thr = INFINITY;
-    if (f.ch_ok && p.out_type == LCE_OUT_BITPACKED) {
+    if (ch_ok && p.out_type == LCE_OUT_BITPACKED) {
         // acc < thr is unchanged by clamping thr to [-K-1, K+1] (|acc| <= K), and then thr is exact in fp32
         f.minus_thr = -(float)max(-p.K - 1, min(p.K + 1, __ldg(p.thr + channel)));
     }
-    f.mult = (f.ch_ok && p.out_type == LCE_OUT_FLOAT32) ? __ldg(p.mult + channel) : 0.f;
-    f.bias = (f.ch_ok && p.out_type == LCE_OUT_FLOAT32) ? __ldg(p.bias + channel) : 0.f;
+    f.mult = (ch_ok && p.out_type == LCE_OUT_FLOAT32) ? __ldg(p.mult + channel) : 0.f;
+    f.bias = (ch_ok && p.out_type == LCE_OUT_FLOAT32) ? __ldg(p.bias + channel) : 0.f;
     f.cout = p.Cout;
     f.cow = p.Cow;
     f.out_words = static_cast<uint32_t *>(p.out) + (ch0 >> 5) + cq;
@@ -716,197 +727,232 @@ __device__ __forceinline__ MxFin mx_fin_context(const MxParams &p, int fw, int l
     f.packp = p.out_packed ? p.out_packed + (ch0 >> 5) + cq : nullptr;
     f.relu = p.activation == LCE_ACT_RELU;
     f.write_float = p.write_float != 0;
-    f.tr = transpose32_setup(lane);
+    f.N = p.N; f.OH = p.OH; f.OW = p.OW; f.Wg = p.Wg; f.Hg = p.Hg;
+    f.Wg_mul = p.Wg_mul; f.Wg_sh = p.Wg_sh; f.Hg_mul = p.Hg_mul; f.Hg_sh = p.Hg_sh;
+    f.pixels = sPix + fw * 64;
+    f.lane_step = ch_ok ? 32 : 0;
+    f.lane_pixels = ch_ok ? f.pixels : sPix + 2 * kFinishers;
     return f;
 }
 
-// Two additions in one instruction: the warps of a CTA share the issue slots (60% of them taken on a 64-channel layer),
-// and what one role saves is time for the others.  56x56x64, 256 images, bits: 29.7 -> 29.0 us.  (The float transforms
-// do not gain from the same for their multiply-adds: 14.1 -> 14.2 us on 56x56x64, 64 images, as graph replays (15.6 called
-// one after another); their stores set the pace.)
-__device__ __forceinline__ void add_pair(float &x, float &y, float c)
+// Output pixel of this lane's position of a tile's chunk, -1 where the position is no output.  The finishers work it out
+// themselves, before the accumulator is ready; as a table written by the loaders it was on those warps' critical chain.
+__device__ __forceinline__ int mx_out_pixel(const MxFin &f, int tile, int c0, int lane)
 {
-    asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %2};\n\tadd.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}" : "+f"(x), "+f"(y) : "f"(c));
+    const int q = tile * f.Nt + c0 + lane;
+    const int row = fast_div(q, f.Wg_mul, f.Wg_sh), c = q - row * f.Wg;
+    const int n = fast_div(row, f.Hg_mul, f.Hg_sh), r = row - n * f.Hg;
+    return c0 + lane < f.Nt && n < f.N && r < f.OH && c < f.OW ? (n * f.OH + r) * f.OW + c : -1;
+}
+
+// The warp has read its last columns of the accumulator
+__device__ __forceinline__ void mx_hand_back(uint64_t *empty_d, int lane)
+{
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncwarp();
+    if (lane == 0) mbar_arrive(empty_d);
 }
 
 // Bit-packed output of one tile (Section 3.2: accumulator compared with the per-channel threshold).
-// Lane = channel; per 32-column chunk the sign of (accumulator - threshold) of 32 positions, then a 32 x 32
-// bit transpose across the warp gives every lane the finished word of one pixel.
-__device__ __forceinline__ void mx_epilogue_bits(const MxFin &f, uint32_t tmem_d, const int32_t *sPix, int lane, uint64_t *empty_d)
+// Lane = channel; per 32-column chunk the sign of (accumulator - threshold) of 32 positions, then a 32 x 32 bit transpose across the warp gives every
+// lane the finished word of one pixel.
+__device__ __forceinline__ void mx_epilogue_bits(const MxFin &f, const Transpose32 &tr, uint32_t tmem_d, int pix, int pix2, int lane, uint64_t *empty_d)
 {
     for (int ck = f.group; ck <= f.last_chunk; ck += f.n_groups) {
         const int c0 = ck * 32;
-        float v[32];
         const bool full = c0 + 32 <= f.Nt;
-        if (full) tmem_ld32(tmem_d + f.lane_off + (uint32_t)c0, v);
-        else tmem_ld16(tmem_d + f.lane_off + (uint32_t)c0, v);
-        if (ck == f.last_chunk) {  // last read of the accumulator by this warp: hand it back before the arithmetic
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            mbar_arrive(empty_d);
-        }
-        // bit j = (acc_j < thr): the sign of acc - thr (both are small integers held exactly), two columns to an addition;
-        // four short chains of shifts instead of one long one
+        uint32_t m = 0u;
 #pragma unroll
-        for (int j = 0; j < 32; j += 2) add_pair(v[j], v[j + 1], f.minus_thr);
-        uint32_t m0 = 0u, m1 = 0u, m2 = 0u, m3 = 0u;
+        for (int half = 0; half < 2; ++half) {
+            if (half == 0 || full) {
+                float v[16];
+                tmem_ld16(tmem_d + f.lane_off + (uint32_t)(c0 + half * 16), v);
+                if (ck == f.last_chunk && (half == 1 || !full)) mx_hand_back(empty_d, lane);  // before the arithmetic
+                // bit j = (acc_j < thr): the sign of acc - thr (both are small integers held exactly), two columns to an
+                // addition; two short chains of shifts instead of one long one
 #pragma unroll
-        for (int j = 7; j >= 0; --j) {
-            m0 = __funnelshift_l(__float_as_uint(v[j]), m0, 1);
-            m1 = __funnelshift_l(__float_as_uint(v[8 + j]), m1, 1);
-            m2 = __funnelshift_l(__float_as_uint(v[16 + j]), m2, 1);
-            m3 = __funnelshift_l(__float_as_uint(v[24 + j]), m3, 1);
+                for (int j = 0; j < 16; j += 2) add_pair(v[j], v[j + 1], f.minus_thr);
+                uint32_t m0 = 0u, m1 = 0u;
+#pragma unroll
+                for (int j = 7; j >= 0; --j) {
+                    m0 = __funnelshift_l(__float_as_uint(v[j]), m0, 1);
+                    m1 = __funnelshift_l(__float_as_uint(v[8 + j]), m1, 1);
+                }
+                m |= (m0 | m1 << 8) << (half * 16);
+            }
         }
-        uint32_t m = m0 | (m1 << 8);
-        if (full) m |= (m2 << 16) | (m3 << 24);
-        const uint32_t word = warp_transpose32(m, f.tr);
-        const int pix = (c0 + lane < f.Nt) ? sPix[c0 + lane] : -1;
-        if (pix >= 0) f.out_words[pix * f.cow] = word;
+        const uint32_t word = warp_transpose32(m, tr);
+        if (pix >= 0) f.out_words[(int64_t)pix * f.cow] = word;
+        pix = pix2;
     }
-    if (f.last_chunk < 0) {  // nothing to read for this warp
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        mbar_arrive(empty_d);
-    }
+    if (f.last_chunk < 0) mx_hand_back(empty_d, lane);  // nothing to read for this warp
 }
 
 // Float / int32 output of one tile (Section 3.2: int -> float, fused activation, one multiply-add;
 // Section 5.3: optional shortcut add and re-quantisation).  A lane holds one channel of 32 positions:
 // for every position the warp writes its 32 consecutive channels as one 128-byte store, so a value
-// costs one multiply-add and one store instruction and nothing is staged.  The re-quantised copy is a
-// warp ballot of the signs: the finished word of the pixel.  Everything the loops need sits in
-// registers before they start (kernel parameters read inside them cost more than the arithmetic).
+// costs one multiply-add and one store instruction and nothing is staged.  The pixels of the positions come from
+// shared memory, -1 where nothing is to be written: one compare a position.
 enum { EPI_FLOAT = 0, EPI_FLOAT_FUSED = 1, EPI_INT32 = 2, EPI_BITS = 3, EPI_PLAIN = 4 };
 
-template <int MODE>
-__device__ __forceinline__ void mx_store_chunk(const float (&v)[32], int cols, const int32_t *sPixChunk, int64_t cout, float *outp,
-                                               bool ch_ok, float mult, float bias)
+// the output pixels of the chunks' positions, for the whole warp to see
+__device__ __forceinline__ void mx_share_pixels(const MxFin &f, int pix, int pix2, int lane)
 {
-    // straight-line code: every store is predicated, nothing branches, so the 32 positions' address
-    // arithmetic, multiply-adds and stores overlap instead of running one position after the other
-#pragma unroll
-    for (int j4 = 0; j4 < 32; j4 += 4) {
-        const int4 pix4 = *reinterpret_cast<const int4 *>(sPixChunk + j4);  // the same for every lane (slots past the tile: never stored)
-        const int pix[4] = {pix4.x, pix4.y, pix4.z, pix4.w};
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const bool st = ch_ok && pix[u] >= 0 && j4 + u < cols;
-            const int64_t o = pix[u] * cout;
-            if (MODE != EPI_INT32) {
-                const float y = __fmaf_rn(v[j4 + u], mult, bias);
-                if (st) outp[o] = y;
-            } else {
-                const int32_t y = __float2int_rn(v[j4 + u]);
-                if (st) reinterpret_cast<int32_t *>(outp)[o] = y;
-            }
-        }
-    }
+    __syncwarp();  // the tile before is through with the array
+    f.pixels[lane] = pix;
+    f.pixels[32 + lane] = pix2;
+    __syncwarp();
 }
 
 template <int MODE>
-__device__ __forceinline__ void mx_epilogue_values(const MxFin &f, uint32_t tmem_d, const int32_t *sPix, int lane, uint64_t *empty_d)
+__device__ __forceinline__ void mx_epilogue_values(const MxFin &f, uint32_t tmem_d, int lane, uint64_t *empty_d)
 {
+    const int32_t *lane_pixels = f.lane_pixels;
     for (int ck = f.group; ck <= f.last_chunk; ck += f.n_groups) {
         const int c0 = ck * 32;
-        const int cols = min(32, f.Nt - c0);
-        float v[32];
-        if (cols == 32) tmem_ld32(tmem_d + f.lane_off + (uint32_t)c0, v);
-        else tmem_ld16(tmem_d + f.lane_off + (uint32_t)c0, v);
-        if (ck == f.last_chunk) {  // last read of the accumulator by this warp
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            mbar_arrive(empty_d);
+        const bool full = c0 + 32 <= f.Nt;
+        // straight-line code: every store is predicated, nothing branches, so the positions' address
+        // arithmetic, multiply-adds and stores overlap instead of running one position after the other
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            if (half == 0 || full) {
+                float v[16];
+                tmem_ld16(tmem_d + f.lane_off + (uint32_t)(c0 + half * 16), v);
+                if (ck == f.last_chunk && (half == 1 || !full)) mx_hand_back(empty_d, lane);
+#pragma unroll
+                for (int j4 = 0; j4 < 16; j4 += 4) {
+                    const int4 o4 = *reinterpret_cast<const int4 *>(lane_pixels + half * 16 + j4);
+                    const int o[4] = {o4.x, o4.y, o4.z, o4.w};
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        float *at = f.outp + (int64_t)o[u] * f.cout;
+                        if (MODE != EPI_INT32) {
+                            const float y = __fmaf_rn(v[j4 + u], f.mult, f.bias);
+                            if (o[u] >= 0) *at = y;
+                        } else {
+                            const int32_t y = __float2int_rn(v[j4 + u]);
+                            if (o[u] >= 0) *reinterpret_cast<int32_t *>(at) = y;
+                        }
+                    }
+                }
+            }
         }
-        mx_store_chunk<MODE>(v, cols, sPix + c0, f.cout, f.outp, f.ch_ok, f.mult, f.bias);
+        lane_pixels += f.lane_step;
     }
-    if (f.last_chunk < 0) {  // nothing to read for this warp
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        mbar_arrive(empty_d);
+    if (f.last_chunk < 0) mx_hand_back(empty_d, lane);  // nothing to read for this warp
+}
+
+// Float output with activation, shortcut add and re-quantised copy fused in (Section 5.3); the latter two only where every
+// channel of the block exists.
+// The shortcut values of a warp's first chunk of a tile are asked for before it waits for the accumulator
+// (mx_shortcut: 32 independent 128-byte loads a warp), those of its next one when it is through with the first.  The
+// re-quantised copy is the sign bits and the bit transpose of the bit-packed form; y + 0 makes -0.0 and NaN, which
+// quantize to 0 bits, positive (PTX: a NaN result has no sign).
+template <bool RES>
+__device__ __forceinline__ void mx_shortcut(const MxFin &f, const int32_t *pixels, float (&r)[32])
+{
+    if (!RES) return;
+#pragma unroll
+    for (int j4 = 0; j4 < 32; j4 += 4) {
+        const int4 o4 = *reinterpret_cast<const int4 *>(pixels + j4);  // the same for every lane
+        const int o[4] = {o4.x, o4.y, o4.z, o4.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const float *at = f.resp + (int64_t)o[u] * f.cout;
+            r[j4 + u] = 0.f;
+            if (o[u] >= 0) r[j4 + u] = __ldg(at);
+        }
     }
 }
 
-// Float output with the shortcut add and the re-quantised copy fused in (Section 5.3).  Per 32-column chunk
-// the warp first asks for the shortcut values of all 32 positions (they do not depend on the accumulator:
-// 32 independent 128-byte loads in flight per warp; with eight the memory latency set the pace), then reads
-// the accumulators 16 columns at a time, and per position does the multiply-add, the add, the 128-byte store
-// and the ballot whose result is the pixel's finished word.
 template <bool RES, bool PACK, bool WRITE_FLOAT>
-__device__ __forceinline__ void mx_epilogue_fused_as(const MxFin &f, uint32_t tmem_d, const int32_t *sPix, int lane, uint64_t *empty_d)
+__device__ __forceinline__ void mx_epilogue_fused(const MxFin &f, const Transpose32 &tr, uint32_t tmem_d, float (&r)[32], int lane, uint64_t *empty_d)
 {
     // which of the three parts (shortcut add, re-quantised copy, float output) a launch has is a template
     // argument: a test of a pointer per position turns the unrolled block below into branchy code that
     // runs at a third of the speed (measured on the plain float transform, and again here)
     const float floor_v = f.relu ? 0.f : -INFINITY;
+    const int32_t *lane_pixels = f.lane_pixels;
     for (int ck = f.group; ck <= f.last_chunk; ck += f.n_groups) {
         const int c0 = ck * 32;
-        const int cols = min(32, f.Nt - c0);  // 32, or 16 in a tile's last chunk
-        const int32_t *pixc = sPix + c0;
+        const bool full = c0 + 32 <= f.Nt;  // otherwise 16 columns, the tile's last
+        if (ck != f.group) mx_shortcut<RES>(f, f.pixels + 32, r);
+        uint32_t m = 0u;
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
-            if (half * 16 < cols) {
-                // the shortcut values of the half's 16 positions first (they do not depend on the accumulator: 16
-                // independent 128-byte loads in flight per warp), then the accumulators
-                float r[16];
-                if (RES) {
-#pragma unroll
-                    for (int j4 = 0; j4 < 16; j4 += 4) {
-                        const int4 p4 = *reinterpret_cast<const int4 *>(pixc + half * 16 + j4);  // the same for every lane
-                        const int pix[4] = {p4.x, p4.y, p4.z, p4.w};
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const bool ld = f.ch_ok && pix[u] >= 0 && half * 16 + j4 + u < cols;
-                            r[j4 + u] = ld ? __ldg(f.resp + (ld ? pix[u] : 0) * f.cout) : 0.f;
-                        }
-                    }
-                }
+            if (half == 0 || full) {
                 float v[16];
-                tmem_ld16x(tmem_d + f.lane_off + (uint32_t)(c0 + half * 16), v);
-                if (ck == f.last_chunk && (half + 1) * 16 >= cols) {  // last read of the accumulator by this warp
-                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                    mbar_arrive(empty_d);
-                }
-                uint32_t my_word = 0u;  // lane u keeps the re-quantised word of the half's position u: one store for the 16
+                tmem_ld16(tmem_d + f.lane_off + (uint32_t)(c0 + half * 16), v);
+                if (ck == f.last_chunk && (half == 1 || !full)) mx_hand_back(empty_d, lane);
 #pragma unroll
                 for (int j4 = 0; j4 < 16; j4 += 4) {
-                    const int4 p4 = *reinterpret_cast<const int4 *>(pixc + half * 16 + j4);
-                    const int pix[4] = {p4.x, p4.y, p4.z, p4.w};
+                    int o[4];
+                    if (WRITE_FLOAT) {
+                        const int4 o4 = *reinterpret_cast<const int4 *>(lane_pixels + half * 16 + j4);
+                        o[0] = o4.x; o[1] = o4.y; o[2] = o4.z; o[3] = o4.w;
+                    }
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        const bool pos_ok = pix[u] >= 0 && half * 16 + j4 + u < cols;  // the same for every lane
                         float y = __fmaf_rn(fmaxf(v[j4 + u], floor_v), f.mult, f.bias);
-                        if (RES) y = __fadd_rn(y, r[j4 + u]);
+                        if (RES) y = __fadd_rn(y, r[half * 16 + j4 + u]);
                         if (WRITE_FLOAT) {
-                            if (f.ch_ok && pos_ok) f.outp[pix[u] * f.cout] = y;
+                            float *at = f.outp + (int64_t)o[u] * f.cout;  // outside the condition: nothing branches
+                            if (o[u] >= 0) *at = y;
                         }
-                        if (PACK) {
-                            const uint32_t word = __ballot_sync(0xffffffffu, f.ch_ok && y < 0.f);
-                            if (lane == j4 + u) my_word = word;
-                        }
+                        if (PACK) v[j4 + u] = y;
                     }
                 }
                 if (PACK) {
-                    const int my_pos = half * 16 + (lane & 15);
-                    const int my_pix = pixc[my_pos];
-                    if (lane < 16 && my_pix >= 0 && my_pos < cols) f.packp[my_pix * f.cow] = my_word;
+                    uint32_t m0 = 0u, m1 = 0u;
+#pragma unroll
+                    for (int j = 0; j < 16; j += 2) add_pair(v[j], v[j + 1], 0.f);
+#pragma unroll
+                    for (int j = 7; j >= 0; --j) {
+                        m0 = __funnelshift_l(__float_as_uint(v[j]), m0, 1);
+                        m1 = __funnelshift_l(__float_as_uint(v[8 + j]), m1, 1);
+                    }
+                    m |= (m0 | m1 << 8) << (half * 16);
                 }
             }
         }
+        if (PACK) {
+            const uint32_t word = warp_transpose32(m, tr);
+            const int pix = lane_pixels[lane];
+            if (pix >= 0) f.packp[(int64_t)pix * f.cow] = word;
+        }
+        lane_pixels += f.lane_step;
     }
-    if (f.last_chunk < 0) {  // nothing to read for this warp
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        mbar_arrive(empty_d);
-    }
+    if (f.last_chunk < 0) mx_hand_back(empty_d, lane);  // nothing to read for this warp
 }
 
-__device__ __forceinline__ void mx_epilogue_fused(const MxFin &f, uint32_t tmem_d, const int32_t *sPix, int lane, uint64_t *empty_d)
+// The finishers' loop over the CTA's tiles.  FORM: which transform; the fused one by its three parts.
+template <int MODE, bool RES, bool PACK, bool WRITE_FLOAT>
+__device__ __forceinline__ bool mx_finish_tiles(const MxParams &p, const MxFin &f, uint64_t *bars, uint32_t tmem_base, int lane, int first_tile, int tile_step)
 {
-    const int form = (f.resp != nullptr ? 4 : 0) | (f.packp != nullptr ? 2 : 0) | (f.write_float ? 1 : 0);
-    switch (form) {
-        case 1: mx_epilogue_fused_as<false, false, true>(f, tmem_d, sPix, lane, empty_d); break;
-        case 2: mx_epilogue_fused_as<false, true, false>(f, tmem_d, sPix, lane, empty_d); break;
-        case 3: mx_epilogue_fused_as<false, true, true>(f, tmem_d, sPix, lane, empty_d); break;
-        case 5: mx_epilogue_fused_as<true, false, true>(f, tmem_d, sPix, lane, empty_d); break;
-        case 6: mx_epilogue_fused_as<true, true, false>(f, tmem_d, sPix, lane, empty_d); break;
-        case 7: mx_epilogue_fused_as<true, true, true>(f, tmem_d, sPix, lane, empty_d); break;
-        default: mx_epilogue_fused_as<false, false, false>(f, tmem_d, sPix, lane, empty_d); break;  // nothing to write: only hands the accumulator back
+    const int T = p.T, n_tiles = p.n_tiles, n_super = p.n_super;
+    Transpose32 tr;
+    if (MODE == EPI_BITS || PACK) tr = transpose32_setup(lane);
+    int it = 0;
+    for (int st = first_tile; st < n_super; st += tile_step) {
+        for (int tile = st * T; tile < st * T + T && tile < n_tiles; ++tile, ++it) {
+            const int buf = it & 1;
+            // what does not depend on the accumulator, before it is there
+            const int pix = mx_out_pixel(f, tile, f.group * 32, lane);
+            const int pix2 = f.last_chunk > f.group ? mx_out_pixel(f, tile, (f.group + f.n_groups) * 32, lane) : -1;
+            float r[32];
+            if (MODE != EPI_BITS) mx_share_pixels(f, pix, pix2, lane);
+            if (MODE == EPI_FLOAT_FUSED) mx_shortcut<RES>(f, f.pixels, r);
+            // the warp goes on together (its transform uses warp-wide shuffles)
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&bars[BAR_FULL_D0 + buf], (uint32_t)(it >> 1) & 1u))) return false;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t tmem_d = tmem_base + (buf ? kD1Col : 0u);
+            uint64_t *empty_d = &bars[BAR_EMPTY_D0 + buf];
+            if (MODE == EPI_FLOAT_FUSED) mx_epilogue_fused<RES, PACK, WRITE_FLOAT>(f, tr, tmem_d, r, lane, empty_d);
+            else if (MODE == EPI_BITS) mx_epilogue_bits(f, tr, tmem_d, pix, pix2, lane, empty_d);
+            else mx_epilogue_values<MODE>(f, tmem_d, lane, empty_d);
+        }
     }
+    return true;
 }
 
 // EPI: EPI_PLAIN carries the three plain output transforms (bit-packed, float, int32; chosen per launch by the
@@ -946,7 +992,7 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     } else if (warp == kIssuerWarp + 1) {
         for (int b = lane; b < BAR_COUNT; b += 32) {
-            const uint32_t count = b <= BAR_FULL_X3 ? kLoaders : (b == BAR_EMPTY_D0 || b == BAR_EMPTY_D1) ? kFinishers : b == BAR_SCALES ? 4 : 1;
+            const uint32_t count = b <= BAR_FULL_X3 ? kLoaders : (b == BAR_EMPTY_D0 || b == BAR_EMPTY_D1) ? kFinishers / 32 : b == BAR_SCALES ? 4 : 1;
             mbar_init(&bars[b], count);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -981,10 +1027,11 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
             fills[0] = prod_g;
             fills[1] = 0;
         }
-    } else if (tid >= kLoaders) {
+    } else if (tid < kFinishers) {
         uint2 *tbl = reinterpret_cast<uint2 *>(smem + p.off_tbl);
+        if (warp == 0) sPix[2 * kFinishers + lane] = -1;  // the pixels of channels that do not exist
         const int even = p.Cw & ~1, paired = p.KH * p.KW * even, words = p.KH * p.KW * p.Cw;
-        for (int e = tid - kLoaders; e < n_mma; e += kFinishers) {
+        for (int e = tid; e < n_mma; e += kFinishers) {
             // A: the pair's place among the resident ones or in its group of streamed ones.  B: the first word's rows, and in
             // the upper half the distance from there to the second word's; an odd last word has a second one of zero
             // weights, whose rows may be any (the next ones: a position buffer has one row to spare)
@@ -998,7 +1045,9 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
     MxLoad ld;
     MxPos stage{0, 0, 0};
     int form = 0;
-    if (tid < kLoaders) {
+    const int ltid = tid - kFinishers;  // a loader's number
+    const bool loader = ltid >= 0 && ltid < kLoaders;
+    if (loader) {
         ld.N = p.N; ld.H = p.H; ld.W = p.W; ld.Cw = p.Cw; ld.Wg = p.Wg; ld.Hg = p.Hg; ld.P = p.P; ld.pt = p.pt; ld.pl = p.pl;
         ld.in = p.in;
         ld.col_words = p.Cw;
@@ -1012,20 +1061,20 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
         }
         ld.across = p.step_across;
         form = mx_form(p);
-        stage = mx_position(first_tile * p.T * p.Nt + tid, p);
+        stage = mx_position(first_tile * p.T * p.Nt + ltid, p);
         asm volatile("griddepcontrol.wait;" ::: "memory");  // the activations may come from the previous kernel
         if (first_tile < p.n_super) {
             // through the general forms, whose staging layout is everybody's: one more copy of every special form
             // costs more in code size than it saves here
-            if (p.n_phase == 1) mx_prefetch<0, MX_S1>(ld, stage, p.Nt + p.halo, raw0, tid, p.cp_words);
-            else mx_prefetch<0, MX_S2>(ld, stage, p.Nt + p.halo, raw0, tid, p.cp_words);
+            if (p.n_phase == 1) mx_prefetch<0, MX_S1>(ld, stage, p.Nt + p.halo, raw0, ltid, p.cp_words);
+            else mx_prefetch<0, MX_S2>(ld, stage, p.Nt + p.halo, raw0, ltid, p.cp_words);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = *tmem_slot;
-    if (warp >= kLoaders / 32 && warp < kLoaders / 32 + 4) {
+    if (warp < 4) {
         // block scales: every byte 0x7F = 2^0 (ue8m0), for all 128 lanes of the 32 scale columns, written by the
         // first four finisher warps (one per lane quarter; they have nothing else to do yet); the issuer
         // waits for the four arrivals before its first MMA
@@ -1041,31 +1090,31 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
     }
 
     bool ok = true;
-    if (tid < kLoaders) {
+    if (loader) {
         // ======================= loaders ==============================================================
-#define LCE_MX_LOAD(CW, FORM) ok = mx_load_tiles<CW, FORM>(p, ld, stage, bars, raw0, sX0, sPix, tid, first_tile, tile_step)
+#define LCE_MX_LOAD(CW, FORM) ok = mx_load_tiles<CW, FORM>(p, ld, stage, bars, raw0, sX0, ltid, first_tile, tile_step)
         LCE_MX_FORMS(LCE_MX_LOAD)
-    } else if (tid < kLoaders + kFinishers) {
+    } else if (tid < kFinishers) {
         // ======================= finishers ============================================================
-        const int fw = warp - kLoaders / 32;  // 0..15: lane quarter fw & 3 (= warp & 3), column group fw >> 2
-        const MxFin fin = mx_fin_context(p, fw, lane, ch0);
+        const MxFin fin = mx_fin_context(p, sPix, warp, lane, ch0);  // lane quarter warp & 3, column group warp >> 2
         asm volatile("griddepcontrol.wait;" ::: "memory");  // outputs and the shortcut tensor: only after the previous kernel
-        const int T = p.T, n_tiles = p.n_tiles, n_super = p.n_super, out_type = p.out_type;
-        int it = 0;
-        for (int st = first_tile; st < n_super && ok; st += tile_step) {
-            for (int k = 0; k < T && st * T + k < n_tiles; ++k, ++it) {
-                const int buf = it & 1;
-                ok = mbar_wait_bounded(&bars[BAR_FULL_D0 + buf], (uint32_t)(it >> 1) & 1u);
-                ok = __all_sync(0xffffffffu, ok);  // the warp goes on together (its epilogue uses warp-wide shuffles and ballots)
-                if (!ok) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t tmem_d = tmem_base + (buf ? kD1Col : 0u);
-                const int32_t *pix = sPix + (it & (kPixSlots - 1)) * kMaxNt;
-                if (EPI == EPI_FLOAT_FUSED) mx_epilogue_fused(fin, tmem_d, pix, lane, &bars[BAR_EMPTY_D0 + buf]);
-                else if (out_type == LCE_OUT_BITPACKED) mx_epilogue_bits(fin, tmem_d, pix, lane, &bars[BAR_EMPTY_D0 + buf]);
-                else if (out_type == LCE_OUT_INT32) mx_epilogue_values<EPI_INT32>(fin, tmem_d, pix, lane, &bars[BAR_EMPTY_D0 + buf]);
-                else mx_epilogue_values<EPI_FLOAT>(fin, tmem_d, pix, lane, &bars[BAR_EMPTY_D0 + buf]);
+#define LCE_MX_FINISH(...) mx_finish_tiles<__VA_ARGS__>(p, fin, bars, tmem_base, lane, first_tile, tile_step)
+        if (EPI == EPI_FLOAT_FUSED) {
+            switch ((fin.resp != nullptr ? 4 : 0) | (fin.packp != nullptr ? 2 : 0) | (fin.write_float ? 1 : 0)) {
+                case 1: ok = LCE_MX_FINISH(EPI_FLOAT_FUSED, false, false, true); break;
+                case 2: ok = LCE_MX_FINISH(EPI_FLOAT_FUSED, false, true, false); break;
+                case 3: ok = LCE_MX_FINISH(EPI_FLOAT_FUSED, false, true, true); break;
+                case 5: ok = LCE_MX_FINISH(EPI_FLOAT_FUSED, true, false, true); break;
+                case 6: ok = LCE_MX_FINISH(EPI_FLOAT_FUSED, true, true, false); break;
+                case 7: ok = LCE_MX_FINISH(EPI_FLOAT_FUSED, true, true, true); break;
+                default: ok = LCE_MX_FINISH(EPI_FLOAT_FUSED, false, false, false); break;  // nothing to write: only hands the accumulator back
             }
+        } else if (p.out_type == LCE_OUT_BITPACKED) {
+            ok = LCE_MX_FINISH(EPI_BITS, false, false, false);
+        } else if (p.out_type == LCE_OUT_INT32) {
+            ok = LCE_MX_FINISH(EPI_INT32, false, false, false);
+        } else {
+            ok = LCE_MX_FINISH(EPI_FLOAT, false, false, false);
         }
     } else if (warp == kIssuerWarp || (warp == kIssuerWarp + 1 && p.resident != 0)) {
         // ======================= MMA issuer: a warp, every lane with the same values ==================
@@ -1329,7 +1378,8 @@ bool mx_covers(const ConvGeom &g)
     if (!mx_frame(g, &pl)) return false;
     const size_t Cw2 = g.Cw + (g.Cw & 1), P = 16 + pl.cover_halo;
     const size_t raw = (pl.n_phase * P * g.Cw + 3) / 4 * 16, table = pl.taps * (Cw2 / 2) * 8;
-    return (kOffDyn + raw + table + 127) / 128 * 128 + 2 * pl.n_phase * Cw2 * P * 16 + 256 + (pl.taps > 1 ? 2 : 1) * Cw2 * 2048 <= kSmemLimit;
+    constexpr size_t kBefore = 8192;  // what lay before these parts when the line was drawn
+    return (kBefore + raw + table + 127) / 128 * 128 + 2 * pl.n_phase * Cw2 * P * 16 + 256 + (pl.taps > 1 ? 2 : 1) * Cw2 * 2048 <= kSmemLimit;
 }
 
 bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
@@ -1482,7 +1532,6 @@ lce_status prepare_bconv_tensor(const ConvGeom &g, PreparedLaunch *prepared)
     const int64_t last_chunk = pl.T > 1 ? (int64_t)(pl.T - 1) * pl.Nt + pl.halo : 0, super_step = (int64_t)pl.ctas_x * pl.T * pl.Nt;
     p.step_across = step(kLoaders);
     p.step_tile = step(pl.Nt);
-    p.step_tile_super = step(super_step - (int64_t)(pl.T - 1) * pl.Nt);
     p.step_chunk_first = step(pl.Nt + pl.halo);
     p.step_chunk_super = step(super_step - last_chunk);
     p.Nt = pl.Nt; p.P = pl.P; p.T = pl.T; p.halo = pl.halo; p.n_tiles = pl.n_tiles; p.n_super = pl.n_super; p.total_q = pl.total_q;

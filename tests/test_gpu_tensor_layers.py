@@ -3,10 +3,11 @@ stride 2 (one phase grid of four), odd and even image sizes, channel remainders,
 of channel words, whose last ones pair up across taps."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 import paper_2011_09398_b200 as lce
-from gpu_util import run_bconv
+from gpu_util import run_bconv, to_dev, to_dev_words, words_to_host
 
 pytestmark = pytest.mark.gpu
 
@@ -39,4 +40,32 @@ def test_tensor_layers_match_the_oracle(shape):
     thr = np.rint(np.sqrt(k * k * cin) * rng.standard_normal(cout)).astype(np.int32)
     got = run_bconv(aw, ww, dict(kwargs, out_type=lce.OUT_BITPACKED), thr=thr, kernel_choice=lce.KERNEL_TENSOR, packed=True)
     np.testing.assert_array_equal(got, oracle.transform_bits(acc, thr))
+    assert lce.lce_device_status() == 0
+
+
+@pytest.mark.parametrize("n,h,w,c", [(1, 9, 9, 64), (40, 15, 13, 128), (9, 20, 17, 256)])
+def test_fused_words_of_special_values(n, h, w, c):
+    """The re-quantised copy is y < 0: 0 for -0.0 and for a NaN of either sign; tiles with one and with two chunks a warp."""
+    rng = np.random.default_rng(n + c)
+    a = (2 * rng.integers(0, 2, size=(n, h, w, c)) - 1).astype(np.int8)
+    wt = (2 * rng.integers(0, 2, size=(c, 3, 3, c)) - 1).astype(np.int8)
+    acc = oracle.bconv2d_acc(a, wt, (1, 1), lce.PAD_SAME_ONE)
+    mult, bias = np.where(rng.integers(0, 2, c), -1.0, 0.0).astype(np.float32), np.full(c, -0.0, np.float32)
+    nan = np.array([0x7FC00000, 0xFFC00000], np.uint32).view(np.float32)
+    special = np.concatenate([nan, np.array([np.inf, -np.inf, -0.0, 0.0, 1e-45, -1e-45, -1.0], np.float32)])
+    residual = rng.choice(special, size=acc.shape).astype(np.float32)
+    desc = lce.make_desc(n, h, w, c, c, out_type=lce.OUT_FLOAT32, kernel_choice=lce.KERNEL_TENSOR, weights_packed=1)
+    weights = lce.lce_bconv2d_pack_weights(desc, to_dev_words(oracle.bitpack_pm1(wt)))
+    with np.errstate(invalid="ignore"):
+        want = oracle.transform_float(acc, mult, bias)
+        for shortcut in (None, residual):
+            y = want if shortcut is None else oracle.add_f32(want, shortcut)
+            for floats in (False, True):
+                out = torch.empty(acc.shape, device="cuda:0") if floats else None
+                words = torch.empty((n, h, w, c // 32), dtype=torch.int32, device="cuda:0")
+                lce.lce_bconv2d_fused(desc, to_dev_words(oracle.bitpack_pm1(a)), weights, to_dev(mult), to_dev(bias),
+                                      None if shortcut is None else to_dev(shortcut), out, words)
+                np.testing.assert_array_equal(words_to_host(words), oracle.bitpack(y))
+                if floats:
+                    np.testing.assert_array_equal(out.cpu().numpy(), y)  # NaN equal to NaN
     assert lce.lce_device_status() == 0
