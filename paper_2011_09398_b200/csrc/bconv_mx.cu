@@ -25,7 +25,7 @@
 //     apart), so every staged position is expanded once for all taps.  T consecutive tiles share one
 //     buffer of T * Nt + halo rows, so the halo a tile reads beyond its own positions is staged once
 //     per T tiles; there are two to four such buffers (as many as shared memory has room for, up to what
-//     lets the loaders run four tiles ahead).
+//     lets the loaders run four tiles ahead), one where a CTA has no second super-tile.
 //   * K is the taps' channel words, 32 values each, two to an instruction (mx_word): the two chunks of its B operand are
 //     rows of one buffer any distance apart, so the last words of an odd count pair up across taps.  A word of zeros
 //     per tap instead cost 9 MMAs for 9 words (32 channels, 3x3; now 5) and 75 for 125 (160 channels, 5x5; now 63:
@@ -186,7 +186,7 @@ struct MxParams {
     int32_t pairs, stages, resident;
     int32_t group_pairs, groups;  // streamed weights: pairs per ring stage, stages' worth of pairs per tile = ceil(pairs / group_pairs)
     int32_t x_bytes;
-    int32_t n_xbuf, ahead;   // position buffers (2..4); tiles the loaders may be ahead of the finished MMAs (2..4)
+    int32_t n_xbuf, ahead;   // position buffers (1..4); tiles the loaders may be ahead of the finished MMAs (2..4)
     int32_t off_tbl, off_w, off_x;    // byte offsets in shared memory
     int32_t cp_words;        // words per cp.async: 4, 2 or 1
     int32_t pad_zero, out_type, activation, write_float;
@@ -400,8 +400,8 @@ __device__ __forceinline__ bool mx_load_tiles(const MxParams &p, const MxLoad &l
             if (it >= ahead) {
                 // At most `ahead` tiles in front of the finished MMAs: those of tile it - ahead are done (a
                 // ring of four barriers, one commit per tile).  That keeps the arrivals on the four full_x
-                // barriers within one phase of what the issuer has seen, and (the MMAs finish in order; ahead
-                // <= (n_xbuf - 1) * T + 1) it means that the super-tile whose position buffer this chunk
+                // barriers within one phase of what the issuer has seen, and (the MMAs finish in order; with more than one
+                // super-tile ahead <= (n_xbuf - 1) * T + 1) it means that the super-tile whose position buffer this chunk
                 // overwrites has been read completely.
                 const int done = it - ahead;
                 if (!mbar_wait_bounded(&bars[BAR_TILE_DONE0 + (done & 3)], (uint32_t)(done >> 2) & 1u)) return false;
@@ -1355,7 +1355,7 @@ struct MxRoom {
     size_t raw_words, x_bytes, off_tbl, off_w, rest;
 };
 
-bool mx_room(const MxPlan &pl, int nt, int T, MxRoom *r)
+bool mx_room(const MxPlan &pl, int nt, int T, int n_xbuf, MxRoom *r)
 {
     // T tiles share one position buffer of T * nt + halo rows: the halo is staged once per T tiles
     r->P = T * nt + pl.halo;
@@ -1365,7 +1365,7 @@ bool mx_room(const MxPlan &pl, int nt, int T, MxRoom *r)
     r->off_tbl = kOffDyn + r->raw_words * 4;
     const size_t fixed = r->off_tbl + (size_t)pl.pairs * 8;  // the table no longer than it is: at 512 channels 3x3 the 8 KB saved are a wider tile
     r->off_w = (fixed + 127) / 128 * 128;
-    r->rest = 2 * r->x_bytes + 256;
+    r->rest = n_xbuf * r->x_bytes + 256;
     return r->off_w + r->rest + (size_t)min(2, pl.pairs) * kPairBytes <= kSmemLimit;
 }
 
@@ -1396,7 +1396,13 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
         for (int T = 1; T <= 8; ++T) {
             if (T > 1 && (T - 1) * ctas_max >= n_tiles) break;   // no CTA would have that many tiles
             MxRoom room;
-            if (!mx_room(*pl, nt, T, &room)) break;
+            // A CTA that has one super-tile needs one position buffer.  28x28x256 at stride 2, 64 images: one tile of 208
+            // positions a CTA instead of two of 112 beside two buffers of four phases, 11.2 -> 9.5 us; 7x7x512, 128 images
+            // 10.7 -> 10.3; 56x56x64, 64 images, float (seven tiles in one super-tile) 13.8 -> 13.5.
+            const int n_super = (n_tiles + T - 1) / T;
+            const int ctas_x = min(ctas_max, n_super);
+            const bool single = n_super <= ctas_x;
+            if (!mx_room(*pl, nt, T, single ? 1 : 2, &room)) break;
             // pairs that fit beside the position buffers: all of them -> resident (one barrier); otherwise a ring of two
             // stages of half the fitting pairs each (a group costs the issuer one wait and one commit, whatever its
             // size: two large groups measured better than three or four smaller ones)
@@ -1411,8 +1417,6 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
                 group_pairs = (pairs + groups - 1) / groups;  // even groups
                 stages = min(kMaxStages, slots / group_pairs);
             }
-            const int n_super = (n_tiles + T - 1) / T;
-            const int ctas_x = min(ctas_max, n_super);
             const int per_cta = ((n_super + ctas_x - 1) / ctas_x) * T;
             // clocks per MMA: 43 + N/2, at least 100 (measured); the loaders need about 400 + 8 clocks per staged
             // position and tile
@@ -1439,10 +1443,10 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
                 // More position buffers where shared memory is left over (thin layers): the loaders may then be
                 // up to four tiles ahead, ahead <= (n_xbuf - 1) * T + 1, and the hand-overs between the roles
                 // (a few hundred clocks each) drop out of the per-tile cycle.
-                int n_xbuf = 2;
-                while (n_xbuf < 4 && (n_xbuf - 1) * T + 1 < 4 && pl->off_x + (size_t)(n_xbuf + 1) * room.x_bytes <= kSmemLimit) ++n_xbuf;
+                int n_xbuf = single ? 1 : 2;
+                while (!single && n_xbuf < 4 && (n_xbuf - 1) * T + 1 < 4 && pl->off_x + (size_t)(n_xbuf + 1) * room.x_bytes <= kSmemLimit) ++n_xbuf;
                 pl->n_xbuf = n_xbuf;
-                pl->ahead = min(4, (n_xbuf - 1) * T + 1);
+                pl->ahead = single ? 4 : min(4, (n_xbuf - 1) * T + 1);
                 pl->smem = pl->off_x + (size_t)n_xbuf * room.x_bytes;
             }
         }

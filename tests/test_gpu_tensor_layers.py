@@ -26,8 +26,12 @@ ODD_WORDS = [
     (2, 7, 7, 480, 64, 5, 2, lce.PAD_VALID), (1, 5, 4, 990, 40, 3, 1, lce.PAD_VALID), (2, 9, 9, 992, 32, 1, 1, lce.PAD_SAME_ONE),
 ]
 
+# CTAs with a single super-tile, and so one position buffer: of one tile whose weights stream, of seven tiles (more than the
+# barriers of a ring), of tiles that the last CTA has fewer of
+ONE_BUFFER = [(64, 28, 28, 256, 40, 3, 2, lce.PAD_SAME_ZERO), (64, 56, 56, 32, 20, 3, 1, lce.PAD_SAME_ONE), (37, 56, 55, 40, 33, 3, 1, lce.PAD_SAME_ZERO)]
 
-@pytest.mark.parametrize("shape", SHAPES + ODD_WORDS, ids=lambda s: "x".join(map(str, s)))
+
+@pytest.mark.parametrize("shape", SHAPES + ODD_WORDS + ONE_BUFFER, ids=lambda s: "x".join(map(str, s)))
 def test_tensor_layers_match_the_oracle(shape):
     n, h, w, cin, cout, k, s, pad = shape
     rng = np.random.default_rng(sum(shape))
