@@ -11,8 +11,8 @@
 // five bits of the word free: they carry popcount(a) in binary, with weights that take 64 of it off, and the
 // threshold is the instruction's third operand, so an output bit is the sign of a matrix result with no arithmetic
 // behind it.  What bounds it is the logic pipe: the gather (nine words per pixel) and collecting those signs.
-// 224x224x3 -> 32, stride 2: batch 256 43 -> 36 us (the popcount loop before it was bound by the popcount unit), batch
-// 64 17 -> 11 us, one image 4.6 -> 2.0 us.
+// 224x224x3 -> 32, stride 2: batch 256 43 -> 36 us (the popcount loop before it was bound by the popcount unit), with all
+// signs of a lane in one register 36 -> 28.6; batch 64 17 -> 11.4 -> 9.5 us, one image 4.6 -> 2.0 us.
 // Other outputs and zero-padding: a thread owns one output pixel and walks all output channels, 32 at a time.
 #include "common.cuh"
 #include "mx_common.cuh"
@@ -123,7 +123,7 @@ __device__ __forceinline__ PatchWords load_patch3(const PatchParams &p, int n, i
     const int y = oh * p.sh - p.pt, x = ow * p.sw - p.pl;
     const uint32_t *at = p.in + ((int64_t)n * p.H + y) * p.W + x;
     PatchWords w;
-    if (__all_sync(0xffffffffu, exists && y >= 0 && x >= 0 && y + 2 < p.H && x + 2 < p.W)) {  // nothing to test
+    if (__all_sync(0xffffffffu, exists && (unsigned)y < (unsigned)max(0, p.H - 2) && (unsigned)x < (unsigned)max(0, p.W - 2))) {  // nothing to test
 #pragma unroll
         for (int kx = 0; kx < 3; ++kx) {
             w.v[kx] = __ldg(at + kx);
@@ -167,14 +167,21 @@ __device__ __forceinline__ uint32_t gather_patch(const PatchParams &p, int n, in
     return patch;
 }
 
+__device__ __forceinline__ void compare_operands(const uint4 &c, int (&c0)[4], int (&c1)[4])
+{
+    asm("mov.b32 %0, %4;\n\tmov.b32 %1, %4;\n\tmov.b32 %2, %5;\n\tmov.b32 %3, %5;" : "=r"(c0[0]), "=r"(c0[1]), "=r"(c0[2]), "=r"(c0[3]) : "r"(c.x), "r"(c.y));
+    asm("mov.b32 %0, %4;\n\tmov.b32 %1, %4;\n\tmov.b32 %2, %5;\n\tmov.b32 %3, %5;" : "=r"(c1[0]), "=r"(c1[1]), "=r"(c1[2]), "=r"(c1[3]) : "r"(c.z), "r"(c.w));
+}
+
 // Bit-packed output, one-padding or none.  A warp takes 32 consecutive output pixels at a time: lane = pixel for the
 // gather, then four groups of 8 pixels x 32 channels.  Row r of matrix tile t is channel 4 (r % 8) + 2 t + r / 8 of the
-// word, so that a lane's four sums of a pixel are four neighbouring bits; three exchanges put the word together, and
-// every lane ends up with the word of one of the 32 pixels.  COUNTED: K <= 27, popcount(a) travels in the word.
+// word, so that a lane's four sums of a pixel are four neighbouring bits, its 32 sums a register of eight nibbles, and one
+// transpose of nibbles over eight lanes leaves every lane with the word of one of the 32 pixels (group by group, by a
+// product, three exchanges and selections each, this took 110 of 270 instructions).  COUNTED: K <= 27, popcount(a) travels in the word.
 constexpr int kLaneWords = 12;  // per lane and 32 channels: eight operand registers, four compare constants
 
 template <bool ONE_WORD, bool COUNTED>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 4)
 bconv_patch_bits_kernel(const PatchParams p, int packed)
 {
     extern __shared__ __align__(16) uint32_t smem[];  // [Cow][3][32 lanes][4]
@@ -222,7 +229,8 @@ bconv_patch_bits_kernel(const PatchParams p, int packed)
     // image, row and column of the lane's pixel, advanced by the grid's stride with carries
     const int step = gridDim.x * kThreads;
     const int step_ow = step % p.OW, step_rows = step / p.OW, step_oh = step_rows % p.OH, step_n = step_rows / p.OH;
-    int64_t m0 = blockIdx.x * kThreads + (int)(threadIdx.x & ~31u);
+    uint32_t m0 = blockIdx.x * kThreads + (threadIdx.x & ~31u);  // at most 2^31 + a step: unsigned
+    const uint32_t M = (uint32_t)p.M;
     int n, oh, ow;
     {
         const int m = (int)m0 + lane, r = m / p.OW;
@@ -234,70 +242,71 @@ bconv_patch_bits_kernel(const PatchParams p, int packed)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const uint4 *slots = reinterpret_cast<const uint4 *>(smem) + lane;
     uint4 w0 = slots[0], w1 = slots[32], c = slots[64];
-    const uint32_t scale = 1u << p.Cin, nibble_at = 1u << (4 * g);
+    int c0[4], c1[4];  // the third operands as the instruction wants them, in registers of their own (no moves in the loop)
+    compare_operands(c, c0, c1);
+    const uint32_t scale = 1u << p.Cin;
+    // the transpose's steps: a lane without the bit keeps its low halves and takes the partner's low halves above them, a
+    // lane with it the high ones
+    const uint32_t by_16 = g & 4 ? 0x3276u : 0x5410u, by_8 = g & 2 ? 0x3715u : 0x6240u, keep_4 = g & 1 ? 0xF0F0F0F0u : 0x0F0F0F0Fu, rot_4 = g & 1 ? 28u : 4u;
     const bool square3 = p.KH == 3 && p.KW == 3;
     PatchWords next{};
-    if (square3) next = load_patch3(p, n, oh, ow, m0 + lane < p.M);
-    for (; m0 < p.M; m0 += step) {
-        const uint32_t patch = square3 ? put_together(next, scale) : m0 + lane < p.M ? gather_patch(p, n, oh, ow, mask) : 0u;
+    if (square3) next = load_patch3(p, n, oh, ow, m0 + lane < M);
+    for (; m0 < M; m0 += step) {
+        const uint32_t patch = square3 ? put_together(next, scale) : m0 + lane < M ? gather_patch(p, n, oh, ow, mask) : 0u;
         ow += step_ow;
         oh += step_oh;
         n += step_n;
         if (ow >= p.OW) { ow -= p.OW; ++oh; }
         if (oh >= p.OH) { oh -= p.OH; ++n; }
-        if (square3) next = load_patch3(p, n, oh, ow, m0 + step + lane < p.M);
+        if (square3) next = load_patch3(p, n, oh, ow, m0 + step + lane < M);
         const int ones = __popc(patch);
         const uint32_t operand = COUNTED ? patch | (uint32_t)ones << 27 : patch;
-        uint32_t b0[4], b1[4];
-        int p0[4], p1[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const uint32_t word = __shfl_sync(0xffffffffu, operand, 8 * i + g);
-            b0[i] = word & a_lo;
-            b1[i] = word & a_hi;
-            if (!COUNTED) {
-                p0[i] = __shfl_sync(0xffffffffu, 64 * ones, 8 * i + 2 * q);
-                p1[i] = __shfl_sync(0xffffffffu, 64 * ones, 8 * i + 2 * q + 1);
-            }
-        }
-        const int64_t pixel = m0 + (g >> 1) * 8 + 2 * q + (g & 1);
+        const uint32_t pixel = m0 + (g >> 1) * 8 + 2 * q + (g & 1);
         for (int wd = 0; wd < (ONE_WORD ? 1 : p.Cow); ++wd) {
-            if (!ONE_WORD) { w0 = slots[wd * 96]; w1 = slots[wd * 96 + 32]; c = slots[wd * 96 + 64]; }
-            uint32_t mine = 0u;
+            if (!ONE_WORD) { w0 = slots[wd * 96]; w1 = slots[wd * 96 + 32]; c = slots[wd * 96 + 64]; compare_operands(c, c0, c1); }
+            // this lane's four neighbouring channels of the pixels 8 i + 2 q and 8 i + 2 q + 1, a nibble of sign bits each
+            uint32_t half[2];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                int d0[4], d1[4];
-                if (COUNTED) {
-                    mma_s8u8(d0, w0.x, w0.y, w0.z, w0.w, b0[i], b1[i], (int)c.x, (int)c.x, (int)c.y, (int)c.y);
-                    mma_s8u8(d1, w1.x, w1.y, w1.z, w1.w, b0[i], b1[i], (int)c.z, (int)c.z, (int)c.w, (int)c.w);
-                } else {
+            for (int h = 0; h < 2; ++h) {
+                uint32_t v = 0u;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) d0[k] = d1[k] = 0;
-                    mma_u8(d0, w0.x, w0.y, w0.z, w0.w, b0[i], b1[i]);
-                    mma_u8(d1, w1.x, w1.y, w1.z, w1.w, b0[i], b1[i]);
+                for (int i = 2 * h + 1; i >= 2 * h; --i) {
+                    const uint32_t word = __shfl_sync(0xffffffffu, operand, 8 * i + g), b0 = word & a_lo, b1 = word & a_hi;
+                    int d0[4], d1[4];
+                    if (COUNTED) {
+                        mma_s8u8(d0, w0.x, w0.y, w0.z, w0.w, b0, b1, c0[0], c0[1], c0[2], c0[3]);
+                        mma_s8u8(d1, w1.x, w1.y, w1.z, w1.w, b0, b1, c1[0], c1[1], c1[2], c1[3]);
+                    } else {
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const int more = k & 1 ? p1[i] : p0[i];
-                        d0[k] = (int)(k & 2 ? c.y : c.x) + more - d0[k];
-                        d1[k] = (int)(k & 2 ? c.w : c.z) + more - d1[k];
+                        for (int k = 0; k < 4; ++k) d0[k] = d1[k] = 0;
+                        const int p0 = __shfl_sync(0xffffffffu, 64 * ones, 8 * i + 2 * q), p1 = __shfl_sync(0xffffffffu, 64 * ones, 8 * i + 2 * q + 1);
+                        mma_u8(d0, w0.x, w0.y, w0.z, w0.w, b0, b1);
+                        mma_u8(d1, w1.x, w1.y, w1.z, w1.w, b0, b1);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const int more = k & 1 ? p1 : p0;
+                            d0[k] = (int)(k & 2 ? c.y : c.x) + more - d0[k];
+                            d1[k] = (int)(k & 2 ? c.w : c.z) + more - d1[k];
+                        }
+                    }
+#pragma unroll
+                    for (int b = 1; b >= 0; --b) {  // the lowest channel last
+                        v = __funnelshift_l((uint32_t)d1[2 + b], v, 1);
+                        v = __funnelshift_l((uint32_t)d1[b], v, 1);
+                        v = __funnelshift_l((uint32_t)d0[2 + b], v, 1);
+                        v = __funnelshift_l((uint32_t)d0[b], v, 1);
                     }
                 }
-                // the sign bits of four channels of a pixel, the lowest channel last
-                const auto nibble = [&](int x0, int x1, int x2, int x3) {
-                    uint32_t v = (uint32_t)x3 >> 31;
-                    v = __funnelshift_l((uint32_t)x2, v, 1);
-                    v = __funnelshift_l((uint32_t)x1, v, 1);
-                    v = __funnelshift_l((uint32_t)x0, v, 1);
-                    asm("mul.lo.u32 %0, %0, %1;" : "+r"(v) : "r"(nibble_at));
-                    return v;
-                };
-                const uint32_t n0 = nibble(d0[0], d0[2], d1[0], d1[2]), n1 = nibble(d0[1], d0[3], d1[1], d1[3]);
-                uint32_t v = (g & 1 ? n1 : n0) | __shfl_xor_sync(0xffffffffu, g & 1 ? n0 : n1, 4);
-                v |= __shfl_xor_sync(0xffffffffu, v, 8);
-                v |= __shfl_xor_sync(0xffffffffu, v, 16);
-                if ((g >> 1) == i) mine = ~v;
+                half[h] = v;
             }
-            if (pixel < p.M) static_cast<uint32_t *>(p.out)[pixel * p.Cow + wd] = mine;
+            // nibble s of lane (g, q) belongs to pixel s of the quad's column q: transposed over the eight g, lane (g, q) holds
+            // all eight nibbles of pixel s = g
+            uint32_t v = __byte_perm(half[0], half[1], 0x5410);
+            v = __byte_perm(v, __shfl_xor_sync(0xffffffffu, v, 16), by_16);
+            v = __byte_perm(v, __shfl_xor_sync(0xffffffffu, v, 8), by_8);
+            const uint32_t y = __shfl_xor_sync(0xffffffffu, v, 4);
+            const uint32_t mine = ~((v & keep_4) | (__funnelshift_l(y, y, rot_4) & ~keep_4));
+            if (pixel < M) static_cast<uint32_t *>(p.out)[ONE_WORD ? pixel : (uint64_t)pixel * (uint32_t)p.Cow + wd] = mine;
         }
     }
 }
