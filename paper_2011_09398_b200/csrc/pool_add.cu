@@ -4,68 +4,93 @@
 // programmatic dependents: they wait for the previous kernel before their first access.
 #include "common.cuh"
 
+#include <string.h>
+
 namespace lce {
 namespace {
 
 constexpr int kThreads = 256;
 
-// A block walks output rows (n, oh); its threads walk the row's words, VEC words at a time (VEC = 4:
-// 128-bit loads and stores, when the word count per pixel allows), so that the only division left
-// per output is a 32-bit one by the words per pixel.  Out-of-image taps are skipped (AND identity
-// = all ones); channel-pad bits stay 0 because they are 0 in every input word.
+// n / d for 0 <= n < 2^31 (fast_div_constants)
+struct FastDiv {
+    uint32_t mul, sh;
+    __device__ __forceinline__ int32_t operator()(int32_t n) const { return (int32_t)(((uint64_t)(uint32_t)n * mul) >> sh); }
+};
+
+struct PoolParams {
+    const uint32_t *in;
+    uint32_t *out;
+    int32_t total, row0, H, W, Cw, OH, OW, PH, PW, sh, sw, pt, pl;  // total: output vectors of the launch, from output row row0 of all images on
+    FastDiv by_cv, by_ow, by_oh;                                    // cv: vectors of a pixel
+};
+
 template <int VEC>
-__global__ void __launch_bounds__(kThreads)
-bmaxpool_kernel(const uint32_t *__restrict__ in, uint32_t *__restrict__ out, int32_t N, int32_t H, int32_t W,
-                int32_t Cw, int32_t OH, int32_t OW, int32_t PH, int32_t PW, int32_t sh, int32_t sw, int32_t pt,
-                int32_t pl)
+struct Words;
+template <>
+struct Words<1> { using type = uint32_t; };
+template <>
+struct Words<2> { using type = uint2; };
+template <>
+struct Words<4> { using type = uint4; };
+
+__device__ __forceinline__ uint32_t both(uint32_t a, uint32_t b) { return a & b; }
+__device__ __forceinline__ uint2 both(const uint2 &a, const uint2 &b) { return make_uint2(a.x & b.x, a.y & b.y); }
+__device__ __forceinline__ uint4 both(const uint4 &a, const uint4 &b) { return make_uint4(a.x & b.x, a.y & b.y, a.z & b.z, a.w & b.w); }
+
+// A thread takes output vectors, VEC words of a pixel (the widest of 1, 2, 4 that divides a pixel's words), wherever rows
+// and images end: a block to an output row left most of its threads idle on the narrow tensors behind a network's first stages
+// (56x56x64, 128 images: 28 pixels of two words; 3.9 us, now 1.9; 56x56x128 4.5, now 2.5).  Out-of-image taps are skipped (AND identity = all
+// ones); channel-pad bits stay 0 because they are 0 in every input word.
+template <int VEC>
+__global__ void __launch_bounds__(kThreads) bmaxpool_kernel(const __grid_constant__ PoolParams p)
 {
+    using V = typename Words<VEC>::type;
+    const int32_t cv = p.Cw / VEC, H = p.H, W = p.W;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int32_t cv = Cw / VEC;            // vectors per pixel
-    const int32_t row_vecs = OW * cv;       // vectors per output row
-    const int32_t rows = N * OH;  // < 2^31: checked on the host
-    for (int32_t row = blockIdx.x; row < rows; row += gridDim.x) {
-        const int32_t n = row / OH, oh = row - n * OH;
-        const int32_t iy0 = oh * sh - pt;
-        const uint32_t *img = in + (int64_t)n * H * W * Cw;
-        uint32_t *orow = out + (int64_t)row * OW * Cw;
-        for (int32_t e = threadIdx.x; e < row_vecs; e += kThreads) {
-            const int32_t ow = e / cv, j = (e - ow * cv) * VEC;
-            const int32_t ix0 = ow * sw - pl;
-            uint32_t acc[VEC];
-            if (PH == 2 && PW == 2 && iy0 >= 0 && iy0 + 1 < H && ix0 >= 0 && ix0 + 1 < W) {
-                // the usual 2x2 window, inside the image: four independent loads in flight, three ANDs
-                const uint32_t *s0 = img + ((int64_t)iy0 * W + ix0) * Cw + j, *s1 = s0 + (int64_t)W * Cw;
-                if (VEC == 4) {
-                    const uint4 a = __ldcs(reinterpret_cast<const uint4 *>(s0)), b = __ldcs(reinterpret_cast<const uint4 *>(s0 + Cw));
-                    const uint4 c = __ldcs(reinterpret_cast<const uint4 *>(s1)), d = __ldcs(reinterpret_cast<const uint4 *>(s1 + Cw));
-                    __stcs(reinterpret_cast<uint4 *>(orow + (int64_t)ow * Cw + j),
-                           make_uint4(a.x & b.x & c.x & d.x, a.y & b.y & c.y & d.y, a.z & b.z & c.z & d.z, a.w & b.w & c.w & d.w));
-                } else {
-                    orow[(int64_t)ow * Cw + j] = __ldcs(s0) & __ldcs(s0 + Cw) & __ldcs(s1) & __ldcs(s1 + Cw);
-                }
-                continue;
-            }
-#pragma unroll
-            for (int v = 0; v < VEC; ++v) acc[v] = 0xffffffffu;
-            for (int32_t ky = 0; ky < PH; ++ky) {
-                const int32_t iy = iy0 + ky;
-                if (iy < 0 || iy >= H) continue;
-                for (int32_t kx = 0; kx < PW; ++kx) {
-                    const int32_t ix = ix0 + kx;
-                    if (ix < 0 || ix >= W) continue;
-                    const uint32_t *src = img + ((int64_t)iy * W + ix) * Cw + j;
-                    if (VEC == 4) {
-                        const uint4 q = __ldg(reinterpret_cast<const uint4 *>(src));
-                        acc[0] &= q.x; acc[1] &= q.y; acc[2] &= q.z; acc[3] &= q.w;
-                    } else {
-                        acc[0] &= __ldg(src);
-                    }
-                }
-            }
-            if (VEC == 4) *reinterpret_cast<uint4 *>(orow + (int64_t)ow * Cw + j) = make_uint4(acc[0], acc[1], acc[2], acc[3]);
-            else orow[(int64_t)ow * Cw + j] = acc[0];
+    const V *const in = reinterpret_cast<const V *>(p.in);
+    V *const out = reinterpret_cast<V *>(p.out);
+    for (uint32_t e = blockIdx.x * kThreads + threadIdx.x; e < (uint32_t)p.total; e += gridDim.x * kThreads) {
+        const int32_t pixel = p.by_cv((int32_t)e), local = p.by_ow(pixel), row = p.row0 + local, n = p.by_oh(row);
+        const int32_t iy0 = (row - n * p.OH) * p.sh - p.pt, ix0 = (pixel - local * p.OW) * p.sw - p.pl;
+        const V *at = in + ((int64_t)n * H + iy0) * W * cv + (int64_t)ix0 * cv + ((int32_t)e - pixel * cv);
+        if (p.PH == 2 && p.PW == 2 && iy0 >= 0 && iy0 + 1 < H && ix0 >= 0 && ix0 + 1 < W) {
+            // the usual 2x2 window, inside the image: four independent loads in flight, three ANDs
+            const V *below = at + (int64_t)W * cv;
+            __stcs(out + e, both(both(__ldcs(at), __ldcs(at + cv)), both(__ldcs(below), __ldcs(below + cv))));
+            continue;
         }
+        V acc;
+        memset(&acc, 0xff, sizeof(acc));
+        for (int32_t ky = 0; ky < p.PH; ++ky) {
+            if (iy0 + ky < 0 || iy0 + ky >= H) continue;
+            for (int32_t kx = 0; kx < p.PW; ++kx)
+                if (ix0 + kx >= 0 && ix0 + kx < W) acc = both(acc, __ldg(at + ((int64_t)ky * W + kx) * cv));
+        }
+        out[e] = acc;
     }
+}
+
+template <int VEC>
+lce_status launch_pool(PoolParams p, int32_t batch, cudaStream_t s)
+{
+    // so many rows at a time that a launch has fewer than 2^31 vectors (and a step of its grid more)
+    const int64_t row = (int64_t)p.OW * (p.Cw / VEC), step = 148 * 16 * kThreads, rows = (int64_t)batch * p.OH;
+    if (row >= (1ll << 31) - step) return LCE_ERR_UNSUPPORTED;
+    const int64_t most = ((1ll << 31) - step) / row;
+    fast_div_constants((uint32_t)(p.Cw / VEC), &p.by_cv.mul, &p.by_cv.sh);
+    fast_div_constants((uint32_t)p.OW, &p.by_ow.mul, &p.by_ow.sh);
+    fast_div_constants((uint32_t)p.OH, &p.by_oh.mul, &p.by_oh.sh);
+    for (int64_t r = 0; r < rows; r += most) {
+        PoolParams q = p;
+        q.row0 = (int32_t)r;
+        q.total = (int32_t)((rows - r < most ? rows - r : most) * row);
+        q.out += r * p.OW * p.Cw;
+        const int64_t blocks = (q.total + (int64_t)kThreads - 1) / kThreads;
+        const lce_status st = launch_dependent(bmaxpool_kernel<VEC>, dim3((unsigned)(blocks < 148 * 16 ? blocks : 148 * 16)), kThreads, 0, s, q);
+        if (st != LCE_OK) return st;
+    }
+    return LCE_OK;
 }
 
 __global__ void __launch_bounds__(kThreads)
@@ -112,15 +137,12 @@ extern "C" lce_status lce_bmaxpool(const uint32_t *in, uint32_t *out, int32_t ba
     const Axis aw = axis_geometry(in_w, pool_w, stride_w, padding);
     if (ah.out <= 0 || aw.out <= 0) return LCE_ERR_INVALID_ARG;
     const int32_t Cw = (channels + 31) / 32;
-    const int64_t total = (int64_t)batch * ah.out * aw.out * Cw;
-    (void)total;
     if ((int64_t)batch * ah.out >= (1ll << 31)) return LCE_ERR_UNSUPPORTED;
-    int64_t blocks = (int64_t)batch * ah.out;  // one block per output row, grid-stride beyond 8 waves of 8 blocks per SM
-    if (blocks > 148 * 8 * 8) blocks = 148 * 8 * 8;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const bool vec = Cw % 4 == 0 && aligned(in, 16) && aligned(out, 16);
-    return launch_dependent(vec ? bmaxpool_kernel<4> : bmaxpool_kernel<1>, dim3((unsigned)blocks), kThreads, 0, s, in, out, batch, in_h, in_w, Cw, ah.out,
-                            aw.out, pool_h, pool_w, stride_h, stride_w, ah.pad_before, aw.pad_before);
+    const PoolParams p{in, out, 0, 0, in_h, in_w, Cw, ah.out, aw.out, pool_h, pool_w, stride_h, stride_w, ah.pad_before, aw.pad_before, {}, {}, {}};
+    if (Cw % 4 == 0 && aligned(in, 16) && aligned(out, 16)) return launch_pool<4>(p, batch, s);
+    if (Cw % 2 == 0 && aligned(in, 8) && aligned(out, 8)) return launch_pool<2>(p, batch, s);
+    return launch_pool<1>(p, batch, s);
 }
 
 extern "C" lce_status lce_add_f32(const float *a, const float *b, float *out, int64_t n, void *stream)

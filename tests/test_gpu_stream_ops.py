@@ -52,3 +52,23 @@ def test_weights_quantized_right_before_the_convolution(cin, k):
         outs.append(lce.lce_bconv2d(desc, x, words))
     for w, out in zip(ws, outs):
         np.testing.assert_array_equal(out.cpu().numpy(), oracle.bconv2d_acc(a, w))
+
+
+# widths of 1, 2, 3, 4 and 6 words (vectors of one, two and four), windows inside and across the edge, buffers that are only
+# 4-byte aligned
+@pytest.mark.parametrize("offset", [0, 1, 2])
+@pytest.mark.parametrize("n,h,w,c,pool,stride,pad", [(3, 9, 7, 32, (2, 2), (2, 2), lce.PAD_VALID), (2, 8, 11, 50, (2, 2), (2, 2), lce.PAD_SAME_ONE), (5, 7, 6, 96, (2, 2), (1, 1), lce.PAD_SAME_ONE),
+                                                     (2, 13, 5, 128, (3, 2), (2, 3), lce.PAD_SAME_ONE), (1, 1, 1, 180, (2, 2), (2, 2), lce.PAD_SAME_ONE), (70, 56, 56, 64, (2, 2), (2, 2), lce.PAD_VALID)])
+def test_maxpool_matches_the_oracle(n, h, w, c, pool, stride, pad, offset):
+    rng = np.random.default_rng(n * h + c)
+    x = np.where(rng.random((n, h, w, c)) < 0.8, -1.0, 1.0).astype(np.float32)
+    words = oracle.bitpack(x)
+    want = oracle.bmaxpool(words, c, pool, stride, pad)
+    src = torch.empty(words.size + offset, dtype=torch.int32, device=DEV)[offset:].view(words.shape)
+    src.copy_(torch.from_numpy(words.view(np.int32)))
+    whole = torch.full((want.size + 128 + offset,), 0x5A5A5A5A, dtype=torch.int32, device=DEV)
+    out = whole[64 + offset:64 + offset + want.size].view(want.shape)
+    lce.lce_bmaxpool(src, c, pool, stride, pad, out)
+    assert guards_intact(whole, 0x5A5A5A5A)
+    np.testing.assert_array_equal(words_to_host(out), want)
+
