@@ -17,6 +17,7 @@ constexpr int kWordsPerWarpPass = 32;  // one warp turns 32x32 floats (4 KB) int
 // handed out four per lane to lanes 0..7, which write them with one 128-bit store each (128
 // contiguous bytes per warp).  Passes are small so that even a 100K-word tensor gives every SM
 // several warps of work: the kernel is latency-bound otherwise.
+template <bool KEEP>
 __global__ void __launch_bounds__(kPackThreads)
 bitpack_aligned_kernel(const float *__restrict__ x, uint32_t *__restrict__ out, int64_t n_words)
 {
@@ -29,7 +30,7 @@ bitpack_aligned_kernel(const float *__restrict__ x, uint32_t *__restrict__ out, 
         if (w0 + kWordsPerWarpPass <= n_words) {
             float v[kWordsPerWarpPass];
 #pragma unroll
-            for (int u = 0; u < kWordsPerWarpPass; ++u) v[u] = __ldcs(x + (w0 + u) * 32 + lane);
+            for (int u = 0; u < kWordsPerWarpPass; ++u) v[u] = KEEP ? __ldg(x + (w0 + u) * 32 + lane) : __ldcs(x + (w0 + u) * 32 + lane);
             uint32_t mine[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
             for (int u = 0; u < kWordsPerWarpPass; ++u) {
@@ -254,7 +255,10 @@ extern "C" lce_status lce_bitpack(const float *x, uint32_t *out, int64_t rows, i
     const int max_blocks = 148 * 8 * 4;
     if (channels % 32 == 0 && aligned(out, 16)) {
         const int64_t passes = (n_words + kWordsPerWarpPass - 1) / kWordsPerWarpPass;
-        return launch_dependent(bitpack_aligned_kernel, dim3(grid_for(passes, kPackThreads / 32, max_blocks)), kPackThreads, 0, s, x, out, n_words);
+        // A tensor that fits in the L2 stays there: it is a shortcut's operand or comes back as one (51 MB again and again 5.7 ->
+        // 4.8 us); a larger one would only push out what is there (205 MB: 30.1 us, 31.8 if kept; the residual stack 217 and 225).
+        const auto kernel = n_words * 128 <= (64ll << 20) ? bitpack_aligned_kernel<true> : bitpack_aligned_kernel<false>;
+        return launch_dependent(kernel, dim3(grid_for(passes, kPackThreads / 32, max_blocks)), kPackThreads, 0, s, x, out, n_words);
     }
     if (channels <= 4 && rows >= 4 && aligned(x, 16) && aligned(out, 16)) {
         if (channels == 1) return launch_few_channels<1>(x, out, rows, max_blocks * 4, s);

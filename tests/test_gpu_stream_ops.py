@@ -72,3 +72,14 @@ def test_maxpool_matches_the_oracle(n, h, w, c, pool, stride, pad, offset):
     assert guards_intact(whole, 0x5A5A5A5A)
     np.testing.assert_array_equal(words_to_host(out), want)
 
+
+@pytest.mark.parametrize("n", [1, 3, 4, 7, 1023, 4 * 148 * 8 * 256 + 5])
+def test_add_from_the_last_element_to_the_first(n):
+    rng = np.random.default_rng(n)
+    a, b = (rng.standard_normal(n).astype(np.float32) for _ in range(2))
+    whole, out = guarded((n,), torch.float32, 9.0)
+    lce.lce_add_f32(to_dev(a), to_dev(b), out)
+    assert guards_intact(whole, 9.0)
+    np.testing.assert_array_equal(out.cpu().numpy(), oracle.add_f32(a, b))
+    ad = to_dev(a)
+    np.testing.assert_array_equal(lce.lce_add_f32(ad, to_dev(b), ad).cpu().numpy(), oracle.add_f32(a, b))  # onto an operand
