@@ -80,7 +80,7 @@ constexpr int kMaxStages = 32;
 // shared-memory map (bytes)
 constexpr int kOffBars = 0;          // full_x[4] tile_done[4] full_d[2] empty_d[2] done[2] scales full_w[32] empty_w[32]
 constexpr int kOffSlot = 1000;       // TMEM base address; 1004 fills issued, 1008 fills consumed
-constexpr int kOffPix = 1024;        // int32[16][2][32]: for every finisher warp the output pixels of the positions it works on, two chunks of a tile at most; int32[32]: -1
+constexpr int kOffPix = 1024;        // int32[16][2][32]: for every finisher warp the output pixels (or offsets) of the positions it works on, two chunks of a tile at most; int32[32]: -1
 constexpr int kOffDyn = 5248;       // raw words, uint2[MMAs of a tile]: operand offsets (A, B; 16-byte units), weight ring, position buffers
 
 enum { BAR_FULL_X0 = 0, BAR_FULL_X3 = 3, BAR_TILE_DONE0, BAR_TILE_DONE3 = BAR_TILE_DONE0 + 3, BAR_FULL_D0, BAR_FULL_D1, BAR_EMPTY_D0, BAR_EMPTY_D1, BAR_DONE, BAR_DONE_B,
@@ -691,9 +691,9 @@ struct MxFin {
     bool relu, write_float;
     int N, OH, OW, Wg, Hg;   // position -> output pixel
     uint32_t Wg_mul, Wg_sh, Hg_mul, Hg_sh;
-    int lane_step;           // from lane_pixels of the first chunk to that of the second
-    int32_t *pixels;         // shared memory: output pixels of the two chunks' positions (one array per warp)
-    const int32_t *lane_pixels;  // the same for this lane; a row of -1 if its channel does not exist
+    int lane_step;           // from lane_positions of the first chunk to that of the second
+    int32_t *positions;      // shared memory: output pixels or offsets of the two chunks' positions (one array per warp)
+    const int32_t *lane_positions;  // the same for this lane; a row of -1 if its channel does not exist
 };
 
 __device__ __forceinline__ MxFin mx_fin_context(const MxParams &p, int32_t *sPix, int fw, int lane, int ch0)
@@ -729,9 +729,9 @@ __device__ __forceinline__ MxFin mx_fin_context(const MxParams &p, int32_t *sPix
     f.write_float = p.write_float != 0;
     f.N = p.N; f.OH = p.OH; f.OW = p.OW; f.Wg = p.Wg; f.Hg = p.Hg;
     f.Wg_mul = p.Wg_mul; f.Wg_sh = p.Wg_sh; f.Hg_mul = p.Hg_mul; f.Hg_sh = p.Hg_sh;
-    f.pixels = sPix + fw * 64;
+    f.positions = sPix + fw * 64;
     f.lane_step = ch_ok ? 32 : 0;
-    f.lane_pixels = ch_ok ? f.pixels : sPix + 2 * kFinishers;
+    f.lane_positions = ch_ok ? f.positions : sPix + 2 * kFinishers;
     return f;
 }
 
@@ -795,19 +795,20 @@ __device__ __forceinline__ void mx_epilogue_bits(const MxFin &f, const Transpose
 // shared memory, -1 where nothing is to be written: one compare a position.
 enum { EPI_FLOAT = 0, EPI_FLOAT_FUSED = 1, EPI_INT32 = 2, EPI_BITS = 3, EPI_PLAIN = 4 };
 
-// the output pixels of the chunks' positions, for the whole warp to see
-__device__ __forceinline__ void mx_share_pixels(const MxFin &f, int pix, int pix2, int lane)
+// the chunks' positions, for the whole warp to see: output pixels, -1 where nothing is to be written, or (the fused form) the
+// offsets of their elements from a channel's first one, which are below 2^31
+__device__ __forceinline__ void mx_share_positions(const MxFin &f, int first, int second, int lane)
 {
     __syncwarp();  // the tile before is through with the array
-    f.pixels[lane] = pix;
-    f.pixels[32 + lane] = pix2;
+    f.positions[lane] = first;
+    f.positions[32 + lane] = second;
     __syncwarp();
 }
 
 template <int MODE>
 __device__ __forceinline__ void mx_epilogue_values(const MxFin &f, uint32_t tmem_d, int lane, uint64_t *empty_d)
 {
-    const int32_t *lane_pixels = f.lane_pixels;
+    const int32_t *lane_positions = f.lane_positions;
     for (int ck = f.group; ck <= f.last_chunk; ck += f.n_groups) {
         const int c0 = ck * 32;
         const bool full = c0 + 32 <= f.Nt;
@@ -821,11 +822,11 @@ __device__ __forceinline__ void mx_epilogue_values(const MxFin &f, uint32_t tmem
                 if (ck == f.last_chunk && (half == 1 || !full)) mx_hand_back(empty_d, lane);
 #pragma unroll
                 for (int j4 = 0; j4 < 16; j4 += 4) {
-                    const int4 o4 = *reinterpret_cast<const int4 *>(lane_pixels + half * 16 + j4);
+                    const int4 o4 = *reinterpret_cast<const int4 *>(lane_positions + half * 16 + j4);
                     const int o[4] = {o4.x, o4.y, o4.z, o4.w};
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        float *at = f.outp + (int64_t)o[u] * f.cout;
+                        float *at = f.outp + (int64_t)o[u] * f.cout;  // outside the condition: nothing branches
                         if (MODE != EPI_INT32) {
                             const float y = __fmaf_rn(v[j4 + u], f.mult, f.bias);
                             if (o[u] >= 0) *at = y;
@@ -837,7 +838,7 @@ __device__ __forceinline__ void mx_epilogue_values(const MxFin &f, uint32_t tmem
                 }
             }
         }
-        lane_pixels += f.lane_step;
+        lane_positions += f.lane_step;
     }
     if (f.last_chunk < 0) mx_hand_back(empty_d, lane);  // nothing to read for this warp
 }
@@ -848,19 +849,20 @@ __device__ __forceinline__ void mx_epilogue_values(const MxFin &f, uint32_t tmem
 // (mx_shortcut: 32 independent 128-byte loads a warp), those of its next one when it is through with the first.  The
 // re-quantised copy is the sign bits and the bit transpose of the bit-packed form; y + 0 makes -0.0 and NaN, which
 // quantize to 0 bits, positive (PTX: a NaN result has no sign).
+// Positions come as offsets of elements: multiplying pixels by the channels at each use took 36.9 us on the 56x56x64 block at 128
+// images, 33.6 now (40.6 with ballots and loads behind the wait); the plain float form, which has registers to spare, is
+// faster with pixels (13.9 us against 14.4 on 56x56x64, 64 images).
 template <bool RES>
-__device__ __forceinline__ void mx_shortcut(const MxFin &f, const int32_t *pixels, float (&r)[32])
+__device__ __forceinline__ void mx_shortcut(const MxFin &f, const int32_t *offsets, float (&r)[32])
 {
     if (!RES) return;
 #pragma unroll
     for (int j4 = 0; j4 < 32; j4 += 4) {
-        const int4 o4 = *reinterpret_cast<const int4 *>(pixels + j4);  // the same for every lane
+        const int4 o4 = *reinterpret_cast<const int4 *>(offsets + j4);  // the same for every lane
         const int o[4] = {o4.x, o4.y, o4.z, o4.w};
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const float *at = f.resp + (int64_t)o[u] * f.cout;
-            r[j4 + u] = 0.f;
-            if (o[u] >= 0) r[j4 + u] = __ldg(at);
+            r[j4 + u] = o[u] >= 0 ? __ldg(f.resp + (o[u] >= 0 ? o[u] : 0)) : 0.f;
         }
     }
 }
@@ -872,11 +874,11 @@ __device__ __forceinline__ void mx_epilogue_fused(const MxFin &f, const Transpos
     // argument: a test of a pointer per position turns the unrolled block below into branchy code that
     // runs at a third of the speed (measured on the plain float transform, and again here)
     const float floor_v = f.relu ? 0.f : -INFINITY;
-    const int32_t *lane_pixels = f.lane_pixels;
+    const int32_t *lane_positions = f.lane_positions;
     for (int ck = f.group; ck <= f.last_chunk; ck += f.n_groups) {
         const int c0 = ck * 32;
         const bool full = c0 + 32 <= f.Nt;  // otherwise 16 columns, the tile's last
-        if (ck != f.group) mx_shortcut<RES>(f, f.pixels + 32, r);
+        if (ck != f.group) mx_shortcut<RES>(f, f.positions + 32, r);
         uint32_t m = 0u;
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
@@ -888,7 +890,7 @@ __device__ __forceinline__ void mx_epilogue_fused(const MxFin &f, const Transpos
                 for (int j4 = 0; j4 < 16; j4 += 4) {
                     int o[4];
                     if (WRITE_FLOAT) {
-                        const int4 o4 = *reinterpret_cast<const int4 *>(lane_pixels + half * 16 + j4);
+                        const int4 o4 = *reinterpret_cast<const int4 *>(lane_positions + half * 16 + j4);
                         o[0] = o4.x; o[1] = o4.y; o[2] = o4.z; o[3] = o4.w;
                     }
 #pragma unroll
@@ -896,8 +898,7 @@ __device__ __forceinline__ void mx_epilogue_fused(const MxFin &f, const Transpos
                         float y = __fmaf_rn(fmaxf(v[j4 + u], floor_v), f.mult, f.bias);
                         if (RES) y = __fadd_rn(y, r[half * 16 + j4 + u]);
                         if (WRITE_FLOAT) {
-                            float *at = f.outp + (int64_t)o[u] * f.cout;  // outside the condition: nothing branches
-                            if (o[u] >= 0) *at = y;
+                            if (o[u] >= 0) f.outp[o[u]] = y;
                         }
                         if (PACK) v[j4 + u] = y;
                     }
@@ -917,10 +918,10 @@ __device__ __forceinline__ void mx_epilogue_fused(const MxFin &f, const Transpos
         }
         if (PACK) {
             const uint32_t word = warp_transpose32(m, tr);
-            const int pix = lane_pixels[lane];
-            if (pix >= 0) f.packp[(int64_t)pix * f.cow] = word;
+            const int o = lane_positions[lane];
+            if (o >= 0) f.packp[o >> 5] = word;  // whole words of channels: 32 values to a word
         }
-        lane_pixels += f.lane_step;
+        lane_positions += f.lane_step;
     }
     if (f.last_chunk < 0) mx_hand_back(empty_d, lane);  // nothing to read for this warp
 }
@@ -940,8 +941,8 @@ __device__ __forceinline__ bool mx_finish_tiles(const MxParams &p, const MxFin &
             const int pix = mx_out_pixel(f, tile, f.group * 32, lane);
             const int pix2 = f.last_chunk > f.group ? mx_out_pixel(f, tile, (f.group + f.n_groups) * 32, lane) : -1;
             float r[32];
-            if (MODE != EPI_BITS) mx_share_pixels(f, pix, pix2, lane);
-            if (MODE == EPI_FLOAT_FUSED) mx_shortcut<RES>(f, f.pixels, r);
+            if (MODE != EPI_BITS) mx_share_positions(f, MODE == EPI_FLOAT_FUSED && pix >= 0 ? pix * f.cout : pix, MODE == EPI_FLOAT_FUSED && pix2 >= 0 ? pix2 * f.cout : pix2, lane);
+            if (MODE == EPI_FLOAT_FUSED) mx_shortcut<RES>(f, f.positions, r);
             // the warp goes on together (its transform uses warp-wide shuffles)
             if (!__all_sync(0xffffffffu, mbar_wait_bounded(&bars[BAR_FULL_D0 + buf], (uint32_t)(it >> 1) & 1u))) return false;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
