@@ -433,9 +433,10 @@ constexpr size_t kSmallSmem = 100 * 1024;  // two CTAs per SM, so that a CTA of 
 // The shape of a launch, by the best of sweeps over tiles, slices and warps on 40 layers (M = 49 .. 50176 pixels,
 // 1 .. 16 channel blocks, 1 .. 36 steps): the smallest tile that leaves few enough CTAs (more than two or three
 // per SM only repeat the set-up), 8 warps, and as many slices as give every warp a job.  Jobs of 16 pixels use a
-// weight operand twice and win where the depth gives enough steps to share out (8 and more); with few steps
-// 8-pixel jobs spread over more warps win.  Tiles of 32 pixels do better with four jobs of 16 pixels than with eight of 8 or
-// sixteen (56x56x64, one image 3.3 -> 2.8 us; 33x33x100, three 4.5 -> 4.2; every job ends in 8 updates of shared sums).
+// weight operand twice and win in tiles of 32 pixels and more, and where the depth gives enough steps to share out (8 and
+// more).  With few steps a second slice is enough in tiles of 16 and 32 pixels, even if half of the warps then have no
+// job: every job ends in 8 updates of shared sums.  One image of 56x56x64 (tiles of 32) 3.3 -> 2.8 us, of 56x56x64 -> 128 at
+// stride 2 (16) 2.8 -> 2.5, three of 33x33x100 (32) 4.5 -> 4.2, 53 of 8x8x160, 1x1 (64) 4.1 -> 3.8.
 // Tiles of 64 pixels in more CTAs than fit at once do better with four warps each; of 16 pixels they do not (14x14x256,
 // three images 3.8 us, 4.9 with four).
 SmallShape small_shape(const ConvGeom &g)
@@ -445,9 +446,9 @@ SmallShape small_shape(const ConvGeom &g)
     const auto ctas = [&](int tile) { return (g.M + tile - 1) / tile * g.Cow; };
     const auto most_ctas = [&](int tile) { return tile == 8 ? 220 : tile == 16 && steps < 8 ? 300 : 420; };
     while (s.tile < 64 && ctas(s.tile) > most_ctas(s.tile) && small_smem(g, 2 * s.tile) <= kSmallSmem) s.tile *= 2;
-    s.groups = s.tile == 32 || (s.tile >= 16 && steps >= 8) ? 2 : 1;
+    s.groups = s.tile >= 32 || (s.tile == 16 && steps >= 8) ? 2 : 1;
     const int jobs = s.tile / (8 * s.groups);           // of one slice
-    const int most = s.tile == 32 || (s.tile == 8 && steps < 32) ? 4 : 8;
+    const int most = s.tile == 32 || (s.tile == 16 && s.groups == 1) || (s.tile == 8 && steps < 32) ? 4 : 8;
     while (s.slices * jobs < most && 2 * s.slices <= steps) s.slices *= 2;
     if (s.tile == 64 && ctas(64) > 400) s.warps = 4;
     s.smem = small_smem(g, s.tile);
