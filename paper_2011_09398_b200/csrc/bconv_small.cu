@@ -434,7 +434,8 @@ constexpr size_t kSmallSmem = 100 * 1024;  // two CTAs per SM, so that a CTA of 
 // 1 .. 16 channel blocks, 1 .. 36 steps): the smallest tile that leaves few enough CTAs (more than two or three
 // per SM only repeat the set-up), 8 warps, and as many slices as give every warp a job.  Jobs of 16 pixels use a
 // weight operand twice and win in tiles of 32 pixels and more, and where the depth gives enough steps to share out (8 and
-// more).  With few steps a second slice is enough in tiles of 16 and 32 pixels, even if half of the warps then have no
+// more).  With few steps (below 8, in tiles of 32 below 20: 10x10x192, 16 images, 14 steps 5.5 -> 5.1 us, 10x10x383, 17
+// images, 27 steps 5.5 -> 6.4) a second slice is enough in tiles of 16 and 32 pixels, even if half of the warps then have no
 // job: every job ends in 8 updates of shared sums.  One image of 56x56x64 (tiles of 32) 3.3 -> 2.8 us, of 56x56x64 -> 128 at
 // stride 2 (16) 2.8 -> 2.5, three of 33x33x100 (32) 4.5 -> 4.2, 53 of 8x8x160, 1x1 (64) 4.1 -> 3.8.
 // Tiles of 64 pixels in more CTAs than fit at once do better with four warps each; of 16 pixels they do not (14x14x256,
@@ -448,7 +449,7 @@ SmallShape small_shape(const ConvGeom &g)
     while (s.tile < 64 && ctas(s.tile) > most_ctas(s.tile) && small_smem(g, 2 * s.tile) <= kSmallSmem) s.tile *= 2;
     s.groups = s.tile >= 32 || (s.tile == 16 && steps >= 8) ? 2 : 1;
     const int jobs = s.tile / (8 * s.groups);           // of one slice
-    const int most = s.tile == 32 || (s.tile == 16 && s.groups == 1) || (s.tile == 8 && steps < 32) ? 4 : 8;
+    const int most = (s.tile == 32 && steps < 20) || (s.tile == 16 && s.groups == 1) || (s.tile == 8 && steps < 32) ? 4 : 8;
     while (s.slices * jobs < most && 2 * s.slices <= steps) s.slices *= 2;
     if (s.tile == 64 && ctas(64) > 400) s.warps = 4;
     s.smem = small_smem(g, s.tile);
