@@ -21,13 +21,20 @@ SHAPES = [
     (1, 8, 8, 1024, 32, 3, 3, 1, ONE), (2, 15, 15, 64, 128, 7, 7, 2, ONE), (10, 60, 60, 32, 64, 3, 3, 3, ZERO), (20, 60, 60, 32, 64, 3, 3, 3, ONE),
 ]
 
+# tiles of 16 pixels (shallow: two slices; deeper: more), 32 (shallow, just below and above the depth at which slices are
+# kept, deep) and 64, the last one of each cut short
+TILES = [
+    (1, 38, 37, 64, 60, 3, 3, 1, ONE), (3, 21, 25, 96, 70, 3, 3, 1, ZERO), (1, 57, 56, 64, 60, 3, 3, 1, ZERO), (16, 12, 12, 252, 90, 3, 3, 1, ONE),
+    (16, 12, 12, 288, 66, 3, 3, 1, ONE), (17, 10, 10, 383, 109, 3, 3, 1, ONE), (41, 14, 13, 64, 64, 1, 1, 1, VALID), (53, 8, 8, 160, 155, 1, 1, 1, ZERO),
+]
+
 
 def is_small(n, h, w, cin, cout, kh, kw, s, pad, out_type):
     plan = lce.lce_bconv2d_plan(lce.make_desc(n, h, w, cin, cout, (kh, kw), (s, s), pad, out_type, weights_packed=1))
     return plan["kernel"] == lce.KERNEL_TILED and not plan["patch"] and plan["pixels_per_thread"] == 0 and plan["tile_pixels"] % 8 == 0
 
 
-@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("shape", SHAPES + TILES, ids=lambda s: "x".join(map(str, s)))
 def test_small_layers_match_the_oracle(shape):
     n, h, w, cin, cout, kh, kw, s, pad = shape
     assert is_small(*shape, lce.OUT_INT32)
