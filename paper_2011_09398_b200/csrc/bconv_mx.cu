@@ -60,6 +60,7 @@
 #include <string.h>
 
 #include "common.cuh"
+#include "mx_columns.cuh"
 #include "mx_common.cuh"
 
 namespace lce {
@@ -70,7 +71,7 @@ constexpr int kLoaders = 256;                                // warps 16-23
 constexpr int kMxThreads = kFinishers + kLoaders + 64;       // + MMA issuer warp + weight producer warp
 constexpr int kIssuerWarp = (kFinishers + kLoaders) / 32;
 constexpr int kProducerTid = (kIssuerWarp + 1) * 32;
-constexpr int kColGroups = kFinishers / 128;                 // finisher warps per TMEM lane quarter
+static_assert(kColGroups == kFinishers / 128, "finisher warps per TMEM lane quarter");
 constexpr int kMaxNt = 224;                                  // tile width (positions); two accumulators + scales fit 512 columns
 constexpr uint32_t kD1Col = 240;                             // TMEM column of the second accumulator buffer
 constexpr uint32_t kSfaCol = 480, kSfbCol = 496;             // block scales (all 1.0) of the A / B operand
@@ -194,9 +195,6 @@ struct MxParams {
     uint16_t tap_rows[kMaxTaps];           // first row of a tap's words in a position buffer, taps in the order of mx_word
     int32_t dup_log2;        // log2 of the copies of the channel block in the 128 rows: 1 for out_c <= 64, 2 for out_c <= 32, else 0
 };
-
-// n / d for 0 <= n < 2^31 with (mul, sh) from the host: floor(n * mul / 2^sh), exact
-__device__ __forceinline__ int fast_div(int n, uint32_t mul, uint32_t sh) { return (int)(((uint64_t)(uint32_t)n * mul) >> sh); }
 
 // ---- loaders --------------------------------------------------------------------------------------------
 // A grid position as image, grid row inside the image and grid column; a thread's positions advance by a few
@@ -674,13 +672,7 @@ __device__ __forceinline__ uint32_t warp_transpose32(uint32_t m, const Transpose
 //
 // What a finisher warp needs for every tile, worked out once before its tile loop (divisions and
 // kernel-parameter reads per tile cost a third of the warp's instructions when they sat in the epilogue).
-// TMEM lane quarter of the warp = warp % 4; with few output channels the 128 rows hold `dup` copies of
-// the channel block, and the warps of copy `sub` take other columns than those of copy 0, so that no
-// finisher warp is idle.
-struct MxFin {
-    int Nt, n_chunks;        // tile width; 32-column chunks of a tile
-    int group, n_groups;     // this warp takes chunks group, group + n_groups, ...
-    int last_chunk;          // its last one (-1: none: nothing to read for this warp)
+struct MxFin : MxColumns, MxGrid {
     uint32_t lane_off;       // TMEM lane offset of its quarter
     float minus_thr, mult, bias;  // this lane's channel: minus its threshold (inf if it does not exist), multiplier, bias
     int cout, cow;
@@ -689,8 +681,6 @@ struct MxFin {
     const float *resp;       // shortcut tensor at this lane's channel, or null
     uint32_t *packp;         // re-quantised copy at this warp's channel word, or null
     bool relu, write_float;
-    int N, OH, OW, Wg, Hg;   // position -> output pixel
-    uint32_t Wg_mul, Wg_sh, Hg_mul, Hg_sh;
     int lane_step;           // from lane_positions of the first chunk to that of the second
     int32_t *positions;      // shared memory: output pixels or offsets of the two chunks' positions (one array per warp)
     const int32_t *lane_positions;  // the same for this lane; a row of -1 if its channel does not exist
@@ -699,16 +689,9 @@ struct MxFin {
 __device__ __forceinline__ MxFin mx_fin_context(const MxParams &p, int32_t *sPix, int fw, int lane, int ch0)
 {
     MxFin f;
-    const int quarter = fw & 3, dl = p.dup_log2;                    // dup = 1 << dl copies of the channel block
-    const int cq = quarter & ((4 >> dl) - 1), sub = quarter >> (2 - dl);
-    const int channel = ch0 + cq * 32 + lane;
-    f.Nt = p.Nt;
-    f.n_chunks = (p.Nt + 31) >> 5;
-    f.group = ((fw >> 2) << dl) + sub;
-    f.n_groups = kColGroups << dl;                                   // 4, 8 or 16
-    const bool real = ch0 + cq * 32 < p.Cout && f.group < f.n_chunks;
-    f.last_chunk = real ? f.group + ((f.n_chunks - 1 - f.group) & ~(f.n_groups - 1)) : -1;
-    f.lane_off = (uint32_t)(quarter * 32) << 16;
+    mx_columns(f, p.Nt, p.Cout, ch0, p.dup_log2, fw);
+    const int cq = f.word, channel = ch0 + cq * 32 + lane;
+    f.lane_off = (uint32_t)((fw & 3) * 32) << 16;
     const bool ch_ok = channel < p.Cout;
     // this lane's constants straight from global memory (constants of the model, never the previous kernel's
     // output): their latency passes while the first tile is being staged
@@ -733,16 +716,6 @@ __device__ __forceinline__ MxFin mx_fin_context(const MxParams &p, int32_t *sPix
     f.lane_step = ch_ok ? 32 : 0;
     f.lane_positions = ch_ok ? f.positions : sPix + 2 * kFinishers;
     return f;
-}
-
-// Output pixel of this lane's position of a tile's chunk, -1 where the position is no output.  The finishers work it out
-// themselves, before the accumulator is ready; as a table written by the loaders it was on those warps' critical chain.
-__device__ __forceinline__ int mx_out_pixel(const MxFin &f, int tile, int c0, int lane)
-{
-    const int q = tile * f.Nt + c0 + lane;
-    const int row = fast_div(q, f.Wg_mul, f.Wg_sh), c = q - row * f.Wg;
-    const int n = fast_div(row, f.Hg_mul, f.Hg_sh), r = row - n * f.Hg;
-    return c0 + lane < f.Nt && n < f.N && r < f.OH && c < f.OW ? (n * f.OH + r) * f.OW + c : -1;
 }
 
 // The warp has read its last columns of the accumulator
@@ -937,9 +910,9 @@ __device__ __forceinline__ bool mx_finish_tiles(const MxParams &p, const MxFin &
     for (int st = first_tile; st < n_super; st += tile_step) {
         for (int tile = st * T; tile < st * T + T && tile < n_tiles; ++tile, ++it) {
             const int buf = it & 1;
-            // what does not depend on the accumulator, before it is there
-            const int pix = mx_out_pixel(f, tile, f.group * 32, lane);
-            const int pix2 = f.last_chunk > f.group ? mx_out_pixel(f, tile, (f.group + f.n_groups) * 32, lane) : -1;
+            // what does not depend on the accumulator, before it is there (the pixels are worked out here: as a table written by
+            // the loaders they were on those warps' critical chain)
+            const int pix = mx_chunk_pixel(f, f, tile, 0, lane), pix2 = mx_chunk_pixel(f, f, tile, 1, lane);
             float r[32];
             if (MODE != EPI_BITS) mx_share_positions(f, MODE == EPI_FLOAT_FUSED && pix >= 0 ? pix * f.cout : pix, MODE == EPI_FLOAT_FUSED && pix2 >= 0 ? pix2 * f.cout : pix2, lane);
             if (MODE == EPI_FLOAT_FUSED) mx_shortcut<RES>(f, f.positions, r);

@@ -7,7 +7,7 @@ import torch
 
 import oracle
 import paper_2011_09398_b200 as lce
-from gpu_util import run_bconv, to_dev, to_dev_words, words_to_host
+from gpu_util import guarded, guards_intact, run_bconv, to_dev, to_dev_words, words_to_host
 
 pytestmark = pytest.mark.gpu
 
@@ -72,4 +72,36 @@ def test_fused_words_of_special_values(n, h, w, c):
                 np.testing.assert_array_equal(words_to_host(words), oracle.bitpack(y))
                 if floats:
                     np.testing.assert_array_equal(out.cpu().numpy(), y)  # NaN equal to NaN
+    assert lce.lce_device_status() == 0
+
+
+# n, h, w, cin, cout, k, stride: channel blocks with one, two or three words missing, one tile and several tiles a CTA
+RAGGED_BLOCKS = [(40, 28, 27, 64, 96, 3, 1), (30, 16, 15, 96, 160, 3, 1), (2, 9, 10, 64, 192, 3, 2), (70, 14, 13, 40, 224, 1, 1), (1, 5, 5, 32, 96, 5, 1)]
+
+
+@pytest.mark.parametrize("shape", RAGGED_BLOCKS, ids=lambda s: "x".join(map(str, s)))
+def test_fused_on_channel_blocks_that_are_partly_empty(shape):
+    """Shortcut add, re-quantised copy and float output, each there and not there: exact, and nothing written beside them."""
+    n, h, w, cin, cout, k, s = shape
+    rng = np.random.default_rng(sum(shape))
+    a = (2 * rng.integers(0, 2, size=(n, h, w, cin)) - 1).astype(np.int8)
+    wt = (2 * rng.integers(0, 2, size=(cout, k, k, cin)) - 1).astype(np.int8)
+    acc = oracle.bconv2d_acc(a, wt, (s, s), lce.PAD_SAME_ONE)
+    mult, bias = rng.uniform(0.5, 1.5, cout).astype(np.float32), rng.standard_normal(cout).astype(np.float32)
+    residual = (rng.standard_normal(acc.shape) * np.sqrt(k * k * cin)).astype(np.float32)
+    desc = lce.make_desc(n, h, w, cin, cout, (k, k), (s, s), out_type=lce.OUT_FLOAT32, kernel_choice=lce.KERNEL_TENSOR, weights_packed=1)
+    x, weights = to_dev_words(oracle.bitpack_pm1(a)), lce.lce_bconv2d_pack_weights(desc, to_dev_words(oracle.bitpack_pm1(wt)))
+    plain = oracle.transform_float(acc, mult, bias)
+    for shortcut in (None, residual):
+        y = plain if shortcut is None else oracle.add_f32(plain, shortcut)
+        for floats, packed in ((True, False), (False, True), (True, True)):
+            whole_f, out = guarded(acc.shape, torch.float32, 12345.0)
+            whole_w, words = guarded(acc.shape[:3] + (cout // 32,), torch.int32, 0x5A5A5A5A)
+            lce.lce_bconv2d_fused(desc, x, weights, to_dev(mult), to_dev(bias), None if shortcut is None else to_dev(shortcut),
+                                  out if floats else None, words if packed else None)
+            if floats:
+                np.testing.assert_array_equal(out.cpu().numpy(), y)
+            if packed:
+                np.testing.assert_array_equal(words_to_host(words), oracle.bitpack(y))
+            assert guards_intact(whole_f, 12345.0) and guards_intact(whole_w, 0x5A5A5A5A)
     assert lce.lce_device_status() == 0
