@@ -1,7 +1,10 @@
 // LceBMaxPool2d (paper Section 3.2: max-pool on packed bits is the bitwise AND of the window,
 // because a 0 bit is +1 and max(sign X) = sign(max X)) and the fp32 residual add that the
 // shortcut pattern of Section 5.3 places between a float-output conv and the next LceQuantize.  Launched as
-// programmatic dependents: they wait for the previous kernel before their first access.
+// programmatic dependents: they wait for the previous kernel before their first access.  They do not let their own
+// dependents start early: a convolution reads its weights and per-channel arrays before it waits, and may take those from a
+// kernel that is still running when the pool or the add starts to wait for it (releasing them at the pool's entry was no
+// faster either: residual stack, 128 images 214.6 us, 213.6 without).
 #include "common.cuh"
 
 #include <string.h>
@@ -46,7 +49,6 @@ __global__ void __launch_bounds__(kThreads) bmaxpool_kernel(const __grid_constan
 {
     using V = typename Words<VEC>::type;
     const int32_t cv = p.Cw / VEC, H = p.H, W = p.W;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const V *const in = reinterpret_cast<const V *>(p.in);
     V *const out = reinterpret_cast<V *>(p.out);

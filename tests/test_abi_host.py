@@ -28,6 +28,19 @@ def declared_symbols(header):
     return sorted(set(re.findall(r"\b(lce_[a-z0-9_]+)\s*\(", text)))
 
 
+def test_only_the_kernels_the_header_names_release_their_dependents_early():
+    """A convolution reads per-channel arrays before it waits for the kernel in front of it, so it matters to callers which
+    kernels let that happen: "this library's convolution kernels and lce_bitpack do"."""
+    header = (ROOT / "include" / "lce.h").read_text().replace("\n *", "")
+    assert "this library's convolution kernels and lce_bitpack do" in re.sub(r"\s+", " ", header)
+    early = set()
+    for source in (ROOT / "paper_2011_09398_b200" / "csrc").glob("*.cu*"):
+        for kernel, body in re.findall(r"__global__[^;{]*?(\w+_kernel)\(.*?\)\s*\{(.*?)\n\}", source.read_text(), flags=re.S):
+            if "griddepcontrol.launch_dependents" in body:
+                early.add(kernel)
+    assert early and all(k.startswith(("bconv", "bitpack_")) for k in early), early
+
+
 def test_every_declared_symbol_is_exported(lib):
     names = declared_symbols("lce.h")
     assert {"lce_bitpack", "lce_bconv2d", "lce_bmaxpool", "lce_device_status_reset"} <= set(names)

@@ -83,3 +83,28 @@ def test_add_from_the_last_element_to_the_first(n):
     np.testing.assert_array_equal(out.cpu().numpy(), oracle.add_f32(a, b))
     ad = to_dev(a)
     np.testing.assert_array_equal(lce.lce_add_f32(ad, to_dev(b), ad).cpu().numpy(), oracle.add_f32(a, b))  # onto an operand
+
+
+@pytest.mark.parametrize("kernel_choice", [lce.KERNEL_AUTO, lce.KERNEL_TENSOR])
+def test_a_pool_between_a_convolution_and_the_reader_of_its_output(kernel_choice):
+    """A convolution may take its biases from what a convolution before the pool wrote: the pool's dependents start when it is
+    through, and so is everything in front of it."""
+    rng = np.random.default_rng(12)
+    x = (2 * rng.integers(0, 2, size=(16, 56, 56, 64)) - 1).astype(np.int8)
+    w = (2 * rng.integers(0, 2, size=(64, 3, 3, 64)) - 1).astype(np.int8)
+    mult, bias = rng.uniform(0.5, 1.5, 64).astype(np.float32), rng.standard_normal(64).astype(np.float32)
+    long_desc = lce.make_desc(16, 56, 56, 64, 64, out_type=lce.OUT_FLOAT32, kernel_choice=lce.KERNEL_DIRECT)
+    desc = lce.make_desc(1, 14, 14, 64, 64, out_type=lce.OUT_FLOAT32, kernel_choice=kernel_choice, weights_packed=1)
+    words = to_dev(oracle.bitpack_pm1(w).view(np.int32))
+    packed, xs, mult_d, bias_d = lce.lce_bconv2d_pack_weights(desc, words), to_dev(oracle.bitpack_pm1(x).view(np.int32)), to_dev(mult), to_dev(bias)
+    small, pooled = xs[:1, :14, :14].contiguous(), torch.empty((1, 7, 7, 2), dtype=torch.int32, device=DEV)
+    tensor_desc = lce.make_desc(16, 56, 56, 64, 64, out_type=lce.OUT_FLOAT32, kernel_choice=lce.KERNEL_TENSOR, weights_packed=1)
+    tensor_packed = lce.lce_bconv2d_pack_weights(tensor_desc, words)
+    first = oracle.transform_float(oracle.bconv2d_acc(x[-1:], w), mult, bias)
+    want = oracle.transform_float(oracle.bconv2d_acc(x[:1, :14, :14], w), mult, first[0, -1, -1])
+    for d, weights in ((long_desc, words), (tensor_desc, tensor_packed)) * 5:
+        biases = torch.full((16, 56, 56, 64), 1e9, device=DEV)
+        lce.lce_bconv2d(d, xs, weights, mult_d, bias_d, None, biases)
+        lce.lce_bmaxpool(small, 64, out=pooled)
+        got = lce.lce_bconv2d(desc, small, packed, mult_d, biases[-1, -1, -1])
+        np.testing.assert_array_equal(got.cpu().numpy(), want)
