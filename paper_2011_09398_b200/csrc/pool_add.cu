@@ -76,10 +76,12 @@ __global__ void __launch_bounds__(kThreads) bmaxpool_kernel(const __grid_constan
 template <int VEC>
 lce_status launch_pool(PoolParams p, int32_t batch, cudaStream_t s)
 {
-    // so many rows at a time that a launch has fewer than 2^31 vectors (and a step of its grid more)
-    const int64_t row = (int64_t)p.OW * (p.Cw / VEC), step = 148 * 16 * kThreads, rows = (int64_t)batch * p.OH;
-    if (row >= (1ll << 31) - step) return LCE_ERR_UNSUPPORTED;
-    const int64_t most = ((1ll << 31) - step) / row;
+    // so many rows at a time that a launch has fewer than 2^31 vectors (a thread's index, a step of the grid more at the end of
+    // its loop, is unsigned)
+    constexpr int64_t kMost = (1ll << 31) - 1;
+    const int64_t row = (int64_t)p.OW * (p.Cw / VEC), rows = (int64_t)batch * p.OH;
+    if (row > kMost) return LCE_ERR_UNSUPPORTED;
+    const int64_t most = kMost / row;
     fast_div_constants((uint32_t)(p.Cw / VEC), &p.by_cv.mul, &p.by_cv.sh);
     fast_div_constants((uint32_t)p.OW, &p.by_ow.mul, &p.by_ow.sh);
     fast_div_constants((uint32_t)p.OH, &p.by_oh.mul, &p.by_oh.sh);

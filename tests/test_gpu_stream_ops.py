@@ -73,6 +73,12 @@ def test_maxpool_matches_the_oracle(n, h, w, c, pool, stride, pad, offset):
     np.testing.assert_array_equal(words_to_host(out), want)
 
 
+def test_maxpool_of_a_row_of_almost_2_to_the_31_words():
+    """A launch's last indices: threads step past the row's end, and past 2^31."""
+    x = torch.randint(-2 ** 31, 2 ** 31, (1, 1, 2 ** 31 - 4096, 1), dtype=torch.int32, device=DEV)
+    assert torch.equal(lce.lce_bmaxpool(x, 32, (1, 1), (1, 1), lce.PAD_VALID), x)
+
+
 @pytest.mark.parametrize("n", [1, 3, 4, 7, 1023, 4 * 148 * 8 * 256 + 5])
 def test_add_from_the_last_element_to_the_first(n):
     rng = np.random.default_rng(n)
