@@ -255,8 +255,8 @@ extern "C" lce_status lce_bitpack(const float *x, uint32_t *out, int64_t rows, i
     const int max_blocks = 148 * 8 * 4;
     if (channels % 32 == 0 && aligned(out, 16)) {
         const int64_t passes = (n_words + kWordsPerWarpPass - 1) / kWordsPerWarpPass;
-        // A tensor that fits in the L2 stays there: it is a shortcut's operand or comes back as one (51 MB again and again 5.7 ->
-        // 4.8 us); a larger one would only push out what is there (205 MB: 30.1 us, 31.8 if kept; the residual stack 217 and 225).
+        // A tensor that fits in the L2 stays there: it is a shortcut's operand or comes back as one (51 MB, quantized and then
+        // added to another tensor, new ones each time: 30.7 -> 27.5 us); a larger one would only push out what is there (205 MB: 30.1 us, 31.8 if kept; the residual stack 217 and 225).
         const auto kernel = n_words * 128 <= (64ll << 20) ? bitpack_aligned_kernel<true> : bitpack_aligned_kernel<false>;
         return launch_dependent(kernel, dim3(grid_for(passes, kPackThreads / 32, max_blocks)), kPackThreads, 0, s, x, out, n_words);
     }

@@ -97,17 +97,18 @@ lce_status launch_pool(PoolParams p, int32_t batch, cudaStream_t s)
     return LCE_OK;
 }
 
-// From the last element to the first: what came before in a network (LceQuantize of one of the operands, or the convolution
-// that wrote it) went through its tensor forwards, so the end of it is still in the L2.  For the same reason
-// the other operand is not kept.  Quantize, pool, dequantize and add of one 205 MB tensor 172.2 -> 167.6 us (a quarter of
-// it: 46.8 -> 42.8).
+// HBM-bound.  Forwards, both operands streamed: what is left in the L2 is the sum, which LceQuantize reads next (Section 5.3).
+// From the last element to the first with the first operand kept, the add was faster only where the same tensors came
+// again and again (quantize, pool, dequantize and add of one 205 MB tensor 164.7 us, 169.0 as it is); with new ones each time it
+// was slower: the four 170.0 us against 169.4 (51 MB 46.5 and 46.2), add and quantize of the sum 126.5 against 121.7 (103 MB 62.4
+// and 59.1; 13 MB the other way, 8.4 and 8.7).
 __global__ void __launch_bounds__(kThreads)
 add_f32_vec4_kernel(const float4 *a, const float4 *b, float4 *out, int64_t n4)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n4; i += (int64_t)gridDim.x * kThreads) {
-        const float4 u = a[n4 - 1 - i], v = __ldcs(b + n4 - 1 - i);
-        out[n4 - 1 - i] = make_float4(__fadd_rn(u.x, v.x), __fadd_rn(u.y, v.y), __fadd_rn(u.z, v.z), __fadd_rn(u.w, v.w));
+        const float4 u = __ldcs(a + i), v = __ldcs(b + i);
+        out[i] = make_float4(__fadd_rn(u.x, v.x), __fadd_rn(u.y, v.y), __fadd_rn(u.z, v.z), __fadd_rn(u.w, v.w));
     }
 }
 

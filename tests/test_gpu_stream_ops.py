@@ -80,7 +80,7 @@ def test_maxpool_of_a_row_of_almost_2_to_the_31_words():
 
 
 @pytest.mark.parametrize("n", [1, 3, 4, 7, 1023, 4 * 148 * 8 * 256 + 5])
-def test_add_from_the_last_element_to_the_first(n):
+def test_add_with_and_without_a_rest_onto_another_tensor_and_onto_an_operand(n):
     rng = np.random.default_rng(n)
     a, b = (rng.standard_normal(n).astype(np.float32) for _ in range(2))
     whole, out = guarded((n,), torch.float32, 9.0)
