@@ -119,7 +119,8 @@ lce_status lce_bconv2d_out_shape(const lce_bconv2d_desc *desc, int32_t *out_h, i
  * aligned (out_c a multiple of 4); a buffer that is only 4-byte aligned is served by the direct kernel
  * under AUTO.  The weights and per-channel arrays are constants of the model: the kernels read them
  * before they wait for the stream's previous kernel where that kernel lets its dependents start early
- * (programmatic dependent launch; this library's convolution kernels and lce_bitpack do), so they must
+ * (programmatic dependent launch; this library's convolution kernels, lce_bitpack and lce_bmaxpool do, the last
+ * one when everything in front of it is complete), so they must
  * not be the output of such a kernel that may still be running (plain weights may: kernels read those after
  * the wait).  What lce_bconv2d_pack_weights, a copy or an ordinary kernel wrote earlier on the stream is
  * complete before this call's kernel is scheduled.

@@ -1,10 +1,7 @@
 // LceBMaxPool2d (paper Section 3.2: max-pool on packed bits is the bitwise AND of the window,
 // because a 0 bit is +1 and max(sign X) = sign(max X)) and the fp32 residual add that the
 // shortcut pattern of Section 5.3 places between a float-output conv and the next LceQuantize.  Launched as
-// programmatic dependents: they wait for the previous kernel before their first access.  They do not let their own
-// dependents start early: a convolution reads its weights and per-channel arrays before it waits, and may take those from a
-// kernel that is still running when the pool or the add starts to wait for it (releasing them at the pool's entry was no
-// faster either: residual stack, 128 images 214.6 us, 213.6 without).
+// programmatic dependents: they wait for the previous kernel before their first access.
 #include "common.cuh"
 
 #include <string.h>
@@ -50,6 +47,10 @@ __global__ void __launch_bounds__(kThreads) bmaxpool_kernel(const __grid_constan
     using V = typename Words<VEC>::type;
     const int32_t cv = p.Cw / VEC, H = p.H, W = p.W;
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    // Behind the wait: the next convolution reads its per-channel arrays before it waits, and those may come from a kernel in
+    // front of the pool, which is complete from here on.  Residual stack, 128 images of 56x56 / 3 of 35x35: released here 212.0 /
+    // 47.6 us, at the entry 212.9 / 47.0, not at all 212.1 / 49.3.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const V *const in = reinterpret_cast<const V *>(p.in);
     V *const out = reinterpret_cast<V *>(p.out);
     for (uint32_t e = blockIdx.x * kThreads + threadIdx.x; e < (uint32_t)p.total; e += gridDim.x * kThreads) {

@@ -28,17 +28,19 @@ def declared_symbols(header):
     return sorted(set(re.findall(r"\b(lce_[a-z0-9_]+)\s*\(", text)))
 
 
-def test_only_the_kernels_the_header_names_release_their_dependents_early():
+def test_kernels_that_release_their_dependents_early_are_those_the_header_names():
     """A convolution reads per-channel arrays before it waits for the kernel in front of it, so it matters to callers which
-    kernels let that happen: "this library's convolution kernels and lce_bitpack do"."""
-    header = (ROOT / "include" / "lce.h").read_text().replace("\n *", "")
-    assert "this library's convolution kernels and lce_bitpack do" in re.sub(r"\s+", " ", header)
-    early = set()
+    kernels let that happen, and that a pool does so only when what is in front of it is complete."""
+    header = re.sub(r"[\s*]+", " ", (ROOT / "include" / "lce.h").read_text())
+    assert "this library's convolution kernels, lce_bitpack and lce_bmaxpool do, the last one when everything in front of it is complete" in header
+    at_entry, behind_wait = set(), set()
     for source in (ROOT / "paper_2011_09398_b200" / "csrc").glob("*.cu*"):
         for kernel, body in re.findall(r"__global__[^;{]*?(\w+_kernel)\(.*?\)\s*\{(.*?)\n\}", source.read_text(), flags=re.S):
             if "griddepcontrol.launch_dependents" in body:
-                early.add(kernel)
-    assert early and all(k.startswith(("bconv", "bitpack_")) for k in early), early
+                before = body[:body.index("griddepcontrol.launch_dependents")]
+                (behind_wait if "griddepcontrol.wait" in before else at_entry).add(kernel)
+    assert at_entry and all(k.startswith(("bconv", "bitpack_")) for k in at_entry), at_entry
+    assert behind_wait == {"bmaxpool_kernel"}
 
 
 def test_every_declared_symbol_is_exported(lib):

@@ -93,8 +93,8 @@ def test_add_with_and_without_a_rest_onto_another_tensor_and_onto_an_operand(n):
 
 @pytest.mark.parametrize("kernel_choice", [lce.KERNEL_AUTO, lce.KERNEL_TENSOR])
 def test_a_pool_between_a_convolution_and_the_reader_of_its_output(kernel_choice):
-    """A convolution may take its biases from what a convolution before the pool wrote: the pool's dependents start when it is
-    through, and so is everything in front of it."""
+    """A convolution may take its biases from what a convolution before the pool wrote: the pool's dependents start when
+    everything in front of the pool is complete."""
     rng = np.random.default_rng(12)
     x = (2 * rng.integers(0, 2, size=(16, 56, 56, 64)) - 1).astype(np.int8)
     w = (2 * rng.integers(0, 2, size=(64, 3, 3, 64)) - 1).astype(np.int8)
