@@ -823,14 +823,16 @@ __device__ __forceinline__ void mx_epilogue_values(const MxFin &f, uint32_t tmem
 // re-quantised copy is the sign bits and the bit transpose of the bit-packed form; y + 0 makes -0.0 and NaN, which
 // quantize to 0 bits, positive (PTX: a NaN result has no sign).
 // Positions come as offsets of elements: multiplying pixels by the channels at each use took 36.9 us on the 56x56x64 block at 128
-// images, 33.6 now (40.6 with ballots and loads behind the wait); the plain float form, which has registers to spare, is
+// images, 34.5 now (40.6 with ballots and loads behind the wait); the plain float form, which has registers to spare, is
 // faster with pixels (13.9 us against 14.4 on 56x56x64, 64 images).
-template <bool RES>
-__device__ __forceinline__ void mx_shortcut(const MxFin &f, const int32_t *offsets, float (&r)[32])
+// With all three parts there are registers for 16 values ahead only, those of the next half chunk: 32 spilled into the loop, 78.5 us
+// on that block with everything, 57.5 now (58.0 with no value before the wait); shortcut and float output 51.3 and 49.3.
+template <bool RES, int AHEAD>
+__device__ __forceinline__ void mx_shortcut(const MxFin &f, const int32_t *offsets, float (&r)[AHEAD])
 {
     if (!RES) return;
 #pragma unroll
-    for (int j4 = 0; j4 < 32; j4 += 4) {
+    for (int j4 = 0; j4 < AHEAD; j4 += 4) {
         const int4 o4 = *reinterpret_cast<const int4 *>(offsets + j4);  // the same for every lane
         const int o[4] = {o4.x, o4.y, o4.z, o4.w};
 #pragma unroll
@@ -840,8 +842,8 @@ __device__ __forceinline__ void mx_shortcut(const MxFin &f, const int32_t *offse
     }
 }
 
-template <bool RES, bool PACK, bool WRITE_FLOAT>
-__device__ __forceinline__ void mx_epilogue_fused(const MxFin &f, const Transpose32 &tr, uint32_t tmem_d, float (&r)[32], int lane, uint64_t *empty_d)
+template <bool RES, bool PACK, bool WRITE_FLOAT, int AHEAD>
+__device__ __forceinline__ void mx_epilogue_fused(const MxFin &f, const Transpose32 &tr, uint32_t tmem_d, float (&r)[AHEAD], int lane, uint64_t *empty_d)
 {
     // which of the three parts (shortcut add, re-quantised copy, float output) a launch has is a template
     // argument: a test of a pointer per position turns the unrolled block below into branchy code that
@@ -851,7 +853,7 @@ __device__ __forceinline__ void mx_epilogue_fused(const MxFin &f, const Transpos
     for (int ck = f.group; ck <= f.last_chunk; ck += f.n_groups) {
         const int c0 = ck * 32;
         const bool full = c0 + 32 <= f.Nt;  // otherwise 16 columns, the tile's last
-        if (ck != f.group) mx_shortcut<RES>(f, f.positions + 32, r);
+        if (AHEAD == 32 && ck != f.group) mx_shortcut<RES>(f, f.positions + 32, r);
         uint32_t m = 0u;
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
@@ -869,12 +871,16 @@ __device__ __forceinline__ void mx_epilogue_fused(const MxFin &f, const Transpos
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         float y = __fmaf_rn(fmaxf(v[j4 + u], floor_v), f.mult, f.bias);
-                        if (RES) y = __fadd_rn(y, r[half * 16 + j4 + u]);
+                        if (RES) y = __fadd_rn(y, r[(half * 16 + j4 + u) & (AHEAD - 1)]);
                         if (WRITE_FLOAT) {
                             if (o[u] >= 0) f.outp[o[u]] = y;
                         }
                         if (PACK) v[j4 + u] = y;
                     }
+                }
+                if (AHEAD == 16) {  // the next 16 columns, while the signs of these are collected
+                    if (half == 0 && full) mx_shortcut<RES>(f, f.positions + (ck == f.group ? 16 : 48), r);
+                    else if (ck != f.last_chunk) mx_shortcut<RES>(f, f.positions + 32, r);
                 }
                 if (PACK) {
                     uint32_t m0 = 0u, m1 = 0u;
@@ -913,7 +919,7 @@ __device__ __forceinline__ bool mx_finish_tiles(const MxParams &p, const MxFin &
             // what does not depend on the accumulator, before it is there (the pixels are worked out here: as a table written by
             // the loaders they were on those warps' critical chain)
             const int pix = mx_chunk_pixel(f, f, tile, 0, lane), pix2 = mx_chunk_pixel(f, f, tile, 1, lane);
-            float r[32];
+            float r[RES && PACK && WRITE_FLOAT ? 16 : 32];
             if (MODE != EPI_BITS) mx_share_positions(f, MODE == EPI_FLOAT_FUSED && pix >= 0 ? pix * f.cout : pix, MODE == EPI_FLOAT_FUSED && pix2 >= 0 ? pix2 * f.cout : pix2, lane);
             if (MODE == EPI_FLOAT_FUSED) mx_shortcut<RES>(f, f.positions, r);
             // the warp goes on together (its transform uses warp-wide shuffles)
