@@ -65,10 +65,11 @@ __global__ void __launch_bounds__(kThreads) bmaxpool_kernel(const __grid_constan
         }
         V acc;
         memset(&acc, 0xff, sizeof(acc));
-        for (int32_t ky = 0; ky < p.PH; ++ky) {
-            if (iy0 + ky < 0 || iy0 + ky >= H) continue;
-            for (int32_t kx = 0; kx < p.PW; ++kx)
-                if (ix0 + kx >= 0 && ix0 + kx < W) acc = both(acc, __ldg(at + ((int64_t)ky * W + kx) * cv));
+        // the window's part inside the image, so that nothing is tested between the loads
+        const int32_t ky1 = min(p.PH, H - iy0), kx0 = max(0, -ix0), kx1 = min(p.PW, W - ix0);
+        for (int32_t ky = max(0, -iy0); ky < ky1; ++ky) {
+            const V *tap = at + ((int64_t)ky * W + kx0) * cv;
+            for (int32_t kx = kx0; kx < kx1; ++kx, tap += cv) acc = both(acc, __ldg(tap));
         }
         out[e] = acc;
     }
