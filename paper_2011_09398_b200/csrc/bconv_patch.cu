@@ -262,6 +262,10 @@ bconv_patch_bits_kernel(const PatchParams p, int packed)
         const int ones = __popc(patch);
         const uint32_t operand = COUNTED ? patch | (uint32_t)ones << 27 : patch;
         const uint32_t pixel = m0 + (g >> 1) * 8 + 2 * q + (g & 1);
+        // Several words one at a time: unrolled, they spill, and two and three words were slower than before the sums of a lane were
+        // transposed at once (224x224x2 -> 40 at stride 2, 16 images 8.4 -> 8.7 us, now 8.0; 56x56x3 -> 96, 64 images 10.05 ->
+        // 10.25, 9.6; 224x224x3 -> 64 at stride 2 18.6 -> 17.5, 16.5; 112x112x1 -> 64, 5x5 38.3 -> 36.1, 36.6).
+#pragma unroll 1
         for (int wd = 0; wd < (ONE_WORD ? 1 : p.Cow); ++wd) {
             if (!ONE_WORD) { w0 = slots[wd * 96]; w1 = slots[wd * 96 + 32]; c = slots[wd * 96 + 64]; compare_operands(c, c0, c1); }
             // this lane's four neighbouring channels of the pixels 8 i + 2 q and 8 i + 2 q + 1, a nibble of sign bits each
