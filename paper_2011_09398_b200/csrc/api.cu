@@ -56,12 +56,13 @@ WeightParts weight_parts(const ConvGeom &g)
 enum KernelPick { PICK_NONE = 0, PICK_DIRECT, PICK_PATCH, PICK_TILED, PICK_TENSOR, PICK_SMALL };
 
 // Which kernel weights packed at load time go to: the one whose estimated time is the shorter.  The estimates (us) were
-// fitted to 180 layers of 2^26 - 2^31 binary MACs, 1x1 - 5x5, 32 - 512 channels, strides 1 and 2 (10% rms each): the
+// fitted to 180 layers of 2^26 - 2^31 binary MACs, 1x1 - 5x5, 32 - 512 channels, strides 1 and 2, as the kernels were then (10%
+// rms each; on 180 others of that range, as they are now, 14% and 11%): the
 // latency kernel pays per output and per 128-deep step of an output, the tensor-core kernel a start-up and the clocks its
 // plan predicts; staging the four phase grids of a stride-2 layer word by word grows with the square of the depth (fewer
-// positions fit a tile).  The slower of the two was picked in 7 of the 180, by 13% on average.  One image of 14x14x64 is
-// 1.7 on the latency kernel and 3.9 on the tensor cores; 21 images of 14x14x256, 1x1 (2^28.0), 5.9 and 4.1; one of
-// 56x56x512, stride 2 (2^30.8), 9.9 and 13.4.  The XOR/POPC kernel was ahead of both in two of the 180.
+// positions fit a tile).  Of those 180 others the slower of the two is picked in 10, by 10% on average and 26% at most.  One
+// image of 14x14x64 is 1.8 on the latency kernel and 3.6 on the tensor cores; 21 images of 14x14x256, 1x1 (2^28.0), 5.7 and
+// 4.0; one of 56x56x512, stride 2 (2^30.8), 9.9 and 12.5.  The XOR/POPC kernel is ahead of both in one of the 180.
 // Where one of the two does not cover the layer the other competes with the integer kernels: from 2^28 (weights
 // resident) or 2^29 MACs (streamed) the tensor cores are ahead, up to 2^29 and 600 CTAs the latency kernel is.
 // `extra`: what the tensor-core kernel costs besides.  PICK_NONE: neither.

@@ -434,9 +434,11 @@ constexpr size_t kSmallSmem = 100 * 1024;  // two CTAs per SM, so that a CTA of 
 // 1 .. 16 channel blocks, 1 .. 36 steps): the smallest tile that leaves few enough CTAs (more than two or three
 // per SM only repeat the set-up), 8 warps, and as many slices as give every warp a job.  Jobs of 16 pixels use a
 // weight operand twice and win in tiles of 32 pixels and more, and where the depth gives enough steps to share out (8 and
-// more).  With few steps (below 8, in tiles of 32 below 20: 10x10x192, 16 images, 14 steps 5.5 -> 5.1 us, 10x10x383, 17
-// images, 27 steps 5.5 -> 6.4) a second slice is enough in tiles of 16 and 32 pixels, even if half of the warps then have no
-// job: every job ends in 8 updates of shared sums.  One image of 56x56x64 (tiles of 32) 3.3 -> 2.8 us, of 56x56x64 -> 128 at
+// more).  With few steps (below 8, in tiles of 32 below 20) a second slice is enough in tiles of 16 and 32 pixels, even if half
+// of the warps then have no job: every job ends in 8 updates of shared sums.  The line at 20 is a compromise, not an edge.  Two
+// slices against four in tiles of 32, us at 14, 16, 18, 21, 23, 25, 27 and 30 steps: 10x10 -> 192, 16 images (300 CTAs) 4.9 /
+// 5.2, 5.6 / 5.6, 5.6 / 6.0, 6.6 / 7.0, 6.7 / 6.8, 7.5 / 7.8, 7.3 / 7.3, 8.6 / 8.7, and much the same with 265 CTAs;
+// 10x10 -> 109, 17 images (216 CTAs) 4.2 / 4.1, 4.7 / 4.4, 4.9 / 4.6, 5.0 / 5.4, 5.1 / 5.2, 5.6 / 5.9, 6.5 / 5.5, 7.3 / 6.6.  One image of 56x56x64 (tiles of 32) 3.3 -> 2.8 us, of 56x56x64 -> 128 at
 // stride 2 (16) 2.8 -> 2.5, three of 33x33x100 (32) 4.5 -> 4.2, 53 of 8x8x160, 1x1 (64) 4.1 -> 3.8.
 // Tiles of 64 pixels in more CTAs than fit at once do better with four warps each; of 16 pixels they do not (14x14x256,
 // three images 3.8 us, 4.9 with four).
