@@ -139,8 +139,9 @@ lce_status lce_bconv2d(const lce_bconv2d_desc *desc, const uint32_t *input, cons
  *   residual   fp32 [batch][oh][ow][out_c] or NULL       out_float fp32 same shape, or NULL
  *   out_packed uint32 [batch][oh][ow][ceil(out_c/32)] or NULL   (at least one output required)
  * The results are bit-identical to lce_bconv2d -> lce_add_f32 -> lce_bitpack run one after the
- * other.  Only shapes the tiled kernels cover (3x3 and 5x5 with equal strides of 1 or 2, 1x1) are accepted; others return
- * LCE_ERR_UNSUPPORTED. */
+ * other.  Accepted are the shapes the tiled kernels cover (3x3 and 5x5 with equal strides of 1 or 2, 1x1) and, on packed weights, with
+ * out_c a multiple of 32 and 16-byte aligned tensors, those of the tensor-core kernel where AUTO takes it or `kernel` names it;
+ * others return LCE_ERR_UNSUPPORTED. */
 lce_status lce_bconv2d_fused(const lce_bconv2d_desc *desc, const uint32_t *input, const uint32_t *weights,
                              const float *multiplier, const float *bias, const float *residual,
                              float *out_float, uint32_t *out_packed, void *stream);
