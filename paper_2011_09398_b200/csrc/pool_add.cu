@@ -66,11 +66,10 @@ __global__ void __launch_bounds__(kThreads) bmaxpool_kernel(const __grid_constan
         V acc;
         memset(&acc, 0xff, sizeof(acc));
         // the window's part inside the image, so that nothing is tested between the loads
-        const int32_t ky1 = min(p.PH, H - iy0), kx0 = max(0, -ix0), kx1 = min(p.PW, W - ix0);
-        for (int32_t ky = max(0, -iy0); ky < ky1; ++ky) {
-            const V *tap = at + ((int64_t)ky * W + kx0) * cv;
-            for (int32_t kx = kx0; kx < kx1; ++kx, tap += cv) acc = both(acc, __ldg(tap));
-        }
+        const int32_t ky0 = max(0, -iy0), kx0 = max(0, -ix0), rows = min(p.PH - ky0, H - max(0, iy0)), columns = min(p.PW - kx0, W - max(0, ix0));
+        const V *line = at + ((int64_t)ky0 * W + kx0) * cv;
+        for (int32_t y = 0; y < rows; ++y, line += (int64_t)W * cv)
+            for (int32_t x = 0; x < columns; ++x) acc = both(acc, __ldg(line + (int64_t)x * cv));
         out[e] = acc;
     }
 }

@@ -55,10 +55,10 @@ def test_weights_quantized_right_before_the_convolution(cin, k):
 
 
 # widths of 1, 2, 3, 4 and 6 words (vectors of one, two and four), windows inside and across the edge, buffers that are only
-# 4-byte aligned
+# 4-byte aligned; windows that reach past both edges and over whole images
 @pytest.mark.parametrize("offset", [0, 1, 2])
 @pytest.mark.parametrize("n,h,w,c,pool,stride,pad", [(3, 9, 7, 32, (2, 2), (2, 2), lce.PAD_VALID), (2, 8, 11, 50, (2, 2), (2, 2), lce.PAD_SAME_ONE), (5, 7, 6, 96, (2, 2), (1, 1), lce.PAD_SAME_ONE),
-                                                     (2, 13, 5, 128, (3, 2), (2, 3), lce.PAD_SAME_ONE), (1, 1, 1, 180, (2, 2), (2, 2), lce.PAD_SAME_ONE), (70, 56, 56, 64, (2, 2), (2, 2), lce.PAD_VALID)])
+                                                     (2, 13, 5, 128, (3, 2), (2, 3), lce.PAD_SAME_ONE), (1, 1, 1, 180, (2, 2), (2, 2), lce.PAD_SAME_ONE), (2, 5, 3, 96, (9, 11), (2, 2), lce.PAD_SAME_ONE), (3, 14, 14, 256, (14, 14), (14, 14), lce.PAD_VALID), (70, 56, 56, 64, (2, 2), (2, 2), lce.PAD_VALID)])
 def test_maxpool_matches_the_oracle(n, h, w, c, pool, stride, pad, offset):
     rng = np.random.default_rng(n * h + c)
     x = np.where(rng.random((n, h, w, c)) < 0.8, -1.0, 1.0).astype(np.float32)
