@@ -466,155 +466,36 @@ __device__ __forceinline__ bool elect_one()
     return pred != 0;
 }
 
-// N MMAs straight from a table of operand offsets, back to back in one block of code: the loads of the
-// block are independent, and between two MMAs there is nothing but the next descriptor's move.  The
-// issuing warp pays about 100 clocks per tcgen05.mma in its instruction stream, whether the instruction
-// is predicated off or not (measured), so blocks come in exact sizes (8, 4, 2, 1) instead of one
-// predicated block of eight.  The whole issuer warp runs this; only the elected lane issues.
-template <int N>
-__device__ __forceinline__ void mx_issue_block(uint32_t tmem_d, const uint2 *tbl, uint32_t a_base, uint32_t b_base, uint32_t desc_hi,
-                                               uint32_t idesc, uint32_t sfa, uint32_t sfb, uint32_t accumulate);
-template <>
-__device__ __forceinline__ void mx_issue_block<8>(uint32_t tmem_d, const uint2 *tbl, uint32_t a_base, uint32_t b_base, uint32_t desc_hi,
-                                                  uint32_t idesc, uint32_t sfa, uint32_t sfb, uint32_t accumulate)
+// One MMA, by one lane.  Descriptors: low words a and b, the same high word
+__device__ __forceinline__ void mx_mma(uint32_t tmem_d, uint32_t a, uint32_t b, uint32_t desc_hi, uint32_t idesc, uint32_t sfa, uint32_t sfb, bool accumulate)
 {
-    uint32_t a[8], b[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const uint2 o = tbl[k];
-        a[k] = a_base + o.x;
-        b[k] = b_base + o.y;
-    }
-    if (elect_one()) {
-        asm volatile(
-            "{\n\t.reg .pred pa, pt;\n\t.reg .b64 da, db;\n\t"
-            "setp.ne.b32 pa, %21, 0;\n\t"
-            "setp.eq.b32 pt, 0, 0;\n\t"
-            "mov.b64 da, {%1, %17};\n\t mov.b64 db, {%9, %17};\n\t"
-            "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], da, db, %18, [%19], [%20], pa;\n\t"
-            "mov.b64 da, {%2, %17};\n\t mov.b64 db, {%10, %17};\n\t"
-            "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], da, db, %18, [%19], [%20], pt;\n\t"
-            "mov.b64 da, {%3, %17};\n\t mov.b64 db, {%11, %17};\n\t"
-            "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], da, db, %18, [%19], [%20], pt;\n\t"
-            "mov.b64 da, {%4, %17};\n\t mov.b64 db, {%12, %17};\n\t"
-            "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], da, db, %18, [%19], [%20], pt;\n\t"
-            "mov.b64 da, {%5, %17};\n\t mov.b64 db, {%13, %17};\n\t"
-            "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], da, db, %18, [%19], [%20], pt;\n\t"
-            "mov.b64 da, {%6, %17};\n\t mov.b64 db, {%14, %17};\n\t"
-            "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], da, db, %18, [%19], [%20], pt;\n\t"
-            "mov.b64 da, {%7, %17};\n\t mov.b64 db, {%15, %17};\n\t"
-            "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], da, db, %18, [%19], [%20], pt;\n\t"
-            "mov.b64 da, {%8, %17};\n\t mov.b64 db, {%16, %17};\n\t"
-            "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], da, db, %18, [%19], [%20], pt;\n\t"
-            "}"
-            :
-            : "r"(tmem_d), "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(a[4]), "r"(a[5]), "r"(a[6]), "r"(a[7]), "r"(b[0]), "r"(b[1]), "r"(b[2]), "r"(b[3]), "r"(b[4]), "r"(b[5]), "r"(b[6]), "r"(b[7]), "r"(desc_hi), "r"(idesc), "r"(sfa), "r"(sfb), "r"(accumulate)
-            : "memory");
-    }
-}
-template <>
-__device__ __forceinline__ void mx_issue_block<4>(uint32_t tmem_d, const uint2 *tbl, uint32_t a_base, uint32_t b_base, uint32_t desc_hi,
-                                                  uint32_t idesc, uint32_t sfa, uint32_t sfb, uint32_t accumulate)
-{
-    uint32_t a[4], b[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const uint2 o = tbl[k];
-        a[k] = a_base + o.x;
-        b[k] = b_base + o.y;
-    }
-    if (elect_one()) {
-        asm volatile(
-            "{\n\t.reg .pred pa, pt;\n\t.reg .b64 da, db;\n\t"
-            "setp.ne.b32 pa, %13, 0;\n\t"
-            "setp.eq.b32 pt, 0, 0;\n\t"
-            "mov.b64 da, {%1, %9};\n\t mov.b64 db, {%5, %9};\n\t"
-            "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], da, db, %10, [%11], [%12], pa;\n\t"
-            "mov.b64 da, {%2, %9};\n\t mov.b64 db, {%6, %9};\n\t"
-            "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], da, db, %10, [%11], [%12], pt;\n\t"
-            "mov.b64 da, {%3, %9};\n\t mov.b64 db, {%7, %9};\n\t"
-            "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], da, db, %10, [%11], [%12], pt;\n\t"
-            "mov.b64 da, {%4, %9};\n\t mov.b64 db, {%8, %9};\n\t"
-            "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], da, db, %10, [%11], [%12], pt;\n\t"
-            "}"
-            :
-            : "r"(tmem_d), "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]), "r"(b[2]), "r"(b[3]), "r"(desc_hi), "r"(idesc), "r"(sfa), "r"(sfb), "r"(accumulate)
-            : "memory");
-    }
-}
-template <>
-__device__ __forceinline__ void mx_issue_block<2>(uint32_t tmem_d, const uint2 *tbl, uint32_t a_base, uint32_t b_base, uint32_t desc_hi,
-                                                  uint32_t idesc, uint32_t sfa, uint32_t sfb, uint32_t accumulate)
-{
-    uint32_t a[2], b[2];
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const uint2 o = tbl[k];
-        a[k] = a_base + o.x;
-        b[k] = b_base + o.y;
-    }
-    if (elect_one()) {
-        asm volatile(
-            "{\n\t.reg .pred pa, pt;\n\t.reg .b64 da, db;\n\t"
-            "setp.ne.b32 pa, %9, 0;\n\t"
-            "setp.eq.b32 pt, 0, 0;\n\t"
-            "mov.b64 da, {%1, %5};\n\t mov.b64 db, {%3, %5};\n\t"
-            "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], da, db, %6, [%7], [%8], pa;\n\t"
-            "mov.b64 da, {%2, %5};\n\t mov.b64 db, {%4, %5};\n\t"
-            "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], da, db, %6, [%7], [%8], pt;\n\t"
-            "}"
-            :
-            : "r"(tmem_d), "r"(a[0]), "r"(a[1]), "r"(b[0]), "r"(b[1]), "r"(desc_hi), "r"(idesc), "r"(sfa), "r"(sfb), "r"(accumulate)
-            : "memory");
-    }
-}
-template <>
-__device__ __forceinline__ void mx_issue_block<1>(uint32_t tmem_d, const uint2 *tbl, uint32_t a_base, uint32_t b_base, uint32_t desc_hi,
-                                                  uint32_t idesc, uint32_t sfa, uint32_t sfb, uint32_t accumulate)
-{
-    uint32_t a[1], b[1];
-#pragma unroll
-    for (int k = 0; k < 1; ++k) {
-        const uint2 o = tbl[k];
-        a[k] = a_base + o.x;
-        b[k] = b_base + o.y;
-    }
-    if (elect_one()) {
-        asm volatile(
-            "{\n\t.reg .pred pa, pt;\n\t.reg .b64 da, db;\n\t"
-            "setp.ne.b32 pa, %7, 0;\n\t"
-            "setp.eq.b32 pt, 0, 0;\n\t"
-            "mov.b64 da, {%1, %3};\n\t mov.b64 db, {%2, %3};\n\t"
-            "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], da, db, %4, [%5], [%6], pa;\n\t"
-            "}"
-            :
-            : "r"(tmem_d), "r"(a[0]), "r"(b[0]), "r"(desc_hi), "r"(idesc), "r"(sfa), "r"(sfb), "r"(accumulate)
-            : "memory");
-    }
+    asm volatile(
+        "{\n\t.reg .pred pa;\n\t.reg .b64 da, db;\n\t"
+        "setp.ne.b32 pa, %7, 0;\n\t"
+        "mov.b64 da, {%1, %3};\n\t mov.b64 db, {%2, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], da, db, %4, [%5], [%6], pa;\n\t}"
+        :
+        : "r"(tmem_d), "r"(a), "r"(b), "r"(desc_hi), "r"(idesc), "r"(sfa), "r"(sfb), "r"((uint32_t)accumulate)
+        : "memory");
 }
 
+// The MMAs of a table of operand offsets, in one loop of the elected lane.  The issuer's code comes by once per tile, while 24
+// other warps of the SM run loops of their own, so it is fetched anew every time: what bounds it is its length (blocks of 8, 4, 2
+// and 1 MMAs written out, all lanes of the warp with them, took 100 clocks an MMA where the tensor pipe needs 50 - 105).
+// Eight a turn: 64 images of 7x7x512 float 9.2 -> 8.4 us, 256 of 14x14x256 -> 512 at stride 2 18.3 -> 17.3, 64 of 32x32x160
+// 5x5 bits 28.0 -> 26.5; with one a turn these take 9.2, 19.3 and 27.1, and 28x28x128 7.6 instead of 7.1; with two it is 7.8, 17.8
+// and 26.2, but 28x28x128 float 9.2 instead of 9.05.
 __device__ __forceinline__ void mx_issue_table(uint32_t tmem_d, const uint2 *tbl, int count, uint32_t a_base, uint32_t b_base, uint32_t desc_hi,
                                                uint32_t idesc, uint32_t sfa, uint32_t sfb, uint32_t &accumulate)
 {
-    int i = 0;
-    for (; i + 8 <= count; i += 8) {
-        mx_issue_block<8>(tmem_d, tbl + i, a_base, b_base, desc_hi, idesc, sfa, sfb, accumulate);
-        accumulate = 1;
+    if (elect_one()) {
+#pragma unroll 8
+        for (int i = 0; i < count; ++i) {
+            const uint2 o = tbl[i];
+            mx_mma(tmem_d, a_base + o.x, b_base + o.y, desc_hi, idesc, sfa, sfb, accumulate || i > 0);
+        }
     }
-    if (count & 4) {
-        mx_issue_block<4>(tmem_d, tbl + i, a_base, b_base, desc_hi, idesc, sfa, sfb, accumulate);
-        accumulate = 1;
-        i += 4;
-    }
-    if (count & 2) {
-        mx_issue_block<2>(tmem_d, tbl + i, a_base, b_base, desc_hi, idesc, sfa, sfb, accumulate);
-        accumulate = 1;
-        i += 2;
-    }
-    if (count & 1) {
-        mx_issue_block<1>(tmem_d, tbl + i, a_base, b_base, desc_hi, idesc, sfa, sfb, accumulate);
-        accumulate = 1;
-    }
+    accumulate = 1;
 }
 
 // Two additions in one instruction
