@@ -169,7 +169,7 @@ lce_status lce_bconv2d_f32(const lce_bconv2d_desc *desc, const float *input, con
  *                       kernel for very few input channels reports LCE_KERNEL_TILED with patch = 1, the
  *                       latency kernel of AUTO LCE_KERNEL_TILED with pixels_per_thread = 0 and tile_pixels,
  *                       warps_per_cta, ctas, shared_bytes).
- *                       For LCE_KERNEL_TENSOR: tile_pixels = grid positions per tile, ctas, shared_bytes,
+ *                       For LCE_KERNEL_TENSOR: tile_pixels = grid positions per accumulator, ctas, shared_bytes,
  *                       weights_resident = 1 when every tap of a channel block stays in shared memory
  *                       (fetched once per CTA; weight_stages = taps), 0 when they stream past once per
  *                       tile (weight_stages = stages of the ring, each a group of consecutive words)

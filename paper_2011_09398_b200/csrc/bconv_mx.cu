@@ -366,6 +366,24 @@ __device__ __forceinline__ int mx_form(const MxParams &p)
     return pairs ? 32 * MX_S2_PAIR + p.Cw : words_ok && p.Cw == 8 ? 32 * MX_S2 + 8 : 32 * MX_S2;
 }
 
+// a loader's registers; the form
+__device__ __forceinline__ int mx_load_setup(const MxParams &p, MxLoad &ld)
+{
+    ld.N = p.N; ld.H = p.H; ld.W = p.W; ld.Cw = p.Cw; ld.Wg = p.Wg; ld.Hg = p.Hg; ld.P = p.P; ld.pt = p.pt; ld.pl = p.pl;
+    ld.in = p.in;
+    ld.col_words = p.Cw;
+    ld.row_words = p.W * p.Cw;
+    ld.image_words = p.H * ld.row_words;
+    ld.origin = p.pt * ld.row_words + p.pl * p.Cw;
+    if (p.stride == 2 && p.n_phase == 1) {  // 1x1: every second pixel of every second row, none of them padding
+        ld.H = p.OH; ld.W = p.OW;
+        ld.col_words *= 2;
+        ld.row_words *= 2;
+    }
+    ld.across = p.step_across;
+    return mx_form(p);
+}
+
 #define LCE_MX_FORMS(CALL)                                                                                                       \
     switch (form) {                                                                                                             \
         case 2: CALL(2, MX_S1); break;                                                                                          \
@@ -909,19 +927,7 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
     const int ltid = tid - kFinishers;  // a loader's number
     const bool loader = ltid >= 0 && ltid < kLoaders;
     if (loader) {
-        ld.N = p.N; ld.H = p.H; ld.W = p.W; ld.Cw = p.Cw; ld.Wg = p.Wg; ld.Hg = p.Hg; ld.P = p.P; ld.pt = p.pt; ld.pl = p.pl;
-        ld.in = p.in;
-        ld.col_words = p.Cw;
-        ld.row_words = p.W * p.Cw;
-        ld.image_words = p.H * ld.row_words;
-        ld.origin = p.pt * ld.row_words + p.pl * p.Cw;
-        if (p.stride == 2 && p.n_phase == 1) {  // 1x1: every second pixel of every second row, none of them padding
-            ld.H = p.OH; ld.W = p.OW;
-            ld.col_words *= 2;
-            ld.row_words *= 2;
-        }
-        ld.across = p.step_across;
-        form = mx_form(p);
+        form = mx_load_setup(p, ld);
         stage = mx_position(first_tile * p.T * p.Nt + ltid, p);
         asm volatile("griddepcontrol.wait;" ::: "memory");  // the activations may come from the previous kernel
         if (first_tile < p.n_super) {
@@ -1092,6 +1098,14 @@ __global__ void __launch_bounds__(kMxThreads, 1) bconv_mx_kernel(const __grid_co
     if (warp == kIssuerWarp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
 }
 
+}  // namespace
+}  // namespace lce
+
+#include "bconv_mx_positions.cuh"
+
+namespace lce {
+namespace {
+
 // ---- load-time weight image -----------------------------------------------------------------------------
 // plain packed words [Cout][KH][KW][Cw] -> e2m1 operand image [channel block][pair of words of K][2][128 channels][16 bytes]
 // in the order of mx_word; channels past Cout, the second word of an odd last one and channels past Cin inside a word are
@@ -1130,6 +1144,7 @@ __global__ void mx_pack_weights_kernel(const uint32_t *w, uint4 *image, int Cout
 
 struct MxPlan {
     int Nt, P, T, stages, resident, group_pairs, groups, n_blocks, ctas_x, n_tiles, n_super, total_q, Wg, Hg, n_phase, Cw, pairs, taps, halo, cover_halo, n_xbuf, ahead;
+    bool positions;  // positions on the TMEM lanes (bconv_mx_positions.cuh)
     size_t raw_words, x_bytes, off_tbl, off_w, off_x, smem;
     double clocks;  // of a CTA's tiles by the cost model
 };
@@ -1243,7 +1258,7 @@ bool mx_covers(const ConvGeom &g)
     return (kBefore + raw + table + 127) / 128 * 128 + 2 * pl.n_phase * Cw2 * P * 16 + 256 + (pl.taps > 1 ? 2 : 1) * Cw2 * 2048 <= kSmemLimit;
 }
 
-bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
+bool mx_plan_as(const ConvGeom &g, int sms, bool positions, MxPlan *pl)
 {
     if (!mx_frame(g, pl)) return false;
     if (!mx_covers(g)) return false;
@@ -1252,7 +1267,8 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
     const int ctas_max = max(1, sms / pl->n_blocks);
     double best = 1e30;
     bool found = false;
-    for (int nt = 16; nt <= kMaxNt; nt += 16) {
+    pl->positions = positions;
+    for (int nt = positions ? kPositionsTile : 16; nt <= (positions ? kPositionsTile : kMaxNt); nt += 16) {
         const int n_tiles = (int)((total_q + nt - 1) / nt);
         for (int T = 1; T <= 8; ++T) {
             if (T > 1 && (T - 1) * ctas_max >= n_tiles) break;   // no CTA would have that many tiles
@@ -1269,6 +1285,7 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
             // size: two large groups measured better than three or four smaller ones)
             const int slots = (int)((kSmemLimit - room.off_w - room.rest) / kPairBytes);
             const bool resident = slots >= pairs;
+            if (positions && !resident) break;
             int stages, group_pairs, groups;
             if (resident) {
                 stages = groups = 1; group_pairs = pairs;
@@ -1315,6 +1332,23 @@ bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
     return found;
 }
 
+// Bit-packed output of up to 96 channels goes with positions on the lanes wherever tiles of 256 positions and all weights fit:
+// of 38 layers of 32 - 512 -> 32 - 96 channels, 1x1 - 5x5, strides 1 and 2, 8 - 256 images, all were faster (0.78 - 0.999 of the
+// time, 0.89 on average; us: 56x56x64 at 8 images 4.88 -> 4.37, at 64 9.8 -> 8.5, at 256 26.6 -> 22.0, 28x28x512 -> 64 at 64 images 15.8 ->
+// 15.4).  With 128 channels an accumulator has 128 columns, three fill TMEM, and it depends: 28x28x128 at 64 images 7.2 -> 8.2,
+// 56x56x64 -> 128 at stride 2, 256 images, 14.7 -> 14.0.  `clocks` stays that of the other form: it is what the choice between this
+// file and the latency kernel is fitted to.
+bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
+{
+    if (!mx_plan_as(g, sms, false, pl)) return false;
+    MxPlan positions;
+    if (g.out_type == LCE_OUT_BITPACKED && g.Cout <= 96 && mx_plan_as(g, sms, true, &positions)) {
+        positions.clocks = pl->clocks;
+        *pl = positions;
+    }
+    return true;
+}
+
 template <int EPI>
 lce_status launch_mx(const MxParams &p, dim3 grid, size_t smem, cudaStream_t s)
 {
@@ -1356,7 +1390,7 @@ lce_status tensor_plan_info(const ConvGeom &g, TensorPlanInfo *info)
 {
     MxPlan pl;
     if (!mx_plan(g, device_sms(), &pl)) return LCE_ERR_UNSUPPORTED;
-    info->tile_positions = pl.Nt;
+    info->tile_positions = pl.positions ? kUnit : pl.Nt;  // of an accumulator
     info->ctas = pl.ctas_x * pl.n_blocks;
     info->weight_stages = pl.resident ? pl.taps : pl.stages;
     info->weights_resident = pl.resident;
@@ -1369,6 +1403,7 @@ lce_status tensor_plan_info(const ConvGeom &g, TensorPlanInfo *info)
 namespace {
 struct MxLaunch {
     MxParams params;
+    int32_t positions;
     dim3 grid;
     size_t smem;
 };
@@ -1383,6 +1418,7 @@ lce_status prepare_bconv_tensor(const ConvGeom &g, PreparedLaunch *prepared)
     l.params = MxParams{};
     l.grid = dim3((unsigned)pl.ctas_x, (unsigned)pl.n_blocks);
     l.smem = pl.smem;
+    l.positions = pl.positions;
     MxParams &p = l.params;
     p.N = g.N; p.H = g.H; p.W = g.W; p.Cw = g.Cw; p.Cout = g.Cout; p.Cow = g.Cow;
     p.OH = g.OH; p.OW = g.OW; p.KH = g.KH; p.KW = g.KW; p.stride = g.sh; p.pt = g.pt; p.pl = g.pl;
@@ -1428,6 +1464,16 @@ lce_status launch_bconv_tensor(const PreparedLaunch &prepared, const uint32_t *i
     p.host_flag = mx_flag_for_launch(s);
     p.cp_words = (p.Cw % 4 == 0 && aligned(in, 16)) ? 4 : (p.Cw % 2 == 0 && aligned(in, 8)) ? 2 : 1;
     p.write_float = out != nullptr;
+    if (l.positions) {
+        MxPositionsParams q;
+        q.m = p;
+        q.n_dim = (p.Cout + 31) / 32 * 32;
+        q.slots = min(4, kPositionsColumns / (2 * q.n_dim));
+        q.wide = p.Cow == 2 && aligned(out, 8) ? 2 : 1;
+        static SmemOptIn opted;
+        if (!opted.ensure(bconv_mx_positions_kernel, l.smem)) return LCE_ERR_CUDA;
+        return launch_dependent(bconv_mx_positions_kernel, l.grid, kPositionsThreads, l.smem, s, q);
+    }
     if (p.out_type == LCE_OUT_FLOAT32 && (residual || out_packed || !out || p.activation != LCE_ACT_NONE))
         return launch_mx<EPI_FLOAT_FUSED>(p, l.grid, l.smem, s);
     return launch_mx<EPI_PLAIN>(p, l.grid, l.smem, s);

@@ -1,0 +1,253 @@
+// The tensor-core kernel for bit-packed output of few channels, with the roles of the operands exchanged: positions are the
+// M dimension (a TMEM lane each), channels the N dimension (32, 64 or 96 columns).  Part of bconv_mx.cu, whose loaders,
+// weight image, grid of positions and barriers it shares.
+//
+// What bounds these layers with channels on the lanes is their finishers (56x56x64: 1620 clocks a tile of 208 positions, its
+// matrix instructions 950), who turn 32 channels x 32 positions of signs around with shuffles and all work on one of two
+// accumulators.  With positions on the lanes a lane has all the channels of its pixel: the signs of 32 columns are the finished
+// word, its words leave in one store, and an accumulator is small enough (128 positions x 64 channels: 64 columns) that several are in
+// flight, read out by four warps each.  The tensor pipe loses nothing: 51 - 59 clocks for 128 x 64 x 64 against 105 for
+// 208 positions x 128 rows, half of which are copies of the channels.  As a graph of ten launches: 56x56x64, 256 images 26.6 -> 22.0 us,
+// 64 images 9.8 -> 8.5; 112x112x32 -> 64 at stride 2, 256 images 30.6 -> 25.6; 56x56x32, 64 images 9.2 -> 7.6.
+//   * tile: 256 positions, two accumulators, issued side by side (the two share the weights' descriptor), handed to the
+//     finishers and back to the loaders with one commit; two to four tiles' accumulators in TMEM;
+//   * finishers: warps 0 - 7 take the even tiles of the CTA, 8 - 15 the odd ones, four warps (lane quarters) to an accumulator;
+//   * issuers: four warps take the tiles in turn, since the loop around the matrix instructions costs as much as they do;
+//   * loops are not unrolled: 28 warps run three different ones, and what bounds them now is how much code that is (two pairs of matrix
+//     instructions written out three times: 23.1 us on 56x56x64, 256 images, once: 22.1);
+//   * thresholds lie in shared memory, one per column.
+// What bounds it now: loaders and issuers at about 1350 clocks a tile each (56x56x64), 10 and more clocks an instruction.
+#pragma once
+
+namespace lce {
+namespace {
+
+constexpr int kUnit = 128;                                  // positions of an accumulator
+constexpr int kPositionsTile = 2 * kUnit;
+constexpr int kPositionsIssuers = 4;
+constexpr int kPositionsThreads = kFinishers + kLoaders + 32 * kPositionsIssuers;
+constexpr int kPositionsColumns = 480;                      // TMEM columns in front of the block scales
+constexpr int BAR_EMPTY_TILE0 = BAR_EMPTY_W0;               // ring of four: the weights are resident, their ring's barriers unused
+static_assert(kPositionsThreads * 72 <= 65536, "registers of a CTA");
+
+struct MxPositionsParams {
+    MxParams m;
+    int32_t n_dim;   // channels of a block, rounded up to whole words
+    int32_t slots;   // tiles whose accumulators TMEM has room for (2..4)
+    int32_t wide;    // words per store: 4, 2 or 1
+};
+
+// v[j] + c[j] < 0 for 16 columns, a bit each
+__device__ __forceinline__ uint32_t mx_column_signs(float (&v)[16], const float *c)
+{
+#pragma unroll
+    for (int j = 0; j < 16; j += 4) {
+        const float4 t = *reinterpret_cast<const float4 *>(c + j);  // the same for every lane
+        asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tadd.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}" : "+f"(v[j]), "+f"(v[j + 1]) : "f"(t.x), "f"(t.y));
+        asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tadd.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}" : "+f"(v[j + 2]), "+f"(v[j + 3]) : "f"(t.z), "f"(t.w));
+    }
+    uint32_t m0 = 0u, m1 = 0u;
+#pragma unroll
+    for (int j = 7; j >= 0; --j) {
+        m0 = __funnelshift_l(__float_as_uint(v[j]), m0, 1);
+        m1 = __funnelshift_l(__float_as_uint(v[8 + j]), m1, 1);
+    }
+    return m0 | m1 << 8;
+}
+
+__device__ __forceinline__ bool mx_positions_finish(const MxPositionsParams &p, uint64_t *bars, const float *thresholds, uint32_t tmem_base, int warp, int lane,
+                                                    int first_tile, int tile_step)
+{
+    MxGrid g;
+    g.N = p.m.N; g.OH = p.m.OH; g.OW = p.m.OW; g.Wg = p.m.Wg; g.Hg = p.m.Hg;
+    g.Wg_mul = p.m.Wg_mul; g.Wg_sh = p.m.Wg_sh; g.Hg_mul = p.m.Hg_mul; g.Hg_sh = p.m.Hg_sh;
+    MxColumns tile_columns;
+    tile_columns.Nt = kPositionsTile;
+    const int T = p.m.T, n_tiles = p.m.n_tiles, n_super = p.m.n_super, slots = p.slots, cow = p.m.Cow, wide = p.wide, words = p.n_dim >> 5;
+    uint32_t *const out = static_cast<uint32_t *>(p.m.out);
+    const int half = warp >> 3, column = (warp & 7) * 32 + lane;
+    const uint32_t tile_cols = (uint32_t)(2 * p.n_dim), tmem = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + ((warp & 4) ? (uint32_t)p.n_dim : 0u);
+    int it = 0, slot = 0;
+    for (int st = first_tile; st < n_super; st += tile_step) {
+        const int end = min(st * T + T, n_tiles);
+#pragma unroll 1
+        for (int tile = st * T; tile < end; ++tile, ++it) {
+            const uint32_t d = tmem + slot * tile_cols;
+            if (++slot == slots) slot = 0;
+            if ((it & 1) != half) continue;
+            const int pixel = mx_out_pixel(tile_columns, g, tile, column);
+            uint32_t *const at = out + (int64_t)pixel * cow;
+            // the warp goes on together
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&bars[BAR_TILE_DONE0 + (it & 3)], (uint32_t)(it >> 2) & 1u))) return false;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            uint32_t before = 0u;
+#pragma unroll 1
+            for (int w = 0; w < words; ++w) {
+                float v[16];
+                tmem_ld16(d + w * 32, v);
+                uint32_t m = mx_column_signs(v, thresholds + w * 32);
+                tmem_ld16(d + w * 32 + 16, v);
+                if (w + 1 == words) mx_hand_back(&bars[BAR_EMPTY_TILE0 + (it & 3)], lane);
+                m |= mx_column_signs(v, thresholds + w * 32 + 16) << 16;
+                if (pixel >= 0) {
+                    if (wide == 1) at[w] = m;
+                    else if (w) *reinterpret_cast<uint2 *>(at) = make_uint2(before, m);
+                }
+                before = m;
+            }
+        }
+    }
+    return true;
+}
+
+__device__ __forceinline__ bool mx_positions_issue(const MxPositionsParams &p, const uint8_t *smem, uint64_t *bars, int32_t *fills, uint32_t tmem_base, int mine, int lane,
+                                                   int first_tile, int tile_step)
+{
+    const uint2 *tbl = reinterpret_cast<const uint2 *>(smem + p.m.off_tbl);
+    // descriptors: see bconv_mx_kernel; here A is the positions and B the weights, N channels
+    const uint32_t idesc = (1u << 7) | (1u << 10) | ((uint32_t)(p.n_dim >> 3) << 17) | (1u << 23) | ((uint32_t)(kUnit >> 4) << 24);
+    const uint32_t desc_hi = 8u | (1u << 14);
+    const int T = p.m.T, n_tiles = p.m.n_tiles, n_super = p.m.n_super, n_xbuf = p.m.n_xbuf, pairs = p.m.pairs, slots = p.slots;
+    const uint32_t w_lo = ((uint32_t)p.m.off_w >> 4) + (smem_u32(smem) >> 4) + (128u << 16);
+    const uint32_t x_lo0 = ((uint32_t)p.m.off_x >> 4) + (smem_u32(smem) >> 4), x_units = (uint32_t)p.m.x_bytes >> 4;
+    const uint32_t n_dim = (uint32_t)p.n_dim, sfa = tmem_base + kSfaCol, sfb = tmem_base + kSfbCol;
+    bool ok = mbar_wait_bounded(&bars[BAR_SCALES], 0) && mbar_wait_bounded(&bars[BAR_FULL_W0], 0);
+    if (lane == 0) fills[1] = 1;
+    int it = 0, xbuf = 0, slot = 0;
+    for (int st = first_tile; st < n_super; st += tile_step, xbuf = xbuf + 1 == n_xbuf ? 0 : xbuf + 1) {
+        const int end = min(T, n_tiles - st * T);
+#pragma unroll 1
+        for (int k = 0; k < end; ++k, ++it) {
+            const uint32_t d = tmem_base + slot * 2 * n_dim;
+            if (++slot == slots) slot = 0;
+            if ((it & (kPositionsIssuers - 1)) != mine) continue;
+            ok = ok && mbar_wait_bounded(&bars[BAR_FULL_X0 + (it & 3)], (uint32_t)(it >> 2) & 1u);
+            // The accumulators must have been read out.  (Their barrier cannot be two phases behind: four tiles ago this warp
+            // waited for the phase before.)
+            if (it >= slots) ok = ok && mbar_wait_bounded(&bars[BAR_EMPTY_TILE0 + ((it - slots) & 3)], (uint32_t)((it - slots) >> 2) & 1u);
+            // the finishers' barrier may not run two phases ahead of those of them that are behind with tile it - 4
+            if (slots == 3 && it >= 4) ok = ok && mbar_wait_bounded(&bars[BAR_EMPTY_TILE0 + (it & 3)], (uint32_t)((it - 4) >> 2) & 1u);
+            if (!__all_sync(0xffffffffu, ok)) return false;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            if (elect_one()) {
+                const uint32_t x_lo = x_lo0 + (uint32_t)xbuf * x_units + (uint32_t)(k * kPositionsTile);
+#pragma unroll 1
+                for (int e = 0; e < pairs; ++e) {
+                    const uint2 o = tbl[e];
+                    mx_mma(d, x_lo + o.y, w_lo + o.x, desc_hi, idesc, sfa, sfb, e > 0);
+                    mx_mma(d + n_dim, x_lo + kUnit + o.y, w_lo + o.x, desc_hi, idesc, sfa, sfb, e > 0);
+                }
+                mma_commit(&bars[BAR_TILE_DONE0 + (it & 3)]);  // to the finishers and to the loaders
+            }
+            __syncwarp();
+        }
+    }
+    return ok;
+}
+
+__global__ void __launch_bounds__(kPositionsThreads, 1) bconv_mx_positions_kernel(const __grid_constant__ MxPositionsParams p)
+{
+    extern __shared__ __align__(1024) uint8_t smem[];
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kOffBars);
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + kOffSlot);
+    int32_t *fills = reinterpret_cast<int32_t *>(smem + kOffSlot + 4);  // [0] weight copies under way, [1] there
+    float *thresholds = reinterpret_cast<float *>(smem + kOffPix);      // of the CTA's channels, negated
+    uint32_t *raw0 = reinterpret_cast<uint32_t *>(smem + kOffDyn);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int first_tile = blockIdx.x, tile_step = gridDim.x;
+
+    // the next kernel of the stream may start setting itself up as soon as every CTA of this one has got here
+    if (tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    // ---- set-up, side by side, as in bconv_mx_kernel ------------------------------------------------------
+    if (warp == kIssuerWarp) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    } else if (warp == kIssuerWarp + 1) {
+        for (int b = lane; b < BAR_COUNT; b += 32)
+            mbar_init(&bars[b], b <= BAR_FULL_X3 ? kLoaders : b >= BAR_EMPTY_TILE0 && b < BAR_EMPTY_TILE0 + 4 ? 8 : b == BAR_SCALES ? 4 : 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        if (lane == 0) {
+            mbar_expect_tx(&bars[BAR_FULL_W0], (uint32_t)(p.m.pairs * kPairBytes));
+            fills[0] = 1;
+            fills[1] = 0;
+        }
+        __syncwarp();
+        const int share = (p.m.pairs + 31) >> 5, first = lane * share, n = min(share, p.m.pairs - first);
+        if (n > 0) bulk_copy_g2s(smem + p.m.off_w + (size_t)first * kPairBytes, p.m.wimg + (size_t)first * kPairBytes, (uint32_t)(n * kPairBytes), &bars[BAR_FULL_W0]);
+    } else if (tid < kFinishers) {
+        uint2 *tbl = reinterpret_cast<uint2 *>(smem + p.m.off_tbl);
+        const int even = p.m.Cw & ~1, paired = p.m.KH * p.m.KW * even, words = p.m.KH * p.m.KW * p.m.Cw;
+        for (int e = tid; e < p.m.pairs; e += kFinishers) {
+            const uint32_t first = word_b_offset(p.m, 2 * e, even, paired);
+            const uint32_t apart = 2 * e < paired ? (uint32_t)p.m.P : 2 * e + 1 < words ? word_b_offset(p.m, 2 * e + 1, even, paired) - first : 1u;
+            tbl[e] = make_uint2((uint32_t)e * (kPairBytes >> 4), first | apart << 16);
+        }
+    }
+    MxLoad ld;
+    MxPos stage{0, 0, 0};
+    int form = 0;
+    const int ltid = tid - kFinishers;  // a loader's number
+    const bool loader = ltid >= 0 && ltid < kLoaders;
+    if (loader) {
+        form = mx_load_setup(p.m, ld);
+        stage = mx_position(first_tile * p.m.T * kPositionsTile + ltid, p.m);
+        asm volatile("griddepcontrol.wait;" ::: "memory");  // the activations may come from the previous kernel
+        if (first_tile < p.m.n_super) {
+            if (p.m.n_phase == 1) mx_prefetch<0, MX_S1>(ld, stage, kPositionsTile + p.m.halo, raw0, ltid, p.m.cp_words);
+            else mx_prefetch<0, MX_S2>(ld, stage, kPositionsTile + p.m.halo, raw0, ltid, p.m.cp_words);
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem_base = *tmem_slot;
+    if (warp < 4) {
+        // block scales: every byte 0x7F = 2^0
+        const uint32_t one = 0x7F7F7F7Fu;
+        const uint32_t taddr = tmem_base + ((uint32_t)(warp * 32) << 16) + kSfaCol;
+#pragma unroll
+        for (int c = 0; c < 32; c += 8)
+            asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(taddr + c), "r"(one) : "memory");
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars[BAR_SCALES]);
+    }
+
+    bool ok = true;
+    if (loader) {
+        uint8_t *sX0 = smem + p.m.off_x;
+#define LCE_MX_LOAD_POSITIONS(CW, FORM) ok = mx_load_tiles<CW, FORM>(p.m, ld, stage, bars, raw0, sX0, ltid, first_tile, tile_step)
+        LCE_MX_FORMS(LCE_MX_LOAD_POSITIONS)
+    } else if (tid < kFinishers) {
+        if (tid < p.n_dim)  // constants of the model.  acc < thr is unchanged by clamping thr to [-K-1, K+1] (|acc| <= K), and then thr is exact in fp32
+            thresholds[tid] = tid < p.m.Cout ? -(float)max(-p.m.K - 1, min(p.m.K + 1, __ldg(p.m.thr + tid))) : INFINITY;
+        asm volatile("bar.sync 1, %0;" ::"n"(kFinishers) : "memory");
+        asm volatile("griddepcontrol.wait;" ::: "memory");  // outputs: only after the previous kernel
+        ok = mx_positions_finish(p, bars, thresholds, tmem_base, warp, lane, first_tile, tile_step);
+    } else {
+        ok = mx_positions_issue(p, smem, bars, fills, tmem_base, warp - kIssuerWarp, lane, first_tile, tile_step);
+    }
+    if (!ok) mx_report_timeout(p.m.host_flag);
+
+    // ---- tear-down: nothing of this CTA may still be in flight when its TMEM and shared memory go ----
+    // When no wait gave up, the finishers have waited for the matrix instructions of every tile and the issuers for the weights.
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    if (!__syncthreads_and(ok)) {
+        if (warp >= kIssuerWarp && elect_one()) {
+            uint64_t *done = &bars[BAR_FULL_W0 + 1 + warp - kIssuerWarp];  // of the unused ring
+            mma_commit(done);                                              // arrives when every MMA this lane issued has finished
+            bool drained = mbar_wait_bounded(done, 0);
+            if (warp == kIssuerWarp) drained = mbar_wait_bounded(&bars[BAR_FULL_W0], 0) && drained;
+            if (!drained) mx_report_timeout(p.m.host_flag);
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+    }
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (warp == kIssuerWarp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
+}
+
+}  // namespace
+}  // namespace lce

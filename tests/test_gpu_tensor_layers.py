@@ -31,7 +31,13 @@ ODD_WORDS = [
 ONE_BUFFER = [(64, 28, 28, 256, 40, 3, 2, lce.PAD_SAME_ZERO), (64, 56, 56, 32, 20, 3, 1, lce.PAD_SAME_ONE), (37, 56, 55, 40, 33, 3, 1, lce.PAD_SAME_ZERO)]
 
 
-@pytest.mark.parametrize("shape", SHAPES + ODD_WORDS + ONE_BUFFER, ids=lambda s: "x".join(map(str, s)))
+# few channels, bits: one, two and three words; one tile of 256 positions, one position more than that, and enough tiles that every
+# ring comes round
+POSITIONS = [(1, 16, 16, 64, 32, 1, 1, lce.PAD_VALID), (1, 1, 257, 40, 64, 1, 1, lce.PAD_VALID), (80, 56, 56, 32, 32, 1, 1, lce.PAD_SAME_ONE), (80, 56, 56, 64, 64, 1, 1, lce.PAD_SAME_ONE),
+             (80, 56, 56, 33, 96, 1, 1, lce.PAD_SAME_ZERO), (70, 55, 56, 32, 41, 3, 1, lce.PAD_SAME_ZERO), (90, 112, 112, 3, 65, 3, 2, lce.PAD_SAME_ONE)]
+
+
+@pytest.mark.parametrize("shape", SHAPES + ODD_WORDS + ONE_BUFFER + POSITIONS, ids=lambda s: "x".join(map(str, s)))
 def test_tensor_layers_match_the_oracle(shape):
     n, h, w, cin, cout, k, s, pad = shape
     rng = np.random.default_rng(sum(shape))
@@ -44,6 +50,24 @@ def test_tensor_layers_match_the_oracle(shape):
     thr = np.rint(np.sqrt(k * k * cin) * rng.standard_normal(cout)).astype(np.int32)
     got = run_bconv(aw, ww, dict(kwargs, out_type=lce.OUT_BITPACKED), thr=thr, kernel_choice=lce.KERNEL_TENSOR, packed=True)
     np.testing.assert_array_equal(got, oracle.transform_bits(acc, thr))
+    assert lce.lce_device_status() == 0
+
+
+@pytest.mark.parametrize("cout,offset", [(64, 0), (64, 1), (64, 2), (40, 1), (96, 1), (32, 3)])
+def test_bits_of_few_channels_at_any_word(cout, offset):
+    """Output words that start on 4 and on 8 bytes, thresholds on, beside and far beyond the accumulators' range."""
+    rng = np.random.default_rng(cout + offset)
+    a, wt = ((2 * rng.integers(0, 2, size=s) - 1).astype(np.int8) for s in ((3, 19, 20, 64), (cout, 3, 3, 64)))
+    acc = oracle.bconv2d_acc(a, wt, (1, 1), lce.PAD_SAME_ONE)
+    thr = rng.choice(np.array([-2**31, -577, -576, -2, 0, 1, 2, 576, 577, 2**31 - 1]), cout).astype(np.int32)
+    desc = lce.make_desc(3, 19, 20, 64, cout, out_type=lce.OUT_BITPACKED, kernel_choice=lce.KERNEL_TENSOR, weights_packed=1)
+    weights = lce.lce_bconv2d_pack_weights(desc, to_dev_words(oracle.bitpack_pm1(wt)))
+    count = acc.shape[0] * acc.shape[1] * acc.shape[2] * ((cout + 31) // 32)
+    whole = torch.full((count + 8,), 0x5A5A5A5A, dtype=torch.int32, device="cuda:0")
+    out = whole[offset:offset + count].view(*acc.shape[:3], -1)
+    lce.lce_bconv2d(desc, to_dev_words(oracle.bitpack_pm1(a)), weights, None, None, to_dev(thr), out)
+    np.testing.assert_array_equal(words_to_host(out.contiguous()), oracle.transform_bits(acc, thr))
+    assert (whole[:offset] == 0x5A5A5A5A).all() and (whole[offset + count:] == 0x5A5A5A5A).all()
     assert lce.lce_device_status() == 0
 
 
