@@ -1231,7 +1231,7 @@ struct MxRoom {
     size_t raw_words, x_bytes, off_tbl, off_w, rest;
 };
 
-bool mx_room(const MxPlan &pl, int nt, int T, int n_xbuf, MxRoom *r)
+bool mx_room(const MxPlan &pl, int nt, int T, int n_xbuf, size_t limit, MxRoom *r)
 {
     // T tiles share one position buffer of T * nt + halo rows: the halo is staged once per T tiles
     r->P = T * nt + pl.halo;
@@ -1242,7 +1242,7 @@ bool mx_room(const MxPlan &pl, int nt, int T, int n_xbuf, MxRoom *r)
     const size_t fixed = r->off_tbl + (size_t)pl.pairs * 8;  // the table no longer than it is: at 512 channels 3x3 the 8 KB saved are a wider tile
     r->off_w = (fixed + 127) / 128 * 128;
     r->rest = n_xbuf * r->x_bytes + 256;
-    return r->off_w + r->rest + (size_t)min(2, pl.pairs) * kPairBytes <= kSmemLimit;
+    return r->off_w + r->rest + (size_t)min(2, pl.pairs) * kPairBytes <= limit;
 }
 
 // Which layers the kernel takes: those whose smallest tile (16 positions) fits beside two whole taps (one of a 1x1 filter)
@@ -1258,8 +1258,9 @@ bool mx_covers(const ConvGeom &g)
     return (kBefore + raw + table + 127) / 128 * 128 + 2 * pl.n_phase * Cw2 * P * 16 + 256 + (pl.taps > 1 ? 2 : 1) * Cw2 * 2048 <= kSmemLimit;
 }
 
-bool mx_plan_as(const ConvGeom &g, int sms, bool positions, MxPlan *pl)
+bool mx_plan_as(const ConvGeom &g, int sms, bool positions, size_t reserved, MxPlan *pl)
 {
+    const size_t limit = kSmemLimit - reserved;
     if (!mx_frame(g, pl)) return false;
     if (!mx_covers(g)) return false;
     const int pairs = pl->pairs, halo = pl->halo;
@@ -1279,11 +1280,11 @@ bool mx_plan_as(const ConvGeom &g, int sms, bool positions, MxPlan *pl)
             const int n_super = (n_tiles + T - 1) / T;
             const int ctas_x = min(ctas_max, n_super);
             const bool single = n_super <= ctas_x;
-            if (!mx_room(*pl, nt, T, single ? 1 : 2, &room)) break;
+            if (!mx_room(*pl, nt, T, single ? 1 : 2, limit, &room)) break;
             // pairs that fit beside the position buffers: all of them -> resident (one barrier); otherwise a ring of two
             // stages of half the fitting pairs each (a group costs the issuer one wait and one commit, whatever its
             // size: two large groups measured better than three or four smaller ones)
-            const int slots = (int)((kSmemLimit - room.off_w - room.rest) / kPairBytes);
+            const int slots = (int)((limit - room.off_w - room.rest) / kPairBytes);
             const bool resident = slots >= pairs;
             if (positions && !resident) break;
             int stages, group_pairs, groups;
@@ -1322,10 +1323,10 @@ bool mx_plan_as(const ConvGeom &g, int sms, bool positions, MxPlan *pl)
                 // up to four tiles ahead, ahead <= (n_xbuf - 1) * T + 1, and the hand-overs between the roles
                 // (a few hundred clocks each) drop out of the per-tile cycle.
                 int n_xbuf = single ? 1 : 2;
-                while (!single && n_xbuf < 4 && (n_xbuf - 1) * T + 1 < 4 && pl->off_x + (size_t)(n_xbuf + 1) * room.x_bytes <= kSmemLimit) ++n_xbuf;
+                while (!single && n_xbuf < 4 && (n_xbuf - 1) * T + 1 < 4 && pl->off_x + (size_t)(n_xbuf + 1) * room.x_bytes <= limit) ++n_xbuf;
                 pl->n_xbuf = n_xbuf;
                 pl->ahead = single ? 4 : min(4, (n_xbuf - 1) * T + 1);
-                pl->smem = pl->off_x + (size_t)n_xbuf * room.x_bytes;
+                pl->smem = pl->off_x + (size_t)n_xbuf * room.x_bytes + reserved;
             }
         }
     }
@@ -1340,9 +1341,9 @@ bool mx_plan_as(const ConvGeom &g, int sms, bool positions, MxPlan *pl)
 // file and the latency kernel is fitted to.
 bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
 {
-    if (!mx_plan_as(g, sms, false, pl)) return false;
+    if (!mx_plan_as(g, sms, false, 0, pl)) return false;
     MxPlan positions;
-    if (g.out_type == LCE_OUT_BITPACKED && g.Cout <= 96 && mx_plan_as(g, sms, true, &positions)) {
+    if (g.out_type == LCE_OUT_BITPACKED && g.Cout <= kPositionsChannels && mx_plan_as(g, sms, true, 0, &positions)) {
         positions.clocks = pl->clocks;
         *pl = positions;
     }
@@ -1355,6 +1356,14 @@ lce_status launch_mx(const MxParams &p, dim3 grid, size_t smem, cudaStream_t s)
     static SmemOptIn opted;
     if (!opted.ensure(bconv_mx_kernel<EPI>, smem)) return LCE_ERR_CUDA;
     return launch_dependent(bconv_mx_kernel<EPI>, grid, kMxThreads, smem, s, p);
+}
+
+template <int FORM>
+lce_status launch_positions(const MxPositionsParams &p, dim3 grid, size_t smem, cudaStream_t s)
+{
+    static SmemOptIn opted;
+    if (!opted.ensure(bconv_mx_positions_kernel<FORM>, smem)) return LCE_ERR_CUDA;
+    return launch_dependent(bconv_mx_positions_kernel<FORM>, grid, kPositionsThreads, smem, s, p);
 }
 
 int mx_dup(const ConvGeom &g) { return g.Cout <= 32 ? 4 : g.Cout <= 64 ? 2 : 1; }
@@ -1403,18 +1412,20 @@ lce_status tensor_plan_info(const ConvGeom &g, TensorPlanInfo *info)
 namespace {
 struct MxLaunch {
     MxParams params;
-    int32_t positions;
     dim3 grid;
     size_t smem;
+    bool positions;
 };
-static_assert(sizeof(MxLaunch) <= sizeof(PreparedLaunch), "PreparedLaunch too small");
-}  // namespace
 
-lce_status prepare_bconv_tensor(const ConvGeom &g, PreparedLaunch *prepared)
+// float output has forms of its own for launches with a shortcut and with a re-quantised copy alone
+struct MxLaunches {
+    MxLaunch plain, copy, shortcut;
+};
+static_assert(sizeof(MxLaunches) <= sizeof(PreparedLaunch), "PreparedLaunch too small");
+
+MxLaunch mx_launch(const ConvGeom &g, const MxPlan &pl)
 {
-    MxPlan pl;
-    if (!mx_plan(g, device_sms(), &pl)) return LCE_ERR_UNSUPPORTED;
-    MxLaunch &l = *reinterpret_cast<MxLaunch *>(prepared->bytes);
+    MxLaunch l;
     l.params = MxParams{};
     l.grid = dim3((unsigned)pl.ctas_x, (unsigned)pl.n_blocks);
     l.smem = pl.smem;
@@ -1449,6 +1460,25 @@ lce_status prepare_bconv_tensor(const ConvGeom &g, PreparedLaunch *prepared)
     p.pad_zero = g.padding == LCE_PAD_SAME_ZERO;
     p.out_type = g.out_type; p.activation = g.activation;
     p.dup_log2 = mx_dup(g) == 4 ? 2 : mx_dup(g) == 2 ? 1 : 0;
+    return l;
+}
+}  // namespace
+
+// Float output of whole words of up to 96 channels goes with positions on the lanes where a shortcut is added or a re-quantised copy
+// written: of 30 such launches (56x56 and 28x28, 64 and 96 channels, 1x1 and 3x3, 32 - 128 images) 27 took 0.58 - 0.96 of the time (us:
+// 56x56x64 at 128 images, copy alone 18.4 -> 15.8, shortcut and copy 34.3 -> 25.3, with the floats 57.6 -> 40.8); the three with a
+// shortcut from 96 to 96 channels have no room for it beside their weights and stay as they are.  Floats alone are bound by their stores
+// and stay, too: 56x56x64 at 64 images 14.1, with positions on the lanes 15.1 (32 bytes of a pixel a store instead of 128).
+lce_status prepare_bconv_tensor(const ConvGeom &g, PreparedLaunch *prepared)
+{
+    MxPlan pl;
+    if (!mx_plan(g, device_sms(), &pl)) return LCE_ERR_UNSUPPORTED;
+    MxLaunches &l = *reinterpret_cast<MxLaunches *>(prepared->bytes);
+    l.plain = l.copy = l.shortcut = mx_launch(g, pl);
+    if (g.out_type == LCE_OUT_FLOAT32 && g.Cout % 32 == 0 && g.Cout <= kPositionsChannels) {
+        if (mx_plan_as(g, device_sms(), true, 0, &pl)) l.copy = mx_launch(g, pl);
+        if (mx_plan_as(g, device_sms(), true, kShortcutBytes, &pl)) l.shortcut = mx_launch(g, pl);
+    }
     return LCE_OK;
 }
 
@@ -1457,7 +1487,8 @@ lce_status launch_bconv_tensor(const PreparedLaunch &prepared, const uint32_t *i
 {
     if (!w_image) return LCE_ERR_UNSUPPORTED;
     if (!aligned(w_image, 16)) return LCE_ERR_ALIGNMENT;
-    const MxLaunch &l = *reinterpret_cast<const MxLaunch *>(prepared.bytes);
+    const MxLaunches &forms = *reinterpret_cast<const MxLaunches *>(prepared.bytes);
+    const MxLaunch &l = residual ? forms.shortcut : out_packed ? forms.copy : forms.plain;
     MxParams p = l.params;
     p.in = in; p.wimg = static_cast<const uint8_t *>(w_image); p.mult = mult; p.bias = bias; p.thr = thr; p.out = out;
     p.residual = residual; p.out_packed = out_packed;
@@ -1470,9 +1501,9 @@ lce_status launch_bconv_tensor(const PreparedLaunch &prepared, const uint32_t *i
         q.n_dim = (p.Cout + 31) / 32 * 32;
         q.slots = min(4, kPositionsColumns / (2 * q.n_dim));
         q.wide = p.Cow == 2 && aligned(out, 8) ? 2 : 1;
-        static SmemOptIn opted;
-        if (!opted.ensure(bconv_mx_positions_kernel, l.smem)) return LCE_ERR_CUDA;
-        return launch_dependent(bconv_mx_positions_kernel, l.grid, kPositionsThreads, l.smem, s, q);
+        q.off_shortcut = (int32_t)l.smem - kShortcutBytes;
+        if (p.out_type == LCE_OUT_BITPACKED) return launch_positions<POSITIONS_BITS>(q, l.grid, l.smem, s);
+        return launch_positions<POSITIONS_FUSED>(q, l.grid, l.smem, s);
     }
     if (p.out_type == LCE_OUT_FLOAT32 && (residual || out_packed || !out || p.activation != LCE_ACT_NONE))
         return launch_mx<EPI_FLOAT_FUSED>(p, l.grid, l.smem, s);

@@ -1,4 +1,4 @@
-// The tensor-core kernel for bit-packed output of few channels, with the roles of the operands exchanged: positions are the
+// The tensor-core kernel for bit-packed output, and float output with a shortcut or a re-quantised copy, of few channels, with the roles of the operands exchanged: positions are the
 // M dimension (a TMEM lane each), channels the N dimension (32, 64 or 96 columns).  Part of bconv_mx.cu, whose loaders,
 // weight image, grid of positions and barriers it shares.
 //
@@ -22,10 +22,12 @@
 namespace lce {
 namespace {
 
+constexpr int kPositionsChannels = 96;                      // at most: with 128 two tiles' accumulators do not fit TMEM
 constexpr int kUnit = 128;                                  // positions of an accumulator
 constexpr int kPositionsTile = 2 * kUnit;
 constexpr int kPositionsIssuers = 4;
 constexpr int kPositionsThreads = kFinishers + kLoaders + 32 * kPositionsIssuers;
+constexpr int kShortcutBytes = kFinishers / 32 * 8192;       // two buffers of 32 positions x 32 channels a finisher warp
 constexpr int kPositionsColumns = 480;                      // TMEM columns in front of the block scales
 constexpr int BAR_EMPTY_TILE0 = BAR_EMPTY_W0;               // ring of four: the weights are resident, their ring's barriers unused
 static_assert(kPositionsThreads * 72 <= 65536, "registers of a CTA");
@@ -34,8 +36,25 @@ struct MxPositionsParams {
     MxParams m;
     int32_t n_dim;   // channels of a block, rounded up to whole words
     int32_t slots;   // tiles whose accumulators TMEM has room for (2..4)
-    int32_t wide;    // words per store: 4, 2 or 1
+    int32_t wide;    // words per store of bit-packed output: 2 or 1
+    int32_t off_shortcut;  // in shared memory: [finisher warp][2][4 KB]
 };
+
+// 16 TMEM lanes x 32 columns by quads of threads: v[4 j + 2 i + e] is lane (thread / 4) + 8 i, column 8 j + 2 (thread % 4) + e
+__device__ __forceinline__ void tmem_ld_quads(uint32_t taddr, float (&v)[16])
+{
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+}
 
 // v[j] + c[j] < 0 for 16 columns, a bit each
 __device__ __forceinline__ uint32_t mx_column_signs(float (&v)[16], const float *c)
@@ -100,6 +119,137 @@ __device__ __forceinline__ bool mx_positions_finish(const MxPositionsParams &p, 
     return true;
 }
 
+// Float output (Section 3.2) with the shortcut add and the re-quantised copy of Section 5.3; whole words of channels.  The accumulator
+// is read in quads: a thread has two neighbouring channels of every eight of four positions, 8 apart, so that the four threads of
+// a quad fill a 32-byte sector with one 8-byte store each, at addresses that differ by constants, and a value costs half a
+// multiply-add and half a store (32 channels of a position as a 128-byte store: an address, a compare and a store each).
+// The shortcut comes through shared memory: a warp copies 32 channels of its 32 positions (4 KB) two steps ahead, 16 bytes a thread,
+// pieces of a row exchanged so that the quads' reads meet every bank once.  Loaded into registers before the accumulator is there
+// it is bound by what the L1 can have under way beside 200 KB of shared memory: 56x56x64, 128 images, shortcut and copy 31.8 us,
+// 25.3 now (34.3 with channels on the lanes; the shortcut's 103 MB take 15.7 at HBM rate).
+template <bool RES, bool PACK, bool WRITE>
+__device__ __forceinline__ bool mx_positions_values(const MxPositionsParams &p, uint64_t *bars, const float *scales, uint8_t *staged, uint32_t tmem_base, int warp, int lane, int first_tile, int tile_step)
+{
+    MxGrid g;
+    g.N = p.m.N; g.OH = p.m.OH; g.OW = p.m.OW; g.Wg = p.m.Wg; g.Hg = p.m.Hg;
+    g.Wg_mul = p.m.Wg_mul; g.Wg_sh = p.m.Wg_sh; g.Hg_mul = p.m.Hg_mul; g.Hg_sh = p.m.Hg_sh;
+    MxColumns tile_columns;
+    tile_columns.Nt = kPositionsTile;
+    const int T = p.m.T, n_tiles = p.m.n_tiles, n_super = p.m.n_super, slots = p.slots, cout = p.n_dim;
+    const int half = warp >> 3, column = (warp & 7) * 32 + lane, quad = lane & 3;
+    const uint32_t tile_cols = (uint32_t)(2 * cout), tmem = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + ((warp & 4) ? (uint32_t)cout : 0u);
+    float *const out = static_cast<float *>(p.m.out) + 2 * quad;
+    const float floor_v = p.m.activation == LCE_ACT_RELU ? 0.f : -INFINITY;
+    scales += 4 * quad;  // multiplier, multiplier, bias, bias of two channels
+    // the shortcut's way: this warp's two buffers, and its next tile's pixels
+    const uint32_t stage = RES ? smem_u32(staged) + (uint32_t)warp * 8192u : 0u;
+    const auto pixel_of = [&](int st, int tile) {  // of the lane's position in a tile, which may lie in the next super-tiles
+        while (tile >= st * T + T && st < n_super) { tile += (tile_step - 1) * T; st += tile_step; }
+        return st < n_super && tile < n_tiles ? mx_out_pixel(tile_columns, g, tile, column) : -1;
+    };
+    const auto copy = [&](int px, int c, uint32_t buffer) {  // 32 channels from c on
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int row = 4 * i + (lane >> 3), from = __shfl_sync(0xffffffffu, px, row);
+            const uint32_t to = buffer + row * 128 + (((lane & 7) ^ (2 * (row & 3))) << 4);
+            const float *src = p.m.residual + (int64_t)from * cout + c + 4 * (lane & 7);
+            if (from >= 0) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to), "l"(src) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    int it = 0, slot = 0, next_pixel = -1, step = 0;
+    if (RES) {
+        next_pixel = pixel_of(first_tile, first_tile * T + half);
+        copy(next_pixel, 0, stage);
+        if (cout > 32) copy(next_pixel, 32, stage + 4096);
+        else copy(pixel_of(first_tile, first_tile * T + half + 2), 0, stage + 4096);
+    }
+    for (int st = first_tile; st < n_super; st += tile_step) {
+        const int end = min(st * T + T, n_tiles);
+#pragma unroll 1
+        for (int tile = st * T; tile < end; ++tile, ++it) {
+            const uint32_t d = tmem + slot * tile_cols;
+            if (++slot == slots) slot = 0;
+            if ((it & 1) != half) continue;
+            const int pixel = RES ? next_pixel : mx_out_pixel(tile_columns, g, tile, column);
+            if (RES) next_pixel = pixel_of(st, tile + 2);
+            int64_t at[4];  // of the thread's four positions, -1: no output
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int px = __shfl_sync(0xffffffffu, pixel, (lane >> 2) + 8 * i);
+                at[i] = px < 0 ? -1 : (int64_t)px * cout;
+            }
+            // the warp goes on together
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&bars[BAR_TILE_DONE0 + (it & 3)], (uint32_t)(it >> 2) & 1u))) {
+                if (RES) asm volatile("cp.async.wait_all;" ::: "memory");  // nothing in flight at the end
+                return false;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll 1
+            for (int c = 0; c < cout; c += 32, ++step) {
+                uint32_t bits[4];
+                const uint32_t from = stage + (uint32_t)(step & 1) * 4096u + (lane >> 2) * 128 + (uint32_t)(quad & 1) * 8u;
+                if (RES) {
+                    asm volatile("cp.async.wait_group 1;" ::: "memory");
+                    __syncwarp();
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float v[16];
+                    tmem_ld_quads(d + c + ((uint32_t)(16 * h) << 16), v);
+                    if (h == 1 && c + 32 == cout) mx_hand_back(&bars[BAR_EMPTY_TILE0 + (it & 3)], lane);
+                    uint32_t m0 = 0u, m1 = 0u;
+#pragma unroll
+                    for (int j = 3; j >= 0; --j) {
+                        const float4 t = *reinterpret_cast<const float4 *>(scales + 2 * c + 16 * j);
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            float y0 = v[4 * j + 2 * i], y1 = v[4 * j + 2 * i + 1];
+                            y0 = fmaxf(y0, floor_v);
+                            y1 = fmaxf(y1, floor_v);
+                            asm("{\n\t.reg .b64 y, s, b;\n\tmov.b64 y, {%0, %1};\n\tmov.b64 s, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tfma.rn.f32x2 y, y, s, b;\n\tmov.b64 {%0, %1}, y;\n\t}" : "+f"(y0), "+f"(y1) : "f"(t.x), "f"(t.y), "f"(t.z), "f"(t.w));
+                            if (RES) {
+                                float r0, r1;
+                                asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(r0), "=f"(r1) : "r"(from + (16 * h + 8 * i) * 128 + (((2 * j + (quad >> 1)) ^ (2 * ((lane >> 2) & 3))) << 4)));
+                                y0 = __fadd_rn(y0, r0);
+                                y1 = __fadd_rn(y1, r1);
+                            }
+                            if (WRITE && at[2 * h + i] >= 0) *reinterpret_cast<float2 *>(out + at[2 * h + i] + c + 8 * j) = make_float2(y0, y1);
+                            if (PACK) {  // the sign of y + 0, which makes -0.0 and NaN positive
+                                uint32_t &m = i ? m1 : m0;
+                                m = __funnelshift_l(__float_as_uint(y1 + 0.f), m << 6, 1);
+                                m = __funnelshift_l(__float_as_uint(y0 + 0.f), m, 1);
+                            }
+                        }
+                    }
+                    bits[2 * h] = m0;
+                    bits[2 * h + 1] = m1;
+                }
+                if (RES) {  // two steps ahead: the same channels or those of this warp's next tile
+                    __syncwarp();
+                    const int ahead = c + 64;
+                    const bool here = ahead < cout;
+                    copy(here ? pixel : cout == 32 ? pixel_of(st, tile + 4) : next_pixel, here ? ahead : ahead - (cout == 32 ? 64 : cout), stage + (uint32_t)(step & 1) * 4096u);
+                }
+                if (PACK) {
+                    uint32_t word = 0u;
+                    int64_t where = -1;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        uint32_t m = bits[i] << (2 * quad);
+                        m |= __shfl_xor_sync(0xffffffffu, m, 1);
+                        m |= __shfl_xor_sync(0xffffffffu, m, 2);
+                        if (quad == i) { word = m; where = at[i]; }
+                    }
+                    if (where >= 0) p.m.out_packed[(where + c) >> 5] = word;
+                }
+            }
+        }
+    }
+    if (RES) asm volatile("cp.async.wait_all;" ::: "memory");
+    return true;
+}
+
 __device__ __forceinline__ bool mx_positions_issue(const MxPositionsParams &p, const uint8_t *smem, uint64_t *bars, int32_t *fills, uint32_t tmem_base, int mine, int lane,
                                                    int first_tile, int tile_step)
 {
@@ -145,6 +295,9 @@ __device__ __forceinline__ bool mx_positions_issue(const MxPositionsParams &p, c
     return ok;
 }
 
+enum { POSITIONS_BITS, POSITIONS_FUSED };  // bit-packed output; float output with a shortcut or a re-quantised copy
+
+template <int FORM>
 __global__ void __launch_bounds__(kPositionsThreads, 1) bconv_mx_positions_kernel(const __grid_constant__ MxPositionsParams p)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -221,11 +374,27 @@ __global__ void __launch_bounds__(kPositionsThreads, 1) bconv_mx_positions_kerne
 #define LCE_MX_LOAD_POSITIONS(CW, FORM) ok = mx_load_tiles<CW, FORM>(p.m, ld, stage, bars, raw0, sX0, ltid, first_tile, tile_step)
         LCE_MX_FORMS(LCE_MX_LOAD_POSITIONS)
     } else if (tid < kFinishers) {
-        if (tid < p.n_dim)  // constants of the model.  acc < thr is unchanged by clamping thr to [-K-1, K+1] (|acc| <= K), and then thr is exact in fp32
+        if (FORM != POSITIONS_BITS) {  // by pairs of channels: two multipliers, two biases
+            if (tid < p.n_dim) {
+                thresholds[4 * (tid >> 1) + (tid & 1)] = __ldg(p.m.mult + tid);
+                thresholds[4 * (tid >> 1) + 2 + (tid & 1)] = __ldg(p.m.bias + tid);
+            }
+        } else if (tid < p.n_dim)  // constants of the model.  acc < thr is unchanged by clamping thr to [-K-1, K+1] (|acc| <= K), and then thr is exact in fp32
             thresholds[tid] = tid < p.m.Cout ? -(float)max(-p.m.K - 1, min(p.m.K + 1, __ldg(p.m.thr + tid))) : INFINITY;
         asm volatile("bar.sync 1, %0;" ::"n"(kFinishers) : "memory");
         asm volatile("griddepcontrol.wait;" ::: "memory");  // outputs: only after the previous kernel
-        ok = mx_positions_finish(p, bars, thresholds, tmem_base, warp, lane, first_tile, tile_step);
+#define LCE_MX_VALUES(...) mx_positions_values<__VA_ARGS__>(p, bars, thresholds, smem + p.off_shortcut, tmem_base, warp, lane, first_tile, tile_step)
+        if (FORM == POSITIONS_BITS) {
+            ok = mx_positions_finish(p, bars, thresholds, tmem_base, warp, lane, first_tile, tile_step);
+        } else {
+            switch ((p.m.residual ? 4 : 0) | (p.m.out_packed ? 2 : 0) | (p.m.write_float ? 1 : 0)) {
+                case 2: ok = LCE_MX_VALUES(false, true, false); break;
+                case 3: ok = LCE_MX_VALUES(false, true, true); break;
+                case 5: ok = LCE_MX_VALUES(true, false, true); break;
+                case 6: ok = LCE_MX_VALUES(true, true, false); break;
+                default: ok = LCE_MX_VALUES(true, true, true); break;
+            }
+        }
     } else {
         ok = mx_positions_issue(p, smem, bars, fills, tmem_base, warp - kIssuerWarp, lane, first_tile, tile_step);
     }

@@ -148,7 +148,7 @@ lce_status launch_dependent(void (*kernel)(Params...), dim3 grid, int threads, s
 // A launch worked out ahead of time for a geometry: everything but the buffers (filled in by the prepare functions,
 // read by the launch functions of the same kernel).
 struct PreparedLaunch {
-    alignas(16) unsigned char bytes[768];
+    alignas(16) unsigned char bytes[1536];
 };
 
 // Kernel entry points implemented in the other translation units.

@@ -99,6 +99,34 @@ def test_fused_words_of_special_values(n, h, w, c):
     assert lce.lce_device_status() == 0
 
 
+@pytest.mark.parametrize("n,h,cout,offset", [(1, 16, 32, 0), (1, 17, 64, 4), (2, 15, 96, 0), (70, 56, 64, 4), (80, 56, 32, 0), (60, 57, 96, 4)])
+def test_fused_of_few_channels(n, h, cout, offset):
+    """Float tensors that start on 16 and on 32 bytes; one tile and so many that every ring comes round; with ReLU."""
+    rng = np.random.default_rng(n + cout + offset)
+    a, wt = ((2 * rng.integers(0, 2, size=s) - 1).astype(np.int8) for s in ((n, h, h, 32), (cout, 1, 1, 32)))
+    acc = oracle.bconv2d_acc(a, wt, (1, 1), lce.PAD_SAME_ONE)
+    mult, bias = rng.uniform(-1.5, 1.5, cout).astype(np.float32), rng.standard_normal(cout).astype(np.float32)
+    desc = lce.make_desc(n, h, h, 32, cout, (1, 1), out_type=lce.OUT_FLOAT32, activation=lce.ACT_RELU, kernel_choice=lce.KERNEL_TENSOR, weights_packed=1)
+    x, weights = to_dev_words(oracle.bitpack_pm1(a)), lce.lce_bconv2d_pack_weights(desc, to_dev_words(oracle.bitpack_pm1(wt)))
+    shortcut = torch.randn(acc.size + 8, device="cuda:0")
+    residual = shortcut[offset:offset + acc.size].view(acc.shape)
+    plain = oracle.transform_float(acc, mult, bias, oracle.ACT_RELU)
+    for res in (None, residual):
+        y = plain if res is None else oracle.add_f32(plain, res.cpu().numpy())
+        for floats, packed in ((True, False), (False, True), (True, True)):
+            whole = torch.full((acc.size + 8,), 12345.0, device="cuda:0")
+            out = whole[offset:offset + acc.size].view(acc.shape)
+            whole_w, words = guarded(acc.shape[:3] + (cout // 32,), torch.int32, 0x5A5A5A5A)
+            lce.lce_bconv2d_fused(desc, x, weights, to_dev(mult), to_dev(bias), res, out if floats else None, words if packed else None)
+            if floats:
+                np.testing.assert_array_equal(out.cpu().numpy(), y)
+                assert (whole[:offset] == 12345.0).all() and (whole[offset + acc.size:] == 12345.0).all()
+            if packed:
+                np.testing.assert_array_equal(words_to_host(words), oracle.bitpack(y))
+                assert guards_intact(whole_w, 0x5A5A5A5A)
+    assert lce.lce_device_status() == 0
+
+
 # n, h, w, cin, cout, k, stride: channel blocks with one, two or three words missing, one tile and several tiles a CTA
 RAGGED_BLOCKS = [(40, 28, 27, 64, 96, 3, 1), (30, 16, 15, 96, 160, 3, 1), (2, 9, 10, 64, 192, 3, 2), (70, 14, 13, 40, 224, 1, 1), (1, 5, 5, 32, 96, 5, 1)]
 
