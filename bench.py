@@ -448,7 +448,7 @@ def run_lce(args):
     bf16 = float(peaks.get("bf16_tflops", 1590.0))
     tensor_peak = bf16 * 1e12 * 4 / 2
     roofline = {
-        "bound": "tensor", "kernel": "bconv_mx_kernel (tcgen05 kind::mxf4, all 8 launches)" if all_tensor else "mixed",
+        "bound": "tensor", "kernel": "bconv_mx_kernel, bconv_mx_positions_kernel (tcgen05 kind::mxf4, all 8 launches)" if all_tensor else "mixed",
         "achieved": achieved / 1e12, "peak": tensor_peak / 1e12, "unit": "T binary-MAC/s (x2 = TFLOP/s)", "frac": achieved / tensor_peak,
         "peak_source": ("MEASURED_PEAKS.json bf16_tflops (burst) x 4 (nominal fp4 : bf16) / 2 FLOP per MAC, of measured" if peaks
                         else "fallback 1590 TFLOP/s bf16 x 4 / 2, of fallback"),
