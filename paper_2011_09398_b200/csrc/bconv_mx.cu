@@ -62,6 +62,7 @@
 #include "common.cuh"
 #include "mx_columns.cuh"
 #include "mx_common.cuh"
+#include "mx_rings.cuh"
 
 namespace lce {
 namespace {

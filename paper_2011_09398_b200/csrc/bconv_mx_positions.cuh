@@ -29,7 +29,8 @@ constexpr int kPositionsIssuers = 4;
 constexpr int kPositionsThreads = kFinishers + kLoaders + 32 * kPositionsIssuers;
 constexpr int kShortcutBytes = kFinishers / 32 * 8192;       // two buffers of 32 positions x 32 channels a finisher warp
 constexpr int kPositionsColumns = 480;                      // TMEM columns in front of the block scales
-constexpr int BAR_EMPTY_TILE0 = BAR_EMPTY_W0;               // ring of four: the weights are resident, their ring's barriers unused
+constexpr int BAR_EMPTY_TILE0 = BAR_EMPTY_W0;               // ring of kEmptyRing: the weights are resident, their ring's barriers unused
+static_assert(kEmptyRing <= kMaxStages, "the accumulators' barriers are in place of the weight ring's");
 static_assert(kPositionsThreads * 72 <= 65536, "registers of a CTA");
 
 struct MxPositionsParams {
@@ -97,7 +98,7 @@ __device__ __forceinline__ bool mx_positions_finish(const MxPositionsParams &p, 
             const int pixel = mx_out_pixel(tile_columns, g, tile, column);
             uint32_t *const at = out + (int64_t)pixel * cow;
             // the warp goes on together
-            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&bars[BAR_TILE_DONE0 + (it & 3)], (uint32_t)(it >> 2) & 1u))) return false;
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&bars[BAR_TILE_DONE0 + mx_ring_slot(it, kTileRing)], mx_ring_parity(it, kTileRing)))) return false;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             uint32_t before = 0u;
 #pragma unroll 1
@@ -106,7 +107,7 @@ __device__ __forceinline__ bool mx_positions_finish(const MxPositionsParams &p, 
                 tmem_ld16(d + w * 32, v);
                 uint32_t m = mx_column_signs(v, thresholds + w * 32);
                 tmem_ld16(d + w * 32 + 16, v);
-                if (w + 1 == words) mx_hand_back(&bars[BAR_EMPTY_TILE0 + (it & 3)], lane);
+                if (w + 1 == words) mx_hand_back(&bars[BAR_EMPTY_TILE0 + mx_ring_slot(it, kEmptyRing)], lane);
                 m |= mx_column_signs(v, thresholds + w * 32 + 16) << 16;
                 if (pixel >= 0) {
                     if (wide == 1) at[w] = m;
@@ -180,7 +181,7 @@ __device__ __forceinline__ bool mx_positions_values(const MxPositionsParams &p, 
                 at[i] = px < 0 ? -1 : (int64_t)px * cout;
             }
             // the warp goes on together
-            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&bars[BAR_TILE_DONE0 + (it & 3)], (uint32_t)(it >> 2) & 1u))) {
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&bars[BAR_TILE_DONE0 + mx_ring_slot(it, kTileRing)], mx_ring_parity(it, kTileRing)))) {
                 if (RES) asm volatile("cp.async.wait_all;" ::: "memory");  // nothing in flight at the end
                 return false;
             }
@@ -197,7 +198,7 @@ __device__ __forceinline__ bool mx_positions_values(const MxPositionsParams &p, 
                 for (int h = 0; h < 2; ++h) {
                     float v[16];
                     tmem_ld_quads(d + c + ((uint32_t)(16 * h) << 16), v);
-                    if (h == 1 && c + 32 == cout) mx_hand_back(&bars[BAR_EMPTY_TILE0 + (it & 3)], lane);
+                    if (h == 1 && c + 32 == cout) mx_hand_back(&bars[BAR_EMPTY_TILE0 + mx_ring_slot(it, kEmptyRing)], lane);
                     uint32_t m0 = 0u, m1 = 0u;
 #pragma unroll
                     for (int j = 3; j >= 0; --j) {
@@ -271,12 +272,10 @@ __device__ __forceinline__ bool mx_positions_issue(const MxPositionsParams &p, c
             const uint32_t d = tmem_base + slot * 2 * n_dim;
             if (++slot == slots) slot = 0;
             if ((it & (kPositionsIssuers - 1)) != mine) continue;
-            ok = ok && mbar_wait_bounded(&bars[BAR_FULL_X0 + (it & 3)], (uint32_t)(it >> 2) & 1u);
-            // The accumulators must have been read out.  (Their barrier cannot be two phases behind: four tiles ago this warp
-            // waited for the phase before.)
-            if (it >= slots) ok = ok && mbar_wait_bounded(&bars[BAR_EMPTY_TILE0 + ((it - slots) & 3)], (uint32_t)((it - slots) >> 2) & 1u);
-            // the finishers' barrier may not run two phases ahead of those of them that are behind with tile it - 4
-            if (slots == 3 && it >= 4) ok = ok && mbar_wait_bounded(&bars[BAR_EMPTY_TILE0 + (it & 3)], (uint32_t)((it - 4) >> 2) & 1u);
+            ok = ok && mbar_wait_bounded(&bars[BAR_FULL_X0 + mx_ring_slot(it, kTileRing)], mx_ring_parity(it, kTileRing));
+            ok = ok && mx_wait_read_out(it, slots, [&](int tile) {
+                return mbar_wait_bounded(&bars[BAR_EMPTY_TILE0 + mx_ring_slot(tile, kEmptyRing)], mx_ring_parity(tile, kEmptyRing));
+            });
             if (!__all_sync(0xffffffffu, ok)) return false;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             if (elect_one()) {
@@ -287,7 +286,7 @@ __device__ __forceinline__ bool mx_positions_issue(const MxPositionsParams &p, c
                     mx_mma(d, x_lo + o.y, w_lo + o.x, desc_hi, idesc, sfa, sfb, e > 0);
                     mx_mma(d + n_dim, x_lo + kUnit + o.y, w_lo + o.x, desc_hi, idesc, sfa, sfb, e > 0);
                 }
-                mma_commit(&bars[BAR_TILE_DONE0 + (it & 3)]);  // to the finishers and to the loaders
+                mma_commit(&bars[BAR_TILE_DONE0 + mx_ring_slot(it, kTileRing)]);  // to the finishers and to the loaders
             }
             __syncwarp();
         }
@@ -318,7 +317,7 @@ __global__ void __launch_bounds__(kPositionsThreads, 1) bconv_mx_positions_kerne
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     } else if (warp == kIssuerWarp + 1) {
         for (int b = lane; b < BAR_COUNT; b += 32)
-            mbar_init(&bars[b], b <= BAR_FULL_X3 ? kLoaders : b >= BAR_EMPTY_TILE0 && b < BAR_EMPTY_TILE0 + 4 ? 8 : b == BAR_SCALES ? 4 : 1);
+            mbar_init(&bars[b], b <= BAR_FULL_X3 ? kLoaders : b >= BAR_EMPTY_TILE0 && b < BAR_EMPTY_TILE0 + kEmptyRing ? 8 : b == BAR_SCALES ? 4 : 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (lane == 0) {
             mbar_expect_tx(&bars[BAR_FULL_W0], (uint32_t)(p.m.pairs * kPairBytes));
