@@ -251,7 +251,7 @@ __device__ __forceinline__ bool mx_positions_values(const MxPositionsParams &p, 
     return true;
 }
 
-__device__ __forceinline__ bool mx_positions_issue(const MxPositionsParams &p, const uint8_t *smem, uint64_t *bars, int32_t *fills, uint32_t tmem_base, int mine, int lane,
+__device__ __forceinline__ bool mx_positions_issue(const MxPositionsParams &p, const uint8_t *smem, uint64_t *bars, uint32_t tmem_base, int mine,
                                                    int first_tile, int tile_step)
 {
     const uint2 *tbl = reinterpret_cast<const uint2 *>(smem + p.m.off_tbl);
@@ -263,7 +263,6 @@ __device__ __forceinline__ bool mx_positions_issue(const MxPositionsParams &p, c
     const uint32_t x_lo0 = ((uint32_t)p.m.off_x >> 4) + (smem_u32(smem) >> 4), x_units = (uint32_t)p.m.x_bytes >> 4;
     const uint32_t n_dim = (uint32_t)p.n_dim, sfa = tmem_base + kSfaCol, sfb = tmem_base + kSfbCol;
     bool ok = mbar_wait_bounded(&bars[BAR_SCALES], 0) && mbar_wait_bounded(&bars[BAR_FULL_W0], 0);
-    if (lane == 0) fills[1] = 1;
     int it = 0, xbuf = 0, slot = 0;
     for (int st = first_tile; st < n_super; st += tile_step, xbuf = xbuf + 1 == n_xbuf ? 0 : xbuf + 1) {
         const int end = min(T, n_tiles - st * T);
@@ -302,7 +301,6 @@ __global__ void __launch_bounds__(kPositionsThreads, 1) bconv_mx_positions_kerne
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kOffBars);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + kOffSlot);
-    int32_t *fills = reinterpret_cast<int32_t *>(smem + kOffSlot + 4);  // [0] weight copies under way, [1] there
     float *thresholds = reinterpret_cast<float *>(smem + kOffPix);      // of the CTA's channels, negated
     uint32_t *raw0 = reinterpret_cast<uint32_t *>(smem + kOffDyn);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -319,11 +317,8 @@ __global__ void __launch_bounds__(kPositionsThreads, 1) bconv_mx_positions_kerne
         for (int b = lane; b < BAR_COUNT; b += 32)
             mbar_init(&bars[b], b <= BAR_FULL_X3 ? kLoaders : b >= BAR_EMPTY_TILE0 && b < BAR_EMPTY_TILE0 + kEmptyRing ? 8 : b == BAR_SCALES ? 4 : 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        if (lane == 0) {
-            mbar_expect_tx(&bars[BAR_FULL_W0], (uint32_t)(p.m.pairs * kPairBytes));
-            fills[0] = 1;
-            fills[1] = 0;
-        }
+        __syncwarp();  // the weights' barrier is another lane's
+        if (lane == 0) mbar_expect_tx(&bars[BAR_FULL_W0], (uint32_t)(p.m.pairs * kPairBytes));
         __syncwarp();
         const int share = (p.m.pairs + 31) >> 5, first = lane * share, n = min(share, p.m.pairs - first);
         if (n > 0) bulk_copy_g2s(smem + p.m.off_w + (size_t)first * kPairBytes, p.m.wimg + (size_t)first * kPairBytes, (uint32_t)(n * kPairBytes), &bars[BAR_FULL_W0]);
@@ -395,7 +390,7 @@ __global__ void __launch_bounds__(kPositionsThreads, 1) bconv_mx_positions_kerne
             }
         }
     } else {
-        ok = mx_positions_issue(p, smem, bars, fills, tmem_base, warp - kIssuerWarp, lane, first_tile, tile_step);
+        ok = mx_positions_issue(p, smem, bars, tmem_base, warp - kIssuerWarp, first_tile, tile_step);
     }
     if (!ok) mx_report_timeout(p.m.host_flag);
 

@@ -2,6 +2,7 @@
 host and walked through in every order in which loaders, issuers, matrix instructions and finishers can take their steps.  No
 order may get stuck, no wait may return for another phase than its own."""
 import ctypes
+import re
 import subprocess
 from pathlib import Path
 
@@ -153,3 +154,15 @@ def test_no_order_of_steps_gets_stuck(walk, slots, ahead):
 def test_a_ring_of_four_and_three_slots_would(walk):
     """The model sees the order in which tile t + 1 is read out before issuer t has looked at tile t - 3."""
     assert walk(3, 4, 18, 4)[0] == 1
+
+
+def test_barriers_initialised_by_lanes_are_there_for_the_warp_before_it_announces_bytes():
+    """Barrier b is initialised by lane b % 32: another lane may use it only behind a __syncwarp()."""
+    seen = 0
+    for source in sorted(CSRC.glob("*.cu*")):
+        text = source.read_text()
+        for at in re.finditer(r"b \+= 32\)\s*\{?[^}]*?mbar_init\(&bars\[b\]", text):
+            announced = text.index("mbar_expect_tx(", at.end())
+            assert "__syncwarp();" in text[at.end():announced], source.name
+            seen += 1
+    assert seen == 2
