@@ -151,7 +151,7 @@ void prepare(const lce_bconv2d_desc *desc, int device, uint32_t form, Prepared *
     const bool rows_aligned = !(form & FORM_ROWS_UNALIGNED);
     p->pick = form & FORM_HOST ? pick_host(desc, p->g, !(form & FORM_NO_IMAGE)) : form & FORM_FUSED ? pick_fused(desc, p->g, p->parts, rows_aligned) : pick_kernel(desc, p->g, desc->weights_packed && p->parts.tensor, rows_aligned);
     if (p->pick == PICK_SMALL) p->status = prepare_bconv_small(p->g, &p->launch);
-    if (p->pick == PICK_TENSOR) p->status = prepare_bconv_tensor(p->g, &p->launch);
+    if (p->pick == PICK_TENSOR) p->status = prepare_bconv_tensor(p->g, form & FORM_FUSED, &p->launch);
 }
 
 // A network repeats few descriptors: the last ones of each host thread are kept.  Working a call out costs 1 - 2 us of

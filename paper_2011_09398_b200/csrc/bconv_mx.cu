@@ -1334,17 +1334,39 @@ bool mx_plan_as(const ConvGeom &g, int sms, bool positions, size_t reserved, MxP
     return found;
 }
 
-// Bit-packed output of up to 96 channels goes with positions on the lanes wherever tiles of 256 positions and all weights fit:
-// of 38 layers of 32 - 512 -> 32 - 96 channels, 1x1 - 5x5, strides 1 and 2, 8 - 256 images, all were faster (0.78 - 0.999 of the
-// time, 0.89 on average; us: 56x56x64 at 8 images 4.88 -> 4.37, at 64 9.8 -> 8.5, at 256 26.6 -> 22.0, 28x28x512 -> 64 at 64 images 15.8 ->
-// 15.4).  With 128 channels an accumulator has 128 columns, three fill TMEM, and it depends: 28x28x128 at 64 images 7.2 -> 8.2,
-// 56x56x64 -> 128 at stride 2, 256 images, 14.7 -> 14.0.  `clocks` stays that of the other form: it is what the choice between this
-// file and the latency kernel is fitted to.
+// Where positions on the lanes pay, given that all weights fit.  A tile is 256 positions whatever the grid, where the other form cuts
+// narrower ones so that every SM has its share: with fewer tiles than SMs, or few in the last wave, SMs have nothing to do.  What the form
+// gains per tile must make up for that, and it gains more the fewer words it stores and the fewer matrix instructions there are.  Both
+// forms as graphs of 20 launches, 1 - 128 images of 7x7 - 112x112, 32 - 512 -> 32 - 96 channels, 1x1 - 5x5, strides 1 and 2 (711 layers
+// with bits, 532 with each fused output); time with positions on the lanes / with channels:
+//   bits: 0.60 - 1.02 where taken.  Left to the other form: 0.94 - 1.22 (14x14x256 -> 64 at 32 images 1.10, 14x14x512 -> 96, 1x1, at
+//     64 images 1.03).
+//   re-quantised copy alone: 0.68 - 1.04; left 0.92 - 1.40 (14x14x96 at 32 images 1.20).
+//   floats or a shortcut: 0.55 - 1.03; left 0.88 - 1.79 (one image of 28x28x96 with all three 1.79).
+enum MxOutput { MX_BITS, MX_COPY, MX_COPY_FLOATS, MX_SHORTCUT_COPY, MX_SHORTCUT_FLOATS, MX_OUTPUTS };  // the last with or without the copy
+
+bool mx_positions_pay(const ConvGeom &g, const MxPlan &pl, int sms, MxOutput output)
+{
+    const int words = (g.Cout + 31) / 32, instructions = pl.pairs * words;  // of 32 channels each
+    const bool one_phase = pl.n_phase == 1;
+    const double waves = (double)pl.n_tiles / sms, full = waves / ceil(waves);
+    if (output == MX_BITS)
+        return one_phase && waves >= 0.5 || full >= 0.6 || one_phase && instructions <= 10 || words == 1 && waves >= 0.35;
+    if (full >= 0.86 || words == 1 && waves >= (one_phase ? 0.5 : 1.0)) return true;
+    if (output == MX_COPY) return pl.pairs <= 8 && full >= 0.6 || one_phase && words <= 2 && instructions <= 8;
+    if (words == 1 && one_phase && instructions <= 10 && waves >= 0.08) return true;
+    return output == MX_SHORTCUT_COPY && waves >= 2.0 || output == MX_SHORTCUT_FLOATS && waves >= 4.0;  // the last wave counts for less
+}
+
+// Bit-packed output of up to 96 channels.  With 128 channels an accumulator has 128 columns, three fill TMEM, and it depends: 28x28x128 at
+// 64 images 7.2 -> 8.2 us, 56x56x64 -> 128 at stride 2, 256 images, 14.7 -> 14.0.  `clocks` stays that of channels on the lanes: it is what
+// the choice between this file and the latency kernel is fitted to, and positions on the lanes are taken where they need no more.
 bool mx_plan_uncached(const ConvGeom &g, int sms, MxPlan *pl)
 {
     if (!mx_plan_as(g, sms, false, 0, pl)) return false;
     MxPlan positions;
-    if (g.out_type == LCE_OUT_BITPACKED && g.Cout <= kPositionsChannels && mx_plan_as(g, sms, true, 0, &positions)) {
+    if (g.out_type == LCE_OUT_BITPACKED && g.Cout <= kPositionsChannels && mx_plan_as(g, sms, true, 0, &positions) &&
+        mx_positions_pay(g, positions, sms, MX_BITS)) {
         positions.clocks = pl->clocks;
         *pl = positions;
     }
@@ -1418,9 +1440,10 @@ struct MxLaunch {
     bool positions;
 };
 
-// float output has forms of its own for launches with a shortcut and with a re-quantised copy alone
+// float output has launches of its own for a re-quantised copy and for a shortcut, taken where they pay
 struct MxLaunches {
     MxLaunch plain, copy, shortcut;
+    bool pays[MX_OUTPUTS];
 };
 static_assert(sizeof(MxLaunches) <= sizeof(PreparedLaunch), "PreparedLaunch too small");
 
@@ -1465,20 +1488,27 @@ MxLaunch mx_launch(const ConvGeom &g, const MxPlan &pl)
 }
 }  // namespace
 
-// Float output of whole words of up to 96 channels goes with positions on the lanes where a shortcut is added or a re-quantised copy
-// written: of 30 such launches (56x56 and 28x28, 64 and 96 channels, 1x1 and 3x3, 32 - 128 images) 27 took 0.58 - 0.96 of the time (us:
-// 56x56x64 at 128 images, copy alone 18.4 -> 15.8, shortcut and copy 34.3 -> 25.3, with the floats 57.6 -> 40.8); the three with a
-// shortcut from 96 to 96 channels have no room for it beside their weights and stay as they are.  Floats alone are bound by their stores
-// and stay, too: 56x56x64 at 64 images 14.1, with positions on the lanes 15.1 (32 bytes of a pixel a store instead of 128).
-lce_status prepare_bconv_tensor(const ConvGeom &g, PreparedLaunch *prepared)
+// Float output of whole words of up to 96 channels, with a shortcut added or a re-quantised copy written, can go with positions on the
+// lanes (us: 56x56x64 at 128 images, copy alone 18.4 -> 15.8, shortcut and copy 34.3 -> 25.3, with the floats 57.6 -> 40.8); a
+// shortcut from 96 to 96 channels, 3x3, has no room beside the weights, as a rule.  Floats alone are bound by their stores and have one
+// form: 56x56x64 at 64 images 14.1, with positions on the lanes 15.1 (32 bytes of a pixel a store instead of 128).
+lce_status prepare_bconv_tensor(const ConvGeom &g, bool fused, PreparedLaunch *prepared)
 {
     MxPlan pl;
-    if (!mx_plan(g, device_sms(), &pl)) return LCE_ERR_UNSUPPORTED;
+    const int sms = device_sms();
+    if (!mx_plan(g, sms, &pl)) return LCE_ERR_UNSUPPORTED;
     MxLaunches &l = *reinterpret_cast<MxLaunches *>(prepared->bytes);
-    l.plain = l.copy = l.shortcut = mx_launch(g, pl);
-    if (g.out_type == LCE_OUT_FLOAT32 && g.Cout % 32 == 0 && g.Cout <= kPositionsChannels) {
-        if (mx_plan_as(g, device_sms(), true, 0, &pl)) l.copy = mx_launch(g, pl);
-        if (mx_plan_as(g, device_sms(), true, kShortcutBytes, &pl)) l.shortcut = mx_launch(g, pl);
+    l.plain = mx_launch(g, pl);
+    memset(l.pays, 0, sizeof(l.pays));
+    if (fused && g.out_type == LCE_OUT_FLOAT32 && g.Cout % 32 == 0 && g.Cout <= kPositionsChannels) {
+        if (mx_plan_as(g, sms, true, 0, &pl)) {
+            l.copy = mx_launch(g, pl);
+            for (MxOutput o : {MX_COPY, MX_COPY_FLOATS}) l.pays[o] = mx_positions_pay(g, pl, sms, o);
+        }
+        if (mx_plan_as(g, sms, true, kShortcutBytes, &pl)) {
+            l.shortcut = mx_launch(g, pl);
+            for (MxOutput o : {MX_SHORTCUT_COPY, MX_SHORTCUT_FLOATS}) l.pays[o] = mx_positions_pay(g, pl, sms, o);
+        }
     }
     return LCE_OK;
 }
@@ -1489,7 +1519,8 @@ lce_status launch_bconv_tensor(const PreparedLaunch &prepared, const uint32_t *i
     if (!w_image) return LCE_ERR_UNSUPPORTED;
     if (!aligned(w_image, 16)) return LCE_ERR_ALIGNMENT;
     const MxLaunches &forms = *reinterpret_cast<const MxLaunches *>(prepared.bytes);
-    const MxLaunch &l = residual ? forms.shortcut : out_packed ? forms.copy : forms.plain;
+    const MxOutput output = residual ? (out ? MX_SHORTCUT_FLOATS : MX_SHORTCUT_COPY) : out ? MX_COPY_FLOATS : MX_COPY;
+    const MxLaunch &l = !(residual || out_packed) || !forms.pays[output] ? forms.plain : residual ? forms.shortcut : forms.copy;
     MxParams p = l.params;
     p.in = in; p.wimg = static_cast<const uint8_t *>(w_image); p.mult = mult; p.bias = bias; p.thr = thr; p.out = out;
     p.residual = residual; p.out_packed = out_packed;

@@ -187,7 +187,7 @@ lce_status launch_bconv_small(const PreparedLaunch &prepared, const uint32_t *in
 bool tensor_covers(const ConvGeom &g);
 size_t tensor_weight_image_bytes(const ConvGeom &g);
 lce_status launch_pack_weights_tensor(const ConvGeom &g, const uint32_t *w, void *image, cudaStream_t s);
-lce_status prepare_bconv_tensor(const ConvGeom &g, PreparedLaunch *prepared);
+lce_status prepare_bconv_tensor(const ConvGeom &g, bool fused, PreparedLaunch *prepared);
 lce_status launch_bconv_tensor(const PreparedLaunch &prepared, const uint32_t *in, const void *w_image, const float *mult,
                                const float *bias, const int32_t *thr, void *out, cudaStream_t s,
                                const float *residual = nullptr, uint32_t *out_packed = nullptr);
