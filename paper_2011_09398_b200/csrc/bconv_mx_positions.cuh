@@ -144,10 +144,7 @@ __device__ __forceinline__ bool mx_positions_values(const MxPositionsParams &p, 
     scales += 4 * quad;  // multiplier, multiplier, bias, bias of two channels
     // the shortcut's way: this warp's two buffers, and its next tile's pixels
     const uint32_t stage = RES ? smem_u32(staged) + (uint32_t)warp * 8192u : 0u;
-    const auto pixel_of = [&](int st, int tile) {  // of the lane's position in a tile, which may lie in the next super-tiles
-        while (tile >= st * T + T && st < n_super) { tile += (tile_step - 1) * T; st += tile_step; }
-        return st < n_super && tile < n_tiles ? mx_out_pixel(tile_columns, g, tile, column) : -1;
-    };
+    const auto pixel_of = [&](int st, int tile) { return mx_pixel_ahead(tile_columns, g, st, tile, column, T, tile_step, n_super, n_tiles); };
     const auto copy = [&](int px, int c, uint32_t buffer) {  // 32 channels from c on
 #pragma unroll
         for (int i = 0; i < 8; ++i) {

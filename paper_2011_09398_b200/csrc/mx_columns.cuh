@@ -64,4 +64,12 @@ LCE_MX_BOTH int mx_chunk_pixel(const MxColumns &f, const MxGrid &g, int tile, in
     return mx_out_pixel(f, g, tile, (f.group + (second ? f.n_groups : 0)) * 32 + lane);
 }
 
+// Output pixel of a column of a tile that may lie behind the super-tile at hand (tiles st * T .. st * T + T - 1): the CTA's next ones are
+// tile_step super-tiles apart.  -1 where that is no output, or the CTA has no such tile.
+LCE_MX_BOTH int mx_pixel_ahead(const MxColumns &f, const MxGrid &g, int st, int tile, int column, int T, int tile_step, int n_super, int n_tiles)
+{
+    while (tile >= st * T + T && st < n_super) { tile += (tile_step - 1) * T; st += tile_step; }
+    return st < n_super && tile < n_tiles ? mx_out_pixel(f, g, tile, column) : -1;
+}
+
 }  // namespace lce
