@@ -50,6 +50,8 @@
 //     transpose across the warp gives each lane the finished word of one pixel.  Float / int32 output
 //     is written straight from the registers: per position a warp stores its 32 consecutive channels as
 //     one 128-byte line.
+//   * few output channels on grids that fill the SMs go with the operands exchanged, positions on the TMEM lanes: a kernel of its own
+//     (bconv_mx_positions.cuh) on the same loaders, weight image and grid, four issuers, no weight ring; mx_positions_pay draws the line.
 //   * launched with programmatic stream serialization, dependents released at kernel entry: set-up and
 //     the weight copies may overlap the tail of the previous kernel of the stream; activations, shortcut
 //     and outputs are touched only after griddepcontrol.wait.
@@ -579,8 +581,8 @@ __device__ __forceinline__ uint32_t warp_transpose32(uint32_t m, const Transpose
 
 // The finishers.  All transforms take the accumulator 16 columns at a time (32 left no register free: the bit-packed one
 // spilled), know their positions' output pixels before the accumulator is there, and do one compare a position.  Instructions
-// bound the thin layers (5900 a tile of 208 positions on 56x56x64): 64 channels, 56x56, 256 images, bits 28.4 -> 26.5 us;
-// 64 images, float 14.0 -> 13.8.  Setting the accumulators to minus the threshold beforehand (tcgen05.st) instead of
+// bound the thin layers (5900 a tile of 208 positions on 56x56x64): 64 channels, 56x56, 64 images, float 14.0 -> 13.8 us; 256 images,
+// bits, 28.4 -> 26.5 (a layer that has gone to bconv_mx_positions.cuh since: 21.8).  Setting the accumulators to minus the threshold beforehand (tcgen05.st) instead of
 // adding it to every value was slower (28.4 -> 36 us): the store waits for the other tile's matrix instructions.
 //
 // What a finisher warp needs for every tile, worked out once before its tile loop (divisions and
@@ -736,10 +738,11 @@ __device__ __forceinline__ void mx_epilogue_values(const MxFin &f, uint32_t tmem
 // re-quantised copy is the sign bits and the bit transpose of the bit-packed form; y + 0 makes -0.0 and NaN, which
 // quantize to 0 bits, positive (PTX: a NaN result has no sign).
 // Positions come as offsets of elements: multiplying pixels by the channels at each use took 36.9 us on the 56x56x64 block at 128
-// images, 34.5 now (40.6 with ballots and loads behind the wait); the plain float form, which has registers to spare, is
+// images, 34.5 then (40.6 with ballots and loads behind the wait; with positions on the lanes, as that block goes now, 25.0); the plain float form, which has registers to spare, is
 // faster with pixels (13.9 us against 14.4 on 56x56x64, 64 images).
 // With all three parts there are registers for 16 values ahead only, those of the next half chunk: 32 spilled into the loop, 78.5 us
-// on that block with everything, 57.5 now (58.0 with no value before the wait); shortcut and float output 51.3 and 49.3.
+// on that block with everything, 57.5 with 16 (58.0 with no value before the wait; 40.6 with positions on the lanes); shortcut and float
+// output 51.3 and 49.3.  What is left here of that form are 96 channels, 3x3, blocks of 128 and more, and grids that do not fill the SMs.
 template <bool RES, int AHEAD>
 __device__ __forceinline__ void mx_shortcut(const MxFin &f, const int32_t *offsets, float (&r)[AHEAD])
 {
@@ -1502,7 +1505,7 @@ MxLaunch mx_launch(const ConvGeom &g, const MxPlan &pl)
 }  // namespace
 
 // Float output of whole words of up to 96 channels, with a shortcut added or a re-quantised copy written, can go with positions on the
-// lanes (us: 56x56x64 at 128 images, copy alone 18.4 -> 15.8, shortcut and copy 34.3 -> 25.3, with the floats 57.6 -> 40.8); a
+// lanes (us: 56x56x64 at 128 images, copy alone 17.9 -> 15.4, shortcut and copy 34.1 -> 25.0, with the floats 57.7 -> 40.6); a
 // shortcut from 96 to 96 channels, 3x3, has no room beside the weights, as a rule.  Floats alone are bound by their stores and have one
 // form: 56x56x64 at 64 images 14.1, with positions on the lanes 15.1 (32 bytes of a pixel a store instead of 128).
 lce_status prepare_bconv_tensor(const ConvGeom &g, bool fused, PreparedLaunch *prepared)

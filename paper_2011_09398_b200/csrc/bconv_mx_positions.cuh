@@ -1,6 +1,6 @@
-// The tensor-core kernel for bit-packed output, and float output with a shortcut or a re-quantised copy, of few channels, with the roles of the operands exchanged: positions are the
-// M dimension (a TMEM lane each), channels the N dimension (32, 64 or 96 columns).  Part of bconv_mx.cu, whose loaders,
-// weight image, grid of positions and barriers it shares.
+// The tensor-core kernel for few output channels (bit-packed; float with a shortcut or a re-quantised copy) with the roles of the
+// operands exchanged: positions are the M dimension (a TMEM lane each), channels the N dimension (32, 64 or 96 columns).  Part of
+// bconv_mx.cu, whose loaders, weight image, grid of positions and barriers it shares, and whose mx_positions_pay says when it is taken.
 //
 // What bounds these layers with channels on the lanes is their finishers (56x56x64: 1620 clocks a tile of 208 positions, its
 // matrix instructions 950), who turn 32 channels x 32 positions of signs around with shuffles and all work on one of two
@@ -16,7 +16,9 @@
 //   * loops are not unrolled: 28 warps run three different ones, and what bounds them now is how much code that is (two pairs of matrix
 //     instructions written out three times: 23.1 us on 56x56x64, 256 images, once: 22.1);
 //   * thresholds lie in shared memory, one per column.
-// What bounds it now: loaders and issuers at about 1350 clocks a tile each (56x56x64), 10 and more clocks an instruction.
+// What bounds it now (56x56x64, 128 images, ncu): bits 46% of the issue slots, the tensor pipe 25% of the cycles; per issue 4.6 warps wait for
+// TMEM, shared or global memory, 2 for the next step of their own chain, 2 for instructions.  A tile takes 0.84 us (128 to 256 images: 12.5 ->
+// 21.8 us, 12 -> 23 tiles a CTA), its 36 matrix instructions 0.55.  With shortcut and copy 57% of the issue slots, 110 MB in 25.0 us.
 #pragma once
 
 namespace lce {
@@ -127,7 +129,7 @@ __device__ __forceinline__ bool mx_positions_finish(const MxPositionsParams &p, 
 // The shortcut comes through shared memory: a warp copies 32 channels of its 32 positions (4 KB) two steps ahead, 16 bytes a thread,
 // pieces of a row exchanged so that the quads' reads meet every bank once.  Loaded into registers before the accumulator is there
 // it is bound by what the L1 can have under way beside 200 KB of shared memory: 56x56x64, 128 images, shortcut and copy 31.8 us,
-// 25.3 now (34.3 with channels on the lanes; the shortcut's 103 MB take 15.7 at HBM rate).
+// 25.0 now (34.1 with channels on the lanes; the shortcut's 103 MB take 15.7 at HBM rate).
 template <bool RES, bool PACK, bool WRITE>
 __device__ __forceinline__ bool mx_positions_values(const MxPositionsParams &p, uint64_t *bars, const float *scales, uint8_t *staged, uint32_t tmem_base, int warp, int lane, int first_tile, int tile_step)
 {
