@@ -37,10 +37,13 @@ def test_bits_on_a_full_grid_have_positions_on_the_lanes(shape):
 def _kernels(call):
     call()  # set up
     torch.cuda.synchronize()
-    with profile(activities=[ProfilerActivity.CUDA]) as p:
-        call()
-        torch.cuda.synchronize()
-    names = [e.key for e in p.key_averages() if "bconv" in e.key]
+    for _ in range(3):  # a profile may come back empty
+        with profile(activities=[ProfilerActivity.CUDA]) as p:
+            call()
+            torch.cuda.synchronize()
+        names = [e.key for e in p.key_averages() if "bconv" in e.key]
+        if names:
+            break
     assert len(names) == 1, names
     return names[0]
 
